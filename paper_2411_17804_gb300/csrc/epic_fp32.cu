@@ -272,6 +272,25 @@ __device__ __forceinline__ void cp_async16_64(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 
+// Starts the copy of `bytes` voltages (2-byte aligned, as all voltages are)
+// to a 16-byte aligned shared buffer, kept at their source's offset in 16
+// bytes (staged_offset): the body goes by 16-byte cp.async whatever the
+// station's sample size, the at most 14 bytes at each end by 2-byte copies (a
+// station of 251 elements, 1,004 bytes a sample, 37 channels x 999 samples at
+// N = 64: 697.0 -> 657.9 us against 2-byte loads for the whole copy).
+__device__ __forceinline__ int staged_offset(const int8_t *src) { return (int)((uintptr_t)src & 15); }
+__device__ __forceinline__ void stage_volt(const int8_t *src, int bytes, unsigned char *buf, int tid, int nthreads) {
+    const int mis = staged_offset(src);
+    unsigned char *dst = buf + mis;
+    const int head = min(bytes, (16 - mis) & 15), body = (bytes - head) >> 4, tail = bytes - head - 16 * body;
+    for (int i = tid; i < body; i += nthreads) cp_async16_64(dst + head + 16 * i, src + head + 16 * i);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    if (tid < (head + tail) >> 1) {
+        const int o = 2 * tid < head ? 2 * tid : 2 * tid + 16 * body;
+        *reinterpret_cast<char2 *>(dst + o) = *reinterpret_cast<const char2 *>(src + o);
+    }
+}
+
 // Shared memory of the N = 64 kernel.  SP samples per phase (2 when the box
 // is at most 32 rows and shared memory allows, else 1); sample si of a phase
 // and pol p keep their H plane at si SO + p PO, SO = 8 (mod 16) too, so that
@@ -285,7 +304,7 @@ struct Epic64Smem {
     static constexpr int SO = (P * PO + 15) / 16 * 16 + 8;   // sample stride
     static constexpr int HB = SP * SO;                        // one of the two H buffers
     static constexpr size_t fixed = sizeof(float2) * (2 * (size_t)HB + 64 * (size_t)k64Xs);
-    __host__ __device__ static size_t vbuf(int ne) { return ((size_t)SP * P * ne * 2 + 15) / 16 * 16; }
+    __host__ __device__ static size_t vbuf(int ne) { return ((size_t)SP * P * ne * 2 + 31) / 16 * 16; }
     __host__ __device__ static size_t cbytes(int ncell) { return TS ? ((size_t)(ncell + 1) * 4 + 15) / 16 * 16 : 0; }
     __host__ __device__ static size_t bytes(int ne, int ncell, int nnz) {
         return fixed + 2 * vbuf(ne) + cbytes(ncell) + (TS ? (size_t)nnz * 16 : 0);
@@ -294,8 +313,8 @@ struct Epic64Smem {
 
 // Same arguments and outputs as epic_fp32_kernel<64, P> (nnz = the table's
 // entry count); PX / PY: the box spans at most 32 cells along x / y.  The
-// int8 voltages of the next phase are copied into shared memory (16-byte
-// cp.async when vec16) while the current one is imaged.
+// int8 voltages of the next phase are copied into shared memory while the
+// current one is imaged.
 //
 // Row tasks: warp w takes rows w and 31 - w (+ 32), so that the rows beyond a
 // box of fewer than 32 spread over the four schedulers.  SP = 2: group g
@@ -306,8 +325,7 @@ template <int P, bool PX, bool PY, int SP, bool TS>
 __global__ void __launch_bounds__(k64Threads, 1)
 epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long len, int box_w, int box_h,
               const int32_t *__restrict__ cstart_g, const int32_t *__restrict__ celem,
-              const float2 *__restrict__ cw, int nnz, float *__restrict__ out, int direct, int accumulate,
-              int vec16) {
+              const float2 *__restrict__ cw, int nnz, float *__restrict__ out, int direct, int accumulate) {
     constexpr int Q = (P == 2) ? 4 : 1;
     using S = Epic64Smem<P, PX, PY, SP, TS>;
     constexpr int PO = S::PO, SO = S::SO, HB = S::HB;
@@ -351,17 +369,8 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
     }
 
     auto load = [&](int ph, int b) {
-        const int bytes = min(SP, n - SP * ph) * vbytes;
-        const int8_t *src = volt + (size_t)(s0 + (long long)SP * ph) * vbytes;
-        unsigned char *dst = vs + (size_t)b * vstride;
-        if (vec16) {
-            for (int i = tid; i < bytes / 16; i += k64Threads) cp_async16_64(dst + 16 * i, src + 16 * i);
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
-        } else {
-            const char2 *s2 = reinterpret_cast<const char2 *>(src);
-            char2 *d2 = reinterpret_cast<char2 *>(dst);
-            for (int i = tid; i < bytes / 2; i += k64Threads) d2[i] = s2[i];
-        }
+        stage_volt(volt + (size_t)(s0 + (long long)SP * ph) * vbytes, min(SP, n - SP * ph) * vbytes,
+                   vs + (size_t)b * vstride, tid, k64Threads);
     };
 
     float acc[8][Q];
@@ -404,7 +413,8 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
         if (it + 1 < nph) load(it + 1, (it + 1) & 1);
         if (it < nph) {
             // row pass of phase it
-            const unsigned char *V = vs + (size_t)(it & 1) * vstride;
+            const unsigned char *V = vs + (size_t)(it & 1) * vstride +
+                                     staged_offset(volt + (size_t)(s0 + (long long)SP * it) * vbytes);
             float2 *H = Hs + (size_t)(it & 1) * HB;
             const int ns = min(SP, n - SP * it);
 #pragma unroll
@@ -535,29 +545,382 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
                 }
             }
         }
-        if (vec16) asm volatile("cp.async.wait_all;\n" ::: "memory");
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
     }
     flush(cur_c, seg);
 }
 
-// img[c] = (accumulate ? img[c] : 0) + sum of the partials of channel c, in
-// CTA order.  CTA b covers samples [b*len, (b+1)*len) of the flat index.
-__global__ void epic_reduce_kernel(const float *__restrict__ part, float *__restrict__ img, int C,
-                                   int T, long long len, int plane, int accumulate) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)C * plane) return;
-    const int c = (int)(i / plane);
-    const int off = (int)(i % plane);
+// ------------------------------------------------------- N = 16 and N = 32
+// Lines in registers as at N = 64, by groups of 4 lanes: with E = N / 4 lane t
+// holds points t + 4 m (m < E) and k = k1 + E k2, so it takes the E-point DFT
+// over m, multiplies output k1 by wN^(t k1), and after one exchange through
+// the group's scratch lane j takes the 4-point DFTs over t of k1 = j + 4 u,
+// ending with X[j + 4 u + E k2].  A phase takes 128 / N samples: 128 groups
+// hold the phase's columns, one (column, sample) each, and the box rows of its
+// (sample, pol) fields are dealt to the same groups.  As at N = 64 the row
+// pass of phase i runs beside the column pass of phase i - 1 (H and the staged
+// voltages double-buffered): one block barrier per phase.  A phase never
+// straddles two channels; at a channel's end the sample slots' sums are added
+// in slot order in shared memory.
+//
+// These grids are latency-bound: one CTA per SM has a few samples of a short
+// cadence, so the time is the chain gather -> row -> column of a phase times
+// the number of phases.  The kernel before this one (below; one thread per
+// whole row and column, two samples per phase) left all but 32 threads idle in
+// its passes and re-walked 32 cells serially per thread.  One 64-element
+// station, one pol, 1024 samples at N = 32: 100.3 -> 18.0 us a call, with the
+// reduction below.
+//
+// Shared layouts: H[plane][y][(k + 4 y) & (N - 1)]: a half-warp writes rows
+// y .. y + 3 (4 adjacent values each) and reads rows t + 4 m of 4 adjacent
+// columns, 16 distinct 8-byte banks both ways; the exchange keeps value k1 of
+// lane t at 4 k1 + ((t + k1) & 3), groups N + 4 float2 apart, conflict-free
+// for the writes (one k1) and the reads (one t).
+constexpr int kSmThreads = 512;                  // 128 groups of 4 lanes
+
+template <int N, int P, bool TS>
+struct EpicSmallSmem {
+    static constexpr int SP = 128 / N;                       // samples per phase
+    static constexpr int XS = N + 4;                         // exchange scratch of a group (float2)
+    static constexpr int HB = SP * P * N * N;                // one of the two H buffers (float2)
+    static constexpr size_t fixed = sizeof(float2) * (2 * (size_t)HB + 128 * (size_t)XS) +
+                                    sizeof(float) * (size_t)(P == 2 ? 4 : 1) * N * N;
+    // staged voltages of a phase, at their source's offset in 16 bytes
+    __host__ __device__ static size_t vbuf(int ne) { return ((size_t)SP * P * ne * 2 + 31) / 16 * 16; }
+    __host__ __device__ static size_t cbytes(int ncell) { return TS ? ((size_t)(ncell + 1) * 4 + 15) / 16 * 16 : 0; }
+    __host__ __device__ static size_t bytes(int ne, int ncell, int nnz) {
+        return fixed + 2 * vbuf(ne) + cbytes(ncell) + (TS ? (size_t)nnz * 16 : 0);
+    }
+};
+
+// E-point DFT of a line's points in one lane; half: the second half is zero.
+template <int E>
+__device__ __forceinline__ void dft_small(float2 (&a)[E], bool half) {
+    if constexpr (E == 8) {
+        if (half) dft8_first4(a);
+        else hai_fft512::dft8(a);
+    } else {
+        hai_fft512::dft4(a[0], a[1], a[2], a[3]);
+    }
+}
+
+// Same arguments and outputs as epic64_kernel.
+template <int N, int P, bool TS>
+__global__ void __launch_bounds__(kSmThreads, 1)
+epic_small_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long len, int box_w, int box_h,
+                  const int32_t *__restrict__ cstart_g, const int32_t *__restrict__ celem,
+                  const float2 *__restrict__ cw, int nnz, float *__restrict__ out, int direct, int accumulate) {
+    constexpr int Q = (P == 2) ? 4 : 1, E = N / 4, U = E / 4, NN = N * N;
+    using S = EpicSmallSmem<N, P, TS>;
+    constexpr int SP = S::SP, XS = S::XS, HB = S::HB;
+    extern __shared__ __align__(16) unsigned char smem[];
+    float2 *Hs = reinterpret_cast<float2 *>(smem);                        // [2][SP][P][N][N]
+    float2 *xs = Hs + 2 * HB + (threadIdx.x >> 2) * XS;                   // this group's scratch
+    float *fimg = reinterpret_cast<float *>(Hs + 2 * HB + 128 * XS);      // [Q][N][N], flush
+    unsigned char *vs = smem + S::fixed;                                  // [2][vstride]
+    const int vbytes = P * ne * 2;                                        // one sample
+    const int vstride = (int)S::vbuf(ne);
+    const int ncell = box_w * box_h;
+    int32_t *cs_s = reinterpret_cast<int32_t *>(vs + 2 * (size_t)vstride);
+    int4 *ent_s = reinterpret_cast<int4 *>(reinterpret_cast<unsigned char *>(cs_s) + S::cbytes(ncell));
+
+    const int tid = threadIdx.x, t = tid & 3, g = tid >> 2;
+    const long long total = (long long)C * T;
+    const long long s0 = (long long)blockIdx.x * len;
+    const long long s1 = min(total, s0 + len);
+    if (s0 >= s1) return;
+    // the range touches at most two channels: phases of the first, then of the second
+    const int c0 = (int)(s0 / T);
+    const long long sb = min(s1, (long long)(c0 + 1) * T);
+    const int n0 = (int)(sb - s0), n1 = (int)(s1 - sb);
+    const int nph0 = (n0 + SP - 1) / SP, nph = nph0 + (n1 + SP - 1) / SP;
+    auto phase = [&](int ph, long long &start) {                          // first sample and count of a phase
+        if (ph < nph0) {
+            start = s0 + (long long)SP * ph;
+            return min(SP, n0 - SP * ph);
+        }
+        start = sb + (long long)SP * (ph - nph0);
+        return min(SP, n1 - SP * (ph - nph0));
+    };
+
+    if (TS) {
+        for (int i = tid; i <= ncell; i += kSmThreads) cs_s[i] = __ldg(cstart_g + i);
+        for (int i = tid; i < nnz; i += kSmThreads) {
+            const float2 w = __ldg(cw + i);
+            ent_s[i] = make_int4(__ldg(celem + i), __float_as_int(w.x), __float_as_int(w.y), 0);
+        }
+    }
+    const int32_t *cstart = TS ? cs_s : cstart_g;
+
+    float2 tw[E];                                                         // wN^(t k), k < E
+#pragma unroll
+    for (int k = 1; k < E; k++) {
+        const int m = t * k * (kTwN / N);                                 // < 64
+        const float2 v = c_tw[m & 31];
+        tw[k] = m < 32 ? v : make_float2(-v.x, -v.y);
+    }
+
+    auto load = [&](int ph, int b) {
+        long long start;
+        const int bytes = phase(ph, start) * vbytes;
+        stage_volt(volt + (size_t)start * vbytes, bytes, vs + (size_t)b * vstride, tid, kSmThreads);
+    };
+
+    float acc[E][Q];
+#pragma unroll
+    for (int k = 0; k < E; k++)
+#pragma unroll
+        for (int q = 0; q < Q; q++) acc[k][q] = 0.f;
+    const int col = g & (N - 1), slot = g / N;           // column pass: column and sample slot of this group
+    auto flush = [&](int c, int sgm) {
+        for (int sl = 0; sl < SP; sl++) {
+            if (slot == sl) {
+                const int lx = (col + N / 2) & (N - 1);
+#pragma unroll
+                for (int u = 0; u < U; u++)
+#pragma unroll
+                    for (int k2 = 0; k2 < 4; k2++) {
+                        const int pix = ((t + 4 * u + E * k2 + N / 2) & (N - 1)) * N + lx;
+#pragma unroll
+                        for (int q = 0; q < Q; q++) {
+                            float *f = fimg + q * NN + pix;
+                            *f = sl ? *f + acc[4 * u + k2][q] : acc[4 * u + k2][q];
+                            acc[4 * u + k2][q] = 0.f;
+                        }
+                    }
+            }
+            __syncthreads();
+        }
+        float *dst = direct ? out + (size_t)c * Q * NN : out + ((size_t)blockIdx.x * 2 + sgm) * Q * NN;
+        for (int i = tid; i < Q * NN; i += kSmThreads) dst[i] = direct && accumulate ? dst[i] + fimg[i] : fimg[i];
+        __syncthreads();
+    };
+    // second half of a line: a[k1] (twiddled) of lane t in, a[4 u + k2] = X[t + 4 u + E k2] out
+    auto finish = [&](float2 (&a)[E]) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < E; k++) xs[4 * k + ((t + k) & 3)] = a[k];
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) a[4 * u + i] = xs[4 * (t + 4 * u) + ((i + t) & 3)];
+            hai_fft512::dft4(a[4 * u], a[4 * u + 1], a[4 * u + 2], a[4 * u + 3]);
+        }
+    };
+
+    load(0, 0);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    for (int it = 0; it <= nph; it++) {
+        if (it + 1 < nph) load(it + 1, (it + 1) & 1);
+        if (it < nph) {
+            // row pass of phase it: task = (sample, pol, box row), rows adjacent
+            long long start;
+            const int ns = phase(it, start);
+            const unsigned char *V = vs + (size_t)(it & 1) * vstride + staged_offset(volt + (size_t)start * vbytes);
+            float2 *H = Hs + (size_t)(it & 1) * HB;
+            const int ntask = ns * P * box_h;
+            for (int base = 0; base < ntask; base += 128) {               // CTA-uniform
+                const int task = base + g;
+                const bool live = task < ntask;
+                if (!__any_sync(0xffffffffu, live)) continue;             // warp-uniform
+                const int f = live ? task / box_h : 0, y = task - f * box_h;
+                float2 a[E];
+#pragma unroll
+                for (int m = 0; m < E; m++) a[m] = make_float2(0.f, 0.f);
+                if (live) {
+                    const char2 *Ev = reinterpret_cast<const char2 *>(V) + (size_t)f * ne;
+                    int cb[E], ce[E];                                     // the cells' entry ranges, loaded first
+#pragma unroll
+                    for (int m = 0; m < E; m++) {
+                        const int x = t + 4 * m;
+                        cb[m] = ce[m] = 0;
+                        if (x < box_w) {
+                            cb[m] = cstart[y * box_w + x];
+                            ce[m] = cstart[y * box_w + x + 1];
+                        }
+                    }
+#pragma unroll
+                    for (int m = 0; m < E; m++)
+                        for (int i = cb[m]; i < ce[m]; i++) {
+                            int el;
+                            float2 wv;                                    // conj(W~)
+                            if (TS) {
+                                const int4 d = ent_s[i];
+                                el = d.x;
+                                wv = make_float2(__int_as_float(d.y), __int_as_float(d.z));
+                            } else {
+                                el = __ldg(celem + i);
+                                wv = __ldg(cw + i);
+                            }
+                            const char2 v = Ev[el];
+                            const float er = (float)v.x, ei = (float)v.y;
+                            a[m].x = fmaf(wv.x, er, fmaf(-wv.y, ei, a[m].x));
+                            a[m].y = fmaf(wv.x, ei, fmaf(wv.y, er, a[m].y));
+                        }
+                }
+                dft_small<E>(a, box_w <= N / 2);
+#pragma unroll
+                for (int k = 1; k < E; k++) a[k] = hai_fft512::cmul(a[k], tw[k]);
+                finish(a);
+                if (live) {
+                    float2 *row = H + ((size_t)f * N + y) * N;
+#pragma unroll
+                    for (int u = 0; u < U; u++)
+#pragma unroll
+                        for (int k2 = 0; k2 < 4; k2++) row[(t + 4 * u + E * k2 + 4 * y) & (N - 1)] = a[4 * u + k2];
+                }
+            }
+        }
+        if (it >= 1) {
+            // column pass of phase it - 1: sample `slot`, column `col`
+            if (it - 1 == nph0) flush(c0, 0);                             // the second channel begins
+            long long start;
+            const int ns = phase(it - 1, start);
+            if (slot < ns) {                                              // warp-uniform: a warp holds 8 columns of a slot
+                const float2 *H = Hs + (size_t)((it - 1) & 1) * HB + (size_t)slot * P * NN;
+                float2 f[P][E];
+#pragma unroll
+                for (int p = 0; p < P; p++) {
+#pragma unroll
+                    for (int m = 0; m < E; m++) {
+                        const int y = t + 4 * m;
+                        f[p][m] = y < box_h ? H[(size_t)p * NN + y * N + ((col + 4 * y) & (N - 1))] : make_float2(0.f, 0.f);
+                    }
+                    dft_small<E>(f[p], box_h <= N / 2);
+#pragma unroll
+                    for (int k = 1; k < E; k++) f[p][k] = hai_fft512::cmul(f[p][k], tw[k]);
+                }
+#pragma unroll
+                for (int p = 0; p < P; p++) finish(f[p]);
+#pragma unroll
+                for (int k = 0; k < E; k++) {
+                    const float2 fx = f[0][k];
+                    acc[k][0] = fmaf(fx.x, fx.x, fmaf(fx.y, fx.y, acc[k][0]));
+                    if (P == 2) {
+                        const float2 fy = f[P - 1][k];
+                        acc[k][Q > 1 ? 1 : 0] = fmaf(fy.x, fy.x, fmaf(fy.y, fy.y, acc[k][Q > 1 ? 1 : 0]));
+                        acc[k][Q > 2 ? 2 : 0] = fmaf(fx.x, fy.x, fmaf(fx.y, fy.y, acc[k][Q > 2 ? 2 : 0]));
+                        acc[k][Q > 3 ? 3 : 0] = fmaf(fx.y, fy.x, fmaf(-fx.x, fy.y, acc[k][Q > 3 ? 3 : 0]));
+                    }
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
+    }
+    flush(n1 > 0 ? c0 + 1 : c0, n1 > 0 ? 1 : 0);
+}
+
+// img[c] = (accumulate ? img[c] : 0) + sum of the partials of channel c.  CTA
+// b covers samples [b*len, (b+1)*len) of the flat index, so only a channel's
+// first CTA can hold it in its second slot.  Thread (x, y) of a block adds the
+// partials b0 + y, b0 + y + G, ... of V adjacent pixels, and row y = 0 adds
+// the G sums in order (deterministic).  A long cadence of few channels has up
+// to one partial per SM and channel: with one thread per pixel walking them all
+// the loads ran one after another on four SMs, and took longer than the
+// imaging they followed; a 64-channel cadence (3 or 4 partials a channel) gains
+// from the wider accesses alone (tensor cores at 64^2: 1093.8 -> 1085.9 us).
+template <int V>
+__global__ void __launch_bounds__(1024) epic_reduce_kernel(const float *__restrict__ part, float *__restrict__ img,
+                                                           int T, long long len, int plane, int accumulate) {
+    extern __shared__ float red[];                          // [G][blockDim.x][V]
+    const int c = blockIdx.y, G = blockDim.y;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int b0 = (int)(((long long)c * T) / len);
     const int b1 = (int)(((long long)(c + 1) * T - 1) / len);
-    float s = 0.f;
-    for (int b = b0; b <= b1; b++) {
-        const int first = (int)(((long long)b * len) / T);
-        const int sgm = c - first;
-        s += part[((size_t)b * 2 + sgm) * plane + off];
+    const int slot0 = c - (int)(((long long)b0 * len) / T);
+    float s[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) s[v] = 0.f;
+    if (i < plane) {
+#pragma unroll 4
+        for (int b = b0 + threadIdx.y; b <= b1; b += G) {
+            const float *src = part + ((size_t)b * 2 + (b == b0 ? slot0 : 0)) * plane + i;
+            if constexpr (V == 4) {
+                const float4 x = *reinterpret_cast<const float4 *>(src);
+                s[0] += x.x;
+                s[1] += x.y;
+                s[2] += x.z;
+                s[3] += x.w;
+            } else {
+                s[0] += *src;
+            }
+        }
     }
-    img[i] = accumulate ? img[i] + s : s;
+    if (G > 1) {
+#pragma unroll
+        for (int v = 0; v < V; v++) red[(threadIdx.y * blockDim.x + threadIdx.x) * V + v] = s[v];
+        __syncthreads();
+        if (threadIdx.y > 0) return;
+        for (int y = 1; y < G; y++)
+#pragma unroll
+            for (int v = 0; v < V; v++) s[v] += red[(y * blockDim.x + threadIdx.x) * V + v];
+    }
+    if (i >= plane) return;
+    float *o = img + (size_t)c * plane + i;
+    if constexpr (V == 4) {
+        float4 x = accumulate ? *reinterpret_cast<const float4 *>(o) : make_float4(0.f, 0.f, 0.f, 0.f);
+        x.x += s[0];
+        x.y += s[1];
+        x.z += s[2];
+        x.w += s[3];
+        *reinterpret_cast<float4 *>(o) = x;
+    } else {
+        *o = accumulate ? *o + s[0] : s[0];
+    }
+}
+
+// Four pixels a thread when the buffers allow 16-byte accesses (planes are
+// multiples of 256 floats); G partials side by side while a channel has four
+// or more for each and the pixels alone leave SMs without threads.
+hai_status reduce_launch(const float *part, float *img, const EpicSplit &sp, int C, int T, int plane, int accumulate,
+                         int sms, cudaStream_t st) {
+    const bool vec = (((uintptr_t)part | (uintptr_t)img) & 15) == 0;
+    const int V = vec ? 4 : 1;
+    const long long work = (long long)C * (plane / V), nb = T / sp.len + 2;
+    int G = 1;
+    while (G < 32 && 4 * G <= nb && work * G < 1024ll * sms) G *= 2;
+    const int X = G < 8 ? 256 / G : 32;
+    const dim3 grid((plane / V + X - 1) / X, C), block(X, G);
+    const size_t smem = G > 1 ? sizeof(float) * V * X * G : 0;
+    if (vec)
+        epic_reduce_kernel<4><<<grid, block, smem, st>>>(part, img, T, sp.len, plane, accumulate);
+    else
+        epic_reduce_kernel<1><<<grid, block, smem, st>>>(part, img, T, sp.len, plane, accumulate);
+    HAI_CUDA_TRY(cudaGetLastError());
+    return HAI_OK;
+}
+
+// The N = 16, 32 kernel, the gather table in shared memory if it fits;
+// *launched = false if even the voltages do not fit.
+template <int N, int P, bool TS>
+hai_status try_small(const int8_t *volt, int C, int T, int ne, const EpicSplit &sp, int box_w, int box_h,
+                     const int32_t *cstart, const int32_t *celem, const float2 *cw, int nnz, float *dst,
+                     int accumulate, int smem_optin, cudaStream_t st, bool *launched) {
+    const size_t smem = EpicSmallSmem<N, P, TS>::bytes(ne, box_w * box_h, nnz);
+    if (*launched || smem > (size_t)smem_optin) return HAI_OK;
+    auto kern = epic_small_kernel<N, P, TS>;
+    HAI_CUDA_TRY(hai_allow_dyn_smem(kern, smem_optin));
+    kern<<<sp.n_cta, kSmThreads, smem, st>>>(volt, C, T, ne, sp.len, box_w, box_h, cstart, celem, cw, nnz, dst,
+                                             sp.direct, accumulate);
+    HAI_CUDA_TRY(cudaGetLastError());
+    *launched = true;
+    return HAI_OK;
+}
+
+template <int N, int P>
+hai_status launch_small(const int8_t *volt, int C, int T, int ne, const EpicSplit &sp, int box_w, int box_h,
+                        const int32_t *cstart, const int32_t *celem, const float2 *cw, int nnz, float *dst,
+                        int accumulate, int smem_optin, cudaStream_t st, bool *launched) {
+    *launched = false;
+    const hai_status s = try_small<N, P, true>(volt, C, T, ne, sp, box_w, box_h, cstart, celem, cw, nnz, dst,
+                                               accumulate, smem_optin, st, launched);
+    if (s != HAI_OK) return s;
+    return try_small<N, P, false>(volt, C, T, ne, sp, box_w, box_h, cstart, celem, cw, nnz, dst, accumulate,
+                                  smem_optin, st, launched);
 }
 
 // The N = 64 kernel in the form the box and the shared memory allow:
@@ -567,9 +930,8 @@ template <int P, bool PX, bool PY, int SP, bool TS>
 void launch64_form(const int8_t *volt, int C, int T, int ne, const EpicSplit &sp, int box_w, int box_h,
                    const int32_t *cstart, const int32_t *celem, const float2 *cw, int nnz, float *dst,
                    int accumulate, size_t smem, cudaStream_t st) {
-    const int vec16 = ((((uintptr_t)volt) & 15) == 0 && ((size_t)P * ne * 2) % 16 == 0) ? 1 : 0;
     epic64_kernel<P, PX, PY, SP, TS><<<sp.n_cta, k64Threads, smem, st>>>(
-        volt, C, T, ne, sp.len, box_w, box_h, cstart, celem, cw, nnz, dst, sp.direct, accumulate, vec16);
+        volt, C, T, ne, sp.len, box_w, box_h, cstart, celem, cw, nnz, dst, sp.direct, accumulate);
 }
 
 template <int P, bool PX, bool PY, int SP, bool TS>
@@ -619,16 +981,6 @@ hai_status launch64_box(const int8_t *volt, int C, int T, int ne, const EpicSpli
 }
 
 template <int P>
-size_t epic64_bytes(int ne, int box_w, int box_h) {
-    // the smallest form (one sample per phase, table in global memory)
-    const bool px = box_w <= 32, py = box_h <= 32;
-    if (px && py) return Epic64Smem<P, true, true, 1, false>::bytes(ne, 0, 0);
-    if (px) return Epic64Smem<P, true, false, 1, false>::bytes(ne, 0, 0);
-    if (py) return Epic64Smem<P, false, true, 1, false>::bytes(ne, 0, 0);
-    return Epic64Smem<P, false, false, 1, false>::bytes(ne, 0, 0);
-}
-
-template <int P>
 hai_status launch64(const int8_t *volt, int C, int T, int ne, const EpicSplit &sp, int box_w, int box_h,
                     const int32_t *cstart, const int32_t *celem, const float2 *cw, int nnz, float *dst,
                     int accumulate, int smem_optin, cudaStream_t st, bool *launched) {
@@ -649,41 +1001,35 @@ hai_status launch64(const int8_t *volt, int C, int T, int ne, const EpicSplit &s
 template <int N, int P>
 hai_status launch_n(const hai_layout *L, const int8_t *volt, int C, int T, float *img, int accumulate,
                     cudaStream_t st) {
-    if (N == 64) {
-        const EpicSplit sp = epic_make_split(C, T, epic_fp32_target_ctas(L->ctx, N));
-        if (!sp.direct && (size_t)sp.n_cta * 2 > L->partial_slots)
-            return hai_fail(HAI_ERR_INVALID_ARG, "epic fp32: partial buffer too small");
-        float *dst = sp.direct ? img : L->d_partials;
-        bool launched = false;
-        if (epic64_bytes<P>(L->n_elem, L->box_w, L->box_h) <= (size_t)L->ctx->smem_optin) {
-            const int pidx = prof_begin(L->ctx, st);
-            hai_status s = launch64<P>(volt, C, T, L->n_elem, sp, L->box_w, L->box_h, L->d_cell_start,
-                                       L->d_entry_elem, L->d_entry_w, L->nnz, dst, accumulate, L->ctx->smem_optin,
-                                       st, &launched);
-            if (s != HAI_OK) return s;
-            prof_end(L->ctx, pidx, st);
-            prof_count(L->ctx, 1);
-            if (!sp.direct) return epic_reduce_launch(L, sp, C, T, img, accumulate, st);
-            return HAI_OK;
-        }
-    }
-    const size_t smem = sizeof(float2) * EpicSmem<N, P>::kBuf +
-                        ((size_t)kSamples * P * L->n_elem * 2 + 15) / 16 * 16;
-    if (smem > (size_t)L->ctx->smem_optin)
-        return hai_fail(HAI_ERR_UNSUPPORTED, "epic fp32: shared memory need exceeds the device limit");
-    auto kern = epic_fp32_kernel<N, P>;
-    HAI_CUDA_TRY(hai_allow_dyn_smem(kern, L->ctx->smem_optin));
+    const int optin = L->ctx->smem_optin;
     const EpicSplit sp = epic_make_split(C, T, epic_fp32_target_ctas(L->ctx, N));
     if (!sp.direct && (size_t)sp.n_cta * 2 > L->partial_slots)
         return hai_fail(HAI_ERR_INVALID_ARG, "epic fp32: partial buffer too small");
     float *dst = sp.direct ? img : L->d_partials;
+    bool launched = false;
     const int pidx = prof_begin(L->ctx, st);
-    kern<<<sp.n_cta, kThreads, smem, st>>>(volt, C, T, L->n_elem, sp.len, L->box_w, L->box_h,
-                                           L->d_cell_start, L->d_entry_elem, L->d_entry_w, dst,
-                                           sp.direct, accumulate);
+    hai_status s = HAI_OK;
+    if constexpr (N == 64)
+        s = launch64<P>(volt, C, T, L->n_elem, sp, L->box_w, L->box_h, L->d_cell_start, L->d_entry_elem,
+                        L->d_entry_w, L->nnz, dst, accumulate, optin, st, &launched);
+    else
+        s = launch_small<N, P>(volt, C, T, L->n_elem, sp, L->box_w, L->box_h, L->d_cell_start, L->d_entry_elem,
+                               L->d_entry_w, L->nnz, dst, accumulate, optin, st, &launched);
+    if (s != HAI_OK) return s;
+    if (!launched) {
+        const size_t smem = sizeof(float2) * EpicSmem<N, P>::kBuf +
+                            ((size_t)kSamples * P * L->n_elem * 2 + 15) / 16 * 16;
+        if (smem > (size_t)optin)
+            return hai_fail(HAI_ERR_UNSUPPORTED, "epic fp32: shared memory need exceeds the device limit");
+        auto kern = epic_fp32_kernel<N, P>;
+        HAI_CUDA_TRY(hai_allow_dyn_smem(kern, optin));
+        kern<<<sp.n_cta, kThreads, smem, st>>>(volt, C, T, L->n_elem, sp.len, L->box_w, L->box_h,
+                                               L->d_cell_start, L->d_entry_elem, L->d_entry_w, dst,
+                                               sp.direct, accumulate);
+        HAI_CUDA_TRY(cudaGetLastError());
+    }
     prof_end(L->ctx, pidx, st);
     prof_count(L->ctx, 1);
-    HAI_CUDA_TRY(cudaGetLastError());
     if (!sp.direct) return epic_reduce_launch(L, sp, C, T, img, accumulate, st);
     return HAI_OK;
 }
@@ -704,14 +1050,10 @@ int epic_fp32_target_ctas(const hai_ctx *ctx, int) { return ctx->num_sms; }
 
 hai_status epic_reduce_launch(const hai_layout *L, const EpicSplit &sp, int C, int T, float *img,
                               int accumulate, cudaStream_t st) {
-    const int Q = (L->n_pol == 2) ? 4 : 1;
-    const int plane = Q * L->grid_n * L->grid_n;
-    const long long n = (long long)C * plane;
-    const int threads = 256;
-    epic_reduce_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(
-        L->d_partials, img, C, T, sp.len, plane, accumulate);
+    const int plane = (L->n_pol == 2 ? 4 : 1) * L->grid_n * L->grid_n;
+    const hai_status s = reduce_launch(L->d_partials, img, sp, C, T, plane, accumulate, L->ctx->num_sms, st);
+    if (s != HAI_OK) return s;
     prof_count(L->ctx, 1);
-    HAI_CUDA_TRY(cudaGetLastError());
     return HAI_OK;
 }
 
@@ -791,11 +1133,14 @@ hai_status launch_static(float *scratch, int ne, int box_w, int box_h, int ncell
     const float2 *cw = reinterpret_cast<const float2 *>(cstart + static_taps_word(ncell, nnz));
     float *partials = scratch + kStaticTableWords;
     bool launched = false;
-    if (N == 64) {
-        hai_status s = launch64<P>(volt, C, T, ne, sp, box_w, box_h, cstart, celem, cw, nnz,
-                                   sp.direct ? img : partials, accumulate, smem_optin, st, &launched);
-        if (s != HAI_OK) return s;
-    }
+    hai_status s = HAI_OK;
+    if constexpr (N == 64)
+        s = launch64<P>(volt, C, T, ne, sp, box_w, box_h, cstart, celem, cw, nnz, sp.direct ? img : partials,
+                        accumulate, smem_optin, st, &launched);
+    else
+        s = launch_small<N, P>(volt, C, T, ne, sp, box_w, box_h, cstart, celem, cw, nnz, sp.direct ? img : partials,
+                               accumulate, smem_optin, st, &launched);
+    if (s != HAI_OK) return s;
     if (!launched) {
         const size_t smem = sizeof(float2) * EpicSmem<N, P>::kBuf + ((size_t)kSamples * P * ne * 2 + 15) / 16 * 16;
         if (smem > (size_t)smem_optin)
@@ -807,14 +1152,7 @@ hai_status launch_static(float *scratch, int ne, int box_w, int box_h, int ncell
                                                sp.direct ? img : partials, sp.direct, accumulate);
         HAI_CUDA_TRY(cudaGetLastError());
     }
-    if (!sp.direct) {
-        const int Q = (P == 2) ? 4 : 1;
-        const int plane = Q * N * N;
-        const long long n = (long long)C * plane;
-        epic_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(partials, img, C, T, sp.len, plane,
-                                                                          accumulate);
-        HAI_CUDA_TRY(cudaGetLastError());
-    }
+    if (!sp.direct) return reduce_launch(partials, img, sp, C, T, (P == 2 ? 4 : 1) * N * N, accumulate, sms, st);
     return HAI_OK;
 }
 
