@@ -25,14 +25,15 @@
 // tiles (<= 112 x 112 cells) of the window of uv cells that on-grid pairs
 // touch, one CTA per (image, grid, tile) with the pairs binned to each tile on
 // the host, and writes its cells with the (-1)^(u+v) checkerboard that puts
-// the phase centre at pixel (N/2, N/2).  The FFTs read their twiddles from
-// a shared-memory table.
+// the phase centre at pixel (N/2, N/2).  The FFTs hold their lines in registers
+// (fft_line.cuh).
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
 #include <vector>
 
+#include "fft_line.cuh"
 #include "hai_internal.h"
 
 namespace {
@@ -149,99 +150,98 @@ __global__ void __launch_bounds__(kThreads) station_grid_kernel(
     }
 }
 
-// Twiddles exp(+2 pi i k / n), k < n / 2, into shared memory: sincospif of
-// 2k / n, the same argument (exact in FP32 for power-of-two n) as pos / half
-// of the butterfly that uses entry k.
-__device__ __forceinline__ void load_twiddles(float2 *tw, int n) {
-    for (int k = threadIdx.x; k < n / 2; k += blockDim.x) {
-        float s, c;
-        sincospif((float)(2 * k) / (float)n, &s, &c);
-        tw[k] = make_float2(c, s);
-    }
-}
+// Row pass, in place on a plane pair (re plane, im plane): lines in registers
+// (fft_line.cuh), 256 / L rows per CTA.  The exchange keeps value k1 of lane t
+// at (L + 1) k1 + t, lines 8 (mod 16) float2 apart at L = 8 and 4 (mod 16) at
+// L = 4: conflict-free both ways.  Global accesses are runs of L floats, whole
+// sectors.  The bound is HBM: every plane is read and written once (1.07 GB on
+// the hierarchical cadence's 512 images at 256^2).  The radix-2 form it
+// replaces made log2 N passes over shared memory and took 604 us there;
+// now 169 us (6.3 TB/s).
+constexpr int kFftThreads = 256;
 
-// In-place radix-2 FFT (exponent +) of n points held in bit-reversed order at
-// x[0], x[stride], ... by one warp; tw as load_twiddles wrote it.
-__device__ void warp_fft(float2 *x, int stride, int n, int log2n, const float2 *tw, int lane) {
-    for (int lh = 0; lh < log2n; lh++) {
-        const int half = 1 << lh, tshift = log2n - 1 - lh;       // twiddle of pos: tw[pos * n / (2 half)]
-        for (int b = lane; b < n / 2; b += 32) {
-            const int pos = b & (half - 1);
-            const int i0 = ((b - pos) << 1) + pos, i1 = i0 + half;
-            const float2 a = x[i0 * stride];
-            const float2 t = cmulf(x[i1 * stride], tw[pos << tshift]);
-            x[i0 * stride] = make_float2(a.x + t.x, a.y + t.y);
-            x[i1 * stride] = make_float2(a.x - t.x, a.y - t.y);
-        }
-        __syncwarp();
-    }
-}
+template <int N>
+struct RowSmem {
+    static constexpr int L = hai_fft::Line<N>::L, E = hai_fft::Line<N>::E;
+    static constexpr int XS = (E * (L + 1) + 15) / 16 * 16 + (L == 8 ? 8 : L == 4 ? 4 : 0);
+};
 
-// Row pass: one warp per row of a plane pair (re plane, im plane).
-__global__ void __launch_bounds__(kThreads) fft_rows_kernel(float *__restrict__ img, int N, int log2n) {
-    extern __shared__ float2 rows[];   // [16][N], then the N / 2 twiddles
-    float2 *tw = rows + (size_t)(kThreads / 32) * N;
-    load_twiddles(tw, N);
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+template <int N>
+__global__ void __launch_bounds__(kFftThreads) fft_rows_kernel(float *__restrict__ img) {
+    constexpr int L = hai_fft::Line<N>::L, E = hai_fft::Line<N>::E, XS = RowSmem<N>::XS, W = kFftThreads / L;
+    __shared__ float2 tw[N], xbuf[W * XS];
+    hai_fft::fill_twiddles<N>(tw);
+    const int t = threadIdx.x % L, w = threadIdx.x / L;
     const int pair = blockIdx.x;       // image * 2 + h
-    const int y = blockIdx.y * (kThreads / 32) + warp;
-    if (y >= N) return;
-    float *pre = img + ((size_t)(pair >> 1) * 4 + 2 * (pair & 1)) * N * N + (size_t)y * N;
+    const int y = blockIdx.y * W + w;
+    const bool live = y < N;
+    float *pre = img + ((size_t)pair * 2 * N + (live ? y : 0)) * N;
     float *pim = pre + (size_t)N * N;
-    float2 *x = rows + (size_t)warp * N;
-    // lane takes the N / 32 consecutive points j = E lane + k: their
-    // bit-reversed slots for one k are a permutation of 32 adjacent entries,
-    // so the stores are free of bank conflicts (j = lane + 32 k would put the
-    // lanes 64 bytes apart)
-    const int E = N / 32;
-    if (E >= 4) {
-        for (int k = 0; k < E; k += 4) {
-            const int j = E * lane + k;
-            const float4 r = *reinterpret_cast<const float4 *>(pre + j), m = *reinterpret_cast<const float4 *>(pim + j);
-            x[__brev(j) >> (32 - log2n)] = make_float2(r.x, m.x);
-            x[__brev(j + 1) >> (32 - log2n)] = make_float2(r.y, m.y);
-            x[__brev(j + 2) >> (32 - log2n)] = make_float2(r.z, m.z);
-            x[__brev(j + 3) >> (32 - log2n)] = make_float2(r.w, m.w);
-        }
-    } else {
-        for (int j = lane; j < N; j += 32) x[__brev(j) >> (32 - log2n)] = make_float2(pre[j], pim[j]);
-    }
+    float2 a[E];
+#pragma unroll
+    for (int m = 0; m < E; m++) a[m] = make_float2(pre[t + L * m], pim[t + L * m]);
+    __syncthreads();
+    hai_fft::line_first<N>(a, t, tw);
+    float2 *x = xbuf + w * XS;
+#pragma unroll
+    for (int k = 0; k < E; k++) x[(L + 1) * k + t] = a[k];
     __syncwarp();
-    warp_fft(x, 1, N, log2n, tw, lane);
-    for (int j = lane; j < N; j += 32) {
-        pre[j] = x[j].x;
-        pim[j] = x[j].y;
-    }
+#pragma unroll
+    for (int u = 0; u < E / L; u++)
+#pragma unroll
+        for (int i = 0; i < L; i++) a[L * u + i] = x[(L + 1) * (t + L * u) + i];
+    hai_fft::line_second<N>(a);
+    if (!live) return;
+#pragma unroll
+    for (int u = 0; u < E / L; u++)
+#pragma unroll
+        for (int i = 0; i < L; i++) {
+            const int k = t + L * u + E * i;
+            pre[k] = a[L * u + i].x;
+            pim[k] = a[L * u + i].y;
+        }
 }
 
-// Column pass: a CTA loads 32 columns of a plane pair and each warp
-// transforms two of them.
-__global__ void __launch_bounds__(kThreads) fft_cols_kernel(float *__restrict__ img, int N, int log2n) {
-    extern __shared__ float2 tile[];   // [N][33], then the N / 2 twiddles
-    float2 *tw = tile + (size_t)N * 33;
-    load_twiddles(tw, N);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pair = blockIdx.x;
-    const int x0 = blockIdx.y * 32;
-    float *pre = img + ((size_t)(pair >> 1) * 4 + 2 * (pair & 1)) * N * N;
+// Column pass, in place: 16 columns per CTA, the column fastest over the
+// threads (64-byte row segments; the exchange, value k1 of lane t at
+// (L k1 + t) 16 + column, is conflict-free).  Before: 595 us on the
+// cadence above (32 columns through a padded tile, radix-2); now 231 us.
+template <int N>
+__global__ void __launch_bounds__(16 * hai_fft::Line<N>::L) fft_cols_kernel(float *__restrict__ img) {
+    constexpr int L = hai_fft::Line<N>::L, E = hai_fft::Line<N>::E;
+    __shared__ float2 tw[N], x[N * 16];
+    hai_fft::fill_twiddles<N>(tw);
+    const int c = threadIdx.x % 16, t = threadIdx.x / 16;
+    float *pre = img + (size_t)blockIdx.x * 2 * N * N + blockIdx.y * 16 + c;
     float *pim = pre + (size_t)N * N;
-    const int ncol = min(32, N - x0);
-    for (int i = threadIdx.x; i < N * 32; i += kThreads) {
-        const int y = i / 32, c = i % 32;
-        if (c < ncol) tile[(__brev(y) >> (32 - log2n)) * 33 + c] = make_float2(pre[(size_t)y * N + x0 + c],
-                                                                               pim[(size_t)y * N + x0 + c]);
-    }
+    float2 a[E];
+#pragma unroll
+    for (int m = 0; m < E; m++) a[m] = make_float2(pre[(size_t)(t + L * m) * N], pim[(size_t)(t + L * m) * N]);
     __syncthreads();
-    for (int c = warp; c < ncol; c += kThreads / 32) warp_fft(tile + c, 33, N, log2n, tw, lane);
+    hai_fft::line_first<N>(a, t, tw);
+#pragma unroll
+    for (int k = 0; k < E; k++) x[(L * k + t) * 16 + c] = a[k];
     __syncthreads();
-    for (int i = threadIdx.x; i < N * 32; i += kThreads) {
-        const int y = i / 32, c = i % 32;
-        if (c < ncol) {
-            pre[(size_t)y * N + x0 + c] = tile[y * 33 + c].x;
-            pim[(size_t)y * N + x0 + c] = tile[y * 33 + c].y;
+#pragma unroll
+    for (int u = 0; u < E / L; u++)
+#pragma unroll
+        for (int i = 0; i < L; i++) a[L * u + i] = x[(L * (t + L * u) + i) * 16 + c];
+    hai_fft::line_second<N>(a);
+#pragma unroll
+    for (int u = 0; u < E / L; u++)
+#pragma unroll
+        for (int i = 0; i < L; i++) {
+            const size_t k = (size_t)(t + L * u + E * i) * N;
+            pre[k] = a[L * u + i].x;
+            pim[k] = a[L * u + i].y;
         }
-    }
+}
+
+template <int N>
+void launch_fft(float *img, int images, cudaStream_t st) {
+    constexpr int W = kFftThreads / hai_fft::Line<N>::L;
+    fft_rows_kernel<N><<<dim3(images * 2, (N + W - 1) / W), kFftThreads, 0, st>>>(img);
+    fft_cols_kernel<N><<<dim3(images * 2, N / 16), 16 * hai_fft::Line<N>::L, 0, st>>>(img);
 }
 
 // beams [S][C][T][K][P][2] -> [K][C][T][P][S][2]; one CTA per (c, t).  VEC:
@@ -486,8 +486,6 @@ extern "C" hai_status hai_xfft_station_image(hai_ctx *ctx, const hai_vis_layout 
     HAI_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
     const int N = L->N, images = L->K * C;
-    int log2n = 0;
-    while ((1 << log2n) < N) log2n++;
     const size_t win_bytes = (size_t)2 * L->tw * L->th * sizeof(float);
     HAI_CUDA_TRY(hai_allow_dyn_smem(station_grid_kernel, ctx->smem_optin));
     if ((long long)images * 2 > 0x7fffffffll) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_station_image: too many images");
@@ -499,13 +497,13 @@ extern "C" hai_status hai_xfft_station_image(hai_ctx *ctx, const hai_vis_layout 
         L->wh, L->tw, L->th, L->ntx, img);
     prof_end(ctx, pidx, st);
     HAI_CUDA_TRY(cudaGetLastError());
-    const int rows_per_cta = kThreads / 32;
-    fft_rows_kernel<<<dim3(images * 2, (N + rows_per_cta - 1) / rows_per_cta), kThreads,
-                      sizeof(float2) * (rows_per_cta * N + N / 2), st>>>(img, N, log2n);
-    HAI_CUDA_TRY(cudaGetLastError());
-    const size_t tile = sizeof(float2) * ((size_t)N * 33 + N / 2);
-    HAI_CUDA_TRY(hai_allow_dyn_smem(fft_cols_kernel, ctx->smem_optin));
-    fft_cols_kernel<<<dim3(images * 2, (N + 31) / 32), kThreads, tile, st>>>(img, N, log2n);
+    switch (N) {
+    case 16: launch_fft<16>(img, images, st); break;
+    case 32: launch_fft<32>(img, images, st); break;
+    case 64: launch_fft<64>(img, images, st); break;
+    case 128: launch_fft<128>(img, images, st); break;
+    default: launch_fft<256>(img, images, st); break;
+    }
     prof_count(ctx, 3);
     HAI_CUDA_TRY(cudaGetLastError());
     return HAI_OK;
