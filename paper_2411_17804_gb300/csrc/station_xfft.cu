@@ -21,11 +21,10 @@
 // gives XX in the real and YY in the imaginary part; XY needs its own complex
 // grid.  The two complex grids are built in the caller's image planes
 // [XX, YY, Re XY, Im XY] (as split re / im planes), which the FFT then
-// transforms in place: no scratch memory.  Gridding runs in shared memory over
-// tiles (<= 112 x 112 cells) of the window of uv cells that on-grid pairs
-// touch, one CTA per (image, grid, tile) with the pairs binned to each tile on
-// the host, and writes its cells with the (-1)^(u+v) checkerboard that puts
-// the phase centre at pixel (N/2, N/2).  The FFTs hold their lines in registers
+// transforms in place: no scratch memory.  Gridding runs over tiles of the uv
+// grid with a thread per cell, the footprints binned to tiles on the host, and
+// writes its cells with the (-1)^(u+v) checkerboard that puts the phase
+// centre at pixel (N/2, N/2).  The FFTs hold their lines in registers
 // (fft_line.cuh).
 #include <math.h>
 #include <string.h>
@@ -38,17 +37,23 @@
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kTileCells = 112;        // uv tile side: 2 x 112^2 floats = 98 KB of shared memory
-constexpr int kTileSmall = 56;         // the smaller side, for layouts with many pairs per tile
-constexpr size_t kTilePairsMin = 4096; // pairs per tile (average) that the smaller side needs
+// Tiles of the periodic uv grid (x = u mod N, y = v mod N), the unit of gridding
+// work: 16 x 16 cells, a thread per cell.
+constexpr int kTile = 16, kTcells = kTile * kTile;
+constexpr int kTileWarps = kTcells / 32;
+constexpr int kImgs = 4;                          // images (beam, channel) a CTA grids together
+constexpr int kFoot = 1024;                       // footprints staged at a time
+constexpr uint32_t kMirror = 1u << 31;            // footprint of the mirror (n, m) of a stored pair
 
-// Gridding record of one stored pair (m >= n): the 2x2 footprints of the pair
-// and of its mirror, as window-relative cell of the lower corner and
-// fractional offsets; du < 0 marks a dropped pair.
-struct PairRec {
-    int16_t du, dv, mu, mv;
-    float fu, fv, mfu, mfv;
+// One chunk of a tile's footprints and, per warp, its gather entries: slot k
+// of lane l at entry base[w] + 32 k + l (zero weights pad the shorter lists).
+struct TileChunk {
+    int32_t foot, nfoot;
+    int32_t base[kTileWarps + 1];
+};
+struct TileEnt {
+    float w;             // bilinear weight
+    int32_t slot;        // footprint within the chunk
 };
 
 __device__ __forceinline__ void pair_of(long long bl, int &m, int &n) {
@@ -80,73 +85,124 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Adds the 2x2 footprint with lower corner (du, dv) (window cells) to the
-// cells that fall inside this CTA's tile [tu0, tu0 + tw) x [tv0, tv0 + th)
-// (tw, th: the tile's own extent; shared rows are tw apart).
-__device__ __forceinline__ void add_footprint(float *wre, float *wim, int tu0, int tv0, int tw, int th, int du, int dv,
-                                              float fu, float fv, float2 g) {
-    const float w[4] = {(1.f - fu) * (1.f - fv), fu * (1.f - fv), (1.f - fu) * fv, fu * fv};
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-        const int cu = du + (t & 1) - tu0, cv = dv + (t >> 1) - tv0;
-        if (w[t] == 0.f || cu < 0 || cu >= tw || cv < 0 || cv >= th) continue;
-        atomicAdd(&wre[cv * tw + cu], w[t] * g.x);
-        atomicAdd(&wim[cv * tw + cu], w[t] * g.y);
+// One pair's visibilities of one image: XX, XY, YX, YY.
+template <bool VEC>
+__device__ __forceinline__ void load_vis(const int32_t *__restrict__ v, int4 &a, int4 &b) {
+    if (VEC) {
+        a = __ldg(reinterpret_cast<const int4 *>(v));
+        b = __ldg(reinterpret_cast<const int4 *>(v) + 1);
+    } else {
+        const int2 *p = reinterpret_cast<const int2 *>(v);
+        const int2 x = __ldg(p), y = __ldg(p + 1), z = __ldg(p + 2), w = __ldg(p + 3);
+        a = make_int4(x.x, x.y, y.x, y.y);
+        b = make_int4(z.x, z.y, w.x, w.y);
     }
 }
 
-// One CTA per (image = (beam, channel), grid h, tile of the uv window):
-// h = 0 builds G_XX + i G_YY into planes 0 / 1, h = 1 builds G_XY into
-// planes 2 / 3.  The CTA grids the pairs binned to its tile, then writes its
-// tile's cells with the checkerboard (the rest of the planes was zeroed).
-__global__ void __launch_bounds__(kThreads) station_grid_kernel(
-    const int32_t *__restrict__ vis, const PairRec *__restrict__ rec, const float2 *__restrict__ phasor,
-    const int32_t *__restrict__ tile_start, const int32_t *__restrict__ tile_pairs, int C, long long nbl, int P,
-    int N, int win_u0, int win_v0, int ww, int wh, int tw, int th, int ntx, float *__restrict__ img) {
-    extern __shared__ float win[];     // [2][th][tw]: re, im
-    const int image = blockIdx.x, h = blockIdx.y, tile = blockIdx.z;
-    const int k = image / C;
-    const int tu0 = (tile % ntx) * tw, tv0 = (tile / ntx) * th;
-    const int tw_eff = min(tw, ww - tu0), th_eff = min(th, wh - tv0);
-    float *wre = win, *wim = win + (size_t)tw * th;
-    for (int i = threadIdx.x; i < 2 * tw * th; i += kThreads) win[i] = 0.f;
-    __syncthreads();
-    const int2 *v = reinterpret_cast<const int2 *>(vis) + (size_t)image * nbl * P * P;
-    const float2 *ph = phasor + (size_t)k * nbl;
-    for (int q = tile_start[tile] + threadIdx.x; q < tile_start[tile + 1]; q += kThreads) {
-        const int bl = tile_pairs[q];
-        const PairRec r = rec[bl];
-        const float2 w = ph[bl];
-        const int2 *vb = v + (size_t)bl * P * P;
-        float2 g, gm;
-        if (h == 0) {
-            const int2 a = vb[0];
-            const float2 xx = cmulf(make_float2((float)a.x, (float)a.y), w);
-            float2 yy = make_float2(0.f, 0.f);
-            if (P == 2) {
-                const int2 b = vb[3];
-                yy = cmulf(make_float2((float)b.x, (float)b.y), w);
-            }
-            g = make_float2(xx.x - yy.y, xx.y + yy.x);                  // XX + i YY
-            gm = make_float2(xx.x + yy.y, -xx.y + yy.x);                // conj(XX) + i conj(YY)
-        } else {
-            const int2 a = vb[1], b = vb[2];
-            g = cmulf(make_float2((float)a.x, (float)a.y), w);          // XY of (m, n)
-            const float2 t = cmulf(make_float2((float)b.x, (float)b.y), w);
-            gm = make_float2(t.x, -t.y);                                // XY of (n, m) = conj(YX~)
-        }
-        add_footprint(wre, wim, tu0, tv0, tw_eff, th_eff, r.du, r.dv, r.fu, r.fv, g);
-        if (r.mu >= 0) add_footprint(wre, wim, tu0, tv0, tw_eff, th_eff, r.mu, r.mv, r.mfu, r.mfv, gm);
+// G_XX + i G_YY into planes 0 / 1 and G_XY into planes 2 / 3 of kImgs images per
+// CTA, one tile of the grid, with the checkerboard.  The tile's footprints (of
+// pairs and of their mirrors) are phased once into shared memory, a chunk at a
+// time, and every cell (thread) then adds its own list of them: no atomics, and
+// a fixed order, so the images are bit-reproducible.  The lists are the same
+// for every image: entries are read once per kImgs images; cells are dealt to
+// the lanes by list length, so a warp's lanes end together.  Tiles are the fast
+// grid index, so a group's visibilities (1 MB an image for 256 stations) come
+// from HBM once and from L2 for the mirrors and the neighbouring tiles.  Grid
+// rows whose tiles are all empty are left unwritten: the FFT passes do not
+// read them.
+//
+// Bound: the divergent loads of the staging (a sector per footprint and image)
+// and shared-memory wavefronts (one 16-byte random read per entry and image).
+// Hierarchical cadence (256 stations, 512 images at 256^2): adding the
+// footprints with shared-memory atomics took 902 us after an 85 us memset of
+// all planes; a lane per image with the cells in registers 798 us (32 lanes a
+// megabyte apart, 1.4 GB read from HBM); this form 616 us.
+template <bool VEC>
+__global__ void __launch_bounds__(kTcells, 3) station_grid_kernel(
+    const int32_t *__restrict__ vis, const uint32_t *__restrict__ foot, const TileEnt *__restrict__ ent,
+    const TileChunk *__restrict__ chunks, const int32_t *__restrict__ tile, const int32_t *__restrict__ tchunk,
+    const uint8_t *__restrict__ cell_of, int ntile, const float2 *__restrict__ phasor, int C, int images,
+    long long nbl, int N, float *__restrict__ img) {
+    extern __shared__ __align__(16) float4 stage[];     // [kImgs][kFoot]; at the end [kImgs][4][256] floats
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int grp = blockIdx.x / ntile, o = blockIdx.x - grp * ntile;
+    const int i0 = grp * kImgs;
+    const int32_t *v[kImgs];
+    const float2 *ph[kImgs];
+#pragma unroll
+    for (int i = 0; i < kImgs; i++) {
+        const int im = min(i0 + i, images - 1);
+        v[i] = vis + (size_t)im * nbl * 8;
+        ph[i] = phasor + (size_t)(im / C) * nbl;
     }
-    __syncthreads();
-    float *pre = img + ((size_t)image * 4 + 2 * h) * N * N, *pim = pre + (size_t)N * N;
-    for (int i = threadIdx.x; i < tw_eff * th_eff; i += kThreads) {
-        const int cu = i % tw_eff, cv = i / tw_eff;
-        const int u = win_u0 + tu0 + cu, v = win_v0 + tv0 + cv;
-        const int x = (u + N) % N, y = (v + N) % N;
-        const float sgn = ((u + v) & 1) ? -1.f : 1.f;
-        pre[(size_t)y * N + x] = sgn * wre[cv * tw_eff + cu];     // rows tw_eff apart, as add_footprint wrote them
-        pim[(size_t)y * N + x] = sgn * wim[cv * tw_eff + cu];
+    float4 acc[kImgs];
+#pragma unroll
+    for (int i = 0; i < kImgs; i++) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int q0 = tchunk[o], q1 = tchunk[o + 1];
+    for (int q = q0; q < q1; q++) {
+        const TileChunk *ch = chunks + q;
+        const int f0 = ch->foot, nf = ch->nfoot;
+        if (q > q0) __syncthreads();                    // the last chunk's gather is done
+        for (int f = tid; f < nf; f += kTcells) {
+            const uint32_t r = __ldg(foot + f0 + f);
+            const bool mirror = r & kMirror;
+            const size_t bl = r & (kMirror - 1);
+            int4 a[kImgs], b[kImgs];
+            float2 w[kImgs];
+#pragma unroll
+            for (int i = 0; i < kImgs; i++) {
+                load_vis<VEC>(v[i] + bl * 8, a[i], b[i]);
+                w[i] = __ldg(ph[i] + bl);
+            }
+#pragma unroll
+            for (int i = 0; i < kImgs; i++) {
+                const float2 xx = cmulf(make_float2((float)a[i].x, (float)a[i].y), w[i]);
+                const float2 yy = cmulf(make_float2((float)b[i].z, (float)b[i].w), w[i]);
+                const float2 xy = cmulf(make_float2((float)(mirror ? b[i].x : a[i].z), (float)(mirror ? b[i].y : a[i].w)), w[i]);
+                // the pair: XX + i YY, XY; its mirror: conj(XX) + i conj(YY), conj(YX)
+                stage[i * kFoot + f] = mirror ? make_float4(xx.x + yy.y, yy.x - xx.y, xy.x, -xy.y)
+                                              : make_float4(xx.x - yy.y, xx.y + yy.x, xy.x, xy.y);
+            }
+        }
+        __syncthreads();
+        const int e1 = ch->base[warp + 1];
+#pragma unroll 2
+        for (int e = ch->base[warp] + lane; e < e1; e += 32) {
+            const float2 x = __ldg(reinterpret_cast<const float2 *>(ent) + e);
+            const int slot = __float_as_int(x.y);
+#pragma unroll
+            for (int i = 0; i < kImgs; i++) {
+                const float4 g = stage[i * kFoot + slot];
+                acc[i].x = fmaf(x.x, g.x, acc[i].x);
+                acc[i].y = fmaf(x.x, g.y, acc[i].y);
+                acc[i].z = fmaf(x.x, g.z, acc[i].z);
+                acc[i].w = fmaf(x.x, g.w, acc[i].w);
+            }
+        }
+    }
+    // the cells back in row order, then out
+    const int t = tile[o], x0 = t % (N / kTile) * kTile, y0 = t / (N / kTile) * kTile;
+    float *cells = reinterpret_cast<float *>(stage);
+    if (q1 > q0) {
+        __syncthreads();
+        const int cell = cell_of[(size_t)o * kTcells + tid];
+        const float sgn = ((cell ^ (cell / kTile)) & 1) ? -1.f : 1.f;     // x0, y0 are even
+#pragma unroll
+        for (int i = 0; i < kImgs; i++) {
+            cells[(i * 4 + 0) * kTcells + cell] = sgn * acc[i].x;
+            cells[(i * 4 + 1) * kTcells + cell] = sgn * acc[i].y;
+            cells[(i * 4 + 2) * kTcells + cell] = sgn * acc[i].z;
+            cells[(i * 4 + 3) * kTcells + cell] = sgn * acc[i].w;
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < kImgs; i++) {
+        if (i0 + i >= images) break;
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+            img[(((size_t)(i0 + i) * 4 + p) * N + y0 + tid / kTile) * N + x0 + tid % kTile] =
+                q1 > q0 ? cells[(i * 4 + p) * kTcells + tid] : 0.f;
     }
 }
 
@@ -157,7 +213,7 @@ __global__ void __launch_bounds__(kThreads) station_grid_kernel(
 // sectors.  The bound is HBM: every plane is read and written once (1.07 GB on
 // the hierarchical cadence's 512 images at 256^2).  The radix-2 form it
 // replaces made log2 N passes over shared memory and took 604 us there;
-// now 169 us (6.3 TB/s).
+// now 169 us (6.3 TB/s).  Only the rows that the gridding wrote are transformed.
 constexpr int kFftThreads = 256;
 
 template <int N>
@@ -167,15 +223,16 @@ struct RowSmem {
 };
 
 template <int N>
-__global__ void __launch_bounds__(kFftThreads) fft_rows_kernel(float *__restrict__ img) {
+__global__ void __launch_bounds__(kFftThreads) fft_rows_kernel(float *__restrict__ img,
+                                                               const int32_t *__restrict__ rows, int nrow) {
     constexpr int L = hai_fft::Line<N>::L, E = hai_fft::Line<N>::E, XS = RowSmem<N>::XS, W = kFftThreads / L;
     __shared__ float2 tw[N], xbuf[W * XS];
     hai_fft::fill_twiddles<N>(tw);
     const int t = threadIdx.x % L, w = threadIdx.x / L;
     const int pair = blockIdx.x;       // image * 2 + h
-    const int y = blockIdx.y * W + w;
-    const bool live = y < N;
-    float *pre = img + ((size_t)pair * 2 * N + (live ? y : 0)) * N;
+    const int r = blockIdx.y * W + w;
+    const bool live = r < nrow;
+    float *pre = img + ((size_t)pair * 2 * N + rows[live ? r : 0]) * N;
     float *pim = pre + (size_t)N * N;
     float2 a[E];
 #pragma unroll
@@ -207,7 +264,8 @@ __global__ void __launch_bounds__(kFftThreads) fft_rows_kernel(float *__restrict
 // (L k1 + t) 16 + column, is conflict-free).  Before: 595 us on the
 // cadence above (32 columns through a padded tile, radix-2); now 231 us.
 template <int N>
-__global__ void __launch_bounds__(16 * hai_fft::Line<N>::L) fft_cols_kernel(float *__restrict__ img) {
+__global__ void __launch_bounds__(16 * hai_fft::Line<N>::L) fft_cols_kernel(float *__restrict__ img,
+                                                                                      const uint8_t *__restrict__ live) {
     constexpr int L = hai_fft::Line<N>::L, E = hai_fft::Line<N>::E;
     __shared__ float2 tw[N], x[N * 16];
     hai_fft::fill_twiddles<N>(tw);
@@ -216,7 +274,10 @@ __global__ void __launch_bounds__(16 * hai_fft::Line<N>::L) fft_cols_kernel(floa
     float *pim = pre + (size_t)N * N;
     float2 a[E];
 #pragma unroll
-    for (int m = 0; m < E; m++) a[m] = make_float2(pre[(size_t)(t + L * m) * N], pim[(size_t)(t + L * m) * N]);
+    for (int m = 0; m < E; m++) {
+        const size_t y = t + L * m;
+        a[m] = live[y] ? make_float2(pre[y * N], pim[y * N]) : make_float2(0.f, 0.f);
+    }
     __syncthreads();
     hai_fft::line_first<N>(a, t, tw);
 #pragma unroll
@@ -238,10 +299,10 @@ __global__ void __launch_bounds__(16 * hai_fft::Line<N>::L) fft_cols_kernel(floa
 }
 
 template <int N>
-void launch_fft(float *img, int images, cudaStream_t st) {
+void launch_fft(float *img, int images, const int32_t *rows, int nrow, const uint8_t *live, cudaStream_t st) {
     constexpr int W = kFftThreads / hai_fft::Line<N>::L;
-    fft_rows_kernel<N><<<dim3(images * 2, (N + W - 1) / W), kFftThreads, 0, st>>>(img);
-    fft_cols_kernel<N><<<dim3(images * 2, N / 16), 16 * hai_fft::Line<N>::L, 0, st>>>(img);
+    fft_rows_kernel<N><<<dim3(images * 2, (nrow + W - 1) / W), kFftThreads, 0, st>>>(img, rows, nrow);
+    fft_cols_kernel<N><<<dim3(images * 2, N / 16), 16 * hai_fft::Line<N>::L, 0, st>>>(img, live);
 }
 
 // beams [S][C][T][K][P][2] -> [K][C][T][P][S][2]; one CTA per (c, t).  VEC:
@@ -297,12 +358,16 @@ struct hai_vis_layout {
     hai_ctx *ctx = nullptr;
     int S = 0, N = 0, P = 0, K = 0;
     long long nbl = 0;
-    int win_u0 = 0, win_v0 = 0, ww = 0, wh = 0;
-    int tw = 0, th = 0, ntx = 0, nty = 0;    // tiles of the window, one CTA each
     long long n_offgrid = 0;
-    PairRec *d_rec = nullptr;
+    int ntile = 0, nrow = 0;                 // tiles in written rows; written rows
+    uint32_t *d_foot = nullptr;              // footprints (pair, mirror bit), tile after tile
+    TileEnt *d_ent = nullptr;                // gather entries
+    TileChunk *d_chunk = nullptr;
+    int32_t *d_tile = nullptr, *d_tchunk = nullptr;   // tiles by footprint count, their first chunks [ntile + 1]
+    uint8_t *d_cell = nullptr;               // [ntile][256] cell of each thread
+    int32_t *d_rows = nullptr;               // the written rows
+    uint8_t *d_live = nullptr;               // [N] whether a row is written
     float2 *d_phasor = nullptr;
-    int32_t *d_tile_start = nullptr, *d_tile_pairs = nullptr;
 };
 
 void vis_layout_dims(const hai_vis_layout *L, int *S, int *N, int *K) {
@@ -313,10 +378,15 @@ void vis_layout_dims(const hai_vis_layout *L, int *S, int *N, int *K) {
 
 static void vis_layout_free(hai_vis_layout *L) {
     if (!L) return;
-    cudaFree(L->d_rec);
+    cudaFree(L->d_foot);
+    cudaFree(L->d_ent);
+    cudaFree(L->d_chunk);
+    cudaFree(L->d_tile);
+    cudaFree(L->d_tchunk);
+    cudaFree(L->d_cell);
+    cudaFree(L->d_rows);
+    cudaFree(L->d_live);
     cudaFree(L->d_phasor);
-    cudaFree(L->d_tile_start);
-    cudaFree(L->d_tile_pairs);
     delete L;
 }
 
@@ -330,36 +400,120 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     if (d->n_pol != 2) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: station images need 2 pols");
     if (hai_fault_injected("alloc")) return hai_fail(HAI_ERR_NO_MEMORY, "hai_vis_layout_create: injected allocation failure");
     const long long nbl = (long long)S * (S + 1) / 2;
-    // footprints in FP64 on the host: lower corner floor(uv) and fraction
-    std::vector<PairRec> rec(nbl);
-    std::vector<long> cu(nbl), cv(nbl), mcu(nbl), mcv(nbl);
-    std::vector<float> fu(nbl), fv(nbl), mfu(nbl), mfv(nbl);
-    std::vector<char> ok(nbl);
-    long umin = N, vmin = N, umax = -N, vmax = -N;
+    // footprints in FP64 on the host: lower corner floor(uv) and fraction, one
+    // record in every tile they touch (counted, then placed)
+    const int nt = N / kTile;
+    struct Foot {
+        uint32_t pair;
+        int16_t cx, cy;                        // lower corner in the tile, -1 .. 15
+        float fu, fv;
+    };
+    std::vector<int32_t> count((size_t)nt * nt, 0);
+    auto each_tile = [&](double u, double v, auto &&f) {
+        const double fu = floor(u), fv = floor(v);
+        const int x = (((int)fu % N) + N) % N, y = (((int)fv % N) + N) % N;
+        const int x1 = (x + 1) % N, y1 = (y + 1) % N;
+        // with one tile a side the wrapped column is in the same tile: its own record
+        const int nx = x % kTile == kTile - 1 ? 2 : 1, ny = y % kTile == kTile - 1 ? 2 : 1;
+        for (int j = 0; j < ny; j++)
+            for (int i = 0; i < nx; i++)
+                f(((j ? y1 : y) / kTile) * nt + (i ? x1 : x) / kTile, i ? -1 : x % kTile, j ? -1 : y % kTile,
+                  (float)(u - fu), (float)(v - fv));
+    };
     long long dropped = 0;
-    for (int m = 0, bl = 0; m < S; m++)
-        for (int n = 0; n <= m; n++, bl++) {
-            const double du = (d->pos_m[2 * m] - d->pos_m[2 * n]) / d->cell_m;
-            const double dv = (d->pos_m[2 * m + 1] - d->pos_m[2 * n + 1]) / d->cell_m;
-            const double a = floor(du), b = floor(dv), ma = floor(-du), mb = floor(-dv);
-            cu[bl] = (long)a;
-            cv[bl] = (long)b;
-            mcu[bl] = (long)ma;
-            mcv[bl] = (long)mb;
-            fu[bl] = (float)(du - a);
-            fv[bl] = (float)(dv - b);
-            mfu[bl] = (float)(-du - ma);
-            mfv[bl] = (float)(-dv - mb);
-            ok[bl] = station_pair_kept(N, du, dv);
-            if (!ok[bl]) {
-                dropped++;
-                continue;
+    auto each_footprint = [&](auto &&f) {      // f(pair with the mirror bit, u, v) of the kept pairs
+        dropped = 0;
+        long long bl = 0;
+        for (int m = 0; m < S; m++)
+            for (int n = 0; n <= m; n++, bl++) {
+                const double du = (d->pos_m[2 * m] - d->pos_m[2 * n]) / d->cell_m;
+                const double dv = (d->pos_m[2 * m + 1] - d->pos_m[2 * n + 1]) / d->cell_m;
+                if (!station_pair_kept(N, du, dv)) {
+                    dropped++;
+                    continue;
+                }
+                f((uint32_t)bl, du, dv);
+                if (m != n) f((uint32_t)bl | kMirror, -du, -dv);     // an auto pair has no mirror
             }
-            umin = std::min(umin, std::min(cu[bl], mcu[bl]));
-            vmin = std::min(vmin, std::min(cv[bl], mcv[bl]));
-            umax = std::max(umax, std::max(cu[bl], mcu[bl]) + 1);
-            vmax = std::max(vmax, std::max(cv[bl], mcv[bl]) + 1);
+    };
+    each_footprint([&](uint32_t, double u, double v) {
+        each_tile(u, v, [&](int p, int, int, float, float) { count[p]++; });
+    });
+    std::vector<uint8_t> live(N, 0);
+    std::vector<int32_t> rows, tiles;
+    for (int ty = 0; ty < nt; ty++) {
+        bool any = false;
+        for (int tx = 0; tx < nt; tx++) any |= count[ty * nt + tx] > 0;
+        if (!any) continue;
+        for (int y = ty * kTile; y < (ty + 1) * kTile; y++) {
+            live[y] = 1;
+            rows.push_back(y);
         }
+        for (int tx = 0; tx < nt; tx++) tiles.push_back(ty * nt + tx);
+    }
+    std::stable_sort(tiles.begin(), tiles.end(), [&](int x, int y) { return count[x] > count[y]; });
+    std::vector<long long> fill(count.size(), 0);
+    long long nfoot = 0;
+    for (int t : tiles) {
+        fill[t] = nfoot;
+        nfoot += count[t];
+    }
+    // entries: at most 4 a footprint, padded within warps; checked as they are placed
+    if (nfoot > 0x0fffffffll) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: too many station pairs");
+    std::vector<Foot> all(std::max<long long>(1, nfoot));
+    each_footprint([&](uint32_t pair, double u, double v) {
+        each_tile(u, v, [&](int p, int cx, int cy, float fu, float fv) {
+            all[fill[p]++] = Foot{pair, (int16_t)cx, (int16_t)cy, fu, fv};
+        });
+    });
+    std::vector<uint32_t> foot(all.size());
+    for (size_t i = 0; i < all.size(); i++) foot[i] = all[i].pair;
+    std::vector<TileEnt> ent;
+    std::vector<TileChunk> chunks;
+    std::vector<int32_t> tchunk(1, 0);
+    std::vector<uint8_t> cell_of(tiles.size() * kTcells);
+    long long f0 = 0;
+    for (size_t o = 0; o < tiles.size(); o++) {
+        const long long f1 = f0 + count[tiles[o]];
+        // f(cell, weight) of a footprint's non-zero cells in the tile
+        auto each_cell = [&](const Foot &r, auto &&f) {
+            for (int t = 0; t < 4; t++) {
+                const int x = r.cx + (t & 1), y = r.cy + (t >> 1);
+                const float w = ((t & 1) ? r.fu : 1.f - r.fu) * ((t >> 1) ? r.fv : 1.f - r.fv);
+                if (x >= 0 && x < kTile && y >= 0 && y < kTile && w != 0.f) f(y * kTile + x, w);
+            }
+        };
+        int total[kTcells] = {}, order[kTcells], thread_of[kTcells];
+        for (long long f = f0; f < f1; f++) each_cell(all[f], [&](int c, float) { total[c]++; });
+        for (int c = 0; c < kTcells; c++) order[c] = c;
+        std::stable_sort(order, order + kTcells, [&](int x, int y) { return total[x] > total[y]; });
+        for (int i = 0; i < kTcells; i++) {
+            thread_of[order[i]] = i;
+            cell_of[o * kTcells + i] = (uint8_t)order[i];
+        }
+        for (long long q = f0; q < f1; q += kFoot) {
+            TileChunk ch;
+            ch.foot = (int32_t)q;
+            ch.nfoot = (int32_t)std::min<long long>(kFoot, f1 - q);
+            int n[kTcells] = {};
+            for (int f = 0; f < ch.nfoot; f++) each_cell(all[q + f], [&](int c, float) { n[thread_of[c]]++; });
+            for (int w = 0; w < kTileWarps; w++) {
+                ch.base[w] = (int32_t)ent.size();
+                ent.resize(ent.size() + 32 * (size_t)*std::max_element(n + 32 * w, n + 32 * w + 32), TileEnt{0.f, 0});
+            }
+            ch.base[kTileWarps] = (int32_t)ent.size();
+            std::fill(n, n + kTcells, 0);
+            for (int f = 0; f < ch.nfoot; f++)
+                each_cell(all[q + f], [&](int c, float w) {
+                    const int i = thread_of[c];
+                    ent[ch.base[i / 32] + 32 * n[i]++ + i % 32] = TileEnt{w, f};
+                });
+            chunks.push_back(ch);
+            if (ent.size() > 0x7fffffffull) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: too many station pairs");
+        }
+        tchunk.push_back((int32_t)chunks.size());
+        f0 = f1;
+    }
     hai_vis_layout *L = new hai_vis_layout();
     L->ctx = ctx;
     L->S = S;
@@ -368,81 +522,25 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     L->K = K;
     L->nbl = nbl;
     L->n_offgrid = dropped;
-    L->win_u0 = (int)umin;
-    L->win_v0 = (int)vmin;
-    L->ww = (int)(umax - umin + 1);
-    L->wh = (int)(vmax - vmin + 1);
-    for (int m = 0, bl = 0; m < S; m++)
-        for (int n = 0; n <= m; n++, bl++) {
-            PairRec &r = rec[bl];
-            if (!ok[bl]) {
-                r = PairRec{-1, -1, -1, -1, 0.f, 0.f, 0.f, 0.f};
-                continue;
-            }
-            r.du = (int16_t)(cu[bl] - umin);
-            r.dv = (int16_t)(cv[bl] - vmin);
-            r.fu = fu[bl];
-            r.fv = fv[bl];
-            // an auto pair has no mirror
-            r.mu = (int16_t)(m == n ? -1 : mcu[bl] - umin);
-            r.mv = (int16_t)(mcv[bl] - vmin);
-            r.mfu = mfu[bl];
-            r.mfv = mfv[bl];
-        }
-    // tiles of at most side^2 cells (2 x 4 bytes each in shared memory); pairs
-    // per tile: every tile that the pair's footprint or its mirror's touches.
-    // The time follows the tiles that hold the densest cells (short
-    // baselines near the window's centre): the smaller side spreads them over
-    // more CTAs, which pays where the tiles stay well filled (measured: 512
-    // stations in a 3 km core 6.1 -> 4.9 ms, 256 stations 0.91 -> 1.17 ms)
-    std::vector<std::vector<int32_t>> lists;
-    int ntile = 0;
-    for (int side : {kTileSmall, kTileCells}) {
-        L->ntx = (L->ww + side - 1) / side;
-        L->nty = (L->wh + side - 1) / side;
-        L->tw = (L->ww + L->ntx - 1) / L->ntx;
-        L->th = (L->wh + L->nty - 1) / L->nty;
-        ntile = L->ntx * L->nty;
-        lists.assign(ntile, {});
-        size_t binned = 0;
-        for (long long bl = 0; bl < nbl; bl++) {
-            const PairRec &r = rec[bl];
-            if (r.du < 0) continue;
-            int seen[8], ns = 0;
-            auto touch = [&](int du, int dv) {
-                for (int t = 0; t < 4; t++) {
-                    const int tx = (du + (t & 1)) / L->tw, ty = (dv + (t >> 1)) / L->th;
-                    const int id = ty * L->ntx + tx;
-                    bool dup = false;
-                    for (int j = 0; j < ns; j++) dup |= seen[j] == id;
-                    if (!dup) seen[ns++] = id;
-                }
-            };
-            touch(r.du, r.dv);
-            if (r.mu >= 0) touch(r.mu, r.mv);
-            for (int j = 0; j < ns; j++) lists[seen[j]].push_back((int32_t)bl);
-            binned += ns;
-        }
-        if (side == kTileCells || binned >= kTilePairsMin * (size_t)ntile) break;
-    }
-    std::vector<int32_t> tstart(ntile + 1, 0), tpairs;
-    for (int t = 0; t < ntile; t++) {
-        tpairs.insert(tpairs.end(), lists[t].begin(), lists[t].end());
-        tstart[t + 1] = (int32_t)tpairs.size();
-    }
+    L->ntile = (int)tiles.size();
+    L->nrow = (int)rows.size();
     double *d_pos = nullptr, *d_dir = nullptr;
     std::vector<double> dirs(2 * (size_t)K, 0.0);
     if (d->dir) std::copy(d->dir, d->dir + 2 * (size_t)K, dirs.begin());
     cudaError_t e = cudaSetDevice(ctx->device);
-    if (e == cudaSuccess) e = cudaMalloc(&L->d_rec, sizeof(PairRec) * nbl);
-    if (e == cudaSuccess) e = cudaMemcpy(L->d_rec, rec.data(), sizeof(PairRec) * nbl, cudaMemcpyHostToDevice);
+    auto put = [&](auto *&dst, const auto &src) {
+        if (e == cudaSuccess) e = cudaMalloc(&dst, sizeof(src[0]) * src.size());
+        if (e == cudaSuccess) e = cudaMemcpy(dst, src.data(), sizeof(src[0]) * src.size(), cudaMemcpyHostToDevice);
+    };
+    put(L->d_foot, foot);
+    put(L->d_ent, ent);
+    put(L->d_chunk, chunks);
+    put(L->d_tile, tiles);
+    put(L->d_tchunk, tchunk);
+    put(L->d_cell, cell_of);
+    put(L->d_rows, rows);
+    put(L->d_live, live);
     if (e == cudaSuccess) e = cudaMalloc(&L->d_phasor, sizeof(float2) * (size_t)K * nbl);
-    if (e == cudaSuccess) e = cudaMalloc(&L->d_tile_start, sizeof(int32_t) * tstart.size());
-    if (e == cudaSuccess) e = cudaMalloc(&L->d_tile_pairs, sizeof(int32_t) * std::max<size_t>(1, tpairs.size()));
-    if (e == cudaSuccess)
-        e = cudaMemcpy(L->d_tile_start, tstart.data(), sizeof(int32_t) * tstart.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !tpairs.empty())
-        e = cudaMemcpy(L->d_tile_pairs, tpairs.data(), sizeof(int32_t) * tpairs.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&d_pos, sizeof(double) * 2 * S);
     if (e == cudaSuccess) e = cudaMalloc(&d_dir, sizeof(double) * 2 * K);
     if (e == cudaSuccess) e = cudaMemcpy(d_pos, d->pos_m, sizeof(double) * 2 * S, cudaMemcpyHostToDevice);
@@ -486,23 +584,23 @@ extern "C" hai_status hai_xfft_station_image(hai_ctx *ctx, const hai_vis_layout 
     HAI_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
     const int N = L->N, images = L->K * C;
-    const size_t win_bytes = (size_t)2 * L->tw * L->th * sizeof(float);
-    HAI_CUDA_TRY(hai_allow_dyn_smem(station_grid_kernel, ctx->smem_optin));
-    if ((long long)images * 2 > 0x7fffffffll) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_station_image: too many images");
-    // cells outside the window stay zero; the tiles write the rest
-    HAI_CUDA_TRY(cudaMemsetAsync(img, 0, sizeof(float) * (size_t)images * 4 * N * N, st));
+    const int groups = (images + kImgs - 1) / kImgs;
+    if ((long long)images * 2 > 0x7fffffffll || (long long)L->ntile * groups > 0x7fffffffll)
+        return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_station_image: too many images");
     const int pidx = prof_begin(ctx, st);
-    station_grid_kernel<<<dim3(images, 2, L->ntx * L->nty), kThreads, win_bytes, st>>>(
-        vis, L->d_rec, L->d_phasor, L->d_tile_start, L->d_tile_pairs, C, L->nbl, L->P, N, L->win_u0, L->win_v0, L->ww,
-        L->wh, L->tw, L->th, L->ntx, img);
+    auto grid = (((uintptr_t)vis & 15) == 0) ? station_grid_kernel<true> : station_grid_kernel<false>;
+    HAI_CUDA_TRY(hai_allow_dyn_smem(grid, ctx->smem_optin));
+    grid<<<(unsigned)(L->ntile * groups), kTcells, sizeof(float4) * kImgs * kFoot, st>>>(
+        vis, L->d_foot, L->d_ent, L->d_chunk, L->d_tile, L->d_tchunk, L->d_cell, L->ntile, L->d_phasor, C, images,
+        L->nbl, N, img);
     prof_end(ctx, pidx, st);
     HAI_CUDA_TRY(cudaGetLastError());
     switch (N) {
-    case 16: launch_fft<16>(img, images, st); break;
-    case 32: launch_fft<32>(img, images, st); break;
-    case 64: launch_fft<64>(img, images, st); break;
-    case 128: launch_fft<128>(img, images, st); break;
-    default: launch_fft<256>(img, images, st); break;
+    case 16: launch_fft<16>(img, images, L->d_rows, L->nrow, L->d_live, st); break;
+    case 32: launch_fft<32>(img, images, L->d_rows, L->nrow, L->d_live, st); break;
+    case 64: launch_fft<64>(img, images, L->d_rows, L->nrow, L->d_live, st); break;
+    case 128: launch_fft<128>(img, images, L->d_rows, L->nrow, L->d_live, st); break;
+    default: launch_fft<256>(img, images, L->d_rows, L->nrow, L->d_live, st); break;
     }
     prof_count(ctx, 3);
     HAI_CUDA_TRY(cudaGetLastError());
