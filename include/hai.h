@@ -408,8 +408,8 @@ hai_status hai_correlate(hai_ctx *ctx, const int8_t *volt, int C, int T, int N, 
  *   img   device float [C][Q][N][N]; overwritten or added to (accumulate)
  * The pair (b, a) is the Hermitian mirror of the stored (a, b).  FP32 grid and
  * FFT; each grid cell sums its contributions in a fixed order, so results are
- * deterministic.  The first call for a layout builds on the host, and copies
- * to the device (synchronously), the per-cell list of K_ab contributions
+ * deterministic.  The first call for a layout builds (synchronously, on the
+ * host and the device) the table of K_ab contributions by patches of the grid
  * (layout-only data, freed with the layout; HAI_ERR_UNSUPPORTED beyond 2e8
  * entries, i.e. N_e(N_e+1)(2K-1)^2 > 2e8); the channels are staged through
  * the context's operand workspace, so calls on one context must not run

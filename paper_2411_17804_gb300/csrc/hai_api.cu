@@ -244,9 +244,10 @@ static void layout_free(hai_layout *L) {
     if (L->big_stream) cudaStreamDestroy(L->big_stream);
     for (cudaEvent_t ev : L->big_ev)
         if (ev) cudaEventDestroy(ev);
-    cudaFree(L->d_xcell);
-    cudaFree(L->d_xent);
-    cudaFree(L->d_xk);
+    cudaFree(L->d_xpatch);
+    cudaFree(L->d_xrec);
+    cudaFree(L->d_xchunk);
+    cudaFree(L->d_xcoef);
     delete L;
 }
 

@@ -88,10 +88,14 @@ struct hai_layout {
     long long big_batch = 0;
     cudaStream_t big_stream = nullptr;  // the fixup of batch i beside batch i + 1's gridding and stage 1
     cudaEvent_t big_ev[2] = {};         // stage 2 done, fixup done
-    // XFFT: per grid cell the (pair, K_ab value, mirror) entries landing there,
-    // built on the first hai_xfft_image call (layout-only data)
-    mutable int32_t *d_xcell = nullptr, *d_xent = nullptr;
-    mutable float2 *d_xk = nullptr;
+    // XFFT: the footprints of K_ab binned to patches of the grid, in chunks, with
+    // their coefficients; built on the first hai_xfft_image call (layout-only data)
+    mutable int32_t *d_xpatch = nullptr;   // first chunk of every patch
+    mutable uint32_t *d_xrec = nullptr;
+    mutable void *d_xchunk = nullptr;
+    mutable float *d_xcoef = nullptr;
+    mutable int xfft_nchunk = 0;
+    mutable bool xfft_real = false;     // real taps: real coefficients
     mutable std::mutex xfft_mu;
     mutable size_t dev_bytes = 0;       // device memory the layout holds (guarded by xfft_mu after creation)
 };

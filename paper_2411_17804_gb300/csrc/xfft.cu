@@ -12,227 +12,362 @@
 // conj(V^{beta alpha}_{ab} K_ab[d]) at lag -d (Hermitian mirror).
 //
 // K_ab and the cells it lands on depend on the layout only.  On a layout's
-// first call the host lists, per grid cell, the (pair, K_ab value, mirror)
-// entries that land there; the imaging is then three kernels per batch of
-// channels:
-//   transpose: the visibilities to [pair][channel][pol pair] (float2), so
-//              that one pair's values for every channel and product are
-//              adjacent;
-//   gather:    per cell, threads over (channel, product) sum the cell's
-//              entries (no atomics; four partial sums combined in a fixed
-//              order: deterministic) and store the cell with the (-1)^(dx+dy)
-//              checkerboard;
-//   FFT:       one CTA per (channel, product) grid: rows then columns,
-//              radix-2 in shared memory, into the image planes.
+// first call the footprints of K_ab (2K - 1 cells a side, and the mirror's) are
+// binned to patches of 4 x 4 cells of the circular grid, and their values on
+// every cell of a patch are computed on the GPU; the imaging is then two kernels
+// per batch of channels:
+//   gather: a warp holds a patch's 16 cells of 32 channels in registers (a lane
+//           per channel) and walks the patch's records, the record's 16
+//           coefficients the same for all lanes;
+//   FFT:    one CTA per (channel, plane pair) adds a cell's partial sums,
+//           applies the (-1)^(dx+dy) checkerboard and transforms rows then
+//           columns in registers (fft_line.cuh) into the image planes.
+// XX and YY grids are Hermitian, so G_XX + i G_YY is one complex grid whose
+// transform holds XX in its real and YY in its imaginary part (an auto's
+// imaginary part, zero from a correlator, would add to the imaginary part of
+// its own image only, which is not kept: it is left out).  Sums run in a fixed
+// order: deterministic.
 #include <math.h>
 
 #include <algorithm>
 #include <vector>
 
+#include "fft_line.cuh"
 #include "hai_internal.h"
 
 namespace {
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
+constexpr int kPs = 4, kPcells = kPs * kPs;      // patch side, cells
+constexpr int kChunk = 256;                       // records of one patch that a CTA sums
+constexpr int kGatherWarps = 8;
+constexpr uint32_t kMirror = 1u << 31, kAuto = 1u << 30;   // record flags beside the stored pair's index
 
-// products: XX = V^00, YY = V^11, XY = V^01; the mirror (b, a) of a stored
-// pair uses V^00, V^11, V^10 (conjugated)
-__constant__ int kProd[3] = {0, 3, 1};
-__constant__ int kMProd[3] = {0, 3, 2};
+// One chunk: records [q0, q1) of a patch.
+struct Chunk {
+    int32_t patch, q0, q1;
+};
 
-// vis [C][nbl][PP] int2 -> vt [nbl][cb][PP] float2 for channels c0 .. c0+cb-1
-__global__ void __launch_bounds__(256) xfft_transpose_kernel(const int32_t *__restrict__ vis, long long nbl, int PP,
-                                                             int c0, int cb, float2 *__restrict__ vt) {
-    const long long n = nbl * cb * PP;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int pp = (int)(i % PP);
-        const long long r = i / PP;
-        const int c = (int)(r % cb);
-        const long long bl = r / cb;
-        const int2 v = reinterpret_cast<const int2 *>(vis)[((size_t)(c0 + c) * nbl + bl) * PP + pp];
-        vt[i] = make_float2((float)v.x, (float)v.y);
+// Coefficients of the records: the value of K_ab (its conjugate for a mirror)
+// on every cell of the record's patch, summed over the lags that fall on the
+// cell of the circular grid; only real parts for a layout of real taps.
+template <bool REAL>
+__global__ void __launch_bounds__(256) xfft_coef_kernel(const Chunk *__restrict__ chunks, const uint32_t *__restrict__ rec,
+                                                        const int32_t *__restrict__ anchors,
+                                                        const float2 *__restrict__ taps, int N, int K,
+                                                        float *__restrict__ coef) {
+    const Chunk ch = chunks[blockIdx.x];
+    const int npx = N / kPs, W = 2 * K - 1;
+    for (int i = threadIdx.x; i < (ch.q1 - ch.q0) * kPcells; i += blockDim.x) {
+        const int q = ch.q0 + i / kPcells, cell = i % kPcells;
+        const uint32_t r = rec[q];
+        const long long bl = r & (kAuto - 1);
+        int a = (int)((sqrt(8.0 * (double)bl + 1.0) - 1.0) * 0.5);
+        while ((long long)(a + 1) * (a + 2) / 2 <= bl) a++;
+        while ((long long)a * (a + 1) / 2 > bl) a--;
+        const int b = (int)(bl - (long long)a * (a + 1) / 2);
+        // the cell's lag relative to the anchors', of the pair (the mirror's lags are negated)
+        int x = ch.patch % npx * kPs + cell % kPs, y = ch.patch / npx * kPs + cell / kPs;
+        if (r & kMirror) {
+            x = (N - x) & (N - 1);
+            y = (N - y) & (N - 1);
+        }
+        const int dx = anchors[2 * a] - anchors[2 * b], dy = anchors[2 * a + 1] - anchors[2 * b + 1];
+        const float2 *ta = taps + (size_t)a * K * K, *tb = taps + (size_t)b * K * K;
+        float2 k = make_float2(0.f, 0.f);
+        // every lag (ex, ey) in (-K, K)^2 congruent to the cell
+        for (int ey = ((y - dy + K - 1) & (N - 1)) - (K - 1); ey <= W - K; ey += N)
+            for (int ex = ((x - dx + K - 1) & (N - 1)) - (K - 1); ex <= W - K; ex += N)
+                for (int vb = max(0, -ey); vb < min(K, K - ey); vb++)
+                    for (int ub = max(0, -ex); ub < min(K, K - ex); ub++) {
+                        // sum over tap pairs with (ua - ub, va - vb) = e of conj(w_a) w_b
+                        const float2 wa = ta[(vb + ey) * K + (ub + ex)], wb = tb[vb * K + ub];
+                        k.x += wa.x * wb.x + wa.y * wb.y;
+                        k.y += wa.x * wb.y - wa.y * wb.x;
+                    }
+        if (REAL) coef[(size_t)q * kPcells + cell] = k.x;
+        else reinterpret_cast<float2 *>(coef)[(size_t)q * kPcells + cell] = make_float2(k.x, r & kMirror ? -k.y : k.y);
     }
 }
 
-// One block per cell; thread j = (channel c, product q), j = c np + q.  The
-// cell's entries are taken four at a time into four partial sums (their loads
-// independent), combined in a fixed order: deterministic.  grid [cb][np][N][N].
-__global__ void __launch_bounds__(256) xfft_gather_kernel(const float2 *__restrict__ vt, const int32_t *__restrict__ cell_start,
-                                                          const int32_t *__restrict__ ent, const float2 *__restrict__ kab,
-                                                          int N, int cb, int np, int PP, float2 *__restrict__ grid) {
-    const int nj = cb * np, NN = N * N;
-    const int cell = blockIdx.x;
-    const int dx = cell % N, dy = cell / N;
-    const float sgn = ((dx + dy) & 1) ? -1.f : 1.f;
-    const int q0 = cell_start[cell], q1 = cell_start[cell + 1];
-    for (int j = threadIdx.x; j < nj; j += blockDim.x) {
-        const int c = j / np, q = j - c * np;
-        const int pd = np == 1 ? 0 : kProd[q], pm = np == 1 ? 0 : kMProd[q];
-        float2 acc[4];
+// Partial sums of one chunk for 32 channels: part[h][channel][chunk][16 cells]
+// (h = 0: G_XX + i G_YY, or G_XX for one pol; h = 1: G_XY).  The warps take the
+// chunk's records in turn and their sums are added in warp order.
+//
+// The work is 16 (real taps) complex multiply-adds a record, lane and plane
+// pair, on operands that are uniform (coefficients) or one 32-byte sector a
+// lane (a pair's products of one channel): bound by issue, then L2.  A per-cell
+// list walked by threads over (channel, product), after a transpose of the
+// visibilities, read each pair's products for each of its 25 cells:
+// 583 us after a 37 us transpose for the 64 channels of a 256-element station,
+// now 193 us.  A chunk of 256 records keeps the patches around zero lag,
+// which hold several thousand, from setting the time.
+template <int P, bool REAL, bool VEC>
+__global__ void __launch_bounds__(32 * kGatherWarps, 2) xfft_gather_kernel(
+    const int32_t *__restrict__ vis, long long nbl, int c0, int cb, const Chunk *__restrict__ chunks, int nchunk,
+    const uint32_t *__restrict__ rec, const float *__restrict__ coef, float2 *__restrict__ part) {
+    constexpr int H = P;                               // plane pairs
+    extern __shared__ float2 sums[];                   // [warps][H][16][33]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const Chunk ch = chunks[blockIdx.x];
+    const int cg = blockIdx.y * 32, c = min(cg + lane, cb - 1);
+    const int32_t *v = vis + (size_t)(c0 + c) * nbl * (2 * P * P);
+    float2 acc[H][kPcells];
 #pragma unroll
-        for (int u = 0; u < 4; u++) acc[u] = make_float2(0.f, 0.f);
-        int e = q0;
-        for (; e + 4 <= q1; e += 4) {
-            int32_t en[4];
-            float2 kv[4], v[4];
+    for (int h = 0; h < H; h++)
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                en[u] = ent[e + u];
-                kv[u] = kab[e + u];
-            }
+        for (int i = 0; i < kPcells; i++) acc[h][i] = make_float2(0.f, 0.f);
+    constexpr int D = 2;                               // records in flight per warp
+    for (int q = ch.q0 + warp; q < ch.q1; q += D * kGatherWarps) {
+        uint32_t r[D];
+        int4 va[D], vb[D];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const long long bl = en[u] & 0x7fffffff;
-                v[u] = vt[(bl * cb + c) * PP + (en[u] < 0 ? pm : pd)];
-            }
+        for (int d = 0; d < D; d++) r[d] = __ldg(rec + min(q + d * kGatherWarps, ch.q1 - 1));
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const float2 t = cmul(v[u], kv[u]);
-                acc[u].x += t.x;
-                acc[u].y += en[u] < 0 ? -t.y : t.y;
+        for (int d = 0; d < D; d++) {
+            const int32_t *p = v + (size_t)(r[d] & (kAuto - 1)) * (2 * P * P);
+            if (P == 1) {
+                const int2 x = __ldg(reinterpret_cast<const int2 *>(p));
+                va[d] = make_int4(x.x, x.y, 0, 0);
+            } else if (VEC) {
+                va[d] = __ldg(reinterpret_cast<const int4 *>(p));
+                vb[d] = __ldg(reinterpret_cast<const int4 *>(p) + 1);
+            } else {
+                const int2 *w = reinterpret_cast<const int2 *>(p);
+                const int2 x = __ldg(w), y = __ldg(w + 1), z = __ldg(w + 2), u = __ldg(w + 3);
+                va[d] = make_int4(x.x, x.y, y.x, y.y);
+                vb[d] = make_int4(z.x, z.y, u.x, u.y);
             }
         }
-        for (; e < q1; e++) {
-            const int32_t en = ent[e];
-            const long long bl = en & 0x7fffffff;
-            const float2 t = cmul(vt[(bl * cb + c) * PP + (en < 0 ? pm : pd)], kab[e]);
-            acc[0].x += t.x;
-            acc[0].y += en < 0 ? -t.y : t.y;
+#pragma unroll
+        for (int d = 0; d < D; d++) {
+            const int qd = q + d * kGatherWarps;
+            if (qd >= ch.q1) break;
+            const bool mirror = r[d] & kMirror, self = r[d] & kAuto;
+            float2 g[H];
+            if (P == 1) {
+                g[0] = make_float2((float)va[d].x, self ? 0.f : mirror ? -(float)va[d].y : (float)va[d].y);
+            } else {
+                const float xr = (float)va[d].x, xi = self ? 0.f : (float)va[d].y;
+                const float yr = (float)vb[d].z, yi = self ? 0.f : (float)vb[d].w;
+                // the pair: XX + i YY, XY; its mirror: conj(XX) + i conj(YY), conj(YX)
+                g[0] = mirror ? make_float2(xr + yi, yr - xi) : make_float2(xr - yi, xi + yr);
+                g[H - 1] = mirror ? make_float2((float)vb[d].x, -(float)vb[d].y) : make_float2((float)va[d].z, (float)va[d].w);
+            }
+            const float4 *cf = reinterpret_cast<const float4 *>(coef) + (size_t)qd * (REAL ? 4 : 8);
+#pragma unroll
+            for (int j = 0; j < (REAL ? 4 : 8); j++) {
+                const float4 k = __ldg(cf + j);
+                if (REAL) {
+                    const float kk[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+#pragma unroll
+                        for (int h = 0; h < H; h++)
+                            acc[h][4 * j + i] = __ffma2_rn(make_float2(kk[i], kk[i]), g[h], acc[h][4 * j + i]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 2; i++) {
+                        const float kr = i ? k.z : k.x, ki = i ? k.w : k.y;
+#pragma unroll
+                        for (int h = 0; h < H; h++) {
+                            float2 &a = acc[h][2 * j + i];
+                            a.x = fmaf(kr, g[h].x, fmaf(-ki, g[h].y, a.x));
+                            a.y = fmaf(kr, g[h].y, fmaf(ki, g[h].x, a.y));
+                        }
+                    }
+                }
+            }
         }
-        const float sx = (acc[0].x + acc[1].x) + (acc[2].x + acc[3].x);
-        const float sy = (acc[0].y + acc[1].y) + (acc[2].y + acc[3].y);
-        grid[((size_t)c * np + q) * NN + cell] = make_float2(sgn * sx, sgn * sy);
+    }
+#pragma unroll
+    for (int h = 0; h < H; h++)
+#pragma unroll
+        for (int i = 0; i < kPcells; i++) sums[((warp * H + h) * kPcells + i) * 33 + lane] = acc[h][i];
+    __syncthreads();
+    for (int i = threadIdx.x; i < H * 32 * kPcells; i += 32 * kGatherWarps) {
+        const int cell = i % kPcells, l = i / kPcells % 32, h = i / (kPcells * 32);
+        if (cg + l >= cb) continue;
+        float2 t = sums[(h * kPcells + cell) * 33 + l];
+#pragma unroll
+        for (int w = 1; w < kGatherWarps; w++) {
+            const float2 u = sums[((w * H + h) * kPcells + cell) * 33 + l];
+            t.x += u.x;
+            t.y += u.y;
+        }
+        part[(((size_t)h * cb + cg + l) * nchunk + blockIdx.x) * kPcells + cell] = t;
     }
 }
 
-// In-place radix-2 FFT (exponent +) of n points in bit-reversed order at
-// x[0], x[s], ... by one warp; tw[k] = exp(+2 pi i k / n), k < n / 2.
-__device__ void warp_fft(float2 *x, int s, int n, int log2n, const float2 *tw, int lane) {
-    for (int lh = 0; lh < log2n; lh++) {
-        const int half = 1 << lh, tshift = log2n - 1 - lh;
-        for (int b = lane; b < n / 2; b += 32) {
-            const int pos = b & (half - 1);
-            const int i0 = ((b - pos) << 1) + pos, i1 = i0 + half;
-            const float2 a = x[i0 * s];
-            const float2 t = cmul(x[i1 * s], tw[pos << tshift]);
-            x[i0 * s] = make_float2(a.x + t.x, a.y + t.y);
-            x[i1 * s] = make_float2(a.x - t.x, a.y - t.y);
+// One CTA per (channel, plane pair): the cells' partial sums (in chunk order)
+// with the checkerboard, rows, columns.  h = 0 -> XX (real part) and YY
+// (imaginary part), h = 1 -> Re XY, Im XY.  Lines in registers, exchanged in
+// their own row or column of the shared tile; the row stride keeps a
+// half-warp's rows on distinct banks.
+template <int N>
+__global__ void __launch_bounds__(N *hai_fft::Line<N>::L) xfft_fft_kernel(const float2 *__restrict__ part,
+                                                                         const int32_t *__restrict__ pstart, int nchunk,
+                                                                         int cb, int P, int c0, float *__restrict__ img,
+                                                                         int accumulate) {
+    constexpr int L = hai_fft::Line<N>::L, E = hai_fft::Line<N>::E, S = N + (L == 8 ? 8 : 4), NT = N * L;
+    __shared__ float2 sm[N * S], tw[N];
+    const int c = blockIdx.x, h = blockIdx.y, tid = threadIdx.x;
+    hai_fft::fill_twiddles<N>(tw);
+    const float2 *src = part + ((size_t)h * cb + c) * nchunk * kPcells;
+    for (int i = tid; i < N * N; i += NT) {           // patch by patch: 128-byte runs
+        const int p = i / kPcells, cell = i % kPcells;
+        const int x = p % (N / kPs) * kPs + cell % kPs, y = p / (N / kPs) * kPs + cell / kPs;
+        float2 s = make_float2(0.f, 0.f);
+        for (int q = pstart[p]; q < pstart[p + 1]; q++) {
+            const float2 v = src[(size_t)q * kPcells + cell];
+            s.x += v.x;
+            s.y += v.y;
         }
+        sm[y * S + x] = (x + y) & 1 ? make_float2(-s.x, -s.y) : s;
+    }
+    __syncthreads();
+    float2 a[E];
+    {
+        const int t = tid % L;
+        float2 *row = sm + (tid / L) * S;
+#pragma unroll
+        for (int m = 0; m < E; m++) a[m] = row[t + L * m];
+        hai_fft::line_first<N>(a, t, tw);
         __syncwarp();
+#pragma unroll
+        for (int k = 0; k < E; k++) row[L * k + ((t + k) & (L - 1))] = a[k];
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < E / L; u++)
+#pragma unroll
+            for (int i = 0; i < L; i++) a[L * u + i] = row[L * (t + L * u) + ((i + t) & (L - 1))];
+        hai_fft::line_second<N>(a);
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < E / L; u++)
+#pragma unroll
+            for (int i = 0; i < L; i++) row[t + L * u + E * i] = a[L * u + i];
     }
+    __syncthreads();
+    const int t = tid / N, x = tid % N;
+    float2 *col = sm + x;
+#pragma unroll
+    for (int m = 0; m < E; m++) a[m] = col[(t + L * m) * S];
+    hai_fft::line_first<N>(a, t, tw);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < E; k++) col[(L * k + t) * S] = a[k];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < E / L; u++)
+#pragma unroll
+        for (int i = 0; i < L; i++) a[L * u + i] = col[(L * (t + L * u) + i) * S];
+    hai_fft::line_second<N>(a);
+    const int Q = P == 2 ? 4 : 1;
+    float *o0 = img + ((size_t)(c0 + c) * Q + 2 * h) * N * N + x;
+#pragma unroll
+    for (int u = 0; u < E / L; u++)
+#pragma unroll
+        for (int i = 0; i < L; i++) {
+            const float2 v = a[L * u + i];
+            float *o = o0 + (size_t)(t + L * u + E * i) * N;
+            *o = accumulate ? *o + v.x : v.x;
+            if (P == 2) o[(size_t)N * N] = accumulate ? o[(size_t)N * N] + v.y : v.y;
+        }
 }
 
-// One CTA per (channel c, product q) grid: the grid lands bit-reversed along
-// both axes in a padded shared tile, rows then columns are transformed in
-// place, and the product goes to its image plane(s): q = 0 -> XX (real part),
-// 1 -> YY (real part), 2 -> Re XY, Im XY.
-__global__ void __launch_bounds__(256) xfft_fft_kernel(const float2 *__restrict__ grid, int N, int log2n, int np, int Q,
-                                                       int c0, float *__restrict__ img, int accumulate) {
-    extern __shared__ float2 sm[];
-    const int S = N + 1;                 // padded row stride
-    float2 *tw = sm + (size_t)N * S;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    const int c = blockIdx.x / np, q = blockIdx.x % np;
-    const float2 *g = grid + (size_t)blockIdx.x * N * N;
-    for (int k = threadIdx.x; k < N / 2; k += blockDim.x) {
-        float s, co;
-        sincospif((float)(2 * k) / (float)N, &s, &co);
-        tw[k] = make_float2(co, s);
-    }
-    for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
-        const int x = i % N, y = i / N;
-        sm[(__brev(y) >> (32 - log2n)) * S + (__brev(x) >> (32 - log2n))] = g[i];
-    }
-    __syncthreads();
-    for (int r = warp; r < N; r += nwarp) warp_fft(sm + (size_t)r * S, 1, N, log2n, tw, lane);
-    __syncthreads();
-    for (int col = warp; col < N; col += nwarp) warp_fft(sm + col, S, N, log2n, tw, lane);
-    __syncthreads();
-    const size_t NN = (size_t)N * N;
-    float *out = img + ((size_t)(c0 + c) * Q) * NN;
-    for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
-        const float2 v = sm[(i / N) * S + (i % N)];
-        if (q < 2) {
-            float *o = out + (size_t)q * NN + i;
-            *o = accumulate ? *o + v.x : v.x;
-        } else {
-            float *o = out + 2 * NN + i, *oi = out + 3 * NN + i;
-            *o = accumulate ? *o + v.x : v.x;
-            *oi = accumulate ? *oi + v.y : v.y;
-        }
-    }
+template <int P, bool REAL, bool VEC>
+hai_status launch_gather(hai_ctx *ctx, const hai_layout *L, const int32_t *vis, long long nbl, int c0, int cb,
+                         float2 *part, cudaStream_t st) {
+    auto kern = xfft_gather_kernel<P, REAL, VEC>;
+    HAI_CUDA_TRY(hai_allow_dyn_smem(kern, ctx->smem_optin));
+    const size_t smem = sizeof(float2) * kGatherWarps * P * kPcells * 33;
+    kern<<<dim3(L->xfft_nchunk, (cb + 31) / 32), 32 * kGatherWarps, smem, st>>>(
+        vis, nbl, c0, cb, static_cast<const Chunk *>(L->d_xchunk), L->xfft_nchunk, L->d_xrec, L->d_xcoef, part);
+    return HAI_OK;
+}
+
+template <int N>
+void launch_fft(const hai_layout *L, const float2 *part, int cb, int c0, float *img, int accumulate, cudaStream_t st) {
+    xfft_fft_kernel<N><<<dim3(cb, L->n_pol), N * hai_fft::Line<N>::L, 0, st>>>(part, L->d_xpatch, L->xfft_nchunk, cb,
+                                                                              L->n_pol, c0, img, accumulate);
 }
 
 }  // namespace
 
-// The layout's per-cell gridding list, built once on the host (FP32 K_ab,
-// summed in the order of the lag loops below) and kept with the layout.
+// The layout's patch records (binned on the host) and their coefficients (on
+// the GPU), built once and kept with the layout.
 static hai_status ensure_table(const hai_layout *L) {
     std::lock_guard<std::mutex> lock(L->xfft_mu);
-    if (L->d_xcell) return HAI_OK;
-    const int N = L->grid_n, K = L->ksize, ne = L->n_elem;
-    // at most 2 (2K-1)^2 entries per stored pair, 12 bytes each on the device
-    const double max_ent = (double)ne * (ne + 1) / 2 * 2.0 * (2 * K - 1) * (2 * K - 1);
+    if (L->d_xpatch) return HAI_OK;
+    const int N = L->grid_n, K = L->ksize, ne = L->n_elem, W = 2 * K - 1, np = N / kPs;
+    // contributions of all pairs to cells: 2 (2K-1)^2 per stored pair at most
+    const double max_ent = (double)ne * (ne + 1) / 2 * 2.0 * W * W;
     if (max_ent > 2.0e8)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_image: the layout's gridding list would exceed 2e8 entries");
-    const float2 *taps = reinterpret_cast<const float2 *>(L->h_taps.data());   // [ne][K][K], as given
     const int32_t *anc = L->h_anchors.data();
-    struct Ent {
-        int32_t cell, e;
-        float2 k;
-    };
-    std::vector<Ent> ents;
-    for (int a = 0, bl = 0; a < ne; a++)
-        for (int b = 0; b <= a; b++, bl++) {
-            const int dx0 = anc[2 * a] - anc[2 * b], dy0 = anc[2 * a + 1] - anc[2 * b + 1];
-            const float2 *ta = taps + (size_t)a * K * K, *tb = taps + (size_t)b * K * K;
-            for (int ey = -(K - 1); ey <= K - 1; ey++)
-                for (int ex = -(K - 1); ex <= K - 1; ex++) {
-                    // K_ab[e] = sum over tap pairs with (ua - ub, va - vb) = e of conj(w_a) w_b
-                    float2 k = make_float2(0.f, 0.f);
-                    for (int vb = std::max(0, -ey); vb < std::min(K, K - ey); vb++)
-                        for (int ub = std::max(0, -ex); ub < std::min(K, K - ex); ub++) {
-                            const float2 wa = ta[(vb + ey) * K + (ub + ex)], wb = tb[vb * K + ub];
-                            k.x += wa.x * wb.x + wa.y * wb.y;
-                            k.y += wa.x * wb.y - wa.y * wb.x;
-                        }
-                    if (k.x == 0.f && k.y == 0.f) continue;
-                    const int dx = (((dx0 + ex) % N) + N) % N, dy = (((dy0 + ey) % N) + N) % N;
-                    ents.push_back({dy * N + dx, bl, k});
-                    if (a != b) ents.push_back({((N - dy) % N) * N + (N - dx) % N, (int32_t)((uint32_t)bl | 0x80000000u), k});
+    // f(patch, record) for every patch that a footprint touches, each once
+    auto each_record = [&](auto &&f) {
+        uint32_t bl = 0;
+        for (int a = 0; a < ne; a++)
+            for (int b = 0; b <= a; b++, bl++)
+                for (int mirror = 0; mirror < (a == b ? 1 : 2); mirror++) {
+                    const int sg = mirror ? -1 : 1;
+                    const int x = (sg * (anc[2 * a] - anc[2 * b]) - (K - 1)) & (N - 1);
+                    const int y = (sg * (anc[2 * a + 1] - anc[2 * b + 1]) - (K - 1)) & (N - 1);
+                    const int nx = std::min(np, (x + W - 1) / kPs - x / kPs + 1);
+                    const int ny = std::min(np, (y + W - 1) / kPs - y / kPs + 1);
+                    const uint32_t r = bl | (mirror ? kMirror : 0u) | (a == b ? kAuto : 0u);
+                    for (int j = 0; j < ny; j++)
+                        for (int i = 0; i < nx; i++) f((y / kPs + j) % np * np + (x / kPs + i) % np, r);
                 }
-        }
-    std::vector<int32_t> start((size_t)N * N + 1, 0), ent(std::max<size_t>(1, ents.size()));
-    std::vector<float2> kv(std::max<size_t>(1, ents.size()));
-    for (const Ent &x : ents) start[x.cell + 1]++;
-    for (int c = 0; c < N * N; c++) start[c + 1] += start[c];
-    {
-        std::vector<int32_t> fill(start.begin(), start.end() - 1);
-        for (const Ent &x : ents) {
-            ent[fill[x.cell]] = x.e;
-            kv[fill[x.cell]++] = x.k;
-        }
+    };
+    std::vector<long long> fill((size_t)np * np + 1, 0);
+    each_record([&](int p, uint32_t) { fill[p + 1]++; });
+    std::vector<Chunk> chunks;
+    std::vector<int32_t> pstart((size_t)np * np + 1, 0);
+    for (int p = 0; p < np * np; p++) {
+        fill[p + 1] += fill[p];
+        for (long long q = fill[p]; q < fill[p + 1]; q += kChunk)
+            chunks.push_back(Chunk{p, (int32_t)q, (int32_t)std::min(q + kChunk, fill[p + 1])});
+        pstart[p + 1] = (int32_t)chunks.size();
     }
-    int32_t *d_start = nullptr, *d_ent = nullptr;
-    float2 *d_k = nullptr;
-    cudaError_t e = cudaMalloc(&d_start, sizeof(int32_t) * start.size());
-    if (e == cudaSuccess) e = cudaMalloc(&d_ent, sizeof(int32_t) * ent.size());
-    if (e == cudaSuccess) e = cudaMalloc(&d_k, sizeof(float2) * kv.size());
-    if (e == cudaSuccess) e = cudaMemcpy(d_start, start.data(), sizeof(int32_t) * start.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_ent, ent.data(), sizeof(int32_t) * ent.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_k, kv.data(), sizeof(float2) * kv.size(), cudaMemcpyHostToDevice);
+    const size_t nrec = (size_t)fill[(size_t)np * np];
+    std::vector<uint32_t> rec(nrec);
+    each_record([&](int p, uint32_t r) { rec[fill[p]++] = r; });
+    bool real = true;
+    for (size_t i = 1; i < L->h_taps.size(); i += 2) real &= L->h_taps[i] == 0.f;
+    const size_t coef_bytes = sizeof(float) * nrec * kPcells * (real ? 1 : 2);
+    int32_t *d_patch = nullptr;
+    uint32_t *d_rec = nullptr;
+    Chunk *d_chunk = nullptr;
+    float *d_coef = nullptr;
+    cudaError_t e = cudaMalloc(&d_patch, sizeof(int32_t) * pstart.size());
+    if (e == cudaSuccess) e = cudaMalloc(&d_rec, sizeof(uint32_t) * nrec);
+    if (e == cudaSuccess) e = cudaMalloc(&d_chunk, sizeof(Chunk) * chunks.size());
+    if (e == cudaSuccess) e = cudaMalloc(&d_coef, coef_bytes);
+    if (e == cudaSuccess) e = cudaMemcpy(d_patch, pstart.data(), sizeof(int32_t) * pstart.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_rec, rec.data(), sizeof(uint32_t) * nrec, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_chunk, chunks.data(), sizeof(Chunk) * chunks.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        (real ? xfft_coef_kernel<true> : xfft_coef_kernel<false>)<<<(unsigned)chunks.size(), 256>>>(
+            d_chunk, d_rec, L->d_anchors, L->d_taps, N, K, d_coef);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
-        cudaFree(d_start);
-        cudaFree(d_ent);
-        cudaFree(d_k);
-        return hai_cuda_fail(e, "hai_xfft_image: gridding list");
+        cudaFree(d_patch);
+        cudaFree(d_rec);
+        cudaFree(d_chunk);
+        cudaFree(d_coef);
+        return hai_cuda_fail(e, "hai_xfft_image: gridding table");
     }
-    L->d_xent = d_ent;
-    L->d_xk = d_k;
-    L->d_xcell = d_start;
-    L->dev_bytes += sizeof(int32_t) * (start.size() + ent.size()) + sizeof(float2) * kv.size();
+    L->d_xrec = d_rec;
+    L->d_xchunk = d_chunk;
+    L->d_xcoef = d_coef;
+    L->xfft_nchunk = (int)chunks.size();
+    L->xfft_real = real;
+    L->d_xpatch = d_patch;
+    L->dev_bytes += sizeof(int32_t) * pstart.size() + sizeof(uint32_t) * nrec + sizeof(Chunk) * chunks.size() + coef_bytes;
     return HAI_OK;
 }
 
@@ -253,26 +388,34 @@ extern "C" hai_status hai_xfft_image(hai_ctx *ctx, const hai_layout *L, const in
     const hai_status ws = hai_workspace(ctx);
     if (ws != HAI_OK) return ws;
     cudaStream_t st = (cudaStream_t)stream;
-    const int P = L->n_pol, PP = P * P, np = (P == 2) ? 3 : 1, Q = (P == 2) ? 4 : 1;
-    int log2n = 0;
-    while ((1 << log2n) < N) log2n++;
+    const int P = L->n_pol;
     const long long nbl = (long long)L->n_elem * (L->n_elem + 1) / 2;
-    // channels per batch: transposed visibilities and grids in the context's workspace
-    const size_t per_chan = sizeof(float2) * ((size_t)nbl * PP + (size_t)np * N * N);
-    const int cmax = (int)std::min<size_t>({(size_t)C, ctx->corr_ws_bytes / per_chan, (size_t)(256 / np) * 256});
-    if (cmax < 1) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_image: one channel exceeds the workspace");
-    float2 *vt = static_cast<float2 *>(ctx->d_corr_ws);
-    const size_t smem = sizeof(float2) * ((size_t)N * (N + 1) + N / 2);
+    // channels per batch: partial sums in the context's workspace
+    const size_t per_chan = sizeof(float2) * (size_t)P * L->xfft_nchunk * kPcells;
+    const int cmax = (int)std::min<size_t>({(size_t)C, ctx->corr_ws_bytes / per_chan, (size_t)32768});
+    // one channel's visibilities and grids as floats keep to the workspace's size too
+    if (cmax < 1 || sizeof(float2) * ((size_t)nbl * P * P + (size_t)(P == 2 ? 3 : 1) * N * N) > ctx->corr_ws_bytes)
+        return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_image: one channel exceeds the workspace");
+    float2 *part = static_cast<float2 *>(ctx->d_corr_ws);
+    const bool vec = ((uintptr_t)vis & 15) == 0;
     const int pidx = prof_begin(ctx, st);
     for (int c0 = 0; c0 < C; c0 += cmax) {
         const int cb = std::min(cmax, C - c0);
-        float2 *grid = vt + (size_t)nbl * cb * PP;
-        const long long n = nbl * cb * PP;
-        xfft_transpose_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 64LL * ctx->num_sms), 256, 0, st>>>(
-            vis, nbl, PP, c0, cb, vt);
-        xfft_gather_kernel<<<N * N, 256, 0, st>>>(vt, L->d_xcell, L->d_xent, L->d_xk, N, cb, np, PP, grid);
-        xfft_fft_kernel<<<cb * np, 256, smem, st>>>(grid, N, log2n, np, Q, c0, img, accumulate);
-        prof_count(ctx, 3);
+        hai_status s;
+        if (P == 1)
+            s = L->xfft_real ? launch_gather<1, true, false>(ctx, L, vis, nbl, c0, cb, part, st)
+                             : launch_gather<1, false, false>(ctx, L, vis, nbl, c0, cb, part, st);
+        else if (L->xfft_real)
+            s = vec ? launch_gather<2, true, true>(ctx, L, vis, nbl, c0, cb, part, st)
+                    : launch_gather<2, true, false>(ctx, L, vis, nbl, c0, cb, part, st);
+        else
+            s = vec ? launch_gather<2, false, true>(ctx, L, vis, nbl, c0, cb, part, st)
+                    : launch_gather<2, false, false>(ctx, L, vis, nbl, c0, cb, part, st);
+        if (s != HAI_OK) return s;
+        if (N == 16) launch_fft<16>(L, part, cb, c0, img, accumulate, st);
+        else if (N == 32) launch_fft<32>(L, part, cb, c0, img, accumulate, st);
+        else launch_fft<64>(L, part, cb, c0, img, accumulate, st);
+        prof_count(ctx, 2);
     }
     prof_end(ctx, pidx, st);
     HAI_CUDA_TRY(cudaGetLastError());
