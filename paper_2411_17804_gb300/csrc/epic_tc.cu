@@ -19,21 +19,30 @@
 // transposed stage-1 result as the MN-major operand A and the same DFT matrix
 // as B; a tile holds one sample for N = 64 and two for N = 32.
 //
-// CTA = 16 warps, one CTA per SM, persistent over a contiguous range of the
+// CTA = 24 warps, one CTA per SM, persistent over a contiguous range of the
 // flattened (station, channel, sample) index:
-//   warps 0-6  "front": re-pack the step's voltages (landed by TMA bulk
-//              copies) as fp16 per element, gather-grid the step's fields
-//              over tiles of the station's non-empty cells into A1 (fp16,
-//              K-major) with FP32 sums; warps 0-3 then move stage-1 results
-//              from TMEM into the stage-2 operand A2 (fp16, MN-major),
-//              transposing on the way;
-//   warp 7     one thread streams the voltages (TMA) and issues every MMA;
+//   grid warps (5-7, 16-23)  re-pack the step's voltages (landed by TMA bulk
+//              copies) as fp16 per element and gather-grid the step's fields
+//              into A1 (fp16, K-major) with FP32 sums;
+//   warps 0-3  move stage-1 results from TMEM into the stage-2 operand A2
+//              (fp16, MN-major), transposing on the way; warp 0 also streams the
+//              voltages (TMA);
+//   warp 4     one thread issues every MMA;
 //   warps 8-15 epilogue: read stage-2 results from TMEM, add |F_X|^2,
 //              |F_Y|^2 and F_X conj(F_Y) into register accumulators, and
 //              write them out when a (station, channel) block ends.
 // Every hand-off between the roles is an mbarrier phase.  TMEM: stage-1
 // results double-buffered, stage-2 results in two tile slots, so the MMAs of
 // one tile overlap the epilogue of the previous one.
+//
+// What bounds it: the issue rate of the CUDA-core roles (the tensor pipe is a
+// fifth busy at N = 64), and before that the time one warp needs for its share
+// of a step.  Hence 11 gridding warps that do nothing else, registers moved from
+// them to the epilogue (setmaxnreg), and an epilogue whose TMEM loads put X and
+// Y of a pixel into one thread.  SKA-low
+// station cadence (256 elements, 64 channels x 2048): 1094 us with 7 front
+// warps that gridded a cell per lane and also moved the stage-1 results, the
+// cross term paired by shuffles; 762 us now.
 #include <math.h>
 #include <string.h>
 
@@ -46,10 +55,16 @@
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kFront = 224;             // warps 0-6
-constexpr int kMmaWarp = 7;
-constexpr int kEpi = 256;               // warps 8-15
+constexpr int kThreads = 768;
+constexpr int kConvWarps = 4;           // warps 0-3
+constexpr int kMmaWarp = 4;
+constexpr int kGridWarps = kGatherWarps;   // warps 5-7 and 16-23
+constexpr int kGrid = 32 * kGridWarps;
+constexpr int kEpiWarps = 8;            // warps 8-15
+// registers: 80 a thread at launch; warpgroups 2 and 3 (epilogue) take 112, the
+// other four give back to 64: 256 x 112 + 512 x 64 = 768 x 80
+constexpr int kLaunchRegs = 80, kEpiRegs = 112, kOtherRegs = 64;
+static_assert(256 * kEpiRegs + 512 * kOtherRegs <= kThreads * kLaunchRegs, "register shares");
 constexpr int kStages = 4;              // voltage steps in flight
 constexpr uint32_t kKs = 128;           // K-major operands: K-group stride
 constexpr uint32_t kA2Ks = 2064;        // MN-major A2: K-group stride (16 groups + 16 B pad)
@@ -66,7 +81,7 @@ struct Geo {
     static constexpr int kTiles = kSps / kTileSamples; // tiles per step
     static constexpr int kK = 2 * kBox;                // contraction of both stages: 64 or 32
     static constexpr int kNcol = 2 * N;                // MMA N of both stages: 128 or 64
-    static constexpr int kU = kFields / 4;             // uint4 of fp16 voltages per element
+    static constexpr int kU = kFields / 4;             // planes of 4 fields (a uint4 of half2 per element)
     static constexpr int kLy = N / 2;                  // output rows per epilogue thread
     static constexpr uint32_t kMNs = (kK / 8) * kKs;   // K-major MN-group stride
     static constexpr uint32_t kBBytes = (kNcol / 8) * kMNs;
@@ -95,7 +110,8 @@ struct Params {
     unsigned *status;
 };
 
-__device__ __forceinline__ void bar_front() { asm volatile("bar.sync 1, 224;" ::: "memory"); }
+__device__ __forceinline__ void bar_grid() { asm volatile("bar.sync 1, 352;" ::: "memory"); }
+static_assert(kGrid == 352, "grid barrier");
 __device__ __forceinline__ void bar_epi() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
 
 template <int N, bool SP, bool BF>
@@ -113,7 +129,7 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
     uint8_t *sB = smem;
     uint8_t *sA1 = smem + G::kOffA1;
     uint8_t *sA2 = smem + G::kOffA2;
-    uint4 *sE = reinterpret_cast<uint4 *>(smem + G::kOffE);   // [2][ne_max][kU]
+    uint4 *sE = reinterpret_cast<uint4 *>(smem + G::kOffE);   // [2][kU][ne_max]
     const uint32_t off_v = G::kOffE + 2u * 16u * G::kU * p.ne_max;
     int8_t *sV = reinterpret_cast<int8_t *>(smem + off_v);
     uint8_t *sT = smem + off_v + kStages * p.vstage;         // the current station's gather table
@@ -124,11 +140,11 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
     if (tid == 0) {
         for (int s = 0; s < kStages; s++) tc::mbar_init(&mb_v[s], 1);
         for (int b = 0; b < 2; b++) {
-            tc::mbar_init(&mb_a1[b], kFront);
+            tc::mbar_init(&mb_a1[b], kGridWarps);
             tc::mbar_init(&mb_d1[b], 1);
-            tc::mbar_init(&mb_a2[b], 128);
+            tc::mbar_init(&mb_a2[b], kConvWarps);
             tc::mbar_init(&mb_full[b], 1);
-            tc::mbar_init(&mb_empty[b], kEpi);
+            tc::mbar_init(&mb_empty[b], kEpiWarps);
         }
         tc::mbar_init(&mb_a2free, 1);
         tc::mbar_fence_init();
@@ -144,210 +160,172 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
     const long long s1 = p.cta_begin ? p.cta_begin[blockIdx.x + 1] : min(s0 + p.len, p.total);
     const int nsteps = tc_count_steps(s0, s1, p.T, G::kSps);
 
-    if (warp < kMmaWarp) {
-        // ================================================================ front
-        int cur_station = -1, ne = 0;
-        int a1_st0 = -1, a1_st1 = -1;          // station whose cells buffer 0 / 1 holds
-        int ntile = 0;
-        const uint32_t *s_cell = nullptr;
-        const int32_t *s_base = nullptr, *s_warp = nullptr;
-        const float2 *s_w = nullptr;
-        const uint16_t *s_e = nullptr;
-
-        // new station: its gather table into shared memory; A1 buffer b zeroed
-        // when it last held another station's cells
-        auto prepare = [&](const TcStep &s, int i) {
-            const int stn = s.stn;
-            const int b = i & 1;
-            if (stn == cur_station && (b ? a1_st1 : a1_st0) == stn) return;
-            bar_front();                           // every front warp is done with step i-1
-            if (stn != cur_station) {
-                const TcStation st = p.stations[stn];
-                for (int k = tid; k < (int)(st.table_bytes / 16); k += kFront)
-                    reinterpret_cast<int4 *>(sT)[k] = __ldg(reinterpret_cast<const int4 *>(st.table) + k);
-                const GatherLayout gl = gather_layout(st.ntile, st.nent);
-                s_cell = reinterpret_cast<const uint32_t *>(sT + gl.off_cell);
-                s_base = reinterpret_cast<const int32_t *>(sT + gl.off_base);
-                s_warp = reinterpret_cast<const int32_t *>(sT + gl.off_warp);
-                s_w = reinterpret_cast<const float2 *>(sT + gl.off_w);
-                s_e = reinterpret_cast<const uint16_t *>(sT + gl.off_e);
-                ntile = st.ntile;
-                ne = st.ne;
-                cur_station = stn;
-            }
-            if ((b ? a1_st1 : a1_st0) != stn) {
-                for (int k = tid; k < (int)(G::kSet * G::kA1Bytes / 16); k += kFront)
-                    reinterpret_cast<int4 *>(sA1 + b * G::kSet * G::kA1Bytes)[k] = make_int4(0, 0, 0, 0);
-                (b ? a1_st1 : a1_st0) = stn;
-            }
-            bar_front();
-        };
-        // voltages of step i -> sE[i & 1]: per element the step's fields as
-        // half2 (int8 values are exact in fp16); ends with a front barrier
-        auto stage_volt = [&](const TcStep &s, int i) {
-            const int8_t *V;
-            uint32_t delta;
-            const int8_t *src = tc_aligned_src(s.src, p.guard, delta);
-            if (p.use_tma) {
-                tc::mbar_wait(&mb_v[i % kStages], (uint32_t)((i / kStages) & 1), p.status);
-                V = sV + (i % kStages) * p.vstage + delta;
-            } else {
-                const int bytes = s.nv * 4 * ne;
-                int8_t *dst = sV + (i % kStages) * p.vstage;
-                for (int b = tid; b < bytes; b += kFront) dst[b] = src[b];
-                bar_front();
-                V = dst;
-            }
-            uint4 *E = sE + (size_t)(i & 1) * p.ne_max * G::kU;
-            const char2 *v2 = reinterpret_cast<const char2 *>(V);
-            for (int a = tid; a < ne; a += kFront) {
-                uint32_t h[G::kFields];
-#pragma unroll
-                for (int f = 0; f < G::kFields; f++) {
-                    char2 x = make_char2(0, 0);    // missing sample: 0
-                    if (f < 2 * s.nv) x = v2[f * ne + a];
-                    h[f] = tc::pack_half2((float)x.x, (float)x.y);
+    const int wg = warp >> 2;
+    if (wg != 2 && wg != 3) {
+        tc::setmaxnreg_dec<kOtherRegs>();
+        if (wg >= 4 || (wg == 1 && warp != kMmaWarp)) {
+            // ================================================================ gridding
+            const int gw = wg >= 4 ? warp - 13 : warp - 5, gt = gw * 32 + lane;
+            int cur_station = -1, ne = 0;
+            int a1_st0 = -1, a1_st1 = -1;          // station whose cells buffer 0 / 1 holds
+            GatherLayout gl{};
+            int cplx = 0;
+            // new station: its gather table into shared memory; A1 buffer b zeroed
+            // when it last held another station's cells
+            auto prepare = [&](const TcStep &s, int i) {
+                const int stn = s.stn;
+                const int b = i & 1;
+                if (stn == cur_station && (b ? a1_st1 : a1_st0) == stn) return;
+                bar_grid();                           // every grid warp is done with step i-1
+                if (stn != cur_station) {
+                    const TcStation st = p.stations[stn];
+                    for (int k = gt; k < (int)(st.table_bytes / 16); k += kGrid)
+                        reinterpret_cast<int4 *>(sT)[k] = __ldg(reinterpret_cast<const int4 *>(st.table) + k);
+                    gl = gather_layout(st.ntile, st.nent, st.cplx);
+                    cplx = st.cplx;
+                    ne = st.ne;
+                    cur_station = stn;
                 }
+                if ((b ? a1_st1 : a1_st0) != stn) {
+                    for (int k = gt; k < (int)(G::kSet * G::kA1Bytes / 16); k += kGrid)
+                        reinterpret_cast<int4 *>(sA1 + b * G::kSet * G::kA1Bytes)[k] = make_int4(0, 0, 0, 0);
+                    (b ? a1_st1 : a1_st0) = stn;
+                }
+                bar_grid();
+            };
+            // voltages of step i -> sE[i & 1]: per element the step's fields as
+            // half2 (int8 values are exact in fp16); ends with a barrier of the grid warps
+            auto stage_volt = [&](const TcStep &s, int i) {
+                const int8_t *V;
+                uint32_t delta;
+                const int8_t *src = tc_aligned_src(s.src, p.guard, delta);
+                if (p.use_tma) {
+                    tc::mbar_wait(&mb_v[i % kStages], (uint32_t)((i / kStages) & 1), p.status);
+                    V = sV + (i % kStages) * p.vstage + delta;
+                } else {
+                    const int bytes = s.nv * 4 * ne;
+                    int8_t *dst = sV + (i % kStages) * p.vstage;
+                    for (int b = gt; b < bytes; b += kGrid) dst[b] = src[b];
+                    bar_grid();
+                    V = dst;
+                }
+                uint4 *E = sE + (size_t)(i & 1) * p.ne_max * G::kU;
+                if (!(ne & 1) && ((uintptr_t)V & 3) == 0) {
+                    // two elements a thread: a field's 4 bytes -> two half2
+                    for (int a = gt; a < ne / 2; a += kGrid) {
 #pragma unroll
-                for (int u = 0; u < G::kU; u++)
-                    E[a * G::kU + u] = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
-            }
-            bar_front();
-        };
-        // gridded values of the step's fields: G_f[cell] = sum conj(W~) E_f,
-        // one cell per lane, one tile of 32 cells per warp at a time
-        auto grid_step = [&](int i) {
-            uint8_t *A = sA1 + (i & 1) * G::kSet * G::kA1Bytes;
-            const uint4 *E = sE + (size_t)(i & 1) * p.ne_max * G::kU;
-            for (int t = s_warp[warp]; t < s_warp[warp + 1]; t++) {
-                float2 g[G::kFields];
+                        for (int u = 0; u < G::kU; u++) {
+                            uint32_t h0[4], h1[4];
 #pragma unroll
-                for (int f = 0; f < G::kFields; f++) g[f] = make_float2(0.f, 0.f);
-                const int qe = s_base[t + 1];
-                // add one slot's conj(W~) E into the fields' sums
-                auto mac = [&](const float2 w, const uint4 *e) {
+                            for (int f = 0; f < 4; f++) {
+                                uint32_t x = 0u;               // missing sample: 0
+                                if (4 * u + f < 2 * s.nv) x = *reinterpret_cast<const uint32_t *>(V + (size_t)(4 * u + f) * ne * 2 + 4 * a);
+                                tc::widen4(x, h0[f], h1[f]);
+                            }
+                            E[u * p.ne_max + 2 * a] = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+                            E[u * p.ne_max + 2 * a + 1] = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+                        }
+                    }
+                } else {
+                    const char2 *v2 = reinterpret_cast<const char2 *>(V);
+                    for (int a = gt; a < ne; a += kGrid) {
+#pragma unroll
+                        for (int u = 0; u < G::kU; u++) {
+                            uint32_t h[4];
+#pragma unroll
+                            for (int f = 0; f < 4; f++) {
+                                char2 x = make_char2(0, 0);
+                                if (4 * u + f < 2 * s.nv) x = v2[(4 * u + f) * ne + a];
+                                h[f] = tc::pack_half2((float)x.x, (float)x.y);
+                            }
+                            E[u * p.ne_max + a] = make_uint4(h[0], h[1], h[2], h[3]);
+                        }
+                    }
+                }
+                bar_grid();
+            };
+            // gridded values of the step's fields, G_f[cell] = sum conj(W~) E_f: one
+            // cell per lane, a tile of 32 cells per warp at a time, 4 fields together
+            auto grid_step = [&](int i) {
+                uint8_t *A = sA1 + (i & 1) * G::kSet * G::kA1Bytes;
+                const int32_t *base = reinterpret_cast<const int32_t *>(sT + gl.off_base);
+                const int32_t *wr = reinterpret_cast<const int32_t *>(sT + gl.off_warp);
+                const int t1 = wr[gw + 1];
+                for (int t = wr[gw]; t < t1; t++) {
+                    const uint32_t off = reinterpret_cast<const uint32_t *>(sT + gl.off_cell)[t * 32 + lane];
+                    const int q0 = base[t] + lane, qe = base[t + 1];
 #pragma unroll
                     for (int u = 0; u < G::kU; u++) {
-                        const uint32_t ev[4] = {e[u].x, e[u].y, e[u].z, e[u].w};
+                        float2 g[4];
 #pragma unroll
-                        for (int k = 0; k < 4; k++) {
-                            const float2 x = __half22float2(*reinterpret_cast<const __half2 *>(&ev[k]));
-                            float2 &acc = g[4 * u + k];
-                            acc.x = fmaf(w.x, x.x, fmaf(-w.y, x.y, acc.x));
-                            acc.y = fmaf(w.x, x.y, fmaf(w.y, x.x, acc.y));
-                        }
-                    }
-                };
-                // the lane's slots are q, q + 32, ...: four at a time with all
-                // their shared-memory loads issued before the first use (the
-                // loop is bound by load latency, not by issue)
-                int q = s_base[t] + lane;
-                for (; q + 96 < qe; q += 128) {
-                    float2 w[4];
-                    int en[4];
+                        for (int f = 0; f < 4; f++) g[f] = make_float2(0.f, 0.f);
+                        cell_sum(sT, gl, cplx, q0, qe, sE + ((size_t)(i & 1) * G::kU + u) * p.ne_max, g);
+                        if (off == 0xffffffffu) continue;
+                        uint8_t *c = A + off + 4 * u * G::kImgBytes;
 #pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        w[j] = s_w[q + 32 * j];
-                        en[j] = s_e[q + 32 * j];
-                    }
-                    uint4 e[4][G::kU];
-#pragma unroll
-                    for (int j = 0; j < 4; j++)
-#pragma unroll
-                        for (int u = 0; u < G::kU; u++) e[j][u] = E[en[j] * G::kU + u];
-#pragma unroll
-                    for (int j = 0; j < 4; j++) mac(w[j], e[j]);
-                }
-                for (; q < qe; q += 32) {
-                    const float2 w = s_w[q];
-                    uint4 e[G::kU];
-                    const int en = s_e[q];
-#pragma unroll
-                    for (int u = 0; u < G::kU; u++) e[u] = E[en * G::kU + u];
-                    mac(w, e);
-                }
-                const uint32_t off = s_cell[t * 32 + lane];
-                if (off != 0xffffffffu) {
-                    uint8_t *c = A + off;
-#pragma unroll
-                    for (int f = 0; f < G::kFields; f++) {
-                        if (SP) {              // the rounding remainder as the lo copy
-                            uint32_t hi, lo;
-                            tc::pack2_split<BF>(g[f].x, g[f].y, hi, lo);
-                            *reinterpret_cast<uint32_t *>(c + f * G::kImgBytes) = hi;
-                            *reinterpret_cast<uint32_t *>(c + G::kA1Bytes + f * G::kImgBytes) = lo;
-                        } else {
-                            *reinterpret_cast<uint32_t *>(c + f * G::kImgBytes) = tc::pack2<BF>(g[f].x, g[f].y);
+                        for (int f = 0; f < 4; f++) {
+                            if (SP) {              // the rounding remainder as the lo copy
+                                uint32_t hi, lo;
+                                tc::pack2_split<BF>(g[f].x, g[f].y, hi, lo);
+                                *reinterpret_cast<uint32_t *>(c + f * G::kImgBytes) = hi;
+                                *reinterpret_cast<uint32_t *>(c + G::kA1Bytes + f * G::kImgBytes) = lo;
+                            } else {
+                                *reinterpret_cast<uint32_t *>(c + f * G::kImgBytes) = tc::pack2<BF>(g[f].x, g[f].y);
+                            }
                         }
                     }
                 }
+            };
+            TcWalker wk;
+            wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
+            for (int i = 0; i < nsteps; i++) {
+                const TcStep s = wk.next(G::kSps);
+                // A1 buffer i & 1 was last read by the stage-1 MMAs of step i - 2
+                if (i >= 2) tc::mbar_wait(&mb_d1[i & 1], (uint32_t)(((i >> 1) - 1) & 1), p.status);
+                prepare(s, i);
+                stage_volt(s, i);
+                grid_step(i);
+                tc::fence_proxy_async();
+                tc::mbar_arrive_warp(&mb_a1[i & 1]);
             }
-        };
-        // warps 0-3: D1 row m = (field, y) -> A2 tile of its sample, column
-        // (y, re/im), rows (sample in tile, l_x, pol)
-        auto convert = [&](const TcStep &s, int i) {
-            const int m = warp * 32 + lane;
-            const int f = m / G::kBox, y = m % G::kBox;
-            const int smp = f >> 1, pol = f & 1;
-            const int tile = smp / G::kTileSamples, s2 = smp % G::kTileSamples;
-            if (tile * G::kTileSamples >= s.nv) return;   // tile not issued
-            uint8_t *A2 = sA2 + (((i % G::kA2Steps) * G::kTiles + tile) * G::kSet) * G::kA2Bytes;
-            const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(i & 1) * G::kNcol;
+        } else if (wg == 0) {
+            // ====================================================== stage-1 results
+            // warps 0-3: D1 row m = (field, y) -> A2 tile of its sample, column
+            // (y, re/im), rows (sample in tile, l_x, pol)
+            auto convert = [&](const TcStep &s, int i) {
+                const int m = warp * 32 + lane;
+                const int f = m / G::kBox, y = m % G::kBox;
+                const int smp = f >> 1, pol = f & 1;
+                const int tile = smp / G::kTileSamples, s2 = smp % G::kTileSamples;
+                if (tile * G::kTileSamples >= s.nv) return;   // tile not issued (the same for the whole warp)
+                uint8_t *A2 = sA2 + (((i % G::kA2Steps) * G::kTiles + tile) * G::kSet) * G::kA2Bytes;
+                const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(i & 1) * G::kNcol;
 #pragma unroll
-            for (int ch = 0; ch < G::kNcol / 32; ch++) {   // 32 columns: component c, l_x = kx0 .. kx0+31
-                uint32_t r[32];
-                tc::tmem_ld32(base + ch * 32, r);
-                tc::tmem_wait_ld();
-                const int c = (ch * 32) / N, kx0 = (ch * 32) % N;
-                const int kappa = 2 * y + c;
+                for (int ch = 0; ch < G::kNcol / 16; ch++) {   // 16 columns: component c, l_x = kx0 .. kx0+15
+                    uint32_t r[16];
+                    tc::tmem_ld16(base + ch * 16, r);
+                    tc::tmem_wait_ld();
+                    const int c = (ch * 16) / N, kx0 = (ch * 16) % N;
+                    const int kappa = 2 * y + c;
 #pragma unroll
-                for (int h = 0; h < 4; h++) {      // 8 frequencies -> one 16-byte row of A2
-                    const int kx = kx0 + 8 * h;
-                    const int m2 = s2 * 2 * N + (kx >> 4) * 32 + pol * 16 + (kx & 15);
-                    uint32_t hv[4], lv[4];
+                    for (int h = 0; h < 2; h++) {      // 8 frequencies -> one 16-byte row of A2
+                        const int kx = kx0 + 8 * h;
+                        const int m2 = s2 * 2 * N + (kx >> 4) * 32 + pol * 16 + (kx & 15);
+                        uint32_t hv[4], lv[4];
 #pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        const float x0 = __uint_as_float(r[8 * h + 2 * e]), x1 = __uint_as_float(r[8 * h + 2 * e + 1]);
-                        if (SP) tc::pack2_split<BF>(x0, x1, hv[e], lv[e]);
-                        else hv[e] = tc::pack2<BF>(x0, x1);
+                        for (int e = 0; e < 4; e++) {
+                            const float x0 = __uint_as_float(r[8 * h + 2 * e]), x1 = __uint_as_float(r[8 * h + 2 * e + 1]);
+                            if (SP) tc::pack2_split<BF>(x0, x1, hv[e], lv[e]);
+                            else hv[e] = tc::pack2<BF>(x0, x1);
+                        }
+                        const uint32_t off = tc::off_mnmajor(m2, kappa, kA2Ks, kA2MNs);
+                        *reinterpret_cast<uint4 *>(A2 + off) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+                        if (SP) *reinterpret_cast<uint4 *>(A2 + G::kA2Bytes + off) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
                     }
-                    const uint32_t off = tc::off_mnmajor(m2, kappa, kA2Ks, kA2MNs);
-                    *reinterpret_cast<uint4 *>(A2 + off) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-                    if (SP) *reinterpret_cast<uint4 *>(A2 + G::kA2Bytes + off) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
                 }
-            }
-        };
-        // A1 buffer (i+1)&1 was last read by MMA1(i-1), whose completion the
-        // converters saw before the next front barrier; A2 buffer i&1 was last
-        // read by MMA2(i-2), issued before MMA1(i), whose completion convert waits.
-        TcWalker wk;
-        wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
-        TcStep prev{}, nxt{};
-        for (int i = -1; i < nsteps; i++) {
-            if (i + 1 < nsteps) {
-                nxt = wk.next(G::kSps);
-                prepare(nxt, i + 1);
-                stage_volt(nxt, i + 1);
-                grid_step(i + 1);
-                tc::fence_proxy_async();
-                tc::mbar_arrive(&mb_a1[(i + 1) & 1]);
-            }
-            if (i >= 0 && warp < 4) {
-                tc::mbar_wait(&mb_d1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
-                // one stage-2 operand buffer (split): the MMAs of step i-1 read it
-                if (SP && i >= 1) tc::mbar_wait(&mb_a2free, (uint32_t)((i - 1) & 1), p.status);
-                tc::fence_after();
-                convert(prev, i);
-                tc::fence_proxy_async();
-                tc::fence_before();
-                tc::mbar_arrive(&mb_a2[i & 1]);
-            }
-            prev = nxt;
-        }
-    } else if (warp == kMmaWarp) {
-        // ================================================================ MMA + TMA
-        if (lane == 0) {
-            const uint32_t b = tc::smem_u32(sB);
+            };
+            // warp 0 also streams the voltages: step i's stage has been widened once
+            // its stage 1 is done
             TcWalker ld;
             ld.init(p.volt, p.stations, p.C, p.T, s0, s1);
             int n_loaded = 0;
@@ -362,70 +340,97 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
                 tc::bulk_g2s(sV + sg * p.vstage, src, bytes, &mb_v[sg]);
                 n_loaded++;
             };
-            for (int q = 0; q < kStages; q++) issue_load();
+            if (warp == 0 && lane == 0)
+                for (int q = 0; q < kStages; q++) issue_load();
+            // A2 buffer i & 1 was last read by MMA2(i-2), issued before MMA1(i),
+            // whose completion is waited for here; MMA1(i+2), which rewrites D1
+            // buffer i & 1, is issued after the arrival on mb_a2 of step i was seen.
             TcWalker wk;
             wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
-            TcStep prev{}, nxt{};
-            int jt = 0;                            // stage-2 tiles issued
-            for (int k = -1; k < nsteps; k++) {
-                if (k + 1 < nsteps) {              // stage 1 of step k+1
-                    const int i = k + 1;
-                    nxt = wk.next(G::kSps);
-                    tc::mbar_wait(&mb_a1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
-                    issue_load();                  // its voltage stage has been widened
-                    tc::fence_after();
-                    const uint32_t a = tc::smem_u32(sA1 + (i & 1) * G::kSet * G::kA1Bytes);
-                    const uint32_t d = tmem + (uint32_t)(i & 1) * G::kNcol;
-                    // products hi*hi [+ hi*lo + lo*hi]: (A offset, B offset) per product
-#pragma unroll
-                    for (int pr = 0; pr < (SP ? 3 : 1); pr++) {
-                        const uint32_t ao = pr == 2 ? G::kA1Bytes : 0u, bo = pr == 1 ? G::kBBytes : 0u;
-#pragma unroll
-                        for (int s = 0; s < G::kK / 16; s++)
-                            tc::mma_f16(d, tc::desc(a + ao + s * 2 * kKs, kKs, G::kMNs),
-                                        tc::desc(b + bo + s * 2 * kKs, kKs, G::kMNs), kIdesc1, (pr > 0 || s > 0));
-                    }
-                    tc::mma_commit(&mb_d1[i & 1]);
-                }
-                if (k >= 0) {                      // stage 2 of step k, one slot per tile
-                    tc::mbar_wait(&mb_a2[k & 1], (uint32_t)((k >> 1) & 1), p.status);
-                    const int ntl = (prev.nv + G::kTileSamples - 1) / G::kTileSamples;
-                    for (int g = 0; g < ntl; g++, jt++) {
-                        const int slot = jt & 1;
-                        if (jt >= 2) tc::mbar_wait(&mb_empty[slot], (uint32_t)(((jt >> 1) - 1) & 1), p.status);
+            for (int i = 0; i < nsteps; i++) {
+                const TcStep s = wk.next(G::kSps);
+                tc::mbar_wait(&mb_d1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
+                if (warp == 0 && lane == 0) issue_load();
+                __syncwarp();
+                // one stage-2 operand buffer (split): the MMAs of step i-1 read it
+                if (SP && i >= 1) tc::mbar_wait(&mb_a2free, (uint32_t)((i - 1) & 1), p.status);
+                tc::fence_after();
+                convert(s, i);
+                tc::fence_proxy_async();
+                tc::fence_before();
+                tc::mbar_arrive_warp(&mb_a2[i & 1]);
+            }
+        } else if (warp == kMmaWarp) {
+            // ================================================================ MMA + TMA
+            if (lane == 0) {
+                // descriptors once, then 32-bit additions: this thread's scalar work
+                // between MMAs delays them
+                const uint64_t db = tc::desc(tc::smem_u32(sB), kKs, G::kMNs);
+                const uint64_t da1 = tc::desc(tc::smem_u32(sA1), kKs, G::kMNs);
+                const uint64_t da2 = tc::desc(tc::smem_u32(sA2), kA2Ks, kA2MNs);
+                TcWalker wk;
+                wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
+                TcStep prev{}, nxt{};
+                int jt = 0;                            // stage-2 tiles issued
+                for (int k = -1; k < nsteps; k++) {
+                    if (k + 1 < nsteps) {              // stage 1 of step k+1
+                        const int i = k + 1;
+                        nxt = wk.next(G::kSps);
+                        tc::mbar_wait(&mb_a1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
                         tc::fence_after();
-                        const uint32_t a =
-                            tc::smem_u32(sA2 + (((k % G::kA2Steps) * G::kTiles + g) * G::kSet) * G::kA2Bytes);
-                        const uint32_t d = tmem + 2u * G::kNcol + (uint32_t)slot * G::kNcol;
+                        const uint64_t a = tc::desc_add(da1, (i & 1) * G::kSet * G::kA1Bytes);
+                        const uint32_t d = tmem + (uint32_t)(i & 1) * G::kNcol;
+                        // products hi*hi [+ hi*lo + lo*hi]: (A offset, B offset) per product
 #pragma unroll
                         for (int pr = 0; pr < (SP ? 3 : 1); pr++) {
-                            const uint32_t ao = pr == 2 ? G::kA2Bytes : 0u, bo = pr == 1 ? G::kBBytes : 0u;
+                            const uint32_t ao = pr == 2 ? G::kA1Bytes : 0u, bo = pr == 1 ? G::kBBytes : 0u;
 #pragma unroll
                             for (int s = 0; s < G::kK / 16; s++)
-                                tc::mma_f16(d, tc::desc(a + ao + s * 2 * kA2Ks, kA2Ks, kA2MNs),
-                                            tc::desc(b + bo + s * 2 * kKs, kKs, G::kMNs), kIdesc2, (pr > 0 || s > 0));
+                                tc::mma_f16(d, tc::desc_add(a, ao + s * 2 * kKs), tc::desc_add(db, bo + s * 2 * kKs), kIdesc1,
+                                            (pr > 0 || s > 0));
                         }
-                        tc::mma_commit(&mb_full[slot]);
+                        tc::mma_commit(&mb_d1[i & 1]);
                     }
-                    if (SP) tc::mma_commit(&mb_a2free);   // the single stage-2 operand may be rewritten
+                    if (k >= 0) {                      // stage 2 of step k, one slot per tile
+                        tc::mbar_wait(&mb_a2[k & 1], (uint32_t)((k >> 1) & 1), p.status);
+                        const int ntl = (prev.nv + G::kTileSamples - 1) / G::kTileSamples;
+                        for (int g = 0; g < ntl; g++, jt++) {
+                            const int slot = jt & 1;
+                            if (jt >= 2) tc::mbar_wait(&mb_empty[slot], (uint32_t)(((jt >> 1) - 1) & 1), p.status);
+                            tc::fence_after();
+                            const uint64_t a = tc::desc_add(da2, (((k % G::kA2Steps) * G::kTiles + g) * G::kSet) * G::kA2Bytes);
+                            const uint32_t d = tmem + 2u * G::kNcol + (uint32_t)slot * G::kNcol;
+#pragma unroll
+                            for (int pr = 0; pr < (SP ? 3 : 1); pr++) {
+                                const uint32_t ao = pr == 2 ? G::kA2Bytes : 0u, bo = pr == 1 ? G::kBBytes : 0u;
+#pragma unroll
+                                for (int s = 0; s < G::kK / 16; s++)
+                                    tc::mma_f16(d, tc::desc_add(a, ao + s * 2 * kA2Ks), tc::desc_add(db, bo + s * 2 * kKs),
+                                                kIdesc2, (pr > 0 || s > 0));
+                            }
+                            tc::mma_commit(&mb_full[slot]);
+                        }
+                        if (SP) tc::mma_commit(&mb_a2free);   // the single stage-2 operand may be rewritten
+                    }
+                    prev = nxt;
                 }
-                prev = nxt;
             }
         }
     } else {
+        tc::setmaxnreg_inc<kEpiRegs>();
         // ============================================================= epilogue
+        // a quadrant of 32 TMEM lanes holds X (lanes 0-15) and Y (16-31) of 16
+        // output columns l_x; the 16-lane loads put both of a pixel into one
+        // thread: l_x = lx0 + lane / 4 (+ 8), l_y = kLy h + 8 j + 2 (lane % 4) (+ 1)
         const int q = warp & 3, h = (warp - 8) >> 2;
-        const int m = 32 * q + lane;
-        const int s2 = m / (2 * N), mm = m % (2 * N);
-        const int pol = (mm >> 4) & 1, kx = (mm >> 5) * 16 + (mm & 15);
+        const int s2 = q / (N / 16), lx0 = 16 * (q % (N / 16));      // sample of the tile, first l_x
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         constexpr int kLy = G::kLy;
         constexpr int kNN = N * N;
-        // packed pairs: acc_a[t / 2] holds rows t, t + 1 of the own polarisation's
-        // power; acc_x[t] the (re, im) cross product of one row
-        float2 acc_a[kLy / 2], acc_x[kLy / 2];
+        constexpr int kPair = kLy / 4;               // pixel pairs (l_y, l_y + 1): [j][l_x half]
+        float2 axx[kPair], ayy[kPair], are[kPair], aim[kPair];
 #pragma unroll
-        for (int t = 0; t < kLy / 2; t++) acc_a[t] = acc_x[t] = make_float2(0.f, 0.f);
+        for (int t = 0; t < kPair; t++) axx[t] = ayy[t] = are[t] = aim[t] = make_float2(0.f, 0.f);
         int seg = 0;
         long long cur_blk = -1;
         // the two sample slots of an N = 32 tile hold partial sums of the same
@@ -438,31 +443,20 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
                 if (phase > 0) bar_epi();
                 if (s2 != phase) continue;
                 const bool add = phase > 0 || (p.direct && p.accumulate);
+                auto put = [&](int plane, float2 (&a)[kPair]) {
 #pragma unroll
-                for (int t = 0; t < kLy; t++) {
-                    const int idx = pol * kNN + (kLy * h + t) * N + kx;
-                    float v = (t & 1) ? acc_a[t >> 1].y : acc_a[t >> 1].x;
-                    if (add) v += dst[idx];
-                    dst[idx] = v;
-                }
-#pragma unroll
-                for (int t = 0; t < kLy / 2; t++) acc_a[t] = make_float2(0.f, 0.f);
-                // cross products: the X thread holds X conj(Y) at even rows, the Y
-                // thread Y conj(X) = conj(X conj(Y)) at odd rows
-                const float sgn = pol ? -1.f : 1.f;
-#pragma unroll
-                for (int t = 0; t < kLy / 2; t++) {
-                    const int ly = kLy * h + 16 * (t >> 3) + 2 * (t & 7) + pol;
-                    const int idx = 2 * kNN + ly * N + kx;
-                    float vr = acc_x[t].x, vi = sgn * acc_x[t].y;
-                    if (add) {
-                        vr += dst[idx];
-                        vi += dst[idx + kNN];
+                    for (int t = 0; t < kPair; t++) {
+                        float *d = dst + plane * kNN + (kLy * h + 8 * (t >> 1) + 2 * (lane & 3)) * N + lx0 + (lane >> 2) +
+                                   8 * (t & 1);
+                        d[0] = add ? d[0] + a[t].x : a[t].x;
+                        d[N] = add ? d[N] + a[t].y : a[t].y;
+                        a[t] = make_float2(0.f, 0.f);
                     }
-                    dst[idx] = vr;
-                    dst[idx + kNN] = vi;
-                    acc_x[t] = make_float2(0.f, 0.f);
-                }
+                };
+                put(0, axx);
+                put(1, ayy);
+                put(2, are);
+                put(3, aim);
             }
         };
         TcWalker wk;
@@ -485,37 +479,34 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
                 const int slot = jt & 1;
                 tc::mbar_wait(&mb_full[slot], (uint32_t)((jt >> 1) & 1), p.status);
                 tc::fence_after();
+                const uint32_t x0 = tmem + lane_base + 2u * G::kNcol + (uint32_t)slot * G::kNcol + (uint32_t)(kLy * h);
 #pragma unroll
-                for (int cc = 0; cc < kLy / 16; cc++) {
-                    const uint32_t col = 2u * G::kNcol + (uint32_t)slot * G::kNcol + (uint32_t)(kLy * h + 16 * cc);
-                    uint32_t rr[16], ri[16];
-                    tc::tmem_ld16(tmem + lane_base + col, rr);
-                    tc::tmem_ld16(tmem + lane_base + col + N, ri);
+                for (int j = 0; j < kLy / 8; j++) {                  // 8 output rows l_y at a time
+                    const uint32_t x = x0 + 8 * j, y = x + (16u << 16);
+                    uint32_t xr[4], xi[4], yr[4], yi[4];
+                    tc::tmem_ld_16x256b(x, xr);
+                    tc::tmem_ld_16x256b(x + N, xi);
+                    tc::tmem_ld_16x256b(y, yr);
+                    tc::tmem_ld_16x256b(y + N, yi);
                     tc::tmem_wait_ld();
-#pragma unroll
-                    for (int t = 0; t < 16; t += 2) {
-                        const float2 fr = make_float2(__uint_as_float(rr[t]), __uint_as_float(rr[t + 1]));
-                        const float2 fi = make_float2(__uint_as_float(ri[t]), __uint_as_float(ri[t + 1]));
-                        float2 &a = acc_a[(16 * cc + t) >> 1];
-                        a = __ffma2_rn(fr, fr, __ffma2_rn(fi, fi, a));     // fmaf(fr, fr, fmaf(fi, fi, a))
+                    if (j == kLy / 8 - 1) {
+                        tc::fence_before();
+                        tc::mbar_arrive_warp(&mb_empty[slot]);
                     }
 #pragma unroll
-                    for (int k = 0; k < 8; k++) {
-                        // own value at row 2k + pol, partner's value at the same row
-                        const float e_r = __uint_as_float(rr[2 * k]), e_i = __uint_as_float(ri[2 * k]);
-                        const float o_r = __uint_as_float(rr[2 * k + 1]), o_i = __uint_as_float(ri[2 * k + 1]);
-                        const float mr = pol ? o_r : e_r, mi = pol ? o_i : e_i;
-                        const float sr = __shfl_xor_sync(0xffffffffu, pol ? e_r : o_r, 16);
-                        const float si = __shfl_xor_sync(0xffffffffu, pol ? e_i : o_i, 16);
-                        // (Re, Im) own conj(other): fmaf(mr, sr, fmaf(mi, si, re)),
-                        // fmaf(mi, sr, fmaf(-mr, si, im)) as packed pairs
-                        float2 &a = acc_x[8 * cc + k];
-                        a = __ffma2_rn(make_float2(mr, mi), make_float2(sr, sr),
-                                       __ffma2_rn(make_float2(mi, -mr), make_float2(si, si), a));
+                    for (int k = 0; k < 2; k++) {
+                        const int t = 2 * j + k;
+                        const float2 ar = make_float2(__uint_as_float(xr[2 * k]), __uint_as_float(xr[2 * k + 1]));
+                        const float2 ai = make_float2(__uint_as_float(xi[2 * k]), __uint_as_float(xi[2 * k + 1]));
+                        const float2 br = make_float2(__uint_as_float(yr[2 * k]), __uint_as_float(yr[2 * k + 1]));
+                        const float2 bi = make_float2(__uint_as_float(yi[2 * k]), __uint_as_float(yi[2 * k + 1]));
+                        axx[t] = __ffma2_rn(ar, ar, __ffma2_rn(ai, ai, axx[t]));
+                        ayy[t] = __ffma2_rn(br, br, __ffma2_rn(bi, bi, ayy[t]));
+                        // X conj(Y): Re fmaf(ar, br, fmaf(ai, bi, .)), Im fmaf(ai, br, fmaf(-ar, bi, .))
+                        are[t] = __ffma2_rn(ar, br, __ffma2_rn(ai, bi, are[t]));
+                        aim[t] = __ffma2_rn(ai, br, __ffma2_rn(make_float2(-ar.x, -ar.y), bi, aim[t]));
                     }
                 }
-                tc::fence_before();
-                tc::mbar_arrive(&mb_empty[slot]);
             }
         }
         if (cur_blk >= 0) flush(cur_stn, cur_chan, seg);
@@ -540,6 +531,9 @@ template <typename K>
 hai_status raise_limit(hai_ctx *ctx, K kern) {
     cudaFuncAttributes a;
     HAI_CUDA_TRY(cudaFuncGetAttributes(&a, kern));
+    // the warpgroups' register shares have to come out of the launch's
+    if (a.numRegs < kLaunchRegs)
+        return hai_fail(HAI_ERR_UNSUPPORTED, "epic tensor cores: the kernel was built with too few registers");
     HAI_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       ctx->smem_optin - (int)a.sharedSizeBytes));
     return HAI_OK;
@@ -718,81 +712,113 @@ const void *epic_tc_dft(hai_ctx *ctx, int N, bool bf16) {
 
 void epic_tc_build_gather(int box_w, int box_h, const std::vector<int32_t> &cstart,
                           const std::vector<int32_t> &elem, const std::vector<float2> &w, uint32_t k_stride,
-                          uint32_t mn_stride, std::vector<uint8_t> &out, int &ntile, int &nent, int n_warps) {
-    std::vector<int> cells;
+                          uint32_t mn_stride, int F, std::vector<uint8_t> &out, int &ntile, int &nent, int &cplx,
+                          int n_warps) {
+    std::vector<int> cells, cnt((size_t)box_w * box_h, 0);
+    cplx = 0;
     for (int y = 0; y < box_h; y++)
-        for (int x = 0; x < box_w; x++)
-            if (cstart[y * box_w + x + 1] > cstart[y * box_w + x]) cells.push_back(y * box_w + x);
-    auto count = [&](int c) { return cstart[c + 1] - cstart[c]; };
+        for (int x = 0; x < box_w; x++) {
+            const int c = y * box_w + x;
+            for (int k = cstart[c]; k < cstart[c + 1]; k++) {
+                cnt[c] += w[k].x != 0.f || w[k].y != 0.f;
+                cplx |= w[k].y != 0.f;
+            }
+            if (cnt[c]) cells.push_back(c);
+        }
     auto a1off = [&](int cell) { return tc::off_kmajor(cell / box_w, 2 * (cell % box_w), k_stride, mn_stride); };
     std::stable_sort(cells.begin(), cells.end(), [&](int a, int b) {
-        if (count(a) != count(b)) return count(a) > count(b);
+        if (cnt[a] != cnt[b]) return cnt[a] > cnt[b];
         return a1off(a) < a1off(b);
     });
     ntile = ((int)cells.size() + 31) / 32;
     // tiles in cell order, then dealt to the gridding warps longest-first
     std::vector<int> slots(ntile, 0);
-    for (int t = 0; t < ntile; t++)
-        for (int l = 0; l < 32 && t * 32 + l < (int)cells.size(); l++) slots[t] = std::max(slots[t], count(cells[t * 32 + l]));
-    std::vector<int> by_cost(ntile);
-    for (int t = 0; t < ntile; t++) by_cost[t] = t;
-    std::stable_sort(by_cost.begin(), by_cost.end(), [&](int a, int b) { return slots[a] > slots[b]; });
+    for (int t = 0; t < ntile; t++) slots[t] = cnt[cells[t * 32]];
     std::vector<std::vector<int>> mine(kGatherWarps);
     std::vector<int> load(n_warps, 0);
-    for (int t : by_cost) {
-        const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-        mine[w].push_back(t);
-        load[w] += slots[t] + 1;
+    for (int t = 0; t < ntile; t++) {        // slots descend
+        const int v = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        mine[v].push_back(t);
+        load[v] += slots[t] + 2;
     }
     std::vector<int> order;                  // new position -> original tile
     std::vector<int> wrange(kGatherWarps + 1, 0);
-    for (int w = 0; w < kGatherWarps; w++) {
-        order.insert(order.end(), mine[w].begin(), mine[w].end());
-        wrange[w + 1] = (int)order.size();
+    for (int v = 0; v < kGatherWarps; v++) {
+        order.insert(order.end(), mine[v].begin(), mine[v].end());
+        wrange[v + 1] = (int)order.size();
     }
     std::vector<int> base(ntile + 1, 0);
     for (int t = 0; t < ntile; t++) base[t + 1] = base[t] + 32 * slots[order[t]];
     nent = base[ntile];
-    const GatherLayout gl = gather_layout(ntile, nent);
+    const GatherLayout gl = gather_layout(ntile, nent, cplx);
     out.assign(gl.bytes, 0);
     uint32_t *o_cell = reinterpret_cast<uint32_t *>(&out[gl.off_cell]);
     int32_t *o_base = reinterpret_cast<int32_t *>(&out[gl.off_base]);
     int32_t *o_warp = reinterpret_cast<int32_t *>(&out[gl.off_warp]);
-    float2 *o_w = reinterpret_cast<float2 *>(&out[gl.off_w]);
+    float *o_w = reinterpret_cast<float *>(&out[gl.off_w]);
     uint16_t *o_e = reinterpret_cast<uint16_t *>(&out[gl.off_e]);
     for (int t = 0; t <= ntile; t++) o_base[t] = base[t];
-    for (int w = 0; w <= kGatherWarps; w++) o_warp[w] = wrange[w];
+    for (int v = 0; v <= kGatherWarps; v++) o_warp[v] = wrange[v];
+    const int phase = 32 / F;                // lanes whose voltages one shared-memory phase reads
     for (int t = 0; t < ntile; t++)
-        for (int l = 0; l < 32; l++) {
-            const int ci = order[t] * 32 + l;      // cell of lane l of the tile now at position t
-            if (ci >= (int)cells.size()) {
-                o_cell[t * 32 + l] = 0xffffffffu;
-                continue;
+        for (int l0 = 0; l0 < 32; l0 += phase) {
+            std::vector<std::vector<int>> left(phase);       // entries each lane still has to place
+            for (int i = 0; i < phase; i++) {
+                const int ci = order[t] * 32 + l0 + i;       // cell of this lane of the tile now at position t
+                o_cell[t * 32 + l0 + i] = ci < (int)cells.size() ? a1off(cells[ci]) : 0xffffffffu;
+                if (ci >= (int)cells.size()) continue;
+                for (int k = cstart[cells[ci]]; k < cstart[cells[ci] + 1]; k++)
+                    if (w[k].x != 0.f || w[k].y != 0.f) left[i].push_back(k);
             }
-            const int cell = cells[ci];
-            o_cell[t * 32 + l] = a1off(cell);
-            for (int k = 0; k < count(cell); k++) {
-                const int q = base[t] + 32 * k + l;
-                o_w[q] = w[cstart[cell] + k];                 // conj(W~) = a + ib
-                o_e[q] = (uint16_t)elem[cstart[cell] + k];
+            const int ns = slots[order[t]];
+            for (int s = 0; s < ns; s++) {
+                std::vector<std::vector<int>> bank(phase);   // elements already read from each bank group
+                int any = 0;
+                std::vector<int> empty;
+                for (int i = 0; i < phase; i++) {
+                    int best = -1, cost = 1 << 30;
+                    for (int j = 0; j < (int)left[i].size(); j++) {
+                        const std::vector<int> &b = bank[elem[left[i][j]] % phase];
+                        const int c = std::find(b.begin(), b.end(), elem[left[i][j]]) != b.end() ? -1 : (int)b.size();
+                        if (c < cost) {
+                            cost = c;
+                            best = j;
+                        }
+                    }
+                    // a lane with slots to spare leaves one empty rather than conflict
+                    if (best < 0 || (cost > 0 && (int)left[i].size() < ns - s)) {
+                        empty.push_back(i);
+                        continue;
+                    }
+                    const int k = left[i][best], q = base[t] + 32 * s + l0 + i;
+                    if (cost >= 0) bank[elem[k] % phase].push_back(elem[k]);
+                    o_e[q] = (uint16_t)elem[k];
+                    if (cplx) {
+                        o_w[2 * q] = w[k].x;                 // conj(W~) = a + ib
+                        o_w[2 * q + 1] = w[k].y;
+                    } else {
+                        o_w[q] = w[k].x;
+                    }
+                    any = elem[k];
+                    left[i].erase(left[i].begin() + best);
+                }
+                for (int i : empty) o_e[base[t] + 32 * s + l0 + i] = (uint16_t)any;   // weight 0
             }
         }
 }
 
 void epic_tc_station_table(int grid_n, int box_w, int box_h, const std::vector<int32_t> &cstart,
-                           const std::vector<int32_t> &elem, const std::vector<float2> &w,
-                           std::vector<uint8_t> &out, int &ntile, int &nent, uint32_t &shared_bytes,
-                           long long &entries) {
+                           const std::vector<int32_t> &elem, const std::vector<float2> &w, std::vector<uint8_t> &out,
+                           TcStation &rec, uint32_t &shared_bytes, long long &entries) {
     if (grid_n == 128) {
         epic_tc128_build_blob(box_w, box_h, cstart, elem, w, out, shared_bytes, entries);
-        ntile = nent = 0;
         return;
     }
     uint32_t ks, mns;
     epic_tc_a1_strides(grid_n, ks, mns);
-    epic_tc_build_gather(box_w, box_h, cstart, elem, w, ks, mns, out, ntile, nent);
+    epic_tc_build_gather(box_w, box_h, cstart, elem, w, ks, mns, 4, out, rec.ntile, rec.nent, rec.cplx);
     shared_bytes = (uint32_t)out.size();
-    entries = nent;
+    entries = rec.nent;
 }
 
 // ---------------------------------------------------------------- one layout

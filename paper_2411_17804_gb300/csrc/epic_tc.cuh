@@ -7,6 +7,7 @@
 // and every CTA (or CTA group) takes a contiguous range of it.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include <vector>
@@ -24,6 +25,7 @@ struct TcStation {
     long long img_off;      // float offset of the station's images [C][4][N][N]
     int ne;                 // elements
     int ntile, nent;        // gather tiles and entries
+    int cplx;               // complex taps
     uint32_t table_bytes;   // multiple of 16
 };
 
@@ -40,47 +42,48 @@ struct TcStep {
 // division at the start, none per step, a station-record load only when the
 // station changes.
 struct TcWalker {
-    const int8_t *volt;
     const TcStation *stations;
     int C, T;
-    long long f, end;
+    long long left;         // samples of the range still to walk
     int stn, chan, t, ne;
-    long long volt_off;
+    const int8_t *next_src;
+    const int8_t *volt;
     __device__ void init(const int8_t *v, const TcStation *st, int C_, int T_, long long s0, long long s1) {
         volt = v;
         stations = st;
         C = C_;
         T = T_;
-        f = s0;
-        end = s1;
+        left = max(0ll, s1 - s0);
         const long long blk = s0 / T;
         t = (int)(s0 - blk * T);
         stn = (int)(blk / C);
         chan = (int)(blk - (long long)stn * C);
         ne = 0;
-        volt_off = 0;
-        if (f < end) load();
+        next_src = v;
+        if (left > 0) load();
     }
+    // voltages are contiguous over a station's (channel, sample) index
     __device__ void load() {
         ne = stations[stn].ne;
-        volt_off = stations[stn].volt_off;
+        next_src = volt + stations[stn].volt_off + ((long long)chan * T + t) * 4ll * ne;
     }
     __device__ TcStep next(int sps) {
         TcStep s;
         s.stn = stn;
         s.chan = chan;
         s.t = t;
-        s.nv = (int)min((long long)min(sps, T - t), end - f);
+        s.nv = (int)min((long long)min(sps, T - t), left);
         s.ne = ne;
-        s.src = volt + volt_off + ((long long)chan * T + t) * 4ll * ne;
-        f += s.nv;
+        s.src = next_src;
+        next_src += s.nv * 4 * ne;
+        left -= s.nv;
         t += s.nv;
         if (t == T) {
             t = 0;
             if (++chan == C) {
                 chan = 0;
                 ++stn;
-                if (f < end) load();
+                if (left > 0) load();
             }
         }
         return s;
@@ -109,40 +112,98 @@ __device__ __forceinline__ int tc_count_steps(long long s0, long long s1, int T,
 // bounding box are dealt into tiles of 32 (one per warp lane), sorted by
 // entry count so a tile's lanes run the same number of slots; a tile's
 // entries are stored slot-major, entry (slot k, lane l) at tile_base + 32 k
-// + l, with zero-weight padding.
+// + l, with zero-weight padding.  Within a lane's list the order is chosen so
+// that the lanes that one shared-memory phase serves together (128 bytes of
+// voltages) read distinct banks, or one element, where they can.
 //   cell offsets   uint32 [ntile * 32]  byte offset of the lane's cell in the
 //                                       stage-1 operand (field 0), or
 //                                       0xffffffff for an unused lane
 //   tile bases     int32 [ntile + 1]    first entry of each tile
 //   warp ranges    int32 [kGatherWarps + 1]  warp w grids tiles [r[w], r[w+1]);
 //                                       tiles are dealt to the warps by
-//                                       longest-first (slots + 1 per tile)
+//                                       longest-first (slots + 2 per tile)
 //   (pad to 16)
-//   weights        float2 [nent]        a + ib = conj(W~)
+//   weights        float [nent]         a of conj(W~) = a + ib; for complex
+//                                       taps float2 [nent] (a, b)
 //   elements       uint16 [nent]
-constexpr int kGatherWarps = 7;
+constexpr int kGatherWarps = 11;        // at most: a kernel may deal to fewer
 struct GatherLayout {
     uint32_t off_cell, off_base, off_warp, off_w, off_e, bytes;
 };
-__host__ __device__ inline GatherLayout gather_layout(int ntile, int nent) {
+__host__ __device__ inline GatherLayout gather_layout(int ntile, int nent, int cplx) {
     GatherLayout t;
     t.off_cell = 0;
     t.off_base = 4u * 32u * ntile;
     t.off_warp = t.off_base + 4u * (ntile + 1);
     t.off_w = (t.off_warp + 4u * (kGatherWarps + 1) + 15u) & ~15u;
-    t.off_e = t.off_w + 8u * nent;
+    t.off_e = t.off_w + (cplx ? 8u : 4u) * nent;
     t.bytes = (t.off_e + 2u * nent + 15u) & ~15u;
     return t;
+}
+
+// Sums of one lane's cell over its slots q, q + 32, .. (< qe): g[f] += conj(W~)
+// E[field f], an element's F half2 voltages in one vector V (uint4: 4 fields,
+// uint2: 2).  tab is the table in shared memory, through its own address (a
+// pointer chosen at run time would make the loads generic).  Each term rounds
+// as fmaf(w.x, x.x, fmaf(-w.y, x.y, re)), fmaf(w.x, x.y, fmaf(w.y, x.x, im)).
+// Slots go four at a time, their loads issued before the first use.
+template <bool CPLX, int F, typename V>
+__device__ __forceinline__ void cell_sum_as(const uint8_t *tab, const GatherLayout &gl, int q, int qe, const V *E,
+                                            float2 (&g)[F]) {
+    static_assert(sizeof(V) == 4 * F, "one half2 a field");
+    const float *wr = reinterpret_cast<const float *>(tab + gl.off_w);
+    const float2 *wc = reinterpret_cast<const float2 *>(tab + gl.off_w);
+    const uint16_t *el = reinterpret_cast<const uint16_t *>(tab + gl.off_e);
+    auto weight = [&](int i) { return CPLX ? wc[i] : make_float2(wr[i], 0.f); };
+    auto mac = [&](const float2 w, const V &e) {
+        const uint32_t *x = reinterpret_cast<const uint32_t *>(&e);
+#pragma unroll
+        for (int f = 0; f < F; f++) {
+            const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(x + f));
+            if (CPLX) g[f] = __ffma2_rn(make_float2(-w.y, w.y), make_float2(v.y, v.x), g[f]);
+            g[f] = __ffma2_rn(make_float2(w.x, w.x), v, g[f]);
+        }
+    };
+    for (; q + 96 < qe; q += 128) {
+        float2 w[4];
+        int en[4];
+        V e[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            en[j] = el[q + 32 * j];
+            w[j] = weight(q + 32 * j);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) e[j] = E[en[j]];
+#pragma unroll
+        for (int j = 0; j < 4; j++) mac(w[j], e[j]);
+    }
+    if (q + 32 < qe) {
+        const int e0 = el[q], e1 = el[q + 32];
+        const float2 w0 = weight(q), w1 = weight(q + 32);
+        const V v0 = E[e0], v1 = E[e1];
+        mac(w0, v0);
+        mac(w1, v1);
+        q += 64;
+    }
+    if (q < qe) mac(weight(q), E[el[q]]);
+}
+template <int F, typename V>
+__device__ __forceinline__ void cell_sum(const uint8_t *tab, const GatherLayout &gl, int cplx, int q, int qe,
+                                         const V *E, float2 (&g)[F]) {
+    if (cplx) cell_sum_as<true>(tab, gl, q, qe, E, g);
+    else cell_sum_as<false>(tab, gl, q, qe, E, g);
 }
 
 // Builds the gather table of one station from its CSR cell lists (cells of
 // the box row-major, cstart[box_w * box_h + 1]).  Cell (x, y) of the box
 // lands at byte tc::off_kmajor(y, 2 x, k_stride, mn_stride) of the stage-1
 // operand.
-// n_warps (<= kGatherWarps) of the front warps get tiles; the others none.
+// Entries of zero weight are left out.  F: half2 fields read per element (the
+// phase is 32 / F lanes).  n_warps (<= kGatherWarps) get tiles; the others none.
 void epic_tc_build_gather(int box_w, int box_h, const std::vector<int32_t> &cstart,
                           const std::vector<int32_t> &elem, const std::vector<float2> &w, uint32_t k_stride,
-                          uint32_t mn_stride, std::vector<uint8_t> &out, int &ntile, int &nent,
+                          uint32_t mn_stride, int F, std::vector<uint8_t> &out, int &ntile, int &nent, int &cplx,
                           int n_warps = kGatherWarps);
 
 // fp16 W'[j][l] = (-1)^j exp(+2 pi i l j / N) as a real matrix entry: row
@@ -191,6 +252,11 @@ int epic_tc_group(int N);
 hai_status epic_tc128_run(hai_ctx *ctx, const TcLaunch &l, cudaStream_t st);
 hai_status epic_tc128_set_attr(hai_ctx *ctx);
 size_t epic_tc128_smem(int ne_max, uint32_t table_max);
+// Gather table (N = 128: blob) of one station: fills the record's table fields;
+// shared_bytes = what the kernel keeps in shared memory.
+void epic_tc_station_table(int grid_n, int box_w, int box_h, const std::vector<int32_t> &cstart,
+                           const std::vector<int32_t> &elem, const std::vector<float2> &w, std::vector<uint8_t> &out,
+                           TcStation &rec, uint32_t &shared_bytes, long long &entries);
 // Per-rank gather blob of one station for the N = 128 kernel;
 // max_rank_bytes = the largest rank table (what a CTA keeps in shared memory).
 void epic_tc128_build_blob(int box_w, int box_h, const std::vector<int32_t> &cstart,

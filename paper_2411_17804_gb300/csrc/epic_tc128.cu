@@ -23,10 +23,18 @@
 // which frees that G buffer for the next-but-one step.  Only a group's owner
 // ever writes its rows, in any copy.
 //
-// Roles as in the N = 32/64 kernel: warps 0-6 front (voltages, gridding,
-// warps 0-3 also move stage-1 results from TMEM into operand B2), warp 7 TMA
-// and MMA issue, warps 8-15 epilogue (register accumulators, 64 per thread).
-// One sample per step.
+// Roles as in the N = 32/64 kernel, 24 warps: warps 0-3 move stage-1 results
+// from TMEM into operand B2, warp 4 TMA and MMA issue, warp 5 ships the gridded
+// rows to the peers, warps 6, 7 and 16-23 voltages and gridding, warps 8-15
+// epilogue (register accumulators, 64 per thread).  One sample per step; the
+// roles of a step hand over by mbarriers, so gridding, shipping, stage 1, its
+// move and stage 2 of successive samples overlap.
+//
+// What bounds it: the latency of that chain (two samples of G in flight) and
+// the gridding warps' share of a sample.  Inter-station EPIC of one beam (256
+// stations, 32 channels x 1000): 2195 us when the seven front warps did the
+// gridding, the shipping and the move in turn, from a table with an entry for
+// every zero weight; 1083 us now (1432 before the MMA descriptors were hoisted).
 #include <math.h>
 #include <string.h>
 
@@ -41,13 +49,19 @@ namespace {
 
 constexpr int kN = 128;
 constexpr int kNN = kN * kN;
-constexpr int kThreads = 512;
-constexpr int kFront = 224;
-constexpr int kMmaWarp = 7;
-constexpr int kEpi = 256;
+constexpr int kThreads = 768;
+constexpr int kConvWarps = 4;                // warps 0-3
+constexpr int kMmaWarp = 4;
+constexpr int kSendWarp = 5;                 // ships G rows to the peers
+constexpr int kGridWarps = 10;               // warps 6, 7 and 16-23
+constexpr int kGrid = 32 * kGridWarps;
+constexpr int kEpiWarps = 8;                 // warps 8-15
+// registers as in the N = 32/64 kernel: 256 x 112 + 512 x 64 = 768 x 80
+constexpr int kLaunchRegs = 80, kEpiRegs = 112, kOtherRegs = 64;
+static_assert(256 * kEpiRegs + 512 * kOtherRegs <= kThreads * kLaunchRegs, "register shares");
+static_assert(kGridWarps <= kGatherWarps, "gather table");
 constexpr int kStages = 4;
 constexpr int kRanks = 4;
-constexpr int kSendWarp = 6;                 // front warp that ships G rows to the peers
 constexpr uint32_t kKs = 128;                // K-major: K-group stride
 constexpr uint32_t kMNs = 16 * kKs;          // K-major, K = 128: MN-group stride (2048)
 constexpr uint32_t kGroupBytes = kMNs;       // 8 rows of a K-major operand
@@ -69,10 +83,10 @@ constexpr uint32_t kD2Col = 128;             // TMEM: D1 at 0 / 64, D2 at 128 / 
 // rank of each 8-row group of the box.
 struct Blob128 {
     uint32_t off[kRanks], bytes[kRanks];
-    int32_t ntile[kRanks], nent[kRanks];
+    int32_t ntile[kRanks], nent[kRanks], cplx[kRanks];
     uint8_t owner[8];
     int32_t box_w, box_h;       // kernel box of the station (cells)
-    uint8_t pad[48];
+    uint8_t pad[32];
 };
 static_assert(sizeof(Blob128) == 128, "blob header");
 
@@ -91,7 +105,8 @@ struct Params {
     unsigned *status;
 };
 
-__device__ __forceinline__ void bar_front() { asm volatile("bar.sync 1, 224;" ::: "memory"); }
+__device__ __forceinline__ void bar_grid() { asm volatile("bar.sync 1, 320;" ::: "memory"); }
+static_assert(kGrid == 320, "grid barrier");
 
 template <bool BF>
 __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) epic_tc128_kernel(const Params p) {
@@ -100,7 +115,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
     constexpr uint32_t kIdesc2 = tc::idesc_f16_as(BF, 128, 128, 0, 1);
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t mb_v[kStages];
-    __shared__ __align__(8) uint64_t mb_a1[2], mb_a1free[2], mb_d1[2], mb_a2, mb_b2free, mb_full[2], mb_empty[2];
+    __shared__ __align__(8) uint64_t mb_g[2], mb_a1[2], mb_a1free[2], mb_d1[2], mb_a2, mb_b2free, mb_full[2], mb_empty[2];
     __shared__ uint32_t tmem_slot;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -123,13 +138,14 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
     if (tid == 0) {
         for (int s = 0; s < kStages; s++) tc::mbar_init(&mb_v[s], 1);
         for (int b = 0; b < 2; b++) {
+            tc::mbar_init(&mb_g[b], kGridWarps);
             tc::mbar_init(&mb_a1[b], 1);
             tc::mbar_init(&mb_a1free[b], kRanks);
             tc::mbar_init(&mb_d1[b], 1);
             tc::mbar_init(&mb_full[b], 1);
-            tc::mbar_init(&mb_empty[b], kEpi);
+            tc::mbar_init(&mb_empty[b], kEpiWarps);
         }
-        tc::mbar_init(&mb_a2, 128);
+        tc::mbar_init(&mb_a2, kConvWarps);
         tc::mbar_init(&mb_b2free, 1);
         tc::mbar_fence_init();
     }
@@ -145,213 +161,207 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
     const long long s1 = p.cta_begin ? p.cta_begin[group + 1] : min(s0 + p.len, p.total);
     const int nsteps = (int)max(0ll, s1 - s0);
 
-    if (warp < kMmaWarp) {
-        // ================================================================ front
-        int cur_station = -1, ne = 0, ntile = 0;
-        int a1_st0 = -1, a1_st1 = -1;          // station whose cells buffer 0 / 1 holds
-        uint32_t own_mask = 0, incoming = 0;
-        uint32_t box_mask = 0, copy_bytes = 0;    // groups inside the box; bytes of a group's box columns
-        bool dead = false;                     // a wait of this thread gave up: send nothing more
-        const uint32_t *s_cell = nullptr;
-        const int32_t *s_base = nullptr, *s_warp = nullptr;
-        const float2 *s_w = nullptr;
-        const uint16_t *s_e = nullptr;
+    const int wg = warp >> 2;
+    if (wg != 2 && wg != 3) {
+        tc::setmaxnreg_dec<kOtherRegs>();
+        if (wg >= 4 || warp > kSendWarp) {
+            // ================================================================ gridding
+            const int gw = wg >= 4 ? warp - 14 : warp - 6, gt = gw * 32 + lane;
+            int cur_station = -1, ne = 0, cplx = 0;
+            GatherLayout gl{};
+            int a1_st0 = -1, a1_st1 = -1;          // station whose cells buffer 0 / 1 holds
+            uint32_t own_mask = 0;
+            uint32_t box_mask = 0, copy_bytes = 0;    // groups inside the box; bytes of a group's box columns
 
-        auto prepare = [&](int stn, int b) {
-            if (stn == cur_station && (b ? a1_st1 : a1_st0) == stn) return;
-            bar_front();
-            if (stn != cur_station) {
-                const TcStation st = p.stations[stn];
-                const Blob128 *hd = reinterpret_cast<const Blob128 *>(st.table);
-                const uint32_t off = hd->off[rank], bytes = hd->bytes[rank];
-                for (int k = tid; k < (int)(bytes / 16); k += kFront)
-                    reinterpret_cast<int4 *>(sT)[k] = __ldg(reinterpret_cast<const int4 *>(st.table + off) + k);
-                const GatherLayout gl = gather_layout(hd->ntile[rank], hd->nent[rank]);
-                s_cell = reinterpret_cast<const uint32_t *>(sT + gl.off_cell);
-                s_base = reinterpret_cast<const int32_t *>(sT + gl.off_base);
-                s_warp = reinterpret_cast<const int32_t *>(sT + gl.off_warp);
-                s_w = reinterpret_cast<const float2 *>(sT + gl.off_w);
-                s_e = reinterpret_cast<const uint16_t *>(sT + gl.off_e);
-                ntile = hd->ntile[rank];
-                ne = st.ne;
-                own_mask = 0;
-                for (int g = 0; g < 8; g++)
-                    if (hd->owner[g] == rank) own_mask |= 1u << g;
-                box_mask = 0;
-                for (int g = 0; g < 8; g++)
-                    if (8 * g < hd->box_h) box_mask |= 1u << g;
-                // K-groups (8 values: 4 cells of (re, im)) that hold box columns
-                copy_bytes = (uint32_t)((2 * hd->box_w + 7) / 8) * kKs;
-                incoming = (uint32_t)__popc(box_mask & ~own_mask) * 2u * copy_bytes;
-                cur_station = stn;
-            }
-            if ((b ? a1_st1 : a1_st0) != stn) {
-                // zero what no other CTA writes into this copy: own groups, groups
-                // outside the box, and the columns past the box of every group
-                uint8_t *A = sA1 + b * kA1Bytes;
-                for (int k = tid; k < (int)(16 * kGroupBytes / 16); k += kFront) {
-                    const uint32_t byte = (uint32_t)k * 16u;
-                    const int g = (byte / kGroupBytes) & 7;
-                    const uint32_t in_group = byte % kGroupBytes;
-                    if ((own_mask & (1u << g)) || !(box_mask & (1u << g)) || in_group >= copy_bytes)
-                        reinterpret_cast<int4 *>(A)[k] = make_int4(0, 0, 0, 0);
+            auto prepare = [&](int stn, int b) {
+                if (stn == cur_station && (b ? a1_st1 : a1_st0) == stn) return;
+                bar_grid();
+                if (stn != cur_station) {
+                    const TcStation st = p.stations[stn];
+                    const Blob128 *hd = reinterpret_cast<const Blob128 *>(st.table);
+                    const uint32_t off = hd->off[rank], bytes = hd->bytes[rank];
+                    for (int k = gt; k < (int)(bytes / 16); k += kGrid)
+                        reinterpret_cast<int4 *>(sT)[k] = __ldg(reinterpret_cast<const int4 *>(st.table + off) + k);
+                    gl = gather_layout(hd->ntile[rank], hd->nent[rank], hd->cplx[rank]);
+                    cplx = hd->cplx[rank];
+                    ne = st.ne;
+                    own_mask = 0;
+                    for (int g = 0; g < 8; g++)
+                        if (hd->owner[g] == rank) own_mask |= 1u << g;
+                    box_mask = 0;
+                    for (int g = 0; g < 8; g++)
+                        if (8 * g < hd->box_h) box_mask |= 1u << g;
+                    // K-groups (8 values: 4 cells of (re, im)) that hold box columns
+                    copy_bytes = (uint32_t)((2 * hd->box_w + 7) / 8) * kKs;
+                    cur_station = stn;
                 }
-                (b ? a1_st1 : a1_st0) = stn;
-            }
-            bar_front();
-        };
-        auto stage_volt = [&](const TcStep &s, int i) {
-            const int8_t *V;
-            uint32_t delta;
-            const int8_t *src = tc_aligned_src(s.src, p.guard, delta);
-            if (p.use_tma) {
-                tc::mbar_wait(&mb_v[i % kStages], (uint32_t)((i / kStages) & 1), p.status);
-                V = sV + (i % kStages) * p.vstage + delta;
-            } else {
-                int8_t *dst = sV + (i % kStages) * p.vstage;
-                for (int b = tid; b < 4 * ne; b += kFront) dst[b] = src[b];
-                bar_front();
-                V = dst;
-            }
-            uint2 *E = sE + (size_t)(i & 1) * ((p.ne_max + 1) & ~1);
-            const char2 *v2 = reinterpret_cast<const char2 *>(V);
-            for (int a = tid; a < ne; a += kFront) {
-                const char2 x = v2[a], y = v2[ne + a];
-                E[a] = make_uint2(tc::pack_half2((float)x.x, (float)x.y), tc::pack_half2((float)y.x, (float)y.y));
-            }
-            bar_front();
-        };
-        auto grid_step = [&](int i) {
-            uint8_t *A = sA1 + (i & 1) * kA1Bytes;
-            const uint2 *E = sE + (size_t)(i & 1) * ((p.ne_max + 1) & ~1);
-            for (int t = s_warp[warp]; t < s_warp[warp + 1]; t++) {
-                float2 g0 = make_float2(0.f, 0.f), g1 = g0;
-                const int qe = s_base[t + 1];
-                // (re, im) += conj(W~) e per pol as packed FMAs, the roundings of
-                // fmaf(w.x, x.x, fmaf(-w.y, x.y, re)) and fmaf(w.x, x.y, fmaf(w.y, x.x, im))
-                auto mac = [&](const float2 w, const uint2 e) {
-                    const float2 x = __half22float2(*reinterpret_cast<const __half2 *>(&e.x));
-                    const float2 y = __half22float2(*reinterpret_cast<const __half2 *>(&e.y));
-                    const float2 wr = make_float2(w.x, w.x), wi = make_float2(-w.y, w.y);
-                    g0 = __ffma2_rn(wr, x, __ffma2_rn(wi, make_float2(x.y, x.x), g0));
-                    g1 = __ffma2_rn(wr, y, __ffma2_rn(wi, make_float2(y.y, y.x), g1));
-                };
-                // the lane's slots q, q + 32, ...: four at a time with every
-                // shared-memory load issued before the first use
-                int q = s_base[t] + lane;
-                for (; q + 96 < qe; q += 128) {
-                    float2 w[4];
-                    int en[4];
-#pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        w[j] = s_w[q + 32 * j];
-                        en[j] = s_e[q + 32 * j];
+                if ((b ? a1_st1 : a1_st0) != stn) {
+                    // zero what no other CTA writes into this copy: own groups, groups
+                    // outside the box, and the columns past the box of every group
+                    uint8_t *A = sA1 + b * kA1Bytes;
+                    for (int k = gt; k < (int)(16 * kGroupBytes / 16); k += kGrid) {
+                        const uint32_t byte = (uint32_t)k * 16u;
+                        const int g = (byte / kGroupBytes) & 7;
+                        const uint32_t in_group = byte % kGroupBytes;
+                        if ((own_mask & (1u << g)) || !(box_mask & (1u << g)) || in_group >= copy_bytes)
+                            reinterpret_cast<int4 *>(A)[k] = make_int4(0, 0, 0, 0);
                     }
-                    uint2 e[4];
-#pragma unroll
-                    for (int j = 0; j < 4; j++) e[j] = E[en[j]];
-#pragma unroll
-                    for (int j = 0; j < 4; j++) mac(w[j], e[j]);
+                    (b ? a1_st1 : a1_st0) = stn;
                 }
-                for (; q < qe; q += 32) mac(s_w[q], E[s_e[q]]);
-                const uint32_t off = s_cell[t * 32 + lane];
-                if (off != 0xffffffffu) {
-                    *reinterpret_cast<uint32_t *>(A + off) = tc::pack2<BF>(g0.x, g0.y);
-                    *reinterpret_cast<uint32_t *>(A + off + kPolBytes) = tc::pack2<BF>(g1.x, g1.y);
+                bar_grid();
+            };
+            auto stage_volt = [&](const TcStep &s, int i) {
+                const int8_t *V;
+                uint32_t delta;
+                const int8_t *src = tc_aligned_src(s.src, p.guard, delta);
+                if (p.use_tma) {
+                    tc::mbar_wait(&mb_v[i % kStages], (uint32_t)((i / kStages) & 1), p.status);
+                    V = sV + (i % kStages) * p.vstage + delta;
+                } else {
+                    int8_t *dst = sV + (i % kStages) * p.vstage;
+                    for (int b = gt; b < 4 * ne; b += kGrid) dst[b] = src[b];
+                    bar_grid();
+                    V = dst;
                 }
-            }
-        };
-        // warp 6: the box columns of the own in-box row groups of G -> the
-        // three other CTAs, one bulk copy per lane (peer, group, pol); then
-        // this CTA's own arrival, expecting the bytes the others send
-        auto send = [&](int i) {
-            const int b = i & 1;
-            uint8_t *A = sA1 + b * kA1Bytes;
-            const uint32_t mine = own_mask & box_mask;
-            const int n_own = __popc(mine);
-            if (!dead)
-                for (int c = lane; c < (kRanks - 1) * n_own * 2; c += 32) {
-                    const int pol = c & 1, k = (c >> 1) % n_own, pi = (c >> 1) / n_own;
-                    const uint32_t peer = (uint32_t)pi + (pi >= (int)rank ? 1u : 0u);
-                    int g = -1;
-                    for (int x = 0, seen = 0; x < 8; x++)
-                        if (mine & (1u << x)) {
-                            if (seen == k) g = x;
-                            seen++;
-                        }
-                    const uint32_t off = (uint32_t)pol * kPolBytes + (uint32_t)g * kGroupBytes;
-                    tc::bulk_s2peer(tc::peer_addr(tc::smem_u32(A + off), peer), A + off, copy_bytes,
-                                    tc::peer_addr(tc::smem_u32(&mb_a1[b]), peer));
-                }
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive_expect_tx(&mb_a1[b], incoming);
-        };
-        // warps 0-3: D1 row (pol, y) -> column (y, re/im) of B2 for the
-        // rows (pol, out re/im, l_x): out re <- (H_r, -H_i), out im <- (H_i, H_r)
-        auto convert = [&](int i) {
-            const int pol = warp >> 1, y = 32 * (warp & 1) + lane;
-            const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(i & 1) * 64u;
-#pragma unroll
-            for (int hh = 0; hh < 2; hh++) {               // l_x in [16 hh, 16 hh + 16)
-                uint32_t hr[16], hi[16];
-                tc::tmem_ld16(base + 16 * hh, hr);
-                tc::tmem_ld16(base + 32 + 16 * hh, hi);
-                tc::tmem_wait_ld();
-#pragma unroll
-                for (int c_in = 0; c_in < 2; c_in++) {
-                    const int kappa = 2 * y + c_in;
-#pragma unroll
-                    for (int c_out = 0; c_out < 2; c_out++) {
-#pragma unroll
-                        for (int h = 0; h < 2; h++) {        // 8 columns l_x -> one 16-byte row
-                            float v[8];
-#pragma unroll
-                            for (int e = 0; e < 8; e++) {
-                                const float r = __uint_as_float(hr[8 * h + e]), im = __uint_as_float(hi[8 * h + e]);
-                                v[e] = c_out == 0 ? (c_in == 0 ? r : -im) : (c_in == 0 ? im : r);
-                            }
-                            const int n2 = pol * 64 + c_out * 32 + 16 * hh + 8 * h;
-                            uint4 u;
-                            u.x = tc::pack2<BF>(v[0], v[1]);
-                            u.y = tc::pack2<BF>(v[2], v[3]);
-                            u.z = tc::pack2<BF>(v[4], v[5]);
-                            u.w = tc::pack2<BF>(v[6], v[7]);
-                            *reinterpret_cast<uint4 *>(sB2 + tc::off_mnmajor(n2, kappa, kB2Ks, kB2MNs)) = u;
-                        }
+                uint2 *E = sE + (size_t)(i & 1) * ((p.ne_max + 1) & ~1);
+                if (!(ne & 1) && ((uintptr_t)V & 3) == 0) {
+                    // two elements a thread: 4 bytes of a pol -> two half2
+                    for (int a = gt; a < ne / 2; a += kGrid) {
+                        uint32_t x0, x1, y0, y1;
+                        tc::widen4(*reinterpret_cast<const uint32_t *>(V + 4 * a), x0, x1);
+                        tc::widen4(*reinterpret_cast<const uint32_t *>(V + 2 * ne + 4 * a), y0, y1);
+                        *reinterpret_cast<uint4 *>(E + 2 * a) = make_uint4(x0, y0, x1, y1);
+                    }
+                } else {
+                    const char2 *v2 = reinterpret_cast<const char2 *>(V);
+                    for (int a = gt; a < ne; a += kGrid) {
+                        const char2 x = v2[a], y = v2[ne + a];
+                        E[a] = make_uint2(tc::pack_half2((float)x.x, (float)x.y), tc::pack_half2((float)y.x, (float)y.y));
                     }
                 }
-            }
-        };
-        TcWalker wk;
-        wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
-        for (int i = -1; i < nsteps; i++) {
-            if (i + 1 < nsteps) {
-                const int j = i + 1, b = j & 1;
+                bar_grid();
+            };
+            auto grid_step = [&](int i) {
+                uint8_t *A = sA1 + (i & 1) * kA1Bytes;
+                const uint2 *E = sE + (size_t)(i & 1) * ((p.ne_max + 1) & ~1);
+                const int32_t *base = reinterpret_cast<const int32_t *>(sT + gl.off_base);
+                const int32_t *wr = reinterpret_cast<const int32_t *>(sT + gl.off_warp);
+                const int t1 = wr[gw + 1];
+                for (int t = wr[gw]; t < t1; t++) {
+                    float2 g[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};       // X, Y
+                    cell_sum(sT, gl, cplx, base[t] + lane, base[t + 1], E, g);
+                    const uint32_t off = reinterpret_cast<const uint32_t *>(sT + gl.off_cell)[t * 32 + lane];
+                    if (off != 0xffffffffu) {
+                        *reinterpret_cast<uint32_t *>(A + off) = tc::pack2<BF>(g[0].x, g[0].y);
+                        *reinterpret_cast<uint32_t *>(A + off + kPolBytes) = tc::pack2<BF>(g[1].x, g[1].y);
+                    }
+                }
+            };
+            TcWalker wk;
+            wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
+            for (int j = 0; j < nsteps; j++) {
+                const int b = j & 1;
                 const TcStep s = wk.next(1);
                 // G buffer b was last read by the stage-1 MMAs of step j - 2 in every CTA
-                if (j >= 2 && !tc::mbar_wait_cluster(&mb_a1free[b], (uint32_t)(((j >> 1) - 1) & 1), p.status))
-                    dead = true;
+                if (j >= 2) tc::mbar_wait_cluster(&mb_a1free[b], (uint32_t)(((j >> 1) - 1) & 1), p.status);
                 prepare(s.stn, b);
                 stage_volt(s, j);
                 grid_step(j);
                 tc::fence_proxy_async();
-                bar_front();
-                if (warp == kSendWarp) send(j);
+                tc::mbar_arrive_warp(&mb_g[b]);
             }
-            if (i >= 0 && warp < 4) {
-                tc::mbar_wait(&mb_d1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
-                if (i >= 1) tc::mbar_wait(&mb_b2free, (uint32_t)((i - 1) & 1), p.status);
-                tc::fence_after();
-                convert(i);
-                tc::fence_proxy_async();
-                tc::fence_before();
-                tc::mbar_arrive(&mb_a2);
+        } else if (warp == kSendWarp) {
+            // ================================================================ shipping
+            int cur_station = -1;
+            uint32_t own_mask = 0, incoming = 0, box_mask = 0, copy_bytes = 0;
+            bool dead = false;                     // a wait gave up: send nothing more
+            auto prepare = [&](int stn) {
+                if (stn == cur_station) return;
+                const Blob128 *hd = reinterpret_cast<const Blob128 *>(p.stations[stn].table);
+                own_mask = box_mask = 0;
+                for (int g = 0; g < 8; g++) {
+                    if (hd->owner[g] == rank) own_mask |= 1u << g;
+                    if (8 * g < hd->box_h) box_mask |= 1u << g;
+                }
+                copy_bytes = (uint32_t)((2 * hd->box_w + 7) / 8) * kKs;
+                incoming = (uint32_t)__popc(box_mask & ~own_mask) * 2u * copy_bytes;
+                cur_station = stn;
+            };
+            // the box columns of the own in-box row groups of G -> the
+            // three other CTAs, one bulk copy per lane (peer, group, pol); then
+            // this CTA's own arrival, expecting the bytes the others send
+            auto send = [&](int i) {
+                const int b = i & 1;
+                uint8_t *A = sA1 + b * kA1Bytes;
+                const uint32_t mine = own_mask & box_mask;
+                const int n_own = __popc(mine);
+                if (!dead)
+                    for (int c = lane; c < (kRanks - 1) * n_own * 2; c += 32) {
+                        const int pol = c & 1, k = (c >> 1) % n_own, pi = (c >> 1) / n_own;
+                        const uint32_t peer = (uint32_t)pi + (pi >= (int)rank ? 1u : 0u);
+                        int g = -1;
+                        for (int x = 0, seen = 0; x < 8; x++)
+                            if (mine & (1u << x)) {
+                                if (seen == k) g = x;
+                                seen++;
+                            }
+                        const uint32_t off = (uint32_t)pol * kPolBytes + (uint32_t)g * kGroupBytes;
+                        tc::bulk_s2peer(tc::peer_addr(tc::smem_u32(A + off), peer), A + off, copy_bytes,
+                                        tc::peer_addr(tc::smem_u32(&mb_a1[b]), peer));
+                    }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive_expect_tx(&mb_a1[b], incoming);
+            };
+            TcWalker wk;
+            wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
+            for (int j = 0; j < nsteps; j++) {
+                const int b = j & 1;
+                prepare(wk.next(1).stn);
+                // the peers' copies of buffer b are free, and this CTA's rows are gridded
+                if (j >= 2 && !tc::mbar_wait_cluster(&mb_a1free[b], (uint32_t)(((j >> 1) - 1) & 1), p.status)) dead = true;
+                if (!tc::mbar_wait(&mb_g[b], (uint32_t)((j >> 1) & 1), p.status)) dead = true;
+                send(j);
             }
-        }
-    } else if (warp == kMmaWarp) {
-        // ================================================================ MMA + TMA
-        if (lane == 0) {
-            const uint32_t b1 = tc::smem_u32(sB1), a2 = tc::smem_u32(sA2), b2 = tc::smem_u32(sB2);
+        } else if (wg == 0) {
+            // ====================================================== stage-1 results
+            // warps 0-3: D1 row (pol, y) -> column (y, re/im) of B2 for the
+            // rows (pol, out re/im, l_x): out re <- (H_r, -H_i), out im <- (H_i, H_r)
+            auto convert = [&](int i) {
+                const int pol = warp >> 1, y = 32 * (warp & 1) + lane;
+                const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(i & 1) * 64u;
+#pragma unroll
+                for (int hh = 0; hh < 2; hh++) {               // l_x in [16 hh, 16 hh + 16)
+                    uint32_t hr[16], hi[16];
+                    tc::tmem_ld16(base + 16 * hh, hr);
+                    tc::tmem_ld16(base + 32 + 16 * hh, hi);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int c_in = 0; c_in < 2; c_in++) {
+                        const int kappa = 2 * y + c_in;
+#pragma unroll
+                        for (int c_out = 0; c_out < 2; c_out++) {
+#pragma unroll
+                            for (int h = 0; h < 2; h++) {        // 8 columns l_x -> one 16-byte row
+                                float v[8];
+#pragma unroll
+                                for (int e = 0; e < 8; e++) {
+                                    const float r = __uint_as_float(hr[8 * h + e]), im = __uint_as_float(hi[8 * h + e]);
+                                    v[e] = c_out == 0 ? (c_in == 0 ? r : -im) : (c_in == 0 ? im : r);
+                                }
+                                const int n2 = pol * 64 + c_out * 32 + 16 * hh + 8 * h;
+                                uint4 u;
+                                u.x = tc::pack2<BF>(v[0], v[1]);
+                                u.y = tc::pack2<BF>(v[2], v[3]);
+                                u.z = tc::pack2<BF>(v[4], v[5]);
+                                u.w = tc::pack2<BF>(v[6], v[7]);
+                                *reinterpret_cast<uint4 *>(sB2 + tc::off_mnmajor(n2, kappa, kB2Ks, kB2MNs)) = u;
+                            }
+                        }
+                    }
+                }
+            };
+            // warp 0 also streams the voltages: step i's stage has been read once its
+            // stage 1 is done
             int n_loaded = 0;
             TcWalker ld;
             ld.init(p.volt, p.stations, p.C, p.T, s0, s1);
@@ -366,60 +376,80 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
                 tc::bulk_g2s(sV + sg * p.vstage, src, bytes, &mb_v[sg]);
                 n_loaded++;
             };
-            for (int q = 0; q < kStages; q++) issue_load();
-            for (int k = -1; k < nsteps; k++) {
-                if (k >= 0) {                      // stage 2 of step k
-                    tc::mbar_wait(&mb_a2, (uint32_t)(k & 1), p.status);
-                    const int slot = k & 1;
-                    if (k >= 2) tc::mbar_wait(&mb_empty[slot], (uint32_t)(((k >> 1) - 1) & 1), p.status);
-                    tc::fence_after();
-                    const uint32_t d = tmem + kD2Col + (uint32_t)slot * 128u;
+            if (warp == 0 && lane == 0)
+                for (int q = 0; q < kStages; q++) issue_load();
+            // D1 buffer i & 1 is rewritten by MMA1(i + 2), issued after the arrival
+            // on mb_a2 of step i was seen
+            for (int i = 0; i < nsteps; i++) {
+                tc::mbar_wait(&mb_d1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
+                if (warp == 0 && lane == 0) issue_load();
+                __syncwarp();
+                if (i >= 1) tc::mbar_wait(&mb_b2free, (uint32_t)((i - 1) & 1), p.status);
+                tc::fence_after();
+                convert(i);
+                tc::fence_proxy_async();
+                tc::fence_before();
+                tc::mbar_arrive_warp(&mb_a2);
+            }
+        } else if (warp == kMmaWarp) {
+            // ================================================================ MMA + TMA
+            if (lane == 0) {
+                const uint32_t b1 = tc::smem_u32(sB1), a2 = tc::smem_u32(sA2), b2 = tc::smem_u32(sB2);
+                // descriptors once, then 32-bit additions: the issuing thread is one of
+                // 24 warps' and its scalar work between MMAs is the sample's period
+                const uint64_t da1[2] = {tc::desc(tc::smem_u32(sA1), kKs, kMNs), tc::desc(tc::smem_u32(sA1) + kA1Bytes, kKs, kMNs)};
+                const uint64_t db1 = tc::desc(b1, kKs, kMNs), da2 = tc::desc(a2, kKs, kMNs), db2 = tc::desc(b2, kB2Ks, kB2MNs);
+                for (int k = -1; k < nsteps; k++) {
+                    if (k + 1 < nsteps) {              // stage 1 of step k+1
+                        const int i = k + 1;
+                        tc::mbar_wait_cluster(&mb_a1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
+                        tc::fence_after();
+                        const uint64_t da = (i & 1) ? da1[1] : da1[0];
+                        const uint32_t d = tmem + (uint32_t)(i & 1) * 64u;
 #pragma unroll
-                    for (int s = 0; s < 8; s++)
-                        tc::mma_f16(d, tc::desc(a2 + s * 2 * kKs, kKs, kMNs), tc::desc(b2 + s * 2 * kB2Ks, kB2Ks, kB2MNs),
-                                    kIdesc2, s > 0);
-                    tc::mma_commit(&mb_full[slot]);
-                    tc::mma_commit(&mb_b2free);
-                }
-                if (k + 1 < nsteps) {              // stage 1 of step k+1
-                    const int i = k + 1;
-                    tc::mbar_wait_cluster(&mb_a1[i & 1], (uint32_t)((i >> 1) & 1), p.status);
-                    issue_load();
-                    tc::fence_after();
-                    const uint32_t a = tc::smem_u32(sA1 + (i & 1) * kA1Bytes);
-                    const uint32_t d = tmem + (uint32_t)(i & 1) * 64u;
+                        for (int s = 0; s < 8; s++)
+                            tc::mma_f16(d, tc::desc_add(da, s * 2 * kKs), tc::desc_add(db1, s * 2 * kKs), kIdesc1, s > 0);
+                        tc::mma_commit(&mb_d1[i & 1]);
+                        // every CTA waits for this only before step i + 2
+                        if (i + 2 < nsteps) tc::mma_commit_multicast(&mb_a1free[i & 1], (uint16_t)((1u << kRanks) - 1));
+                    }
+                    if (k >= 0) {                      // stage 2 of step k
+                        tc::mbar_wait(&mb_a2, (uint32_t)(k & 1), p.status);
+                        const int slot = k & 1;
+                        if (k >= 2) tc::mbar_wait(&mb_empty[slot], (uint32_t)(((k >> 1) - 1) & 1), p.status);
+                        tc::fence_after();
+                        const uint32_t d = tmem + kD2Col + (uint32_t)slot * 128u;
 #pragma unroll
-                    for (int s = 0; s < 8; s++)
-                        tc::mma_f16(d, tc::desc(a + s * 2 * kKs, kKs, kMNs), tc::desc(b1 + s * 2 * kKs, kKs, kMNs),
-                                    kIdesc1, s > 0);
-                    tc::mma_commit(&mb_d1[i & 1]);
-                    // every CTA waits for this only before step i + 2
-                    if (i + 2 < nsteps) tc::mma_commit_multicast(&mb_a1free[i & 1], (uint16_t)((1u << kRanks) - 1));
+                        for (int s = 0; s < 8; s++)
+                            tc::mma_f16(d, tc::desc_add(da2, s * 2 * kKs), tc::desc_add(db2, s * 2 * kB2Ks), kIdesc2, s > 0);
+                        tc::mma_commit(&mb_full[slot]);
+                        tc::mma_commit(&mb_b2free);
+                    }
                 }
             }
         }
     } else {
+        tc::setmaxnreg_inc<kEpiRegs>();
         // ============================================================= epilogue
         const int q = warp & 3, h = (warp - 8) >> 2;
         const int ly = 32 * q + lane;
         const int lx0 = 32 * (int)rank + 16 * h;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        // packed accumulators: pw[t] = (|X|^2, |Y|^2), cx[t] = (Re, Im) X conj(Y)
-        float2 pw[16], cx[16];
+        // pixel pairs (l_x, l_x + 1): adjacent TMEM columns, so the packed operands
+        // come out of the loads as they are
+        float2 axx[8], ayy[8], are[8], aim[8];
 #pragma unroll
-        for (int t = 0; t < 16; t++) pw[t] = cx[t] = make_float2(0.f, 0.f);
+        for (int t = 0; t < 8; t++) axx[t] = ayy[t] = are[t] = aim[t] = make_float2(0.f, 0.f);
         int seg = 0;
         long long cur_blk = -1;
         auto flush = [&](int stn, int c, int sgm) {
             float *dst = p.direct ? p.img + p.stations[stn].img_off + (size_t)c * 4 * kNN
                                   : p.partials + ((size_t)group * 2 + sgm) * 4 * kNN;
-            // plane pl: component c (0 = .x, 1 = .y) of the pairs in a
-            auto put = [&](int pl, const float2 (&a)[16], int c) {
+            auto put = [&](int pl, float2 (&a)[8]) {
                 float4 *d4 = reinterpret_cast<float4 *>(dst + (size_t)pl * kNN + (size_t)ly * kN + lx0);
 #pragma unroll
                 for (int v = 0; v < 4; v++) {
-                    float4 o = c ? make_float4(a[4 * v].y, a[4 * v + 1].y, a[4 * v + 2].y, a[4 * v + 3].y)
-                                 : make_float4(a[4 * v].x, a[4 * v + 1].x, a[4 * v + 2].x, a[4 * v + 3].x);
+                    float4 o = make_float4(a[2 * v].x, a[2 * v].y, a[2 * v + 1].x, a[2 * v + 1].y);
                     if (p.direct && p.accumulate) {
                         const float4 old = d4[v];
                         o.x += old.x;
@@ -428,14 +458,13 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
                         o.w += old.w;
                     }
                     d4[v] = o;
+                    a[2 * v] = a[2 * v + 1] = make_float2(0.f, 0.f);
                 }
             };
-            put(0, pw, 0);
-            put(1, pw, 1);
-            put(2, cx, 0);
-            put(3, cx, 1);
-#pragma unroll
-            for (int t = 0; t < 16; t++) pw[t] = cx[t] = make_float2(0.f, 0.f);
+            put(0, axx);
+            put(1, ayy);
+            put(2, are);
+            put(3, aim);
         };
         TcWalker wk;
         wk.init(p.volt, p.stations, p.C, p.T, s0, s1);
@@ -466,20 +495,20 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
                 tc::tmem_wait_ld();
                 if (qt == 3) {
                     tc::fence_before();
-                    tc::mbar_arrive(&mb_empty[slot]);
+                    tc::mbar_arrive_warp(&mb_empty[slot]);
                 }
 #pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const int t = 4 * qt + e;
-                    const float a_r = __uint_as_float(ar[e]), a_i = __uint_as_float(ai[e]);
-                    const float b_r = __uint_as_float(br[e]), b_i = __uint_as_float(bi[e]);
-                    // |X|^2 = fmaf(a_r, a_r, fmaf(a_i, a_i, .)), |Y|^2 likewise;
-                    // Re X conj(Y) = fmaf(a_r, b_r, fmaf(a_i, b_i, .)),
-                    // Im X conj(Y) = fmaf(a_i, b_r, fmaf(-a_r, b_i, .)): packed pairs
-                    const float2 re = make_float2(a_r, b_r), im = make_float2(a_i, b_i);
-                    pw[t] = __ffma2_rn(re, re, __ffma2_rn(im, im, pw[t]));
-                    cx[t] = __ffma2_rn(make_float2(a_r, a_i), make_float2(b_r, b_r),
-                                       __ffma2_rn(make_float2(a_i, -a_r), make_float2(b_i, b_i), cx[t]));
+                for (int e = 0; e < 2; e++) {
+                    const int t = 2 * qt + e;
+                    const float2 xr = make_float2(__uint_as_float(ar[2 * e]), __uint_as_float(ar[2 * e + 1]));
+                    const float2 xi = make_float2(__uint_as_float(ai[2 * e]), __uint_as_float(ai[2 * e + 1]));
+                    const float2 yr = make_float2(__uint_as_float(br[2 * e]), __uint_as_float(br[2 * e + 1]));
+                    const float2 yi = make_float2(__uint_as_float(bi[2 * e]), __uint_as_float(bi[2 * e + 1]));
+                    axx[t] = __ffma2_rn(xr, xr, __ffma2_rn(xi, xi, axx[t]));
+                    ayy[t] = __ffma2_rn(yr, yr, __ffma2_rn(yi, yi, ayy[t]));
+                    // X conj(Y): Re fmaf(xr, yr, fmaf(xi, yi, .)), Im fmaf(xi, yr, fmaf(-xr, yi, .))
+                    are[t] = __ffma2_rn(xr, yr, __ffma2_rn(xi, yi, are[t]));
+                    aim[t] = __ffma2_rn(xi, yr, __ffma2_rn(make_float2(-xr.x, -xr.y), yi, aim[t]));
                 }
             }
         }
@@ -547,8 +576,8 @@ void epic_tc128_build_blob(int box_w, int box_h, const std::vector<int32_t> &cst
                     }
                 cs[c + 1] = (int32_t)el.size();
             }
-        // warp 6 sends the rows to the other CTAs instead of gridding
-        epic_tc_build_gather(box_w, box_h, cs, el, ww, kKs, kMNs, tabs[r], hd.ntile[r], hd.nent[r], kGatherWarps - 1);
+        epic_tc_build_gather(box_w, box_h, cs, el, ww, kKs, kMNs, 2, tabs[r], hd.ntile[r], hd.nent[r], hd.cplx[r],
+                             kGridWarps);
         hd.bytes[r] = (uint32_t)tabs[r].size();
         max_rank_bytes = std::max(max_rank_bytes, hd.bytes[r]);
         max_rank_entries = std::max<long long>(max_rank_entries, hd.nent[r]);
@@ -601,6 +630,13 @@ hai_status epic_tc128_run(hai_ctx *ctx, const TcLaunch &l, cudaStream_t st) {
 }
 
 hai_status epic_tc128_set_attr(hai_ctx *ctx) {
+    // the warpgroups' register shares have to come out of the launch's
+    for (auto kern : {epic_tc128_kernel<false>, epic_tc128_kernel<true>}) {
+        cudaFuncAttributes a;
+        HAI_CUDA_TRY(cudaFuncGetAttributes(&a, kern));
+        if (a.numRegs < kLaunchRegs)
+            return hai_fail(HAI_ERR_UNSUPPORTED, "epic tensor cores: the kernel was built with too few registers");
+    }
     HAI_CUDA_TRY(hai_allow_dyn_smem(epic_tc128_kernel<false>, ctx->smem_optin));
     HAI_CUDA_TRY(hai_allow_dyn_smem(epic_tc128_kernel<true>, ctx->smem_optin));
     return HAI_OK;

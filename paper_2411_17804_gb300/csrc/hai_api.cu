@@ -349,8 +349,7 @@ extern "C" hai_status hai_layout_create(hai_ctx *ctx, const hai_layout_desc *d, 
         std::vector<uint8_t> tab;
         TcStation rec = {};
         uint32_t shared_bytes = 0;
-        epic_tc_station_table(n, L->box_w, L->box_h, count, elem, w, tab, rec.ntile, rec.nent, shared_bytes,
-                              L->tc_entries);
+        epic_tc_station_table(n, L->box_w, L->box_h, count, elem, w, tab, rec, shared_bytes, L->tc_entries);
         L->tc_tables_bytes = shared_bytes;
         L->tc_blob_bytes = tab.size();
         e = dmalloc(&L->d_tc_tables, tab.size());

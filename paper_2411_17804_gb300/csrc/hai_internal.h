@@ -144,12 +144,6 @@ int epic_fp32_target_ctas(const hai_ctx *ctx, int grid_n);
 hai_status epic_tc_launch(const hai_layout *L, const int8_t *volt, int C, int T, float *img,
                           int accumulate, cudaStream_t st, int split, int bf16);
 bool epic_tc_supported(const hai_layout *L);
-// Gather table of a layout for the tensor-core kernel of its grid side;
-// shared_bytes = what the kernel keeps in shared memory.
-void epic_tc_station_table(int grid_n, int box_w, int box_h, const std::vector<int32_t> &cstart,
-                           const std::vector<int32_t> &elem, const std::vector<float2> &w,
-                           std::vector<uint8_t> &out, int &ntile, int &nent, uint32_t &shared_bytes,
-                           long long &entries);
 hai_status epic_reduce_launch(const hai_layout *L, const EpicSplit &sp, int C, int T, float *img,
                               int accumulate, cudaStream_t st);
 // FP32 EPIC for N = 128, 256, 512 (row FFTs to a scratch, then column FFTs,

@@ -45,6 +45,12 @@ __device__ __forceinline__ uint64_t desc(uint32_t saddr, uint32_t k_stride, uint
     return d;
 }
 
+// A descriptor `bytes` further on (a multiple of 16; the address stays below
+// 256 KB, so the 14-bit field does not carry): one 32-bit addition.
+__device__ __forceinline__ uint64_t desc_add(uint64_t d, uint32_t bytes) {
+    return (d & 0xffffffff00000000ull) | ((uint32_t)d + (bytes >> 4));
+}
+
 // Instruction descriptor of kind::f16 with FP16 A and B, FP32 accumulator.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int a_mn_major, int b_mn_major) {
     return (1u << 4) | ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16) |
@@ -125,6 +131,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr));
 }
 
+// 16 lanes x 8 consecutive 32-bit columns as a fragment: thread i receives in
+// r[0], r[1] columns 2 (i % 4), + 1 of lane i / 4, and in r[2], r[3] those of
+// lane i / 4 + 8, counted from the lane of taddr (a multiple of 16).
+__device__ __forceinline__ void tmem_ld_16x256b(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // the inverse of tmem_ld16: thread i writes lane (quadrant base + i),
@@ -156,6 +171,19 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *m, uint32_t byte
                  "r"(bytes)
                  : "memory");
 }
+
+// One arrival for the warp, after every lane's work so far.
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t *m) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(m);
+}
+
+// Register limits of a warpgroup (all its warps execute it): the shares of a
+// block must add up to at most the registers it was launched with.
+template <int R>
+__device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R)); }
+template <int R>
+__device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R)); }
 
 // Test the phase; the hardware may suspend the thread for a short while
 // (hint: 20 us) while the phase is incomplete.
@@ -328,6 +356,18 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
 __device__ __forceinline__ uint32_t pack_bf162(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t *>(&h);
+}
+
+// Four int8 (two complex values) -> two half2, exact: the bits 0x6400 | (x ^ 0x80)
+// hold 1024 + 128 + x.
+__device__ __forceinline__ void widen4(uint32_t x, uint32_t &lo, uint32_t &hi) {
+    const __half2 bias = __floats2half2_rn(1152.f, 1152.f);
+    x ^= 0x80808080u;
+    const uint32_t p0 = __byte_perm(x, 0x64646464u, 0x4140), p1 = __byte_perm(x, 0x64646464u, 0x4342);
+    const __half2 h0 = __hsub2(*reinterpret_cast<const __half2 *>(&p0), bias);
+    const __half2 h1 = __hsub2(*reinterpret_cast<const __half2 *>(&p1), bias);
+    lo = *reinterpret_cast<const uint32_t *>(&h0);
+    hi = *reinterpret_cast<const uint32_t *>(&h1);
 }
 
 // Two values rounded to the 16-bit operand type (FP16, or BF16 if BF) and
