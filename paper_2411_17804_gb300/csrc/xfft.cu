@@ -12,21 +12,21 @@
 // conj(V^{beta alpha}_{ab} K_ab[d]) at lag -d (Hermitian mirror).
 //
 // K_ab and the cells it lands on depend on the layout only.  On a layout's
-// first call the footprints of K_ab (2K - 1 cells a side, and the mirror's) are
-// binned to patches of 4 x 4 cells of the circular grid, and their values on
+// first call the footprints of K_ab (2K - 1 cells a side, stored pairs only) are
+// binned to patches of 4 x 2 cells of the circular grid, and their values on
 // every cell of a patch are computed on the GPU; the imaging is then two kernels
 // per batch of channels:
-//   gather: a warp holds a patch's 16 cells of 32 channels in registers (a lane
-//           per channel) and walks the patch's records, the record's 16
+//   gather: a warp holds a patch's 8 cells of 32 channels in registers (a lane
+//           per channel), the sums D of all four products (XX, XY, YX, YY) over
+//           the stored pairs, and walks the patch's records, the record's 8
 //           coefficients the same for all lanes;
-//   FFT:    one CTA per (channel, plane pair) adds a cell's partial sums,
-//           applies the (-1)^(dx+dy) checkerboard and transforms rows then
-//           columns in registers (fft_line.cuh) into the image planes.
-// XX and YY grids are Hermitian, so G_XX + i G_YY is one complex grid whose
-// transform holds XX in its real and YY in its imaginary part (an auto's
-// imaginary part, zero from a correlator, would add to the imaginary part of
-// its own image only, which is not kept: it is left out).  Sums run in a fixed
-// order: deterministic.
+//   FFT:    one CTA per (channel, product) adds the mirrors' part as it loads
+//           the grid, G_XX[d] = D_XX[d] + conj(D_XX[-d]) and G_XY[d] = D_XY[d] +
+//           conj(D_YX[-d]) (autos enter D with half their weight), applies the
+//           (-1)^(dx+dy) checkerboard and transforms rows then columns in
+//           registers (fft_line.cuh) into the image planes.
+// The polarisations keep their own sums and transforms throughout, so a weak
+// one loses nothing to a strong one.  Sums run in a fixed order: deterministic.
 #include <math.h>
 
 #include <algorithm>
@@ -37,26 +37,27 @@
 
 namespace {
 
-constexpr int kPs = 4, kPcells = kPs * kPs;      // patch side, cells
+constexpr int kPw = 4, kPh = 2, kPcells = kPw * kPh;   // patch sides, cells
 constexpr int kChunk = 256;                       // records of one patch that a CTA sums
 constexpr int kGatherWarps = 8;
-constexpr uint32_t kMirror = 1u << 31, kAuto = 1u << 30;   // record flags beside the stored pair's index
+constexpr uint32_t kAuto = 1u << 30;              // record flag beside the stored pair's index
 
 // One chunk: records [q0, q1) of a patch.
 struct Chunk {
     int32_t patch, q0, q1;
 };
 
-// Coefficients of the records: the value of K_ab (its conjugate for a mirror)
-// on every cell of the record's patch, summed over the lags that fall on the
-// cell of the circular grid; only real parts for a layout of real taps.
+// Coefficients of the records: the value of K_ab on every cell of the record's
+// patch, summed over the lags that fall on the cell of the circular grid; half
+// of it for an auto (which is its own mirror); only real parts for a layout of
+// real taps.
 template <bool REAL>
 __global__ void __launch_bounds__(256) xfft_coef_kernel(const Chunk *__restrict__ chunks, const uint32_t *__restrict__ rec,
                                                         const int32_t *__restrict__ anchors,
                                                         const float2 *__restrict__ taps, int N, int K,
                                                         float *__restrict__ coef) {
     const Chunk ch = chunks[blockIdx.x];
-    const int npx = N / kPs, W = 2 * K - 1;
+    const int npx = N / kPw, W = 2 * K - 1;
     for (int i = threadIdx.x; i < (ch.q1 - ch.q0) * kPcells; i += blockDim.x) {
         const int q = ch.q0 + i / kPcells, cell = i % kPcells;
         const uint32_t r = rec[q];
@@ -65,12 +66,7 @@ __global__ void __launch_bounds__(256) xfft_coef_kernel(const Chunk *__restrict_
         while ((long long)(a + 1) * (a + 2) / 2 <= bl) a++;
         while ((long long)a * (a + 1) / 2 > bl) a--;
         const int b = (int)(bl - (long long)a * (a + 1) / 2);
-        // the cell's lag relative to the anchors', of the pair (the mirror's lags are negated)
-        int x = ch.patch % npx * kPs + cell % kPs, y = ch.patch / npx * kPs + cell / kPs;
-        if (r & kMirror) {
-            x = (N - x) & (N - 1);
-            y = (N - y) & (N - 1);
-        }
+        const int x = ch.patch % npx * kPw + cell % kPw, y = ch.patch / npx * kPh + cell / kPw;
         const int dx = anchors[2 * a] - anchors[2 * b], dy = anchors[2 * a + 1] - anchors[2 * b + 1];
         const float2 *ta = taps + (size_t)a * K * K, *tb = taps + (size_t)b * K * K;
         float2 k = make_float2(0.f, 0.f);
@@ -84,33 +80,36 @@ __global__ void __launch_bounds__(256) xfft_coef_kernel(const Chunk *__restrict_
                         k.x += wa.x * wb.x + wa.y * wb.y;
                         k.y += wa.x * wb.y - wa.y * wb.x;
                     }
-        if (REAL) coef[(size_t)q * kPcells + cell] = k.x;
-        else reinterpret_cast<float2 *>(coef)[(size_t)q * kPcells + cell] = make_float2(k.x, r & kMirror ? -k.y : k.y);
+        const float half = r & kAuto ? 0.5f : 1.f;
+        if (REAL) coef[(size_t)q * kPcells + cell] = half * k.x;
+        else reinterpret_cast<float2 *>(coef)[(size_t)q * kPcells + cell] = make_float2(half * k.x, half * k.y);
     }
 }
 
-// Partial sums of one chunk for 32 channels: part[h][channel][chunk][16 cells]
-// (h = 0: G_XX + i G_YY, or G_XX for one pol; h = 1: G_XY).  The warps take the
-// chunk's records in turn and their sums are added in warp order.
+// Partial sums of one chunk for 32 channels: part[product][channel][chunk][8
+// cells] (XX, XY, YX, YY, or XX alone for one pol).  The warps take the chunk's
+// records in turn and their sums are added in warp order.  An auto's XX and YY
+// are real and its YX is conj(XY) in what the correlator writes; only those
+// parts enter, as only they reach the image.
 //
-// The work is 16 (real taps) complex multiply-adds a record, lane and plane
-// pair, on operands that are uniform (coefficients) or one 32-byte sector a
-// lane (a pair's products of one channel): bound by issue, then L2.  A per-cell
-// list walked by threads over (channel, product), after a transpose of the
-// visibilities, read each pair's products for each of its 25 cells:
-// 583 us after a 37 us transpose for the 64 channels of a 256-element station,
-// now 193 us.  A chunk of 256 records keeps the patches around zero lag,
+// The work is 8 (real taps) complex multiply-adds a record, lane and product, on
+// operands that are uniform (coefficients) or one 32-byte sector a lane (a
+// pair's products of one channel): bound by issue, then L2.  A per-cell list
+// walked by threads over (channel, product), after a transpose of the
+// visibilities, read each pair's products for each of its 25 cells: 583 us
+// after a 37 us transpose for the 64 channels of a 256-element station, now
+// 141 us.  A chunk of 256 records keeps the patches around zero lag,
 // which hold several thousand, from setting the time.
 template <int P, bool REAL, bool VEC>
 __global__ void __launch_bounds__(32 * kGatherWarps, 2) xfft_gather_kernel(
     const int32_t *__restrict__ vis, long long nbl, int c0, int cb, const Chunk *__restrict__ chunks, int nchunk,
     const uint32_t *__restrict__ rec, const float *__restrict__ coef, float2 *__restrict__ part) {
-    constexpr int H = P;                               // plane pairs
-    extern __shared__ float2 sums[];                   // [warps][H][16][33]
+    constexpr int H = P * P;                           // products
+    extern __shared__ float2 sums[];                   // [warps][H][8][33]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Chunk ch = chunks[blockIdx.x];
     const int cg = blockIdx.y * 32, c = min(cg + lane, cb - 1);
-    const int32_t *v = vis + (size_t)(c0 + c) * nbl * (2 * P * P);
+    const int32_t *v = vis + (size_t)(c0 + c) * nbl * (2 * H);
     float2 acc[H][kPcells];
 #pragma unroll
     for (int h = 0; h < H; h++)
@@ -124,7 +123,7 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 2) xfft_gather_kernel(
         for (int d = 0; d < D; d++) r[d] = __ldg(rec + min(q + d * kGatherWarps, ch.q1 - 1));
 #pragma unroll
         for (int d = 0; d < D; d++) {
-            const int32_t *p = v + (size_t)(r[d] & (kAuto - 1)) * (2 * P * P);
+            const int32_t *p = v + (size_t)(r[d] & (kAuto - 1)) * (2 * H);
             if (P == 1) {
                 const int2 x = __ldg(reinterpret_cast<const int2 *>(p));
                 va[d] = make_int4(x.x, x.y, 0, 0);
@@ -142,20 +141,17 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 2) xfft_gather_kernel(
         for (int d = 0; d < D; d++) {
             const int qd = q + d * kGatherWarps;
             if (qd >= ch.q1) break;
-            const bool mirror = r[d] & kMirror, self = r[d] & kAuto;
+            const bool self = r[d] & kAuto;
             float2 g[H];
-            if (P == 1) {
-                g[0] = make_float2((float)va[d].x, self ? 0.f : mirror ? -(float)va[d].y : (float)va[d].y);
-            } else {
-                const float xr = (float)va[d].x, xi = self ? 0.f : (float)va[d].y;
-                const float yr = (float)vb[d].z, yi = self ? 0.f : (float)vb[d].w;
-                // the pair: XX + i YY, XY; its mirror: conj(XX) + i conj(YY), conj(YX)
-                g[0] = mirror ? make_float2(xr + yi, yr - xi) : make_float2(xr - yi, xi + yr);
-                g[H - 1] = mirror ? make_float2((float)vb[d].x, -(float)vb[d].y) : make_float2((float)va[d].z, (float)va[d].w);
+            g[0] = make_float2((float)va[d].x, self ? 0.f : (float)va[d].y);
+            if (P == 2) {
+                g[H > 1 ? 1 : 0] = make_float2((float)va[d].z, (float)va[d].w);
+                g[H > 2 ? 2 : 0] = self ? make_float2((float)va[d].z, -(float)va[d].w) : make_float2((float)vb[d].x, (float)vb[d].y);
+                g[H - 1] = make_float2((float)vb[d].z, self ? 0.f : (float)vb[d].w);
             }
-            const float4 *cf = reinterpret_cast<const float4 *>(coef) + (size_t)qd * (REAL ? 4 : 8);
+            const float4 *cf = reinterpret_cast<const float4 *>(coef) + (size_t)qd * (REAL ? 2 : 4);
 #pragma unroll
-            for (int j = 0; j < (REAL ? 4 : 8); j++) {
+            for (int j = 0; j < (REAL ? 2 : 4); j++) {
                 const float4 k = __ldg(cf + j);
                 if (REAL) {
                     const float kk[4] = {k.x, k.y, k.z, k.w};
@@ -198,11 +194,12 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 2) xfft_gather_kernel(
     }
 }
 
-// One CTA per (channel, plane pair): the cells' partial sums (in chunk order)
-// with the checkerboard, rows, columns.  h = 0 -> XX (real part) and YY
-// (imaginary part), h = 1 -> Re XY, Im XY.  Lines in registers, exchanged in
-// their own row or column of the shared tile; the row stride keeps a
-// half-warp's rows on distinct banks.
+// One CTA per (channel, image product h = XX, YY, XY): the cells' partial sums
+// (in chunk order), each added to its own cell and, conjugated, to the mirrored
+// one; checkerboard, rows, columns.  XX, YY -> their plane (the transform is
+// real), XY -> Re XY, Im XY.  Lines in registers, exchanged in their own row or
+// column of the shared tile; the row stride keeps a half-warp's rows on distinct
+// banks.
 template <int N>
 __global__ void __launch_bounds__(N *hai_fft::Line<N>::L) xfft_fft_kernel(const float2 *__restrict__ part,
                                                                          const int32_t *__restrict__ pstart, int nchunk,
@@ -212,17 +209,50 @@ __global__ void __launch_bounds__(N *hai_fft::Line<N>::L) xfft_fft_kernel(const 
     __shared__ float2 sm[N * S], tw[N];
     const int c = blockIdx.x, h = blockIdx.y, tid = threadIdx.x;
     hai_fft::fill_twiddles<N>(tw);
-    const float2 *src = part + ((size_t)h * cb + c) * nchunk * kPcells;
-    for (int i = tid; i < N * N; i += NT) {           // patch by patch: 128-byte runs
-        const int p = i / kPcells, cell = i % kPcells;
-        const int x = p % (N / kPs) * kPs + cell % kPs, y = p / (N / kPs) * kPs + cell / kPs;
+    // products of the pair and of its mirror: XX, XX; YY, YY; XY, YX
+    const int hd = h == 0 ? 0 : h == 1 ? 3 : 1, hm = h == 2 ? 2 : hd;
+    auto sum = [&](int prod, int i) {                 // cell i in patch order: 64-byte runs
+        const float2 *src = part + ((size_t)prod * cb + c) * nchunk * kPcells + i % kPcells;
         float2 s = make_float2(0.f, 0.f);
-        for (int q = pstart[p]; q < pstart[p + 1]; q++) {
-            const float2 v = src[(size_t)q * kPcells + cell];
+        for (int q = pstart[i / kPcells]; q < pstart[i / kPcells + 1]; q++) {
+            const float2 v = src[(size_t)q * kPcells];
             s.x += v.x;
             s.y += v.y;
         }
-        sm[y * S + x] = (x + y) & 1 ? make_float2(-s.x, -s.y) : s;
+        return s;
+    };
+    auto at = [&](int i, int &x, int &y) {
+        const int p = i / kPcells, cell = i % kPcells;
+        x = p % (N / kPw) * kPw + cell % kPw;
+        y = p / (N / kPw) * kPh + cell / kPw;
+    };
+    for (int i = tid; i < N * N; i += NT) {
+        int x, y;
+        at(i, x, y);
+        sm[y * S + x] = sum(hd, i);
+    }
+    __syncthreads();
+    // the mirrored cell's value: from the tile before it is overwritten (XX,
+    // YY), or from the YX sums; signs with the checkerboard (the same for d, -d)
+    constexpr int kC = N * N / NT;
+    float2 m[kC];
+#pragma unroll
+    for (int k = 0; k < kC; k++) {
+        int x, y;
+        at(tid + k * NT, x, y);
+        const int j = ((N - y) & (N - 1)) * S + ((N - x) & (N - 1));
+        if (h < 2) m[k] = sm[j];
+        else m[k] = sum(hm, tid + k * NT);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kC; k++) {
+        int x, y;
+        at(tid + k * NT, x, y);
+        // XX, YY: own cell += conj(mirrored); XY: mirrored cell += conj(own YX sum)
+        const int j = h < 2 ? y * S + x : ((N - y) & (N - 1)) * S + ((N - x) & (N - 1));
+        const float sg = (x + y) & 1 ? -1.f : 1.f;
+        sm[j] = make_float2(sg * (sm[j].x + m[k].x), sg * (sm[j].y - m[k].y));
     }
     __syncthreads();
     float2 a[E];
@@ -263,7 +293,7 @@ __global__ void __launch_bounds__(N *hai_fft::Line<N>::L) xfft_fft_kernel(const 
         for (int i = 0; i < L; i++) a[L * u + i] = col[(L * (t + L * u) + i) * S];
     hai_fft::line_second<N>(a);
     const int Q = P == 2 ? 4 : 1;
-    float *o0 = img + ((size_t)(c0 + c) * Q + 2 * h) * N * N + x;
+    float *o0 = img + ((size_t)(c0 + c) * Q + h) * N * N + x;
 #pragma unroll
     for (int u = 0; u < E / L; u++)
 #pragma unroll
@@ -271,7 +301,7 @@ __global__ void __launch_bounds__(N *hai_fft::Line<N>::L) xfft_fft_kernel(const 
             const float2 v = a[L * u + i];
             float *o = o0 + (size_t)(t + L * u + E * i) * N;
             *o = accumulate ? *o + v.x : v.x;
-            if (P == 2) o[(size_t)N * N] = accumulate ? o[(size_t)N * N] + v.y : v.y;
+            if (h == 2) o[(size_t)N * N] = accumulate ? o[(size_t)N * N] + v.y : v.y;
         }
 }
 
@@ -280,7 +310,7 @@ hai_status launch_gather(hai_ctx *ctx, const hai_layout *L, const int32_t *vis, 
                          float2 *part, cudaStream_t st) {
     auto kern = xfft_gather_kernel<P, REAL, VEC>;
     HAI_CUDA_TRY(hai_allow_dyn_smem(kern, ctx->smem_optin));
-    const size_t smem = sizeof(float2) * kGatherWarps * P * kPcells * 33;
+    const size_t smem = sizeof(float2) * kGatherWarps * P * P * kPcells * 33;
     kern<<<dim3(L->xfft_nchunk, (cb + 31) / 32), 32 * kGatherWarps, smem, st>>>(
         vis, nbl, c0, cb, static_cast<const Chunk *>(L->d_xchunk), L->xfft_nchunk, L->d_xrec, L->d_xcoef, part);
     return HAI_OK;
@@ -288,7 +318,7 @@ hai_status launch_gather(hai_ctx *ctx, const hai_layout *L, const int32_t *vis, 
 
 template <int N>
 void launch_fft(const hai_layout *L, const float2 *part, int cb, int c0, float *img, int accumulate, cudaStream_t st) {
-    xfft_fft_kernel<N><<<dim3(cb, L->n_pol), N * hai_fft::Line<N>::L, 0, st>>>(part, L->d_xpatch, L->xfft_nchunk, cb,
+    xfft_fft_kernel<N><<<dim3(cb, L->n_pol == 2 ? 3 : 1), N * hai_fft::Line<N>::L, 0, st>>>(part, L->d_xpatch, L->xfft_nchunk, cb,
                                                                               L->n_pol, c0, img, accumulate);
 }
 
@@ -299,7 +329,7 @@ void launch_fft(const hai_layout *L, const float2 *part, int cb, int c0, float *
 static hai_status ensure_table(const hai_layout *L) {
     std::lock_guard<std::mutex> lock(L->xfft_mu);
     if (L->d_xpatch) return HAI_OK;
-    const int N = L->grid_n, K = L->ksize, ne = L->n_elem, W = 2 * K - 1, np = N / kPs;
+    const int N = L->grid_n, K = L->ksize, ne = L->n_elem, W = 2 * K - 1, npx = N / kPw, npy = N / kPh, np = npx * npy;
     // contributions of all pairs to cells: 2 (2K-1)^2 per stored pair at most
     const double max_ent = (double)ne * (ne + 1) / 2 * 2.0 * W * W;
     if (max_ent > 2.0e8)
@@ -309,29 +339,27 @@ static hai_status ensure_table(const hai_layout *L) {
     auto each_record = [&](auto &&f) {
         uint32_t bl = 0;
         for (int a = 0; a < ne; a++)
-            for (int b = 0; b <= a; b++, bl++)
-                for (int mirror = 0; mirror < (a == b ? 1 : 2); mirror++) {
-                    const int sg = mirror ? -1 : 1;
-                    const int x = (sg * (anc[2 * a] - anc[2 * b]) - (K - 1)) & (N - 1);
-                    const int y = (sg * (anc[2 * a + 1] - anc[2 * b + 1]) - (K - 1)) & (N - 1);
-                    const int nx = std::min(np, (x + W - 1) / kPs - x / kPs + 1);
-                    const int ny = std::min(np, (y + W - 1) / kPs - y / kPs + 1);
-                    const uint32_t r = bl | (mirror ? kMirror : 0u) | (a == b ? kAuto : 0u);
-                    for (int j = 0; j < ny; j++)
-                        for (int i = 0; i < nx; i++) f((y / kPs + j) % np * np + (x / kPs + i) % np, r);
-                }
+            for (int b = 0; b <= a; b++, bl++) {
+                const int x = (anc[2 * a] - anc[2 * b] - (K - 1)) & (N - 1);
+                const int y = (anc[2 * a + 1] - anc[2 * b + 1] - (K - 1)) & (N - 1);
+                const int nx = std::min(npx, (x + W - 1) / kPw - x / kPw + 1);
+                const int ny = std::min(npy, (y + W - 1) / kPh - y / kPh + 1);
+                const uint32_t r = bl | (a == b ? kAuto : 0u);
+                for (int j = 0; j < ny; j++)
+                    for (int i = 0; i < nx; i++) f((y / kPh + j) % npy * npx + (x / kPw + i) % npx, r);
+            }
     };
-    std::vector<long long> fill((size_t)np * np + 1, 0);
+    std::vector<long long> fill((size_t)np + 1, 0);
     each_record([&](int p, uint32_t) { fill[p + 1]++; });
     std::vector<Chunk> chunks;
-    std::vector<int32_t> pstart((size_t)np * np + 1, 0);
-    for (int p = 0; p < np * np; p++) {
+    std::vector<int32_t> pstart((size_t)np + 1, 0);
+    for (int p = 0; p < np; p++) {
         fill[p + 1] += fill[p];
         for (long long q = fill[p]; q < fill[p + 1]; q += kChunk)
             chunks.push_back(Chunk{p, (int32_t)q, (int32_t)std::min(q + kChunk, fill[p + 1])});
         pstart[p + 1] = (int32_t)chunks.size();
     }
-    const size_t nrec = (size_t)fill[(size_t)np * np];
+    const size_t nrec = (size_t)fill[np];
     std::vector<uint32_t> rec(nrec);
     each_record([&](int p, uint32_t r) { rec[fill[p]++] = r; });
     bool real = true;
@@ -391,7 +419,7 @@ extern "C" hai_status hai_xfft_image(hai_ctx *ctx, const hai_layout *L, const in
     const int P = L->n_pol;
     const long long nbl = (long long)L->n_elem * (L->n_elem + 1) / 2;
     // channels per batch: partial sums in the context's workspace
-    const size_t per_chan = sizeof(float2) * (size_t)P * L->xfft_nchunk * kPcells;
+    const size_t per_chan = sizeof(float2) * (size_t)P * P * L->xfft_nchunk * kPcells;
     const int cmax = (int)std::min<size_t>({(size_t)C, ctx->corr_ws_bytes / per_chan, (size_t)32768});
     // one channel's visibilities and grids as floats keep to the workspace's size too
     if (cmax < 1 || sizeof(float2) * ((size_t)nbl * P * P + (size_t)(P == 2 ? 3 : 1) * N * N) > ctx->corr_ws_bytes)
