@@ -18,7 +18,13 @@
 //            XY CTA also writes YX[-d] = conj(XY[d]) (I_YX = conj(I_XY)).
 // N = 512 keeps each line in registers instead: 64 threads per line, three
 // radix-8 passes and two shared-memory exchanges (fft512.cuh), the inverse
-// transform taken as conj(FFT(conj(x))); 8 lines per CTA in both passes.
+// transform taken as conj(FFT(conj(x))); 8 lines per CTA in both passes.  The XX
+// and YY images are real, so their rows go two to a transform, only columns 0 ..
+// 256 are kept between the passes, and the column pass writes the others as
+// R[-d] = conj(R[d]).  Persistent CTAs build the twiddle tables once.  16 channels
+// of the lattice: every product as a complex image, tables built by every CTA
+// (3,072 a pass), 39 + 57 us; 28 + 52 us now (bound: L2 and the exchanges'
+// barriers; 335 MB cross L2 where the image and the grid alone are 201).
 #include <algorithm>
 
 #include "fft512.cuh"
@@ -129,29 +135,57 @@ __global__ void __launch_bounds__(kThreads) fc_cols_kernel(int N, int log2n, int
     }
 }
 
-// N = 512, rows: CTA = 8 rows of one (channel, product), thread (r, tau).
-__global__ void __launch_bounds__(512) fc512_rows_kernel(const float *__restrict__ img, int P,
-                                                         float2 *__restrict__ out) {
+// N = 512: items of a channel in each pass.  Rows: 32 of 16 rows for each of XX
+// and YY, 64 of 8 rows for XY.  Columns: 33 of 8 columns (0 .. 256) for each of
+// XX and YY, 64 for XY.
+__host__ __device__ constexpr int fc512_items(int P, bool cols) { return P == 2 ? (cols ? 33 + 33 + 64 : 32 + 32 + 64) : cols ? 33 : 32; }
+
+// Rows: thread (r, tau) of line r.  A real plane's line holds rows y, y + 1 as
+// z = (row_y, row_y+1), whose transform splits into X_y[k] = (Z[k] + conj Z[-k])
+// / 2 and X_y+1[k] = (Z[k] - conj Z[-k]) / 2i.
+__global__ void __launch_bounds__(512, 3) fc512_rows_kernel(const float *__restrict__ img, int P, int C,
+                                                            float2 *__restrict__ out) {
     constexpr int N = 512;
     extern __shared__ float2 sm[];
     float2 *tw = sm;                                          // [kTwFloat2]
-    float2 *bufs = sm + hai_fft512::kTwFloat2;                // [8][kFftBuf]
     hai_fft512::fill_fft512_tables(tw);
-    const int r = threadIdx.x >> 6, tau = threadIdx.x & 63;
-    const int np = (P == 2) ? 3 : 1, Q = (P == 2) ? 4 : 1;
-    const int c = blockIdx.x / np, pr = blockIdx.x % np;
-    const int y = blockIdx.y * 8 + r;
-    const size_t NN = (size_t)N * N;
-    const float *re = img + ((size_t)c * Q + (pr == 2 ? 2 : pr)) * NN + (size_t)y * N;
-    float2 a[8];
-#pragma unroll
-    for (int m = 0; m < 8; m++)                               // conj of the input: exponent -
-        a[m] = make_float2(__ldg(re + tau + 64 * m), pr == 2 ? -__ldg(re + NN + tau + 64 * m) : 0.f);
     __syncthreads();
-    hai_fft512::fft512<false>(a, tau, bufs + r * hai_fft512::kFftBuf, tw, [] { __syncthreads(); });
-    float2 *dst = out + ((size_t)c * P * P + out_plane(pr, P)) * NN + (size_t)y * N;
+    const int r = threadIdx.x >> 6, tau = threadIdx.x & 63;
+    float2 *buf = sm + hai_fft512::kTwFloat2 + r * hai_fft512::kFftBuf;
+    const int per = fc512_items(P, false), Q = (P == 2) ? 4 : 1;
+    const size_t NN = (size_t)N * N;
+    for (int it = blockIdx.x; it < C * per; it += gridDim.x) {
+        const int c = it / per, k = it % per, pr = k >> 5 > 2 ? 2 : k >> 5;
+        const bool real = pr < 2;
+        const int y = real ? 16 * (k & 31) + 2 * r : 8 * (k - 64) + r;
+        // second component: the next row (real plane), or the next plane
+        const float *re = img + ((size_t)c * Q + pr) * NN + (size_t)y * N, *im = re + (real ? N : NN);
+        float2 a[8];
 #pragma unroll
-    for (int j = 0; j < 8; j++) dst[tau + 64 * j] = make_float2(a[j].x, -a[j].y);
+        for (int m = 0; m < 8; m++)                           // conj of the input: exponent -
+            a[m] = make_float2(__ldg(re + tau + 64 * m), -__ldg(im + tau + 64 * m));
+        hai_fft512::fft512<false>(a, tau, buf, tw, [] { __syncthreads(); });
+        float2 *dst = out + ((size_t)c * P * P + out_plane(pr, P)) * NN + (size_t)y * N;
+        if (!real) {                                          // CTA-uniform
+#pragma unroll
+            for (int j = 0; j < 8; j++) dst[tau + 64 * j] = make_float2(a[j].x, -a[j].y);
+            __syncthreads();
+            continue;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 8; j++) buf[tau + 64 * j] = make_float2(a[j].x, -a[j].y);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 5; j++) {
+            const int kx = tau + 64 * j;
+            if (kx > N / 2) break;
+            const float2 z = buf[kx], w = buf[(N - kx) & (N - 1)];
+            dst[kx] = make_float2(0.5f * (z.x + w.x), 0.5f * (z.y - w.y));
+            dst[N + kx] = make_float2(0.5f * (z.y + w.y), 0.5f * (w.x - z.x));
+        }
+        __syncthreads();
+    }
 }
 
 // N = 512, columns: CTA = 8 adjacent columns of one (channel, product).  The
@@ -163,7 +197,7 @@ __global__ void __launch_bounds__(512) fc512_rows_kernel(const float *__restrict
 // its column; times (-1)^(dx+dy) / N^2; the XY CTA also writes the YX mirror.
 constexpr int kTs = 514;
 
-__global__ void __launch_bounds__(512) fc512_cols_kernel(int P, float2 *__restrict__ out) {
+__global__ void __launch_bounds__(512, 3) fc512_cols_kernel(int P, int C, float2 *__restrict__ out) {
     constexpr int N = 512;
     extern __shared__ float2 sm[];
     float2 *tw = sm;
@@ -171,45 +205,56 @@ __global__ void __launch_bounds__(512) fc512_cols_kernel(int P, float2 *__restri
     float2 *tile = bufs;
     static_assert(8 * kTs <= 8 * hai_fft512::kFftBuf, "tile inside the exchange buffers");
     hai_fft512::fill_fft512_tables(tw);
+    __syncthreads();
     const int col = threadIdx.x >> 6, tau = threadIdx.x & 63;
     const int lc = threadIdx.x & 7, lr = threadIdx.x >> 3;     // row-segment mapping: column, row of 64
-    const int np = (P == 2) ? 3 : 1;
-    const int c = blockIdx.x / np, pr = blockIdx.x % np;
-    const int x0 = blockIdx.y * 8;
+    const int per = fc512_items(P, true);
     const size_t NN = (size_t)N * N;
-    float2 *plane = out + ((size_t)c * P * P + out_plane(pr, P)) * NN;
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int y = lr + 64 * k;
-        tile[lc * kTs + y] = plane[(size_t)y * N + x0 + lc];
-    }
-    __syncthreads();
-    float2 a[8];
-#pragma unroll
-    for (int m = 0; m < 8; m++) {                             // conj of the input: exponent -
-        const float2 v = tile[col * kTs + tau + 64 * m];
-        a[m] = make_float2(v.x, -v.y);
-    }
-    __syncthreads();
-    hai_fft512::fft512<false>(a, tau, bufs + col * hai_fft512::kFftBuf, tw, [] { __syncthreads(); });
-    __syncthreads();                                          // exchange buffers free: the tile again
     const float inv = 1.0f / (float)NN;
-    const int dx = x0 + col;
+    for (int it = blockIdx.x; it < C * per; it += gridDim.x) {
+        const int c = it / per, k0 = it % per, pr = k0 < 33 ? 0 : k0 < 66 ? 1 : 2;
+        const bool real = pr < 2;
+        const int x0 = 8 * (k0 - 33 * pr);
+        const int ncol = real ? min(8, N / 2 + 1 - x0) : 8;
+        float2 *plane = out + ((size_t)c * P * P + out_plane(pr, P)) * NN;
+        float2 *mirror = real ? plane : out + ((size_t)c * P * P + 2) * NN;
+        if (lc < ncol) {
 #pragma unroll
-    for (int j = 0; j < 8; j++) {
-        const int dy = tau + 64 * j;
-        const float s = ((dx + dy) & 1) ? -inv : inv;
-        tile[col * kTs + dy] = make_float2(a[j].x * s, -a[j].y * s);
-    }
-    __syncthreads();
-    float2 *mirror = (pr == 2) ? out + ((size_t)c * P * P + 2) * NN : nullptr;   // YX
+            for (int k = 0; k < 8; k++) {
+                const int y = lr + 64 * k;
+                tile[lc * kTs + y] = plane[(size_t)y * N + x0 + lc];
+            }
+        }
+        __syncthreads();
+        float2 a[8];
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int dy = lr + 64 * k;
-        const float2 v = tile[lc * kTs + dy];
-        plane[(size_t)dy * N + x0 + lc] = v;
-        if (mirror)
-            mirror[(size_t)((N - dy) & (N - 1)) * N + ((N - x0 - lc) & (N - 1))] = make_float2(v.x, -v.y);
+        for (int m = 0; m < 8; m++) {                         // conj of the input: exponent -
+            const float2 v = col < ncol ? tile[col * kTs + tau + 64 * m] : make_float2(0.f, 0.f);
+            a[m] = make_float2(v.x, -v.y);
+        }
+        __syncthreads();
+        hai_fft512::fft512<false>(a, tau, bufs + col * hai_fft512::kFftBuf, tw, [] { __syncthreads(); });
+        __syncthreads();                                      // exchange buffers free: the tile again
+        const int dxc = x0 + col;
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int dy = tau + 64 * j;
+            const float s = ((dxc + dy) & 1) ? -inv : inv;
+            tile[col * kTs + dy] = make_float2(a[j].x * s, -a[j].y * s);
+        }
+        __syncthreads();
+        const int dx = x0 + lc;
+        if (lc < ncol) {
+            const bool twin = !real || (dx != 0 && dx != N / 2);
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                const int dy = lr + 64 * k;
+                const float2 v = tile[lc * kTs + dy];
+                plane[(size_t)dy * N + dx] = v;
+                if (twin) mirror[(size_t)((N - dy) & (N - 1)) * N + ((N - dx) & (N - 1))] = make_float2(v.x, -v.y);
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -240,8 +285,11 @@ extern "C" hai_status hai_fft_correlate(hai_ctx *ctx, const float *img, int C, i
         HAI_CUDA_TRY(hai_allow_dyn_smem(fc512_rows_kernel, ctx->smem_optin));
         HAI_CUDA_TRY(hai_allow_dyn_smem(fc512_cols_kernel, ctx->smem_optin));
         const int pidx = prof_begin(ctx, st);
-        fc512_rows_kernel<<<dim3(C * np, N / 8), 512, smem512, st>>>(img, P, out);
-        fc512_cols_kernel<<<dim3(C * np, N / 8), 512, smem512, st>>>(P, out);
+        if ((long long)C * fc512_items(P, true) > 0x7fffffffll)
+            return hai_fail(HAI_ERR_UNSUPPORTED, "hai_fft_correlate: too many channels");
+        const int resident = 3 * ctx->num_sms;
+        fc512_rows_kernel<<<std::min(resident, C * fc512_items(P, false)), 512, smem512, st>>>(img, P, C, out);
+        fc512_cols_kernel<<<std::min(resident, C * fc512_items(P, true)), 512, smem512, st>>>(P, C, out);
         prof_end(ctx, pidx, st);
         prof_count(ctx, 2);
         HAI_CUDA_TRY(cudaGetLastError());
