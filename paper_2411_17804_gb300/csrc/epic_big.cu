@@ -626,7 +626,8 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
     const uint32_t bbytes = (uint32_t)kKb2 * V::BTile;     // one DFT operand part of an l_y block
     if (warp == 0) {
         if (lane == 0) {
-            long long gs = 0, gk = 0;                      // samples and k blocks loaded
+            long long gs = 0;                              // samples loaded
+            int st = 0, fill = 0;                          // ring stage, times it has been filled before
             int cur_lyb = -1;
             for (long long u = u0; u < u1;) {
                 const long long it = u / tb;
@@ -650,15 +651,17 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
                         tc::bulk_prefetch_l2(p.a2 + pre, kKb2 * kTile16);
                         if constexpr (SP) tc::bulk_prefetch_l2(p.a2lo + pre, kKb2 * kTile16);
                     }
-                    for (int kb = 0; kb < kKb2; kb++, gk++) {
-                        const int st = (int)(gk % V::S2Stages);
-                        if (gk >= V::S2Stages)
-                            tc::mbar_wait(&aempty[st], (uint32_t)(((gk / V::S2Stages) - 1) & 1), p.status);
+                    for (int kb = 0; kb < kKb2; kb++) {
+                        if (fill) tc::mbar_wait(&aempty[st], (uint32_t)((fill - 1) & 1), p.status);
                         tc::mbar_arrive_expect_tx(&afull[st], V::AStage);
                         tc::bulk_g2s(sA0 + (size_t)st * V::AStage, p.a2 + base + (size_t)kb * kTile16, kTile16, &afull[st]);
                         if constexpr (SP)
                             tc::bulk_g2s(sA0 + (size_t)st * V::AStage + kTile16, p.a2lo + base + (size_t)kb * kTile16,
                                          kTile16, &afull[st]);
+                        if (++st == V::S2Stages) {
+                            st = 0;
+                            fill++;
+                        }
                     }
                 }
                 u += s1 - s0;
@@ -669,10 +672,12 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
         // split), one commit per k block (frees the A stage) and one per sample
         // (fills the accumulator)
         if (lane == 0) {
-            long long gs = 0, gk = 0;
-            int cur_lyb = -1;
-            uint32_t bph = 0;
-            const uint32_t sb0 = tc::smem_u32(sB), sa0 = tc::smem_u32(sA0);
+            long long gs = 0;
+            int cur_lyb = -1, st = 0;
+            uint32_t bph = 0, aph = 0;                     // phases of bfull, of the ring
+            // descriptors once, then 32-bit additions: scalar work between the MMAs
+            // on this thread delays them
+            const uint64_t db0 = tc::desc(tc::smem_u32(sB), kKBytes, kKMN), da0 = tc::desc(tc::smem_u32(sA0), kMKs, kMMN);
             for (long long u = u0; u < u1;) {
                 const long long it = u / tb;
                 const int s0 = (int)(u % tb), s1 = (int)std::min<long long>(tb, s0 + (u1 - u));
@@ -687,28 +692,31 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
                     if (gs >= 2) tc::mbar_wait(&dempty[b], (uint32_t)(((gs >> 1) - 1) & 1), p.status);
                     tc::fence_after();
                     const uint32_t d = tmem + (uint32_t)b * V::NM;
-                    for (int kb = 0; kb < kKb2; kb++, gk++) {
-                        const int st = (int)(gk % V::S2Stages);
+                    for (int kb = 0; kb < kKb2; kb++) {
                         // a stage filled by bulk copies (async proxy, completed on the
                         // mbarrier) needs no tcgen05 fence before the MMAs read it; the
                         // fence above orders them after the epilogue's TMEM reads
-                        tc::mbar_wait(&afull[st], (uint32_t)((gk / V::S2Stages) & 1), p.status);
-                        const uint32_t a = sa0 + (uint32_t)st * V::AStage;
-                        const uint32_t bq = sb0 + (uint32_t)kb * V::BTile;
+                        tc::mbar_wait(&afull[st], aph, p.status);
+                        const uint64_t a = tc::desc_add(da0, (uint32_t)st * V::AStage);
+                        const uint64_t bq = tc::desc_add(db0, (uint32_t)kb * V::BTile);
 #pragma unroll
                         for (int j = 0; j < 4; j++) {
                             const uint32_t acc0 = (kb > 0 || j > 0) ? 1u : 0u;
-                            const uint64_t da = tc::desc(a + j * 2 * kMKs, kMKs, kMMN);
-                            const uint64_t db = tc::desc(bq + j * 2 * kKBytes, kKBytes, kKMN);
+                            const uint64_t da = tc::desc_add(a, j * 2 * kMKs);
+                            const uint64_t db = tc::desc_add(bq, j * 2 * kKBytes);
                             tc::mma_f16(d, da, db, kIdesc, acc0);
                             if constexpr (SP) {
-                                const uint64_t dal = tc::desc(a + kTile16 + j * 2 * kMKs, kMKs, kMMN);
-                                const uint64_t dbl = tc::desc(bq + bbytes + j * 2 * kKBytes, kKBytes, kKMN);
+                                const uint64_t dal = tc::desc_add(a, kTile16 + j * 2 * kMKs);
+                                const uint64_t dbl = tc::desc_add(bq, bbytes + j * 2 * kKBytes);
                                 tc::mma_f16(d, da, dbl, kIdesc, 1u);
                                 tc::mma_f16(d, dal, db, kIdesc, 1u);
                             }
                         }
                         tc::mma_commit(&aempty[st]);
+                        if (++st == V::S2Stages) {
+                            st = 0;
+                            aph ^= 1;
+                        }
                     }
                     tc::mma_commit(&dfull[b]);
                 }
@@ -716,53 +724,50 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
             }
         }
     } else if (warp >= 2) {
-        // epilogue, warps 2-17: thread row m = (l_x, pol) of TMEM lane
-        // quadrant q, group h of Ly l_y values
+        // epilogue, warps 2-17: TMEM lane quadrant q (X in lanes 0-15, Y in 16-31
+        // of 16 output columns l_x), group h of Ly l_y values.  The 16-lane loads
+        // put X and Y of a pixel into one thread, l_x = 16 q + lane / 4 (+ 8),
+        // l_y = Ly h + 8 j + 2 (lane % 4) (+ 1), and adjacent l_y into adjacent
+        // registers: no shuffles, which took a quarter of the shared-memory
+        // bandwidth that the MMAs read their operands through, and no selects.
         const int ew = warp - 2, q = warp & 3, h = ew >> 2;
-        const int m = 32 * q + lane;
-        const int pol = (m >> 4) & 1, kx = (m >> 5) * 16 + (m & 15);
+        const int kx = 16 * q + (lane >> 2);
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        constexpr int kLy = V::Ly;
+        constexpr int kLy = V::Ly, kPair = kLy / 4;        // pixel pairs (l_y, l_y + 1): [j][l_x half]
         const size_t NN = (size_t)g.N * g.N;
-        float2 acc_a[kLy / 2], acc_x[kLy / 2];
+        float2 axx[kPair], ayy[kPair], are[kPair], aim[kPair];
         long long gs = 0;
         for (long long u = u0; u < u1;) {
             const long long it = u / tb;
             const int s0 = (int)(u % tb), s1 = (int)std::min<long long>(tb, s0 + (u1 - u));
             const int lyb = (int)(it / per_lyb), rem = (int)(it % per_lyb), c = rem / g.lb2, lxb = rem % g.lb2;
 #pragma unroll
-            for (int t = 0; t < kLy / 2; t++) acc_a[t] = acc_x[t] = make_float2(0.f, 0.f);
+            for (int t = 0; t < kPair; t++) axx[t] = ayy[t] = are[t] = aim[t] = make_float2(0.f, 0.f);
             for (int s = s0; s < s1; s++, gs++) {
                 const int b = (int)(gs & 1);
                 if (lane == 0) tc::mbar_wait(&dfull[b], (uint32_t)((gs >> 1) & 1), p.status);
                 __syncwarp();
                 tc::fence_after();
-                // 8 l_y at a time (re and im: 16 registers): the pixel pairs
-                // (2k, 2k + 1) of the cross term stay inside each group
 #pragma unroll
-                for (int g8 = 0; g8 < kLy / 8; g8++) {
-                    const uint32_t col = (uint32_t)b * V::NM + (uint32_t)(kLy * h + 8 * g8);
-                    uint32_t rr[8], ri[8];
-                    tc::tmem_ld8(tmem + lane_base + col, rr);
-                    tc::tmem_ld8(tmem + lane_base + col + V::W, ri);
+                for (int j = 0; j < kLy / 8; j++) {
+                    const uint32_t x = tmem + lane_base + (uint32_t)b * V::NM + (uint32_t)(kLy * h + 8 * j), y = x + (16u << 16);
+                    uint32_t xr[4], xi[4], yr[4], yi[4];
+                    tc::tmem_ld_16x256b(x, xr);
+                    tc::tmem_ld_16x256b(x + V::W, xi);
+                    tc::tmem_ld_16x256b(y, yr);
+                    tc::tmem_ld_16x256b(y + V::W, yi);
                     tc::tmem_wait_ld();
 #pragma unroll
-                    for (int k = 0; k < 8; k += 2) {
-                        const float2 fr = make_float2(__uint_as_float(rr[k]), __uint_as_float(rr[k + 1]));
-                        const float2 fi = make_float2(__uint_as_float(ri[k]), __uint_as_float(ri[k + 1]));
-                        float2 &a = acc_a[(8 * g8 + k) >> 1];
-                        a = __ffma2_rn(fr, fr, __ffma2_rn(fi, fi, a));
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        const float e_r = __uint_as_float(rr[2 * k]), e_i = __uint_as_float(ri[2 * k]);
-                        const float o_r = __uint_as_float(rr[2 * k + 1]), o_i = __uint_as_float(ri[2 * k + 1]);
-                        const float mr = pol ? o_r : e_r, mi = pol ? o_i : e_i;
-                        const float sr = __shfl_xor_sync(0xffffffffu, pol ? e_r : o_r, 16);
-                        const float si = __shfl_xor_sync(0xffffffffu, pol ? e_i : o_i, 16);
-                        float2 &a = acc_x[4 * g8 + k];
-                        a = __ffma2_rn(make_float2(mr, mi), make_float2(sr, sr),
-                                       __ffma2_rn(make_float2(mi, -mr), make_float2(si, si), a));
+                    for (int r = 0; r < 2; r++) {
+                        const int t = 2 * j + r;
+                        const float2 ar = make_float2(__uint_as_float(xr[2 * r]), __uint_as_float(xr[2 * r + 1]));
+                        const float2 ai = make_float2(__uint_as_float(xi[2 * r]), __uint_as_float(xi[2 * r + 1]));
+                        const float2 br = make_float2(__uint_as_float(yr[2 * r]), __uint_as_float(yr[2 * r + 1]));
+                        const float2 bi = make_float2(__uint_as_float(yi[2 * r]), __uint_as_float(yi[2 * r + 1]));
+                        axx[t] = __ffma2_rn(ar, ar, __ffma2_rn(ai, ai, axx[t]));
+                        ayy[t] = __ffma2_rn(br, br, __ffma2_rn(bi, bi, ayy[t]));
+                        are[t] = __ffma2_rn(ar, br, __ffma2_rn(ai, bi, are[t]));
+                        aim[t] = __ffma2_rn(ai, br, __ffma2_rn(make_float2(-ar.x, -ar.y), bi, aim[t]));
                     }
                 }
                 tc::fence_before();
@@ -786,26 +791,18 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
                 ps = (size_t)V::W * 64;
                 add = false;
             }
+            auto put = [&](int plane, const float2 (&a)[kPair]) {
 #pragma unroll
-            for (int t = 0; t < kLy; t++) {
-                float *d = dst + pol * ps + (size_t)(kLy * h + t) * rs + kx;
-                float v = (t & 1) ? acc_a[t >> 1].y : acc_a[t >> 1].x;
-                if (add) v += *d;
-                *d = v;
-            }
-            const float sgn = pol ? -1.f : 1.f;
-#pragma unroll
-            for (int t = 0; t < kLy / 2; t++) {
-                const int ly = kLy * h + 16 * (t >> 3) + 2 * (t & 7) + pol;
-                float *d = dst + 2 * ps + (size_t)ly * rs + kx;
-                float vr = acc_x[t].x, vi = sgn * acc_x[t].y;
-                if (add) {
-                    vr += d[0];
-                    vi += d[ps];
+                for (int t = 0; t < kPair; t++) {
+                    float *d = dst + plane * ps + (size_t)(kLy * h + 8 * (t >> 1) + 2 * (lane & 3)) * rs + kx + 8 * (t & 1);
+                    d[0] = add ? d[0] + a[t].x : a[t].x;
+                    d[rs] = add ? d[rs] + a[t].y : a[t].y;
                 }
-                d[0] = vr;
-                d[ps] = vi;
-            }
+            };
+            put(0, axx);
+            put(1, ayy);
+            put(2, are);
+            put(3, aim);
             u += s1 - s0;
         }
     }
