@@ -22,7 +22,7 @@
 // grid.  The two complex grids are built in the caller's image planes
 // [XX, YY, Re XY, Im XY] (as split re / im planes), which the FFT then
 // transforms in place: no scratch memory.  Gridding runs over tiles of the uv
-// grid with a thread per cell, the footprints binned to tiles on the host, and
+// grid with a thread per cell, the pairs binned to tiles on the host, and
 // writes its cells with the (-1)^(u+v) checkerboard that puts the phase
 // centre at pixel (N/2, N/2).  The FFTs hold their lines in registers
 // (fft_line.cuh).
@@ -37,23 +37,31 @@
 
 namespace {
 
-// Tiles of the periodic uv grid (x = u mod N, y = v mod N), the unit of gridding
-// work: 16 x 16 cells, a thread per cell.
+// Tiles of the periodic uv grid (x = u mod N, y = v mod N), 16 x 16 cells with a
+// thread per cell.  The unit of gridding work is a tile and its mirror: tile t
+// along an axis holds the lower corners 16 t .. 16 t + 15, whose mirrors' lower
+// corners fall in tile -t - 1, so that a pair's visibilities are read once for
+// both of its footprints.
 constexpr int kTile = 16, kTcells = kTile * kTile;
-constexpr int kTileWarps = kTcells / 32;
+constexpr int kGridThreads = 2 * kTcells;         // the tile's cells, then the mirror tile's
+constexpr int kGridWarps = kGridThreads / 32;
 constexpr int kImgs = 4;                          // images (beam, channel) a CTA grids together
-constexpr int kFoot = 1024;                       // footprints staged at a time
-constexpr uint32_t kMirror = 1u << 31;            // footprint of the mirror (n, m) of a stored pair
+constexpr int kFoot = 512;                        // pairs staged at a time
+constexpr int kFootRow = kFoot + 4;               // float4 per staged row: direct and mirrored values 4 banks apart
 
-// One chunk of a tile's footprints and, per warp, its gather entries: slot k
-// of lane l at entry base[w] + 32 k + l (zero weights pad the shorter lists).
+// One chunk of a unit's pairs and, per warp, its gather entries: slot k of lane
+// l at entry base[w] + 32 k + l (zero weights pad the shorter lists).
 struct TileChunk {
     int32_t foot, nfoot;
-    int32_t base[kTileWarps + 1];
+    int32_t base[kGridWarps + 1];
 };
 struct TileEnt {
     float w;             // bilinear weight
-    int32_t slot;        // footprint within the chunk
+    int32_t slot;        // pair within the chunk; + kFootRow: its mirror's value
+};
+// Tiles of a unit (mirror < 0: none), and its first chunk.
+struct TileUnit {
+    int32_t tile, mirror, chunk;
 };
 
 __device__ __forceinline__ void pair_of(long long bl, int &m, int &n) {
@@ -85,83 +93,72 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// One pair's visibilities of one image: XX, XY, YX, YY.
-template <bool VEC>
-__device__ __forceinline__ void load_vis(const int32_t *__restrict__ v, int4 &a, int4 &b) {
-    if (VEC) {
-        a = __ldg(reinterpret_cast<const int4 *>(v));
-        b = __ldg(reinterpret_cast<const int4 *>(v) + 1);
-    } else {
-        const int2 *p = reinterpret_cast<const int2 *>(v);
-        const int2 x = __ldg(p), y = __ldg(p + 1), z = __ldg(p + 2), w = __ldg(p + 3);
-        a = make_int4(x.x, x.y, y.x, y.y);
-        b = make_int4(z.x, z.y, w.x, w.y);
-    }
-}
-
 // G_XX + i G_YY into planes 0 / 1 and G_XY into planes 2 / 3 of kImgs images per
-// CTA, one tile of the grid, with the checkerboard.  The tile's footprints (of
-// pairs and of their mirrors) are phased once into shared memory, a chunk at a
-// time, and every cell (thread) then adds its own list of them: no atomics, and
-// a fixed order, so the images are bit-reproducible.  The lists are the same
-// for every image: entries are read once per kImgs images; cells are dealt to
-// the lanes by list length, so a warp's lanes end together.  Tiles are the fast
+// CTA, one tile of the grid and its mirror, with the checkerboard.  The unit's
+// pairs are phased once into shared memory, a chunk at a time, as the value of
+// the pair (XX + i YY, XY) and that of its mirror (conj(XX) + i conj(YY),
+// conj(YX)), and every cell (thread) then adds its own list of them: no atomics,
+// and a fixed order, so the images are bit-reproducible.  Two lanes share a
+// pair's 32-byte sector (XX, XY | YX, YY) and exchange XX for YY; one then holds
+// the pair's value and the other the mirror's.  The lists are the same for every
+// image: entries and phasors are read once per kImgs images; cells are dealt to
+// the lanes by list length, so a warp's lanes end together.  Units are the fast
 // grid index, so a group's visibilities (1 MB an image for 256 stations) come
-// from HBM once and from L2 for the mirrors and the neighbouring tiles.  Grid
-// rows whose tiles are all empty are left unwritten: the FFT passes do not
-// read them.
+// from HBM once and from L2 for the neighbouring tiles.  Grid rows whose tiles
+// are all empty are left unwritten: the FFT passes do not read them.
 //
-// Bound: the divergent loads of the staging (a sector per footprint and image)
-// and shared-memory wavefronts (one 16-byte random read per entry and image).
+// Bound: shared-memory wavefronts (one 16-byte random read per entry and image).
 // Hierarchical cadence (256 stations, 512 images at 256^2): adding the
 // footprints with shared-memory atomics took 902 us after an 85 us memset of
 // all planes; a lane per image with the cells in registers 798 us (32 lanes a
-// megabyte apart, 1.4 GB read from HBM); this form 616 us.
+// megabyte apart, 1.4 GB read from HBM); a tile at a time with a lane per
+// footprint's two 16-byte loads 616 us (32 lines a load); this form 511 us.
 template <bool VEC>
-__global__ void __launch_bounds__(kTcells, 3) station_grid_kernel(
+__global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
     const int32_t *__restrict__ vis, const uint32_t *__restrict__ foot, const TileEnt *__restrict__ ent,
-    const TileChunk *__restrict__ chunks, const int32_t *__restrict__ tile, const int32_t *__restrict__ tchunk,
-    const uint8_t *__restrict__ cell_of, int ntile, const float2 *__restrict__ phasor, int C, int images,
-    long long nbl, int N, float *__restrict__ img) {
-    extern __shared__ __align__(16) float4 stage[];     // [kImgs][kFoot]; at the end [kImgs][4][256] floats
+    const TileChunk *__restrict__ chunks, const TileUnit *__restrict__ unit, const uint8_t *__restrict__ cell_of,
+    int nunit, const float2 *__restrict__ phasor, int C, int images, long long nbl, int N, float *__restrict__ img) {
+    extern __shared__ __align__(16) float4 stage[];     // [kImgs][2][kFootRow]; at the end [kImgs][4][512] floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int grp = blockIdx.x / ntile, o = blockIdx.x - grp * ntile;
-    const int i0 = grp * kImgs;
-    const int32_t *v[kImgs];
-    const float2 *ph[kImgs];
-#pragma unroll
-    for (int i = 0; i < kImgs; i++) {
-        const int im = min(i0 + i, images - 1);
-        v[i] = vis + (size_t)im * nbl * 8;
-        ph[i] = phasor + (size_t)(im / C) * nbl;
-    }
+    const int grp = blockIdx.x / nunit, o = blockIdx.x - grp * nunit;
+    const int i0 = grp * kImgs, i1 = min(i0 + kImgs, images) - 1;
+    const bool same = i0 / C == i1 / C;                 // one beam: one phasor for all images
     float4 acc[kImgs];
 #pragma unroll
     for (int i = 0; i < kImgs; i++) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int q0 = tchunk[o], q1 = tchunk[o + 1];
+    const int half = lane & 1;                          // XX, XY or YX, YY
+    const int q0 = unit[o].chunk, q1 = unit[o + 1].chunk;
     for (int q = q0; q < q1; q++) {
         const TileChunk *ch = chunks + q;
         const int f0 = ch->foot, nf = ch->nfoot;
         if (q > q0) __syncthreads();                    // the last chunk's gather is done
-        for (int f = tid; f < nf; f += kTcells) {
-            const uint32_t r = __ldg(foot + f0 + f);
-            const bool mirror = r & kMirror;
-            const size_t bl = r & (kMirror - 1);
-            int4 a[kImgs], b[kImgs];
+        // whole warps stay in the loop for the exchange
+        for (int fw = (tid >> 1) & ~15; fw < nf; fw += kGridThreads / 2) {
+            const int f = fw + (lane >> 1);
+            const size_t bl = __ldg(foot + f0 + min(f, nf - 1));
+            int4 x[kImgs];
             float2 w[kImgs];
 #pragma unroll
             for (int i = 0; i < kImgs; i++) {
-                load_vis<VEC>(v[i] + bl * 8, a[i], b[i]);
-                w[i] = __ldg(ph[i] + bl);
+                const int im = min(i0 + i, images - 1);
+                const int32_t *v = vis + ((size_t)im * nbl + bl) * 8 + 4 * half;
+                if (VEC) {
+                    x[i] = __ldg(reinterpret_cast<const int4 *>(v));
+                } else {
+                    const int2 a = __ldg(reinterpret_cast<const int2 *>(v)), b = __ldg(reinterpret_cast<const int2 *>(v) + 1);
+                    x[i] = make_int4(a.x, a.y, b.x, b.y);
+                }
+                w[i] = i > 0 && same ? w[0] : __ldg(phasor + (size_t)(im / C) * nbl + bl);
             }
 #pragma unroll
             for (int i = 0; i < kImgs; i++) {
-                const float2 xx = cmulf(make_float2((float)a[i].x, (float)a[i].y), w[i]);
-                const float2 yy = cmulf(make_float2((float)b[i].z, (float)b[i].w), w[i]);
-                const float2 xy = cmulf(make_float2((float)(mirror ? b[i].x : a[i].z), (float)(mirror ? b[i].y : a[i].w)), w[i]);
-                // the pair: XX + i YY, XY; its mirror: conj(XX) + i conj(YY), conj(YX)
-                stage[i * kFoot + f] = mirror ? make_float4(xx.x + yy.y, yy.x - xx.y, xy.x, -xy.y)
-                                              : make_float4(xx.x - yy.y, xx.y + yy.x, xy.x, xy.y);
+                const float2 u = cmulf(make_float2((float)x[i].x, (float)x[i].y), w[i]);      // XX or YX
+                const float2 v = cmulf(make_float2((float)x[i].z, (float)x[i].w), w[i]);      // XY or YY
+                const float sx = __shfl_xor_sync(0xffffffffu, half ? v.x : u.x, 1);
+                const float sy = __shfl_xor_sync(0xffffffffu, half ? v.y : u.y, 1);           // YY or XX
+                if (f < nf)
+                    stage[(i * 2 + half) * kFootRow + f] = half ? make_float4(sx + v.y, v.x - sy, u.x, -u.y)
+                                                                : make_float4(u.x - sy, u.y + sx, v.x, v.y);
             }
         }
         __syncthreads();
@@ -172,7 +169,7 @@ __global__ void __launch_bounds__(kTcells, 3) station_grid_kernel(
             const int slot = __float_as_int(x.y);
 #pragma unroll
             for (int i = 0; i < kImgs; i++) {
-                const float4 g = stage[i * kFoot + slot];
+                const float4 g = stage[i * 2 * kFootRow + slot];
                 acc[i].x = fmaf(x.x, g.x, acc[i].x);
                 acc[i].y = fmaf(x.x, g.y, acc[i].y);
                 acc[i].z = fmaf(x.x, g.z, acc[i].z);
@@ -181,28 +178,31 @@ __global__ void __launch_bounds__(kTcells, 3) station_grid_kernel(
         }
     }
     // the cells back in row order, then out
-    const int t = tile[o], x0 = t % (N / kTile) * kTile, y0 = t / (N / kTile) * kTile;
+    const int side = tid / kTcells, tc = tid % kTcells;
     float *cells = reinterpret_cast<float *>(stage);
     if (q1 > q0) {
         __syncthreads();
-        const int cell = cell_of[(size_t)o * kTcells + tid];
-        const float sgn = ((cell ^ (cell / kTile)) & 1) ? -1.f : 1.f;     // x0, y0 are even
+        const int cell = cell_of[(size_t)o * kGridThreads + tid];
+        const float sgn = ((cell ^ (cell / kTile)) & 1) ? -1.f : 1.f;     // tiles start on even cells
 #pragma unroll
         for (int i = 0; i < kImgs; i++) {
-            cells[(i * 4 + 0) * kTcells + cell] = sgn * acc[i].x;
-            cells[(i * 4 + 1) * kTcells + cell] = sgn * acc[i].y;
-            cells[(i * 4 + 2) * kTcells + cell] = sgn * acc[i].z;
-            cells[(i * 4 + 3) * kTcells + cell] = sgn * acc[i].w;
+            float *d = cells + (size_t)i * 4 * kGridThreads + side * kTcells + cell;
+            d[0] = sgn * acc[i].x;
+            d[kGridThreads] = sgn * acc[i].y;
+            d[2 * kGridThreads] = sgn * acc[i].z;
+            d[3 * kGridThreads] = sgn * acc[i].w;
         }
         __syncthreads();
     }
+    const int t = side ? unit[o].mirror : unit[o].tile;
+    if (t < 0) return;
+    const int x = t % (N / kTile) * kTile + tc % kTile, y = t / (N / kTile) * kTile + tc / kTile;
 #pragma unroll
     for (int i = 0; i < kImgs; i++) {
         if (i0 + i >= images) break;
 #pragma unroll
         for (int p = 0; p < 4; p++)
-            img[(((size_t)(i0 + i) * 4 + p) * N + y0 + tid / kTile) * N + x0 + tid % kTile] =
-                q1 > q0 ? cells[(i * 4 + p) * kTcells + tid] : 0.f;
+            img[(((size_t)(i0 + i) * 4 + p) * N + y) * N + x] = q1 > q0 ? cells[(i * 4 + p) * kGridThreads + tid] : 0.f;
     }
 }
 
@@ -359,12 +359,12 @@ struct hai_vis_layout {
     int S = 0, N = 0, P = 0, K = 0;
     long long nbl = 0;
     long long n_offgrid = 0;
-    int ntile = 0, nrow = 0;                 // tiles in written rows; written rows
-    uint32_t *d_foot = nullptr;              // footprints (pair, mirror bit), tile after tile
+    int nunit = 0, nrow = 0;                 // tile units in written rows; written rows
+    uint32_t *d_foot = nullptr;              // stored pairs, unit after unit
     TileEnt *d_ent = nullptr;                // gather entries
     TileChunk *d_chunk = nullptr;
-    int32_t *d_tile = nullptr, *d_tchunk = nullptr;   // tiles by footprint count, their first chunks [ntile + 1]
-    uint8_t *d_cell = nullptr;               // [ntile][256] cell of each thread
+    TileUnit *d_unit = nullptr;              // units by pair count [nunit + 1]
+    uint8_t *d_cell = nullptr;               // [nunit][512] cell of each thread
     int32_t *d_rows = nullptr;               // the written rows
     uint8_t *d_live = nullptr;               // [N] whether a row is written
     float2 *d_phasor = nullptr;
@@ -381,8 +381,7 @@ static void vis_layout_free(hai_vis_layout *L) {
     cudaFree(L->d_foot);
     cudaFree(L->d_ent);
     cudaFree(L->d_chunk);
-    cudaFree(L->d_tile);
-    cudaFree(L->d_tchunk);
+    cudaFree(L->d_unit);
     cudaFree(L->d_cell);
     cudaFree(L->d_rows);
     cudaFree(L->d_live);
@@ -400,30 +399,37 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     if (d->n_pol != 2) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: station images need 2 pols");
     if (hai_fault_injected("alloc")) return hai_fail(HAI_ERR_NO_MEMORY, "hai_vis_layout_create: injected allocation failure");
     const long long nbl = (long long)S * (S + 1) / 2;
-    // footprints in FP64 on the host: lower corner floor(uv) and fraction, one
-    // record in every tile they touch (counted, then placed)
+    // footprints in FP64 on the host: lower corner floor(uv) and fraction; a pair
+    // is recorded once in every unit (tile and mirror tile) that its footprint or
+    // its mirror's touches (counted, then placed)
     const int nt = N / kTile;
-    struct Foot {
-        uint32_t pair;
-        int16_t cx, cy;                        // lower corner in the tile, -1 .. 15
+    auto mirror_of = [&](int t) { return (nt - 1 - t / nt) * nt + nt - 1 - t % nt; };
+    auto unit_of = [&](int t) { return std::min(t, mirror_of(t)); };
+    struct Hit {
+        int tile, mirrored, cx, cy;            // lower corner in the tile, -1 .. 15
         float fu, fv;
     };
-    std::vector<int32_t> count((size_t)nt * nt, 0);
-    auto each_tile = [&](double u, double v, auto &&f) {
-        const double fu = floor(u), fv = floor(v);
-        const int x = (((int)fu % N) + N) % N, y = (((int)fv % N) + N) % N;
-        const int x1 = (x + 1) % N, y1 = (y + 1) % N;
-        // with one tile a side the wrapped column is in the same tile: its own record
-        const int nx = x % kTile == kTile - 1 ? 2 : 1, ny = y % kTile == kTile - 1 ? 2 : 1;
-        for (int j = 0; j < ny; j++)
-            for (int i = 0; i < nx; i++)
-                f(((j ? y1 : y) / kTile) * nt + (i ? x1 : x) / kTile, i ? -1 : x % kTile, j ? -1 : y % kTile,
-                  (float)(u - fu), (float)(v - fv));
+    // the tiles that the two footprints of a pair touch
+    auto hits_of = [&](double du, double dv, bool autos, Hit (&h)[8]) {
+        int n = 0;
+        for (int m = 0; m < (autos ? 1 : 2); m++) {
+            const double u = m ? -du : du, v = m ? -dv : dv, fu = floor(u), fv = floor(v);
+            const int x = (((int)fu % N) + N) % N, y = (((int)fv % N) + N) % N;
+            const int x1 = (x + 1) % N, y1 = (y + 1) % N;
+            // with one tile a side the wrapped column is in the same tile: its own hit
+            const int nx = x % kTile == kTile - 1 ? 2 : 1, ny = y % kTile == kTile - 1 ? 2 : 1;
+            for (int j = 0; j < ny; j++)
+                for (int i = 0; i < nx; i++)
+                    h[n++] = Hit{((j ? y1 : y) / kTile) * nt + (i ? x1 : x) / kTile, m, i ? -1 : x % kTile,
+                                 j ? -1 : y % kTile, (float)(u - fu), (float)(v - fv)};
+        }
+        return n;
     };
     long long dropped = 0;
-    auto each_footprint = [&](auto &&f) {      // f(pair with the mirror bit, u, v) of the kept pairs
+    auto each_pair = [&](auto &&f) {           // f(pair, hits, n) of the kept pairs
         dropped = 0;
         long long bl = 0;
+        Hit h[8];
         for (int m = 0; m < S; m++)
             for (int n = 0; n <= m; n++, bl++) {
                 const double du = (d->pos_m[2 * m] - d->pos_m[2 * n]) / d->cell_m;
@@ -432,25 +438,28 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
                     dropped++;
                     continue;
                 }
-                f((uint32_t)bl, du, dv);
-                if (m != n) f((uint32_t)bl | kMirror, -du, -dv);     // an auto pair has no mirror
+                f((uint32_t)bl, h, hits_of(du, dv, m == n, h));    // an auto pair has no mirror
             }
     };
-    each_footprint([&](uint32_t, double u, double v) {
-        each_tile(u, v, [&](int p, int, int, float, float) { count[p]++; });
-    });
+    auto each_unit = [&](const Hit *h, int n, auto &&f) {          // f(unit) once for every unit hit
+        for (int i = 0; i < n; i++) {
+            bool seen = false;
+            for (int j = 0; j < i; j++) seen |= unit_of(h[j].tile) == unit_of(h[i].tile);
+            if (!seen) f(unit_of(h[i].tile));
+        }
+    };
+    std::vector<int32_t> count((size_t)nt * nt, 0);
+    each_pair([&](uint32_t, const Hit *h, int n) { each_unit(h, n, [&](int u) { count[u]++; }); });
+    // written rows: those of a tile row (or its mirror's) with a pair in it
     std::vector<uint8_t> live(N, 0);
     std::vector<int32_t> rows, tiles;
-    for (int ty = 0; ty < nt; ty++) {
-        bool any = false;
-        for (int tx = 0; tx < nt; tx++) any |= count[ty * nt + tx] > 0;
-        if (!any) continue;
-        for (int y = ty * kTile; y < (ty + 1) * kTile; y++) {
-            live[y] = 1;
-            rows.push_back(y);
-        }
-        for (int tx = 0; tx < nt; tx++) tiles.push_back(ty * nt + tx);
-    }
+    for (int t = 0; t < nt * nt; t++)
+        if (count[t])
+            for (int r : {t / nt, nt - 1 - t / nt}) std::fill(live.begin() + r * kTile, live.begin() + (r + 1) * kTile, 1);
+    for (int y = 0; y < N; y++)
+        if (live[y]) rows.push_back(y);
+    for (int t = 0; t < nt * nt; t++)
+        if (unit_of(t) == t && live[t / nt * kTile]) tiles.push_back(t);
     std::stable_sort(tiles.begin(), tiles.end(), [&](int x, int y) { return count[x] > count[y]; });
     std::vector<long long> fill(count.size(), 0);
     long long nfoot = 0;
@@ -458,62 +467,85 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
         fill[t] = nfoot;
         nfoot += count[t];
     }
-    // entries: at most 4 a footprint, padded within warps; checked as they are placed
     if (nfoot > 0x0fffffffll) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: too many station pairs");
-    std::vector<Foot> all(std::max<long long>(1, nfoot));
-    each_footprint([&](uint32_t pair, double u, double v) {
-        each_tile(u, v, [&](int p, int cx, int cy, float fu, float fv) {
-            all[fill[p]++] = Foot{pair, (int16_t)cx, (int16_t)cy, fu, fv};
+    std::vector<uint32_t> foot(std::max<long long>(1, nfoot));
+    struct Where {
+        int m, n;
+    };
+    std::vector<Where> who(foot.size());
+    {
+        long long bl = 0;
+        std::vector<Where> of((size_t)nbl);
+        for (int m = 0; m < S; m++)
+            for (int n = 0; n <= m; n++) of[bl++] = Where{m, n};
+        each_pair([&](uint32_t pair, const Hit *h, int n) {
+            each_unit(h, n, [&](int u) {
+                who[fill[u]] = of[pair];
+                foot[fill[u]++] = pair;
+            });
         });
-    });
-    std::vector<uint32_t> foot(all.size());
-    for (size_t i = 0; i < all.size(); i++) foot[i] = all[i].pair;
+    }
     std::vector<TileEnt> ent;
     std::vector<TileChunk> chunks;
-    std::vector<int32_t> tchunk(1, 0);
-    std::vector<uint8_t> cell_of(tiles.size() * kTcells);
+    std::vector<TileUnit> units;
+    std::vector<uint8_t> cell_of(tiles.size() * kGridThreads);
     long long f0 = 0;
     for (size_t o = 0; o < tiles.size(); o++) {
         const long long f1 = f0 + count[tiles[o]];
-        // f(cell, weight) of a footprint's non-zero cells in the tile
-        auto each_cell = [&](const Foot &r, auto &&f) {
-            for (int t = 0; t < 4; t++) {
-                const int x = r.cx + (t & 1), y = r.cy + (t >> 1);
-                const float w = ((t & 1) ? r.fu : 1.f - r.fu) * ((t >> 1) ? r.fv : 1.f - r.fv);
-                if (x >= 0 && x < kTile && y >= 0 && y < kTile && w != 0.f) f(y * kTile + x, w);
+        const int ta = tiles[o], tb = mirror_of(ta) == ta ? -1 : mirror_of(ta);
+        units.push_back(TileUnit{ta, tb, (int32_t)chunks.size()});
+        // f(cell of the unit, weight, mirrored) of the non-zero cells of pair k in the unit
+        auto each_cell = [&](long long k, auto &&f) {
+            Hit h[8];
+            const int m = who[k].m, n = who[k].n;
+            const double du = (d->pos_m[2 * m] - d->pos_m[2 * n]) / d->cell_m;
+            const double dv = (d->pos_m[2 * m + 1] - d->pos_m[2 * n + 1]) / d->cell_m;
+            const int nh = hits_of(du, dv, m == n, h);
+            for (int i = 0; i < nh; i++) {
+                const Hit &r = h[i];
+                if (r.tile != ta && r.tile != tb) continue;
+                for (int t = 0; t < 4; t++) {
+                    const int x = r.cx + (t & 1), y = r.cy + (t >> 1);
+                    const float w = ((t & 1) ? r.fu : 1.f - r.fu) * ((t >> 1) ? r.fv : 1.f - r.fv);
+                    if (x >= 0 && x < kTile && y >= 0 && y < kTile && w != 0.f)
+                        f((r.tile == ta ? 0 : kTcells) + y * kTile + x, w, r.mirrored);
+                }
             }
         };
-        int total[kTcells] = {}, order[kTcells], thread_of[kTcells];
-        for (long long f = f0; f < f1; f++) each_cell(all[f], [&](int c, float) { total[c]++; });
-        for (int c = 0; c < kTcells; c++) order[c] = c;
-        std::stable_sort(order, order + kTcells, [&](int x, int y) { return total[x] > total[y]; });
-        for (int i = 0; i < kTcells; i++) {
+        int total[kGridThreads] = {}, order[kGridThreads], thread_of[kGridThreads];
+        for (long long k = f0; k < f1; k++) each_cell(k, [&](int c, float, int) { total[c]++; });
+        for (int side = 0; side < 2; side++) {
+            int *o0 = order + side * kTcells;
+            for (int c = 0; c < kTcells; c++) o0[c] = side * kTcells + c;
+            std::stable_sort(o0, o0 + kTcells, [&](int x, int y) { return total[x] > total[y]; });
+        }
+        for (int i = 0; i < kGridThreads; i++) {
             thread_of[order[i]] = i;
-            cell_of[o * kTcells + i] = (uint8_t)order[i];
+            cell_of[o * kGridThreads + i] = (uint8_t)(order[i] % kTcells);
         }
         for (long long q = f0; q < f1; q += kFoot) {
             TileChunk ch;
             ch.foot = (int32_t)q;
             ch.nfoot = (int32_t)std::min<long long>(kFoot, f1 - q);
-            int n[kTcells] = {};
-            for (int f = 0; f < ch.nfoot; f++) each_cell(all[q + f], [&](int c, float) { n[thread_of[c]]++; });
-            for (int w = 0; w < kTileWarps; w++) {
+            int n[kGridThreads] = {};
+            for (int f = 0; f < ch.nfoot; f++) each_cell(q + f, [&](int c, float, int) { n[thread_of[c]]++; });
+            for (int w = 0; w < kGridWarps; w++) {
                 ch.base[w] = (int32_t)ent.size();
                 ent.resize(ent.size() + 32 * (size_t)*std::max_element(n + 32 * w, n + 32 * w + 32), TileEnt{0.f, 0});
             }
-            ch.base[kTileWarps] = (int32_t)ent.size();
-            std::fill(n, n + kTcells, 0);
+            ch.base[kGridWarps] = (int32_t)ent.size();
+            std::fill(n, n + kGridThreads, 0);
             for (int f = 0; f < ch.nfoot; f++)
-                each_cell(all[q + f], [&](int c, float w) {
+                each_cell(q + f, [&](int c, float w, int mirrored) {
                     const int i = thread_of[c];
-                    ent[ch.base[i / 32] + 32 * n[i]++ + i % 32] = TileEnt{w, f};
+                    ent[ch.base[i / 32] + 32 * n[i]++ + i % 32] = TileEnt{w, mirrored * kFootRow + f};
                 });
             chunks.push_back(ch);
             if (ent.size() > 0x7fffffffull) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: too many station pairs");
         }
-        tchunk.push_back((int32_t)chunks.size());
         f0 = f1;
     }
+    units.push_back(TileUnit{-1, -1, (int32_t)chunks.size()});
     hai_vis_layout *L = new hai_vis_layout();
     L->ctx = ctx;
     L->S = S;
@@ -522,7 +554,7 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     L->K = K;
     L->nbl = nbl;
     L->n_offgrid = dropped;
-    L->ntile = (int)tiles.size();
+    L->nunit = (int)tiles.size();
     L->nrow = (int)rows.size();
     double *d_pos = nullptr, *d_dir = nullptr;
     std::vector<double> dirs(2 * (size_t)K, 0.0);
@@ -535,8 +567,7 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     put(L->d_foot, foot);
     put(L->d_ent, ent);
     put(L->d_chunk, chunks);
-    put(L->d_tile, tiles);
-    put(L->d_tchunk, tchunk);
+    put(L->d_unit, units);
     put(L->d_cell, cell_of);
     put(L->d_rows, rows);
     put(L->d_live, live);
@@ -585,14 +616,13 @@ extern "C" hai_status hai_xfft_station_image(hai_ctx *ctx, const hai_vis_layout 
     cudaStream_t st = (cudaStream_t)stream;
     const int N = L->N, images = L->K * C;
     const int groups = (images + kImgs - 1) / kImgs;
-    if ((long long)images * 2 > 0x7fffffffll || (long long)L->ntile * groups > 0x7fffffffll)
+    if ((long long)images * 2 > 0x7fffffffll || (long long)L->nunit * groups > 0x7fffffffll)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_station_image: too many images");
     const int pidx = prof_begin(ctx, st);
     auto grid = (((uintptr_t)vis & 15) == 0) ? station_grid_kernel<true> : station_grid_kernel<false>;
     HAI_CUDA_TRY(hai_allow_dyn_smem(grid, ctx->smem_optin));
-    grid<<<(unsigned)(L->ntile * groups), kTcells, sizeof(float4) * kImgs * kFoot, st>>>(
-        vis, L->d_foot, L->d_ent, L->d_chunk, L->d_tile, L->d_tchunk, L->d_cell, L->ntile, L->d_phasor, C, images,
-        L->nbl, N, img);
+    grid<<<(unsigned)(L->nunit * groups), kGridThreads, sizeof(float4) * kImgs * 2 * kFootRow, st>>>(
+        vis, L->d_foot, L->d_ent, L->d_chunk, L->d_unit, L->d_cell, L->nunit, L->d_phasor, C, images, L->nbl, N, img);
     prof_end(ctx, pidx, st);
     HAI_CUDA_TRY(cudaGetLastError());
     switch (N) {
