@@ -10,9 +10,10 @@
 // CTA (no partial images, no reduction).  The SM shares start from the cost
 // model and hai_plan_autotune refits them from measured class times.
 //
-// Cost model of one sample of a station, in SM cycles: a fixed part for the
-// two DFT stages and the epilogue plus a part per gather entry of the
-// gridding step (entries of the largest rank for N = 128).
+// Cost model of one sample of a station, in SM cycles (of all four SMs of a
+// cluster for N = 128): a fixed part for the two DFT stages and the epilogue
+// plus a part per gather entry of the gridding step (entries of the largest
+// rank for N = 128).
 //
 // Second level (hai_plan_set_hierarchy, Section 6): after the station images
 // the same graph beamforms every station (int8 weights, exact int32 sums,
@@ -51,8 +52,15 @@ struct PlanClass {
     cudaEvent_t done = nullptr;
 };
 
-double model_fixed(int N) { return N == 32 ? 350.0 : N == 64 ? 700.0 : 1100.0; }
-double model_entry(int N) { return N == 32 ? 0.5 : N == 64 ? 0.75 : 1.0; }
+// Fitted to the kernels alone on whole shares (4 blocks of 64 samples per CTA or
+// cluster): 930 SM cycles at N = 32 whatever the station, 1,540 (80 elements) to
+// 1,970 (300) at N = 64, 10,500 (384) to 13,800 (1024) on the four SMs of an
+// N = 128 cluster.  On 96 uneven stations (32 channels, 64 samples) shares
+// from 350 + 0.5, 700 + 0.75 and 1,100 + 1.0 an entry, the last without the
+// other three SMs, kept the N = 128 class running alone for a third of a replay:
+// 5,504 us, with these 3,322 us (the three classes end within 12% of each other).
+double model_fixed(int N) { return N == 32 ? 910.0 : N == 64 ? 1380.0 : 8500.0; }
+double model_entry(int N) { return N == 32 ? 0.05 : N == 64 ? 0.21 : 2.0; }
 
 }  // namespace
 
