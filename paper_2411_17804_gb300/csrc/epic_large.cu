@@ -599,12 +599,17 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
         // layout's second stream into one of two row scratches, so that the
         // row pass of batch i overlaps the column pass of batch i - 1; columns:
         // the 4 x 128-point warp transforms for boxes of at most 128 rows, else
-        // radix-8 as the rows.  Batches of 2 channels x as many samples as a
-        // scratch holds (512 at a 128-row box): the column pass reads and
-        // writes its image columns once per batch, and the two streams meet
-        // once per batch.
+        // radix-8 as the rows.  A batch is some channels x as many samples as a
+        // scratch holds (1,024 of them at a 128-row box): the column pass reads
+        // and writes its image columns once per batch, and the two streams meet
+        // once per batch.  Its CTAs (128 a channel, two on an SM) all take the
+        // same time, so the channels are those whose CTAs need the fewest waves,
+        // as long as a batch keeps 128 samples: 7 of 16 channels are 3 + 3 + 1
+        // waves where batches of 2 are 8 of 0.84 (lattice, 100 samples: 2193 us
+        // with batches of 2, 1979 us).
         constexpr int kRpc = 8;
-        constexpr int kCb = 2;
+        static_assert(kColsQ == kCols512, "CTAs per channel");
+        constexpr int kMinSamples = 128;
         const uint8_t *tabs = static_cast<const uint8_t *>(L->d_large_scratch) + 2 * kH512Bytes;
         const float2 *twq = reinterpret_cast<const float2 *>(tabs);
         const float2 *tw8 = twq + kTwq;
@@ -618,8 +623,19 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
         cudaEvent_t const *ev = L->large_ev;            // 0, 1: rows done (scratch 0, 1); 2, 3: columns done; 4: fork / join
         HAI_CUDA_TRY(cudaEventRecord(ev[4], st));
         HAI_CUDA_TRY(cudaStreamWaitEvent(rst, ev[4], 0));
-        const int cb_max = std::min(C, kCb);
         const long long fields512 = (long long)(kH512Bytes / field_bytes);
+        const int slots = 2 * L->ctx->num_sms;
+        auto waves = [&](int cb) { return (cb * (512 / kColsQ) + slots - 1) / slots; };
+        const int most = (int)std::max<long long>(std::min(2, C), std::min<long long>(C, fields512 / ((long long)P * std::min(T, kMinSamples))));
+        int cb_max = 1;
+        long long best = -1;
+        for (int cb = 1; cb <= std::min(most, 64); cb++) {
+            const long long w = (long long)(C / cb) * waves(cb) + (C % cb ? waves(C % cb) : 0);
+            if (best < 0 || w < best) {
+                best = w;
+                cb_max = cb;
+            }
+        }
         const int tb512 = (int)std::max<long long>(1, std::min<long long>(T, fields512 / ((long long)cb_max * P)));
         int i = 0;
         for (int t0 = 0; t0 < T; t0 += tb512) {
