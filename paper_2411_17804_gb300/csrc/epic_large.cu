@@ -20,7 +20,7 @@
 // the rows as radix-8 transforms over 64 threads, the columns of a box of at
 // most 128 rows as four 128-point transforms per warp (see below), the
 // column data staged through shared memory a few samples ahead.  There the
-// batches are large (2 channels x 512 samples at a 128-row box, 1 GB of row
+// batches are large (1,024 samples of a channel at a 128-row box, 1 GB of row
 // output) and alternate between two scratches in HBM: the row pass of one
 // batch runs on a second stream beside the column pass of the previous one.
 // As in the small-grid FP32 kernel the box sits at the transform's origin:
@@ -176,63 +176,120 @@ __global__ void __launch_bounds__(512) large_cols_kernel(const float2 *__restric
 // ------------------------------------------------------------------ N = 512
 // The 512-point transforms of the dense grids in registers: fft512.cuh.
 
-// Row pass, N = 512: blockIdx.x = field of the batch, blockIdx.y = group of
-// RPC box rows; thread (r = tid / 64, tau): the row's cells x = tau + 64 m
-// gathered from the layout's table, the transform, H[field][y][l] written
-// for every l (coalesced: l = tau + 64 j).  The twiddle tables come from
-// tw_g (built on the host) into shared memory.
-template <int RPC>
-__global__ void __launch_bounds__(64 * RPC) large512_rows_kernel(
-    const int8_t *__restrict__ volt, int T, int P, int ne, int box_w, int box_h,
-    const int32_t *__restrict__ cell_start, const int32_t *__restrict__ entry_elem,
-    const float2 *__restrict__ entry_w, const int4 *__restrict__ cell_tab, const float2 *__restrict__ tw_g, Batch bt,
-    float2 *__restrict__ H) {
+// Row pass, N = 512: a block keeps one group of RPC box rows (blockIdx.y) and
+// walks the samples of the batch, blockIdx.x and every gridDim.x-th after it;
+// thread (r = tid / 64, tau): the row's cells x = tau + 64 m gathered from the
+// layout's table, both polarisations in one transform of packed pairs,
+// H[sample][y][l] written for every l (coalesced: l = tau + 64 j).  The twiddle
+// tables come from tw_g (built on the host) into shared memory once.  ONE: at
+// most one entry a cell and 128 cells a row (cell_tab: element and weight in
+// one load): the thread's two cells stay in registers and the next sample's
+// voltages are loaded while this one is transformed.
+//
+// Bound: the exchanges' barriers and latency (issue slots 43% busy).  Lattice,
+// 200 samples: 81 us with a block per 8 rows of one polarisation (every block
+// loading the tables), 73 us for packed pairs in such blocks, 50 us like this.
+template <int RPC, bool ONE>
+__global__ void __launch_bounds__(64 * RPC, 4) large512_rows_kernel(
+    const int8_t *__restrict__ volt, int T, int ne, int box_w, int box_h, const int32_t *__restrict__ cell_start,
+    const int32_t *__restrict__ entry_elem, const float2 *__restrict__ entry_w, const int4 *__restrict__ cell_tab,
+    const float2 *__restrict__ tw_g, Batch bt, ulonglong2 *__restrict__ H) {
     extern __shared__ float4 sm4[];
     float2 *tw = reinterpret_cast<float2 *>(sm4);      // [kTwFloat2]
-    float2 *bufs = tw + kTwFloat2;                      // [RPC][kFftBuf]
+    ulonglong2 *bufs = reinterpret_cast<ulonglong2 *>(tw + kTwFloat2);   // [RPC][kFftBuf]
     static_assert(kTwFloat2 % 2 == 0, "tables copied as float4");
     for (int i = threadIdx.x; i < kTwFloat2 / 2; i += blockDim.x)
         sm4[i] = reinterpret_cast<const float4 *>(tw_g)[i];
     const int r = threadIdx.x >> 6, tau = threadIdx.x & 63;
-    const int f = blockIdx.x;
-    const int pol = f % P, tt = (f / P) % bt.tb, cc = f / (P * bt.tb);
-    const int y = blockIdx.y * RPC + r;
-    const char2 *E = reinterpret_cast<const char2 *>(volt) +
-                     ((((size_t)(bt.c0 + cc) * T + (bt.t0 + tt)) * P + pol) * ne);
-    float2 a[8];
+    const int y = blockIdx.y * RPC + r, nf = bt.cb * bt.tb;
+    auto sample = [&](int f) {
+        const int tt = f % bt.tb, cc = f / bt.tb;
+        return reinterpret_cast<const char2 *>(volt) + ((size_t)(bt.c0 + cc) * T + (bt.t0 + tt)) * 2 * ne;
+    };
+    int el[2] = {-1, -1};
+    float2 w[2];                                       // conj(W~)
+    char2 vx[2], vy[2];
+    auto fetch = [&](const char2 *E) {
 #pragma unroll
-    for (int m = 0; m < 8; m++) {
-        const int x = tau + 64 * m;
-        float2 g = make_float2(0.f, 0.f);
-        if (y < box_h && x < box_w) {
-            const int cell = y * box_w + x;
-            if (cell_tab) {                             // one entry at most: element and weight in one load
-                const int4 d = cell_tab[cell];
-                if (d.x >= 0) {
-                    const char2 e = E[d.x];
-                    const float2 w = make_float2(__int_as_float(d.y), __int_as_float(d.z));
-                    g.x = fmaf(w.x, (float)e.x, -w.y * (float)e.y);
-                    g.y = fmaf(w.x, (float)e.y, w.y * (float)e.x);
-                }
-            } else {
-                for (int k = cell_start[cell]; k < cell_start[cell + 1]; k++) {
-                    const char2 e = E[entry_elem[k]];
-                    const float2 w = entry_w[k];        // conj(W~)
-                    g.x = fmaf(w.x, (float)e.x, fmaf(-w.y, (float)e.y, g.x));
-                    g.y = fmaf(w.x, (float)e.y, fmaf(w.y, (float)e.x, g.y));
-                }
+        for (int m = 0; m < 2; m++)
+            if (el[m] >= 0) {
+                vx[m] = E[el[m]];
+                vy[m] = E[ne + el[m]];
+            }
+    };
+    if (ONE) {
+#pragma unroll
+        for (int m = 0; m < 2; m++) {
+            const int x = tau + 64 * m;
+            w[m] = make_float2(0.f, 0.f);
+            vx[m] = vy[m] = make_char2(0, 0);
+            if (y < box_h && x < box_w) {
+                const int4 d = cell_tab[y * box_w + x];
+                el[m] = d.x;
+                w[m] = make_float2(__int_as_float(d.y), __int_as_float(d.z));
             }
         }
-        a[m] = g;
+        if ((int)blockIdx.x < nf) fetch(sample(blockIdx.x));
     }
     __syncthreads();
-    if (box_w <= 128) fft512<true>(a, tau, bufs + r * kFftBuf, tw, [] { __syncthreads(); });
-    else fft512<false>(a, tau, bufs + r * kFftBuf, tw, [] { __syncthreads(); });
-    if (y < box_h) {
-        float2 *out = H + ((size_t)f * box_h + y) * 512;
+    for (int f = blockIdx.x; f < nf; f += gridDim.x) {
+        c2 a[8];
+        if (ONE) {
 #pragma unroll
-        for (int j = 0; j < 8; j++) out[tau + 64 * j] = a[j];
+            for (int m = 0; m < 8; m++) a[m] = {0, 0};
+#pragma unroll
+            for (int m = 0; m < 2; m++)
+                if (el[m] >= 0) {
+                    const float ex = (float)vx[m].x, ey = (float)vx[m].y, dx = (float)vy[m].x, dy = (float)vy[m].y;
+                    a[m] = {pack2(fmaf(w[m].x, ex, -w[m].y * ey), fmaf(w[m].x, dx, -w[m].y * dy)),
+                            pack2(fmaf(w[m].x, ey, w[m].y * ex), fmaf(w[m].x, dy, w[m].y * dx))};
+                }
+            if (f + (int)gridDim.x < nf) fetch(sample(f + gridDim.x));
+        } else {
+            const char2 *E = sample(f);
+#pragma unroll
+            for (int m = 0; m < 8; m++) {
+                const int x = tau + 64 * m;
+                float2 g = make_float2(0.f, 0.f), h = make_float2(0.f, 0.f);
+                if (y < box_h && x < box_w) {
+                    const int cell = y * box_w + x;
+                    for (int k = cell_start[cell]; k < cell_start[cell + 1]; k++) {
+                        const char2 e = E[entry_elem[k]], d = E[ne + entry_elem[k]];
+                        const float2 v = entry_w[k];
+                        g.x = fmaf(v.x, (float)e.x, fmaf(-v.y, (float)e.y, g.x));
+                        g.y = fmaf(v.x, (float)e.y, fmaf(v.y, (float)e.x, g.y));
+                        h.x = fmaf(v.x, (float)d.x, fmaf(-v.y, (float)d.y, h.x));
+                        h.y = fmaf(v.x, (float)d.y, fmaf(v.y, (float)d.x, h.y));
+                    }
+                }
+                a[m] = {pack2(g.x, h.x), pack2(g.y, h.y)};
+            }
+        }
+        if (ONE || box_w <= 128) fft512<true>(a, tau, bufs + r * kFftBuf, tw, [] { __syncthreads(); });
+        else fft512<false>(a, tau, bufs + r * kFftBuf, tw, [] { __syncthreads(); });
+        if (y < box_h) {
+            ulonglong2 *out = H + ((size_t)f * box_h + y) * 512;
+#pragma unroll
+            for (int j = 0; j < 8; j++) out[tau + 64 * j] = Xchg<c2>::put(a[j]);
+        }
+        __syncthreads();                                // exchange buffers free for the next sample
     }
+}
+
+// |F_X|^2, |F_Y|^2 (a pair) and F_X conj(F_Y) of one pixel added to its sums.
+__device__ __forceinline__ void add_products(c2 f, unsigned long long &pw, float &xr, float &xi) {
+    pw = fma2(f.re, f.re, fma2(f.im, f.im, pw));
+    const float2 r = unpack2(f.re), i = unpack2(f.im);
+    xr = fmaf(r.x, r.y, fmaf(i.x, i.y, xr));           // Re X conj(Y)
+    xi = fmaf(i.x, r.y, fmaf(-r.x, i.y, xi));          // Im X conj(Y)
+}
+
+// The four sums of a pixel into the image planes (or onto them).
+__device__ __forceinline__ void put_products(float *dst, size_t plane, int add, unsigned long long pw, float xr, float xi) {
+    const float2 p = unpack2(pw);
+    const float v[4] = {p.x, p.y, xr, xi};
+#pragma unroll
+    for (int q = 0; q < 4; q++) dst[q * plane] = add ? v[q] + dst[q * plane] : v[q];
 }
 
 // Column pass, N = 512, two polarisations, boxes taller than 128 rows:
@@ -244,59 +301,40 @@ __global__ void __launch_bounds__(64 * RPC) large512_rows_kernel(
 // the (-1)^j phase centre).
 constexpr int kCols512 = 4;                  // columns per CTA: 256 threads, two CTAs per SM
 
-__global__ void __launch_bounds__(64 * kCols512, 2) large512_cols_kernel(const float2 *__restrict__ H, int box_h,
+__global__ void __launch_bounds__(64 * kCols512, 2) large512_cols_kernel(const ulonglong2 *__restrict__ H, int box_h,
                                                                        Batch bt, float *__restrict__ img, int add) {
-    extern __shared__ float2 sm[];
-    float2 *tw = sm;                                    // [kTwFloat2]
-    float2 *bufs = sm + kTwFloat2;                      // [2 pols][kCols512 columns][kFftBuf]
+    extern __shared__ float4 sm4[];
+    float2 *tw = reinterpret_cast<float2 *>(sm4);       // [kTwFloat2]
+    ulonglong2 *bufs = reinterpret_cast<ulonglong2 *>(tw + kTwFloat2);   // [kCols512 columns][kFftBuf]
     fill_fft512_tables(tw);
     const int c = threadIdx.x >> 6, tau = threadIdx.x & 63;
     const int cc = blockIdx.x, l0 = blockIdx.y * kCols512;
-    float acc[4][8];
+    unsigned long long pw[8];
+    float xr[8], xi[8];
 #pragma unroll
-    for (int q = 0; q < 4; q++)
-#pragma unroll
-        for (int j = 0; j < 8; j++) acc[q][j] = 0.f;
-    // input m (row tau + 64 m) of polarisation p of sample tt of this channel
-    auto in = [&](int tt, int p, int m) -> float2 {
-        const size_t f = ((size_t)cc * bt.tb + tt) * 2 + p;
-        const int yy = tau + 64 * m;
-        return yy < box_h ? H[(f * box_h + yy) * 512 + l0 + c] : make_float2(0.f, 0.f);
-    };
+    for (int j = 0; j < 8; j++) {
+        pw[j] = 0;
+        xr[j] = xi[j] = 0.f;
+    }
     __syncthreads();
     for (int tt = 0; tt < bt.tb; tt++) {
-        float2 x[8], yv[8];
+        c2 x[8];
+        const ulonglong2 *src = H + ((size_t)cc * bt.tb + tt) * box_h * 512 + l0 + c;
 #pragma unroll
         for (int m = 0; m < 8; m++) {
-            x[m] = in(tt, 0, m);
-            yv[m] = in(tt, 1, m);
+            const int yy = tau + 64 * m;
+            x[m] = yy < box_h ? Xchg<c2>::get(src[(size_t)yy * 512]) : c2{0, 0};
         }
         fft512<false>(x, tau, bufs + c * kFftBuf, tw, [] { __syncthreads(); });
-        fft512<false>(yv, tau, bufs + (kCols512 + c) * kFftBuf, tw, [] { __syncthreads(); });
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-            const float2 a = x[j], b = yv[j];
-            acc[0][j] = fmaf(a.x, a.x, fmaf(a.y, a.y, acc[0][j]));
-            acc[1][j] = fmaf(b.x, b.x, fmaf(b.y, b.y, acc[1][j]));
-            acc[2][j] = fmaf(a.x, b.x, fmaf(a.y, b.y, acc[2][j]));      // Re X conj(Y)
-            acc[3][j] = fmaf(a.y, b.x, fmaf(-a.x, b.y, acc[3][j]));     // Im X conj(Y)
-        }
+        for (int j = 0; j < 8; j++) add_products(x[j], pw[j], xr[j], xi[j]);
         __syncthreads();                                // exchange buffers free for the next sample
     }
-    const int ch = bt.c0 + cc;
     const size_t NN = (size_t)512 * 512;
-    const int ox = (l0 + c + 256) & 511;
+    float *dst = img + (size_t)(bt.c0 + cc) * 4 * NN + ((l0 + c + 256) & 511);
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        float *dst = img + ((size_t)ch * 4 + q) * NN + ox;
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-            const int oy = (tau + 64 * j + 256) & 511;
-            float v = acc[q][j];
-            if (add) v += dst[(size_t)oy * 512];
-            dst[(size_t)oy * 512] = v;
-        }
-    }
+    for (int j = 0; j < 8; j++)
+        put_products(dst + (size_t)((tau + 64 * j + 256) & 511) * 512, NN, add, pw[j], xr[j], xi[j]);
 }
 
 // ------------------------------------------------------------------ N = 512, box <= 128 x 128
@@ -326,22 +364,23 @@ constexpr size_t kH512Bytes = (size_t)1 << 30;   // each of the two row scratche
 // 16-point DFT, exponent +, natural order in and out: m = m1 + 4 m2,
 // k = ka + 4 kb; 4-point DFTs over m2, twiddles w16^(m1 ka), 4-point DFTs
 // over m1.
-__device__ __forceinline__ void dft16(float2 (&a)[16]) {
-    const float c8 = 0.92387953251128674f, s8 = 0.38268343236508978f, h = 0.70710678118654752f;
+__device__ __forceinline__ void dft16(c2 (&a)[16]) {
+    const float c8 = 0.92387953251128674f, s8 = 0.38268343236508978f;
 #pragma unroll
     for (int m1 = 0; m1 < 4; m1++) dft4(a[m1], a[m1 + 4], a[m1 + 8], a[m1 + 12]);   // a[m1 + 4 ka]
     a[5] = cmul(a[5], make_float2(c8, s8));                                         // w16^1
-    a[9] = make_float2(h * (a[9].x - a[9].y), h * (a[9].x + a[9].y));               // w16^2
+    a[9] = crot<1>(a[9]);                                                           // w16^2
     a[13] = cmul(a[13], make_float2(s8, c8));                                       // w16^3
-    a[6] = make_float2(h * (a[6].x - a[6].y), h * (a[6].x + a[6].y));               // w16^2
-    a[10] = cmuli(a[10]);                                                           // w16^4
-    a[14] = make_float2(-h * (a[14].x + a[14].y), h * (a[14].x - a[14].y));         // w16^6
+    a[6] = crot<1>(a[6]);                                                           // w16^2
+    a[14] = crot<3>(a[14]);                                                         // w16^6
     a[7] = cmul(a[7], make_float2(s8, c8));                                         // w16^3
-    a[11] = make_float2(-h * (a[11].x + a[11].y), h * (a[11].x - a[11].y));         // w16^6
+    a[11] = crot<3>(a[11]);                                                         // w16^6
     a[15] = cmul(a[15], make_float2(-c8, -s8));                                     // w16^9
 #pragma unroll
-    for (int ka = 0; ka < 4; ka++) dft4(a[4 * ka], a[4 * ka + 1], a[4 * ka + 2], a[4 * ka + 3]);   // a[4 ka + kb]
-    float2 o[16];
+    for (int ka = 0; ka < 4; ka++)
+        if (ka == 2) dft4<true>(a[8], a[9], a[10], a[11]);                          // a[10] w16^4 = a[10] i
+        else dft4(a[4 * ka], a[4 * ka + 1], a[4 * ka + 2], a[4 * ka + 3]);          // a[4 ka + kb]
+    c2 o[16];
 #pragma unroll
     for (int ka = 0; ka < 4; ka++)
 #pragma unroll
@@ -350,55 +389,32 @@ __device__ __forceinline__ void dft16(float2 (&a)[16]) {
     for (int k = 0; k < 16; k++) a[k] = o[k];
 }
 
-// Two 512-point transforms (the two polarisations) by one warp, as above;
-// xb: the warp's two exchange buffers (2 kXq float2), tw: Pq and Tq in shared
-// memory.  Entry: x[m] = h_X[t + 8 m], y[m] = h_Y[t + 8 m].
-__device__ __forceinline__ void fft512q2(float2 (&x)[16], float2 (&y)[16], int r, int t, float2 *xb,
-                                         const float2 *tw) {
+// A 512-point transform of both polarisations by one warp, as above; xb: the
+// warp's exchange buffer (kXq pairs), tw: Pq and Tq in shared memory.  Entry:
+// x[m] = h[t + 8 m].
+__device__ __forceinline__ void fft512q2(c2 (&x)[16], int r, int t, ulonglong2 *xb, const float2 *tw) {
     const float2 *pr = tw + r * kPr + t;
 #pragma unroll
-    for (int m = 0; m < 16; m++) {
-        const float2 w = pr[8 * m];
-        x[m] = cmul(x[m], w);
-        y[m] = cmul(y[m], w);
-    }
+    for (int m = 0; m < 16; m++) x[m] = cmul(x[m], pr[8 * m]);
     dft16(x);
-    dft16(y);
     const float2 *tq = tw + 4 * kPr + t;
 #pragma unroll
-    for (int k = 1; k < 16; k++) {
-        const float2 w = tq[8 * k];
-        x[k] = cmul(x[k], w);
-        y[k] = cmul(y[k], w);
-    }
-    float2 *wx = xb + r * 152 + t, *wy = wx + kXq;
+    for (int k = 1; k < 16; k++) x[k] = cmul(x[k], tq[8 * k]);
+    ulonglong2 *w = xb + r * 152 + t;
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
-        wx[9 * k] = x[k];
-        wy[9 * k] = y[k];
-    }
+    for (int k = 0; k < 16; k++) w[9 * k] = Xchg<c2>::put(x[k]);
     __syncwarp();
-    const float2 *rx = xb + r * 152 + 9 * t, *ry = rx + kXq;
-    float2 a0[8], a1[8], b0[8], b1[8];
+    const ulonglong2 *rd = xb + r * 152 + 9 * t;
 #pragma unroll
-    for (int s = 0; s < 8; s++) {
-        a0[s] = rx[s];
-        a1[s] = rx[72 + s];
-        b0[s] = ry[s];
-        b1[s] = ry[72 + s];
-    }
-    __syncwarp();                                        // the buffers are free again
-    dft8(a0);
-    dft8(a1);
-    dft8(b0);
-    dft8(b1);
+    for (int h = 0; h < 2; h++) {
+        c2 a[8];
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        x[k] = a0[k];
-        x[8 + k] = a1[k];
-        y[k] = b0[k];
-        y[8 + k] = b1[k];
+        for (int s = 0; s < 8; s++) a[s] = Xchg<c2>::get(rd[72 * h + s]);
+        dft8(a);
+#pragma unroll
+        for (int k = 0; k < 8; k++) x[8 * h + k] = a[k];
     }
+    __syncwarp();                                        // the buffer is free again
 }
 
 __device__ __forceinline__ void load_twq(float2 *dst, const float2 *__restrict__ src) {
@@ -409,95 +425,89 @@ __device__ __forceinline__ void load_twq(float2 *dst, const float2 *__restrict__
 
 // Column pass, boxes of at most 128 rows: one warp per (image column l_x,
 // channel of the batch), four adjacent columns per block.  For each sample
-// the block copies the four columns of both pols (box_h rows of H, 32 bytes
-// per row: whole L2 sectors) into shared memory asynchronously two samples
-// ahead; each warp transforms its column along y and adds |F_X|^2, |F_Y|^2
+// the block copies the four columns (box_h rows of H, 64 bytes per row) into
+// shared memory asynchronously two samples ahead; each warp transforms its
+// column along y, both polarisations as packed pairs, and adds |F_X|^2, |F_Y|^2
 // and F_X conj(F_Y) into 64 register accumulators (16 rows l_y per lane); at
-// the end the column is read, added to and written once (output pixel
-// shifted by N/2).  The staged rows are kRowQ float2 apart so that a warp's
-// reads of rows t + 8 m hit distinct banks.
+// the end the column is read, added to and written once (output pixel shifted
+// by N/2).  The staged rows are kRowQ pairs apart so that a warp's reads of
+// rows t + 8 m hit distinct banks.
+//
+// Bound: the issue slots (53% busy) and latency at 12 warps an SM; packed pairs
+// need 159 registers where two scalar transforms side by side needed 190 and
+// two blocks an SM.  Lattice, 200 samples: 205 us -> 130 us.
+constexpr int kCtasQ = 3;                     // blocks per SM
 constexpr int kColsQ = 4;                     // columns (warps) per block
-constexpr int kRowQ = 6;                      // float2 per staged row (4 used)
+constexpr int kRowQ = 5;                      // pairs per staged row (4 used)
 constexpr int kPfq = 3;                       // sample stages in flight
-constexpr int kStageQ = 2 * 128 * kRowQ;      // float2 per stage (2 pols x 128 rows)
+constexpr int kStageQ = 128 * kRowQ;          // pairs per stage
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-__global__ void __launch_bounds__(32 * kColsQ, 2) large512q_cols_kernel(const float2 *__restrict__ H, int box_h,
-                                                                      const float2 *__restrict__ twq, Batch bt,
-                                                                      float *__restrict__ img, int add) {
+__global__ void __launch_bounds__(32 * kColsQ, kCtasQ) large512q_cols_kernel(const ulonglong2 *__restrict__ H, int box_h,
+                                                                           const float2 *__restrict__ twq, Batch bt,
+                                                                           float *__restrict__ img, int add) {
     extern __shared__ float4 smq[];
     float2 *tw = reinterpret_cast<float2 *>(smq);                 // [kTwq]
-    float2 *pb = tw + kTwq;                                       // [kPfq][2 pols][128 rows][kRowQ]
-    float2 *xb = pb + kPfq * kStageQ;                             // [kColsQ][2 kXq]
+    ulonglong2 *pb = reinterpret_cast<ulonglong2 *>(tw + kTwq);   // [kPfq][128 rows][kRowQ]
+    ulonglong2 *xb = pb + kPfq * kStageQ;                         // [kColsQ][kXq]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 3, t = lane & 7;
     const int lx0 = blockIdx.x * kColsQ, lx = lx0 + warp, cc = blockIdx.y;
-    xb += warp * 2 * kXq;
+    xb += warp * kXq;
     load_twq(tw, twq);
-    for (int i = threadIdx.x; i < kPfq * kStageQ; i += blockDim.x) pb[i] = make_float2(0.f, 0.f);
+    for (int i = threadIdx.x; i < kPfq * kStageQ; i += blockDim.x) pb[i] = make_ulonglong2(0, 0);
     __syncthreads();                                              // rows >= box_h stay zero
-    auto issue = [&](int tt) {                                    // two 16-byte copies per (pol, row)
-        const size_t f0 = ((size_t)cc * bt.tb + tt) * 2;
-        float2 *dst = pb + (tt % kPfq) * kStageQ;
-        for (int i = threadIdx.x; i < 2 * 128 * 2; i += blockDim.x) {
-            const int u = i & 1, p = i >> 8, yy = (i >> 1) & 127;
-            if (yy < box_h)
-                cp_async16(dst + (p * 128 + yy) * kRowQ + 2 * u, H + (((f0 + p) * box_h + yy) * 512 + lx0 + 2 * u));
-        }
+    const int cu = threadIdx.x & 3, cy = threadIdx.x >> 2;        // copies: column cu, rows cy + 32 i
+    const ulonglong2 *from = H + (size_t)cc * bt.tb * box_h * 512 + (size_t)cy * 512 + lx0 + cu;
+    const size_t per_sample = (size_t)box_h * 512;
+    int fill = 0;                                                 // stage filled next
+    auto issue = [&] {
+        ulonglong2 *dst = pb + fill * kStageQ + cy * kRowQ + cu;
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (cy + 32 * i < box_h) cp_async16(dst + 32 * i * kRowQ, from + (size_t)(32 * i) * 512);
+        from += per_sample;
+        if (++fill == kPfq) fill = 0;
     };
-    float acc[4][16];
+    unsigned long long pw[16];
+    float xr[16], xi[16];
 #pragma unroll
-    for (int q = 0; q < 4; q++)
-#pragma unroll
-        for (int j = 0; j < 16; j++) acc[q][j] = 0.f;
-    issue(0);
+    for (int j = 0; j < 16; j++) {
+        pw[j] = 0;
+        xr[j] = xi[j] = 0.f;
+    }
+    issue();
     cp_async_commit();
-    if (bt.tb > 1) issue(1);
+    if (bt.tb > 1) issue();
     cp_async_commit();
+    int cur = 0;
     for (int tt = 0; tt < bt.tb; tt++) {
-        __syncthreads();                                          // the stage refilled next was read last sample
-        if (tt + 2 < bt.tb) issue(tt + 2);
+        cp_async_wait1();
+        __syncthreads();                                          // sample tt's copies landed (every thread's);
+        if (tt + 2 < bt.tb) issue();                              // the stage refilled was read last sample
         cp_async_commit();
-        cp_async_wait2();
-        __syncthreads();                                          // sample tt's copies (every thread's) landed
-        const float2 *src = pb + (tt % kPfq) * kStageQ + t * kRowQ + warp;
-        float2 x[16], yv[16];
+        const ulonglong2 *src = pb + cur * kStageQ + t * kRowQ + warp;
+        if (++cur == kPfq) cur = 0;
+        c2 x[16];
 #pragma unroll
-        for (int m = 0; m < 16; m++) {
-            x[m] = src[8 * m * kRowQ];
-            yv[m] = src[(128 + 8 * m) * kRowQ];
-        }
-        fft512q2(x, yv, r, t, xb, tw);
+        for (int m = 0; m < 16; m++) x[m] = Xchg<c2>::get(src[8 * m * kRowQ]);
+        fft512q2(x, r, t, xb, tw);
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-            const float2 a = x[j], b = yv[j];
-            acc[0][j] = fmaf(a.x, a.x, fmaf(a.y, a.y, acc[0][j]));
-            acc[1][j] = fmaf(b.x, b.x, fmaf(b.y, b.y, acc[1][j]));
-            acc[2][j] = fmaf(a.x, b.x, fmaf(a.y, b.y, acc[2][j]));      // Re X conj(Y)
-            acc[3][j] = fmaf(a.y, b.x, fmaf(-a.x, b.y, acc[3][j]));     // Im X conj(Y)
-        }
+        for (int j = 0; j < 16; j++) add_products(x[j], pw[j], xr[j], xi[j]);
     }
-    const int ch = bt.c0 + cc;
     const size_t NN = (size_t)512 * 512;
-    const int ox = (lx + 256) & 511;
+    float *dst = img + (size_t)(bt.c0 + cc) * 4 * NN + ((lx + 256) & 511);
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        float *dst = img + ((size_t)ch * 4 + q) * NN + ox;
+    for (int h = 0; h < 2; h++)
 #pragma unroll
-        for (int h = 0; h < 2; h++)
-#pragma unroll
-            for (int k2 = 0; k2 < 8; k2++) {
-                const int oy = (4 * t + r + 32 * h + 64 * k2 + 256) & 511;
-                float v = acc[q][8 * h + k2];
-                if (add) v += dst[(size_t)oy * 512];
-                dst[(size_t)oy * 512] = v;
-            }
-    }
+        for (int k2 = 0; k2 < 8; k2++)
+            put_products(dst + (size_t)((4 * t + r + 32 * h + 64 * k2 + 256) & 511) * 512, NN, add, pw[8 * h + k2],
+                         xr[8 * h + k2], xi[8 * h + k2]);
 }
 
 }  // namespace
@@ -595,28 +605,31 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
     float2 *H = static_cast<float2 *>(L->d_large_scratch);
     const int pidx = prof_begin(L->ctx, st);
     if (N == 512 && P == 2) {
-        // rows: register-resident radix-8 transforms, 8 rows per CTA, on the
+        // rows: register-resident radix-8 transforms, 4 rows per CTA, on the
         // layout's second stream into one of two row scratches, so that the
         // row pass of batch i overlaps the column pass of batch i - 1; columns:
         // the 4 x 128-point warp transforms for boxes of at most 128 rows, else
         // radix-8 as the rows.  A batch is some channels x as many samples as a
         // scratch holds (1,024 of them at a 128-row box): the column pass reads
         // and writes its image columns once per batch, and the two streams meet
-        // once per batch.  Its CTAs (128 a channel, two on an SM) all take the
-        // same time, so the channels are those whose CTAs need the fewest waves,
-        // as long as a batch keeps 128 samples: 7 of 16 channels are 3 + 3 + 1
-        // waves where batches of 2 are 8 of 0.84 (lattice, 100 samples: 2193 us
-        // with batches of 2, 1979 us).
-        constexpr int kRpc = 8;
+        // once per batch.  Its CTAs (128 a channel, kCtasQ on an SM) all take
+        // the same time, so the channels are those whose CTAs need the fewest
+        // waves, as long as a batch keeps 128 samples: 16 channels go as 7 + 7 + 2
+        // in 2 + 2 + 1 waves (lattice, 100 samples, with two CTAs an SM then:
+        // batches of 2 channels 2193 us, by waves 1979 us).
+        constexpr int kRpc = 4;
         static_assert(kColsQ == kCols512, "CTAs per channel");
         constexpr int kMinSamples = 128;
         const uint8_t *tabs = static_cast<const uint8_t *>(L->d_large_scratch) + 2 * kH512Bytes;
         const float2 *twq = reinterpret_cast<const float2 *>(tabs);
         const float2 *tw8 = twq + kTwq;
-        const size_t rs_smem = sizeof(float2) * (kTwFloat2 + kRpc * (size_t)kFftBuf);
+        const size_t rs_smem = sizeof(float2) * (kTwFloat2 + 2 * kRpc * (size_t)kFftBuf);
         const size_t cs_smem = sizeof(float2) * (kTwFloat2 + 2 * kCols512 * (size_t)kFftBuf);
-        const size_t cq_smem = sizeof(float2) * (kTwq + (size_t)kPfq * kStageQ + (size_t)kColsQ * 2 * kXq);
-        HAI_CUDA_TRY(hai_allow_dyn_smem(large512_rows_kernel<kRpc>, L->ctx->smem_optin));
+        const size_t cq_smem = sizeof(float2) * (kTwq + 2 * (kPfq * (size_t)kStageQ + kColsQ * (size_t)kXq));
+        const int4 *cell_tab = static_cast<const int4 *>(L->d_large_cell);
+        const auto rows = cell_tab && L->box_w <= 128 ? large512_rows_kernel<kRpc, true> : large512_rows_kernel<kRpc, false>;
+        const int row_groups = (L->box_h + kRpc - 1) / kRpc, row_ctas = std::max(1, 4 * L->ctx->num_sms / row_groups);
+        HAI_CUDA_TRY(hai_allow_dyn_smem(rows, L->ctx->smem_optin));
         HAI_CUDA_TRY(hai_allow_dyn_smem(large512_cols_kernel, L->ctx->smem_optin));
         HAI_CUDA_TRY(hai_allow_dyn_smem(large512q_cols_kernel, L->ctx->smem_optin));
         cudaStream_t rst = L->large_stream;
@@ -624,7 +637,7 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
         HAI_CUDA_TRY(cudaEventRecord(ev[4], st));
         HAI_CUDA_TRY(cudaStreamWaitEvent(rst, ev[4], 0));
         const long long fields512 = (long long)(kH512Bytes / field_bytes);
-        const int slots = 2 * L->ctx->num_sms;
+        const int slots = (L->box_h <= 128 ? kCtasQ : 2) * L->ctx->num_sms;
         auto waves = [&](int cb) { return (cb * (512 / kColsQ) + slots - 1) / slots; };
         const int most = (int)std::max<long long>(std::min(2, C), std::min<long long>(C, fields512 / ((long long)P * std::min(T, kMinSamples))));
         int cb_max = 1;
@@ -642,17 +655,16 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
             const int tb = std::min(tb512, T - t0);
             for (int c0 = 0; c0 < C; c0 += cb_max, i++) {
                 const int buf = i & 1;
-                float2 *Hb = reinterpret_cast<float2 *>(static_cast<uint8_t *>(L->d_large_scratch) + buf * kH512Bytes);
+                ulonglong2 *Hb = reinterpret_cast<ulonglong2 *>(static_cast<uint8_t *>(L->d_large_scratch) + buf * kH512Bytes);
                 Batch bt;
                 bt.c0 = c0;
                 bt.cb = std::min(cb_max, C - c0);
                 bt.t0 = t0;
                 bt.tb = tb;
                 if (i >= 2) HAI_CUDA_TRY(cudaStreamWaitEvent(rst, ev[2 + buf], 0));   // columns of batch i - 2 done
-                large512_rows_kernel<kRpc><<<dim3(bt.cb * tb * P, (L->box_h + kRpc - 1) / kRpc), 64 * kRpc, rs_smem,
-                                             rst>>>(volt, T, P, L->n_elem, L->box_w, L->box_h, L->d_cell_start,
-                                                    L->d_entry_elem, L->d_entry_w,
-                                                    static_cast<const int4 *>(L->d_large_cell), tw8, bt, Hb);
+                rows<<<dim3(std::min(bt.cb * tb, row_ctas), row_groups), 64 * kRpc, rs_smem, rst>>>(
+                    volt, T, L->n_elem, L->box_w, L->box_h, L->d_cell_start, L->d_entry_elem, L->d_entry_w, cell_tab, tw8,
+                    bt, Hb);
                 HAI_CUDA_TRY(cudaEventRecord(ev[buf], rst));
                 HAI_CUDA_TRY(cudaStreamWaitEvent(st, ev[buf], 0));
                 const int add = (t0 > 0 || accumulate) ? 1 : 0;
