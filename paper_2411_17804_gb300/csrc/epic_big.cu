@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
     // contiguous tile range of this CTA; tiles are (l_x block, field), field fastest
     const long long r0 = p.ntiles * blockIdx.x / gridDim.x, r1 = p.ntiles * (blockIdx.x + 1) / gridDim.x;
     if (warp == 0) {
-        if (lane == 0) {
+        if (tc::elect()) {
             long long gs = 0;
             int cur_lb = -1;
             for (long long tile = r0; tile < r1; tile++) {
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (tc::elect()) {
             long long gs = 0;
             int cur_lb = -1;
             uint32_t bph = 0;
@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
     const long long u1 = unit_start(p.units, gridDim.x, blockIdx.x + 1);
     const uint32_t bbytes = (uint32_t)kKb2 * V::BTile;     // one DFT operand part of an l_y block
     if (warp == 0) {
-        if (lane == 0) {
+        if (tc::elect()) {
             long long gs = 0;                              // samples loaded
             int st = 0, fill = 0;                          // ring stage, times it has been filled before
             int cur_lyb = -1;
@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(576, 1) big_s2_kernel(const S2Params p) {
         // one thread issues the MMAs: per k block 4 K-steps (x 3 products when
         // split), one commit per k block (frees the A stage) and one per sample
         // (fills the accumulator)
-        if (lane == 0) {
+        if (tc::elect()) {
             long long gs = 0;
             int cur_lyb = -1, st = 0;
             uint32_t bph = 0, aph = 0;                     // phases of bfull, of the ring

@@ -34,7 +34,9 @@
 // the gridding warps' share of a sample.  Inter-station EPIC of one beam (256
 // stations, 32 channels x 1000): 2195 us when the seven front warps did the
 // gridding, the shipping and the move in turn, from a table with an entry for
-// every zero weight; 1083 us now (1432 before the MMA descriptors were hoisted).
+// every zero weight; 1083 us before
+// the MMAs were issued behind an elected lane (1432 before their descriptors were
+// hoisted), 1044 us now.
 #include <math.h>
 #include <string.h>
 
@@ -393,7 +395,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
             }
         } else if (warp == kMmaWarp) {
             // ================================================================ MMA + TMA
-            if (lane == 0) {
+            if (tc::elect()) {
                 const uint32_t b1 = tc::smem_u32(sB1), a2 = tc::smem_u32(sA2), b2 = tc::smem_u32(sB2);
                 // descriptors once, then 32-bit additions: the issuing thread is one of
                 // 24 warps' and its scalar work between MMAs is the sample's period

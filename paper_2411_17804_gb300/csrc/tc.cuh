@@ -63,6 +63,19 @@ __host__ __device__ constexpr uint32_t idesc_f16_as(bool bf16, int M, int N, int
     return idesc_f16(M, N, a_mn_major, b_mn_major) | (bf16 ? ((1u << 7) | (1u << 10)) : 0u);
 }
 
+// One thread of a converged warp: true for one lane.  The compiler knows that the
+// branch it guards runs in one thread and keeps the descriptors of an issue loop in
+// uniform registers; behind `lane == 0` it moves every operand there for each
+// instruction (8 MMAs of 128 x 32 x 16 with their commit, back to back: 66 cycles
+// each behind lane == 0, 41 behind elect; 128 x 64: 48; 64 x 64: 34).  For loops
+// that issue little else: the N = 64 kernel, whose issuer waits on two pipelines,
+// was slower with it (760 -> 774 us a cadence of 80 SKA stations).
+__device__ __forceinline__ bool elect() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 // D[tmem] (+)= A * B^T, issued by one thread.
 __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
                                         uint32_t accumulate) {
