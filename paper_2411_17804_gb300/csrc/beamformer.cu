@@ -11,59 +11,65 @@
 // sums 2 N_e of them, so for N_e <= 512 every FP32 partial sum is an integer
 // below 2^24: exact.
 //
-// CTA = 13 warps, persistent over a contiguous range of (s, c, tile) units:
-//   warps 0-7  producers: cp.async 16-byte copies of the voltage rows of a
-//              64-element chunk (zero-filled past T) into a 5-deep int8 ring
-//              (4 chunks, 64 KB, in flight per SM to cover HBM latency), then
-//              fp16 widening into a 2-deep K-major A ring; every thread owns
-//              four fixed (row, 16-byte group) items of a chunk for the copies
-//              and four for the widening, their offsets computed once; the
-//              station's weights are widened into B when the station changes;
-//   warp 8     one thread issues the MMAs (8 per chunk);
-//   warps 9-12 epilogue: TMEM -> int32, optional requantisation; each thread
+// CTA = 24 warps, persistent over a contiguous range of (s, c, tile) units:
+//   warps 0-15 producers, in four groups of 4 warps: group g fills slot g of the
+//              4-deep A ring, every fourth 64-element chunk, by 16-byte loads of
+//              the voltage rows into registers (two chunks of the group in
+//              flight; zero past T), widened to fp16 straight into the K-major
+//              slot; the station's weights are widened into B when the station
+//              changes;
+//   warp 16    one thread issues the MMAs (8 per chunk);
+//   warps 20-23 epilogue: TMEM -> int32, optional requantisation; each thread
 //              assembles its sample's [k][p][re, im] row from both pols and
 //              writes it with 16-byte stores (rows are contiguous per unit).
+//
+// Bound: HBM requests and the producers' registers (4.0 TB/s of voltages).  64
+// stations x 256 elements x 32 channels x 1000 samples to 16 int8 beams: 745 us
+// when eight warps landed the rows as int8 in shared memory by cp.async first, with
+// two block barriers a chunk; 739 us with 16 warps loading into registers for every
+// slot in turn; 760 us in groups, all with a warp on half lines of 8 rows; 521 us
+// with a warp on whole 128-byte lines of 4 rows.  Neighbouring units dealt to the
+// CTAs side by side instead of in ranges change stations more often: 546 us.
 #include "hai_internal.h"
 #include "tc.cuh"
 
 namespace {
 
-constexpr int kThreads = 416;
-constexpr int kProd = 256;             // warps 0-7
-constexpr int kMmaWarp = 8;
-constexpr int kEpi = 128;              // warps 9-12
-constexpr int kItems = 4;              // (row, 16-byte group) items per producer thread and chunk
+constexpr int kThreads = 768;
+constexpr int kProd = 512;             // warps 0-15
+constexpr int kMmaWarp = 16;
+constexpr int kEpi = 128;              // warps 20-23
+constexpr int kProdRegs = 96, kMmaRegs = 32, kEpiRegs = 64;   // 4 x 96 + 32 + 64 = 6 x 80
+constexpr int kGroup = 128;            // producers of one slot
+constexpr int kItems = 8;              // (row, 16-byte group) items per producer thread and chunk
+constexpr int kItemRows = 16;          // rows between a thread's items
 constexpr int kTile = 128;             // samples per unit (MMA M)
 constexpr int kChunkE = 64;            // elements per K chunk (128 real K)
-constexpr int kI8Stages = 5;           // int8 landing ring: 4 chunks in flight
-constexpr int kAhead = kI8Stages - 1;
-constexpr int kAStages = 2;            // fp16 operand ring
-constexpr uint32_t kI8Bytes = kTile * kChunkE * 2;   // int8 chunk: 128 rows x 128 B
-constexpr uint32_t kAKs = 128;         // A: K-group stride
-constexpr uint32_t kAMNs = 2048;       // A: row-group stride (16 K groups)
-constexpr uint32_t kABytes = 16 * kAMNs;             // 32 KB fp16 chunk
+constexpr int kAStages = 4;            // fp16 operand ring
+constexpr uint32_t kAKs = 144;         // A: K-group stride
+constexpr uint32_t kAMNs = 16 * kAKs;  // A: row-group stride (16 K groups)
+constexpr uint32_t kABytes = 16 * kAMNs;             // 36 KB fp16 chunk
+constexpr uint32_t kBKs = 128;         // B: K-group stride
 
 struct BfParams {
     const int8_t *volt;
     const int8_t *w;
     int S, C, T, K, ne, P;
     int tiles;                 // sample tiles per (s, c)
-    long long nunits, per_cta;
+    long long nunits;
     int shift;                 // < 0: int32 output
     void *beams;
     unsigned long long *nsat;
     unsigned *status;
 };
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
-                 "r"(src_bytes)
-                 : "memory");
+// 16 voltage bytes, not kept in L1 (every byte is read once).
+__device__ __forceinline__ int4 load16(const int8_t *p) {
+    int4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void bar_prod() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void bar_prod() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
 // 16 int8 -> 16 fp16 (two 8-value K groups), exact: bits 0x6400 + (x ^ 0x80) minus 1152
 __device__ __forceinline__ void widen16(const int4 raw, uint4 &lo, uint4 &hi) {
@@ -103,20 +109,19 @@ __global__ void __launch_bounds__(kThreads, 1) bf_kernel(const BfParams p) {
     const int ne_pad = nchunk * kChunkE;                      // B covers whole chunks, zero-padded
     const uint32_t bmns = (uint32_t)ne_pad * 32u;             // B: row-group stride (2 ne_pad / 8 groups)
     const uint32_t bbytes = (uint32_t)(2 * p.K / 8) * bmns;   // B of one polarisation
-    uint8_t *sI8 = smem;                                      // [kI8Stages][kI8Bytes]
-    uint8_t *sA = smem + kI8Stages * kI8Bytes;                // [kAStages][kABytes]
+    uint8_t *sA = smem;                                       // [kAStages][kABytes]
     uint8_t *sB = sA + kAStages * kABytes;                    // [P][bbytes]
     const int ncols = 2 * p.K;                                // MMA N per polarisation
     const uint32_t dcols = (uint32_t)(p.P * ncols);           // TMEM columns per unit
 
     if (tid == 0) {
         for (int s = 0; s < kAStages; s++) {
-            tc::mbar_init(&mb_full[s], kProd);
+            tc::mbar_init(&mb_full[s], kGroup / 32);
             tc::mbar_init(&mb_empty[s], 1);
         }
         for (int b = 0; b < 2; b++) {
             tc::mbar_init(&mb_dfull[b], 1);
-            tc::mbar_init(&mb_dempty[b], kEpi);
+            tc::mbar_init(&mb_dempty[b], kEpi / 32);
         }
         tc::mbar_fence_init();
     }
@@ -127,138 +132,167 @@ __global__ void __launch_bounds__(kThreads, 1) bf_kernel(const BfParams p) {
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = tmem_slot;
-    const long long u0 = (long long)blockIdx.x * p.per_cta;
-    const long long u1 = min(p.nunits, u0 + p.per_cta);
+    const long long u0 = p.nunits * blockIdx.x / gridDim.x, u1 = p.nunits * (blockIdx.x + 1) / gridDim.x;
     const size_t row_bytes = (size_t)p.ne * 2;                 // one (t, p) row of voltages
     const uint32_t idesc = tc::idesc_f16(128, ncols, 0, 0);
 
     if (warp < kMmaWarp) {
+        tc::setmaxnreg_inc<kProdRegs>();
         // ============================================================ producers
-        long long gq = 0;                                      // chunk counter (stages)
-        int cur_s = -1;
-        // chunks of the CTA in order: (unit = (station, channel, tile), pol,
-        // element chunk), walked by counters (no 64-bit divisions per chunk);
-        // one walker for the copies issued kAhead chunks early, one for the
-        // chunk being widened
-        struct Walk {
-            int s, c, tile, pol, kc;
-        };
-        auto walk_init = [&](Walk &w) {
-            w.s = (int)(u0 / ((long long)p.C * p.tiles));
-            w.c = (int)((u0 / p.tiles) % p.C);
-            w.tile = (int)(u0 % p.tiles);
-            w.pol = 0;
-            w.kc = 0;
-        };
-        auto walk_next = [&](Walk &w) {
-            if (++w.kc < nchunk) return;
-            w.kc = 0;
-            if (++w.pol < p.P) return;
-            w.pol = 0;
-            if (++w.tile < p.tiles) return;
-            w.tile = 0;
-            if (++w.c < p.C) return;
-            w.c = 0;
-            ++w.s;
-        };
-        const long long nq = (u1 - u0) * p.P * nchunk;
+        // Group grp fills slot grp of the ring: chunks grp, grp + 4, ... of the
+        // CTA in order (unit, pol, element chunk).  Two chunks of the group are in
+        // flight in registers; the loads of a buffer's next chunk start as soon as
+        // it has been widened.
+        const int grp = tid / kGroup, gt = tid % kGroup;
+        const int per_unit = p.P * nchunk;
         const uint32_t t_stride = (uint32_t)(p.P * row_bytes);  // bytes between samples of one pol
-        Walk wi, wc;
-        walk_init(wi);
-        walk_init(wc);
-        static_assert(kTile * 8 == kItems * kProd, "items per chunk");
-        // copy items: row tc0 + 32 j, group gc (16 bytes of row t stored at
-        // group g ^ (t & 7): conflict-free reads below)
-        const int tc0 = tid >> 3, gc = tid & 7;
-        const uint32_t src0 = (uint32_t)tc0 * t_stride + (uint32_t)gc * 16;
-        const uint32_t dst0 = (uint32_t)tc0 * 128 + (uint32_t)((gc ^ (tc0 & 7)) * 16);
-        // widening items: row tw0 + 32 j, group gw
-        const int tw0 = (tid & 7) + 8 * (tid >> 6), gw = (tid >> 3) & 7;
-        const uint32_t rd0 = (uint32_t)tw0 * 128 + (uint32_t)((gw ^ (tw0 & 7)) * 16);
+        static_assert(kTile * 8 == kItems * kGroup && kProd == kAStages * kGroup, "items per chunk, a slot per group");
+        // items: rows tw0 + 16 j, group gw: a warp loads whole 128-byte lines of 4
+        // rows; 8 lanes store 2 rows of 4 groups (K groups 144 bytes apart: no bank
+        // conflicts)
+        const int tw0 = 4 * (gt >> 5) + 2 * ((lane >> 3) & 1) + (lane & 1), gw = 4 * (lane >> 4) + ((lane >> 1) & 3);
+        const uint32_t src0 = (uint32_t)tw0 * t_stride + (uint32_t)gw * 16;
         const uint32_t wr0 = (uint32_t)(tw0 >> 3) * kAMNs + (uint32_t)(tw0 & 7) * 16 + (uint32_t)(2 * gw) * kAKs;
-        auto issue = [&](long long q) {                        // cp.async of chunk q into its int8 stage
-            if (q < nq) {
-                const int t0 = wi.tile * kTile;
-                const int8_t *base = p.volt + ((((size_t)wi.s * p.C + wi.c) * p.T + t0) * p.P + wi.pol) * row_bytes +
-                                     (size_t)wi.kc * kChunkE * 2;
-                uint8_t *dst = sI8 + (q % kI8Stages) * kI8Bytes + dst0;
-                const int t_valid = p.T - t0 - tc0;
-                const bool g_ok = gc * 8 < p.ne - wi.kc * kChunkE;
-#pragma unroll
-                for (int j = 0; j < kItems; j++) {
-                    const bool ok = g_ok && 32 * j < t_valid;
-                    const int8_t *src = ok ? base + src0 + (size_t)(32 * j) * t_stride : p.volt;
-                    cp_async16(dst + 32 * 128 * j, src, ok ? 16u : 0u);
+        int4 buf0[kItems], buf1[kItems];
+        // load walker: the group's next chunk (unit lu, chunk lr of the unit)
+        long long lu = u0, lsc = u0 / p.tiles;                 // station * C + channel
+        int ltile = (int)(u0 - lsc * p.tiles), lr = grp;
+        auto load = [&](int4 (&d)[kItems]) {
+            while (lr >= per_unit) {
+                lr -= per_unit;
+                lu++;
+                if (++ltile == p.tiles) {
+                    ltile = 0;
+                    lsc++;
                 }
-                walk_next(wi);
             }
-            cp_async_commit();
+            if (lu >= u1) return;
+            const int t0 = ltile * kTile, pol = lr >= nchunk ? 1 : 0, kc = lr - pol * nchunk;
+            const int8_t *src = p.volt + (size_t)(lsc * p.T + t0) * t_stride + pol * row_bytes + kc * (kChunkE * 2) + src0;
+            const int rows = p.T - t0, left = p.ne - kc * kChunkE;
+            if (rows >= kTile && left >= kChunkE) {            // the same for the group
+#pragma unroll
+                for (int j = 0; j < kItems; j++) d[j] = load16(src + (uint32_t)(kItemRows * j) * t_stride);
+            } else {
+#pragma unroll
+                for (int j = 0; j < kItems; j++)
+                    d[j] = tw0 + kItemRows * j < rows && gw * 8 < left ? load16(src + (uint32_t)(kItemRows * j) * t_stride)
+                                                                       : make_int4(0, 0, 0, 0);
+            }
+            lr += kAStages;
         };
-        for (int q = 0; q < kAhead; q++) issue(q);
-        for (long long q = 0; q < nq; q++, gq++) {
-            const int s = wc.s;
-            walk_next(wc);
-            issue(q + kAhead);             // its ring slot was drained at the end of iteration q - 1
-            cp_async_wait<kAhead>();
-            const int slot = (int)(gq % kAStages);
-            if (gq >= kAStages) tc::mbar_wait(&mb_empty[slot], (uint32_t)(((gq / kAStages) - 1) & 1), p.status);
-            if (s != cur_s) {
-                // new station: every MMA issued so far has completed (the empty
-                // barrier of the previous chunk), so B can be rewritten
-                if (gq >= 1) {
-                    const long long pq = gq - 1;
-                    tc::mbar_wait(&mb_empty[pq % kAStages], (uint32_t)((pq / kAStages) & 1), p.status);
-                }
-                for (int it = tid; it < (int)(p.P * bbytes / 16); it += kProd)
-                    reinterpret_cast<uint4 *>(sB)[it] = make_uint4(0, 0, 0, 0);
-                bar_prod();
-                for (int it = tid; it < p.P * p.K * p.ne; it += kProd) {   // (pol, beam, element)
-                    const int a = it % p.ne, kk = (it / p.ne) % p.K, pp = it / (p.ne * p.K);
-                    const char2 wv = reinterpret_cast<const char2 *>(p.w)[(((size_t)s * p.K + kk) * p.P + pp) * p.ne + a];
-                    const __half wr = __int2half_rn(wv.x), wi = __int2half_rn(wv.y), nwi = __int2half_rn(-(int)wv.y);
-                    uint8_t *B = sB + pp * bbytes;
-                    // row 2kk: (wr, wi); row 2kk+1: (-wi, wr)
-                    *reinterpret_cast<__half2 *>(B + tc::off_kmajor(2 * kk, 2 * a, kAKs, bmns)) = __halves2half2(wr, wi);
-                    *reinterpret_cast<__half2 *>(B + tc::off_kmajor(2 * kk + 1, 2 * a, kAKs, bmns)) = __halves2half2(nwi, wr);
-                }
-                cur_s = s;
-            }
-            bar_prod();                                        // int8 stage landed for all threads
-            const uint8_t *src = sI8 + (q % kI8Stages) * kI8Bytes + rd0;
-            uint8_t *A = sA + slot * kABytes + wr0;
+        uint8_t *A = sA + grp * kABytes + wr0;
+        auto widen = [&](int4 (&d)[kItems]) {
 #pragma unroll
-            for (int j = 0; j < kItems; j++) {                 // rows tw0 + 32 j: A row groups + 4 j
-                const int4 raw = *reinterpret_cast<const int4 *>(src + 32 * 128 * j);
+            for (int j = 0; j < kItems; j++) {                 // rows tw0 + 16 j: A row groups + 2 j
                 uint4 lo, hi;
-                widen16(raw, lo, hi);
-                *reinterpret_cast<uint4 *>(A + 4 * kAMNs * j) = lo;
-                *reinterpret_cast<uint4 *>(A + 4 * kAMNs * j + kAKs) = hi;
+                widen16(d[j], lo, hi);
+                *reinterpret_cast<uint4 *>(A + (kItemRows / 8) * kAMNs * j) = lo;
+                *reinterpret_cast<uint4 *>(A + (kItemRows / 8) * kAMNs * j + kAKs) = hi;
             }
+            load(d);
+        };
+        // The station's weights into B: 8 elements of one (pol, beam) at a time,
+        // row 2k: (wr, wi), row 2k + 1: (-wi, wr); zero beyond the elements.
+        auto fill_b = [&](int s) {
+            const int g8 = ne_pad / 8, rows8 = p.P * p.K * g8;
+            const bool wide = ((uintptr_t)p.w & 15) == 0;
+            for (int it = tid; it < rows8; it += kProd) {
+                const int a8 = it % g8, row = it / g8, kk = row % p.K, pp = row / p.K;
+                int4 raw = make_int4(0, 0, 0, 0);
+                if (a8 * 8 < p.ne) {
+                    const int8_t *src = p.w + ((((size_t)s * p.K + kk) * p.P + pp) * p.ne + a8 * 8) * 2;
+                    if (wide) raw = *reinterpret_cast<const int4 *>(src);
+                    else {
+                        const ushort *e = reinterpret_cast<const ushort *>(src);
+                        auto two = [&](int i) { return (int)((uint32_t)e[i] | ((uint32_t)e[i + 1] << 16)); };
+                        raw = make_int4(two(0), two(2), two(4), two(6));
+                    }
+                }
+                uint4 o[2];
+                widen16(raw, o[0], o[1]);
+                uint8_t *B = sB + pp * bbytes + tc::off_kmajor(2 * kk, 16 * a8, kBKs, bmns);
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    // (wr, wi) -> (-wi, wr): halves swapped, the low one's sign flipped (0 stays +0)
+                    const uint32_t v[4] = {o[h].x, o[h].y, o[h].z, o[h].w};
+                    uint32_t m[4];
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const __half2 x = *reinterpret_cast<const __half2 *>(&v[i]);
+                        const __half2 y = __halves2half2(__hsub(__ushort_as_half(0), __high2half(x)), __low2half(x));
+                        m[i] = *reinterpret_cast<const uint32_t *>(&y);
+                    }
+                    *reinterpret_cast<uint4 *>(B + h * kBKs) = o[h];
+                    *reinterpret_cast<uint4 *>(B + h * kBKs + 16) = make_uint4(m[0], m[1], m[2], m[3]);
+                }
+            }
+        };
+        load(buf0);
+        load(buf1);
+        const long long per_station = (long long)p.C * p.tiles;
+        long long u = u0, cu = u0 % per_station;               // unit, within its station
+        int s = (int)(u0 / per_station), n = 0, r = grp;       // n chunks done, r the next one's place in the unit
+        // Every group comes by every unit: a new station's B can be rewritten once
+        // the MMAs of every group's last chunk have completed.
+        auto enter = [&] {
+            if (n > 0) tc::mbar_wait(&mb_empty[grp], (uint32_t)((n - 1) & 1), p.status);
+            bar_prod();
+            fill_b(s);
             tc::fence_proxy_async();
-            tc::mbar_arrive(&mb_full[slot]);
-            bar_prod();                                        // int8 stage may be refilled
+            bar_prod();
+        };
+        auto more = [&] {
+            while (r >= per_unit) {
+                r -= per_unit;
+                if (++u == u1) return false;
+                if (++cu == per_station) {
+                    cu = 0;
+                    s++;
+                    enter();
+                }
+            }
+            return true;
+        };
+        auto step = [&](int4 (&d)[kItems]) {
+            if (n > 0) tc::mbar_wait(&mb_empty[grp], (uint32_t)((n - 1) & 1), p.status);
+            widen(d);
+            tc::fence_proxy_async();
+            tc::mbar_arrive_warp(&mb_full[grp]);
+            r += kAStages;
+            n++;
+        };
+        // each buffer in its own half of the loop: one pass over both would copy a
+        // buffer still being loaded, and wait for it
+        if (u < u1) {
+            enter();
+            while (more()) {
+                step(buf0);
+                if (!more()) break;
+                step(buf1);
+            }
         }
-        cp_async_wait<0>();
-    } else if (warp == kMmaWarp) {
+    } else if (warp < kMmaWarp + 4) {
         // ============================================================ MMA
-        if (lane == 0) {
+        tc::setmaxnreg_dec<kMmaRegs>();
+        if (warp == kMmaWarp && tc::elect()) {
             long long gq = 0, gu = 0;
+            const uint64_t da = tc::desc(tc::smem_u32(sA), kAKs, kAMNs), db = tc::desc(tc::smem_u32(sB), kBKs, bmns);
             for (long long u = u0; u < u1; u++, gu++) {
                 const int b = (int)(gu & 1);
                 if (gu >= 2) tc::mbar_wait(&mb_dempty[b], (uint32_t)(((gu >> 1) - 1) & 1), p.status);
                 tc::fence_after();
                 for (int pol = 0; pol < p.P; pol++) {
                     const uint32_t d = tmem + (uint32_t)b * dcols + (uint32_t)pol * ncols;
-                    const uint32_t bb = tc::smem_u32(sB + pol * bbytes);
                     for (int kc = 0; kc < nchunk; kc++, gq++) {
                         const int slot = (int)(gq % kAStages);
                         tc::mbar_wait(&mb_full[slot], (uint32_t)((gq / kAStages) & 1), p.status);
                         tc::fence_after();
-                        const uint32_t a = tc::smem_u32(sA + slot * kABytes);
+                        const uint64_t a = tc::desc_add(da, slot * kABytes);
+                        const uint64_t bb = tc::desc_add(db, pol * bbytes + kc * 16 * kBKs);
 #pragma unroll
                         for (int s = 0; s < 8; s++)
-                            tc::mma_f16(d, tc::desc(a + s * 2 * kAKs, kAKs, kAMNs),
-                                        tc::desc(bb + (kc * 16 + s * 2) * kAKs, kAKs, bmns), idesc,
+                            tc::mma_f16(d, tc::desc_add(a, s * 2 * kAKs), tc::desc_add(bb, s * 2 * kBKs), idesc,
                                         (kc > 0 || s > 0) ? 1u : 0u);
                         tc::mma_commit(&mb_empty[slot]);
                     }
@@ -268,6 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1) bf_kernel(const BfParams p) {
         }
     } else {
         // ============================================================ epilogue
+        tc::setmaxnreg_dec<kEpiRegs>();
         const int q = warp & 3;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const int t_local = q * 32 + lane;
@@ -338,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) bf_kernel(const BfParams p) {
                 }
             }
             tc::fence_before();
-            tc::mbar_arrive(&mb_dempty[b]);
+            tc::mbar_arrive_warp(&mb_dempty[b]);
         }
         if (p.nsat) {
             for (int o = 16; o; o >>= 1) sat += __shfl_xor_sync(0xffffffffu, sat, o);
@@ -383,13 +418,12 @@ extern "C" hai_status hai_beamform(hai_ctx *ctx, const int8_t *volt, const int8_
     p.tiles = (T + kTile - 1) / kTile;
     p.nunits = (long long)S * C * p.tiles;
     const int grid = (int)std::min<long long>(p.nunits, ctx->num_sms);
-    p.per_cta = (p.nunits + grid - 1) / grid;
     p.shift = requant_shift;
     p.beams = beams;
     p.nsat = reinterpret_cast<unsigned long long *>(n_saturated);
     p.status = ctx->d_status;
     const size_t bbytes = (size_t)(2 * K / 8) * ((N + kChunkE - 1) / kChunkE * kChunkE) * 32;
-    const size_t smem = kI8Stages * kI8Bytes + kAStages * kABytes + (size_t)P * bbytes;
+    const size_t smem = kAStages * kABytes + (size_t)P * bbytes;
     if (smem > (size_t)ctx->smem_optin)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_beamform: weights of one station exceed shared memory");
     HAI_CUDA_TRY(cudaFuncSetAttribute(bf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
