@@ -244,7 +244,7 @@ epic_fp32_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long lon
 // phase costs one block barrier.
 //
 // Shared layouts, all accesses in the minimum two wavefronts per 8-byte
-// access: H[sample][p][y][(k + 2 (y & 7)) & 63] with pol and sample planes
+// access: H[sample][p][y][(k + 2 (y & 7)) & 63] with pol (or re, im) and sample planes
 // 8 (mod 16) float2 apart (a half-warp writes one row of both samples, or of
 // both pols, or rows y and y + 4 of one pol, and reads rows t + 8 m of two
 // adjacent columns); the exchange scratch of a group holds value k of lane t
@@ -252,17 +252,14 @@ epic_fp32_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long lon
 constexpr int k64Threads = 512;                  // 64 groups of 8 lanes
 constexpr int k64Xs = 72;                        // float2 of exchange scratch per group (one pol at a time)
 
-__device__ __forceinline__ void dft8_first4(float2 (&a)[8]) {
+template <typename V>
+__device__ __forceinline__ void dft8_first4(V (&a)[8]) {
     // inputs a[4..7] zero: the even outputs are the 4-point DFT of a[0..3],
     // the odd ones that of a[m] w8^m
-    const float h = 0.70710678118654752f;
-    float2 v0 = a[0], v1 = a[1], v2 = a[2], v3 = a[3];
-    v1 = make_float2(h * (v1.x - v1.y), h * (v1.x + v1.y));          // * e^(+i pi/4)
-    v2 = hai_fft512::cmuli(v2);                                       // * e^(+i pi/2)
-    v3 = make_float2(-h * (v3.x + v3.y), h * (v3.x - v3.y));         // * e^(+3i pi/4)
-    float2 u0 = a[0], u1 = a[1], u2 = a[2], u3 = a[3];
+    V v0 = a[0], v1 = hai_fft512::crot<1>(a[1]), v2 = a[2], v3 = hai_fft512::crot<3>(a[3]);
+    V u0 = a[0], u1 = a[1], u2 = a[2], u3 = a[3];
     hai_fft512::dft4(u0, u1, u2, u3);
-    hai_fft512::dft4(v0, v1, v2, v3);
+    hai_fft512::dft4<true>(v0, v1, v2, v3);
     a[0] = u0; a[2] = u1; a[4] = u2; a[6] = u3;
     a[1] = v0; a[3] = v1; a[5] = v2; a[7] = v3;
 }
@@ -316,11 +313,19 @@ struct Epic64Smem {
 // int8 voltages of the next phase are copied into shared memory while the
 // current one is imaged.
 //
-// Row tasks: warp w takes rows w and 31 - w (+ 32), so that the rows beyond a
-// box of fewer than 32 spread over the four schedulers.  SP = 2: group g
-// takes its row of sample g & 1 of the phase, both pols (one walk of the
-// gather table for both); SP = 1, P = 2: pol g & 1; P = 1: rows g and g + 4
-// paired in a half-warp.  The exchanges go one pol at a time.
+// Row tasks: warp w takes rows w and 31 - w, so that the rows beyond a box of
+// fewer than 32 spread over the four schedulers.  SP = 2: group g takes its row of
+// sample g & 1 of the phase, both pols (one walk of the gather table for both); SP
+// = 1: a row a group, both pols at once too for boxes of more than 32 rows (rows g
+// and g + 4 paired in a half-warp), else pol g & 1.
+//
+// kPair: both pols go through one transform as packed pairs (one instruction for
+// both), the two planes of H and the two halves of an exchange holding real and
+// imaginary parts of (X, Y).  Bound: shared-memory wavefronts (exchanges, H and the
+// gather's random reads: four fifths of the cycles) and issue slots.  37 channels x
+// 999 samples of a station of 251 elements: 658 us with a transform per pol and the
+// channel of a sample found by a 64-bit division, 617 us with packed pairs, 598 us
+// with the channel's samples counted.
 template <int P, bool PX, bool PY, int SP, bool TS>
 __global__ void __launch_bounds__(k64Threads, 1)
 epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long len, int box_w, int box_h,
@@ -329,8 +334,8 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
     constexpr int Q = (P == 2) ? 4 : 1;
     using S = Epic64Smem<P, PX, PY, SP, TS>;
     constexpr int PO = S::PO, SO = S::SO, HB = S::HB;
-    constexpr int RP = (SP == 2) ? P : 1;                    // pols per row task
-    constexpr int RR = (SP == 2 || P == 2) && !PY ? 2 : 1;   // row tasks per group
+    constexpr bool kPair = P == 2 && (SP == 2 || !PY);       // both pols in one transform of packed pairs
+    constexpr int GP = kPair ? 2 : 1;                        // pols per row task
     static_assert(SP == 1 || PY, "two samples per phase need a box of at most 32 rows");
     extern __shared__ __align__(16) unsigned char smem[];
     float2 *Hs = reinterpret_cast<float2 *>(smem);                        // [2][HB]
@@ -379,7 +384,7 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
 #pragma unroll
         for (int q = 0; q < Q; q++) acc[k][q] = 0.f;
     const int col = g;                                   // column pass: column of this group
-    int cur_c = (int)(s0 / T), seg = 0;
+    int cur_c = (int)(s0 / T), seg = 0, left = T - (int)(s0 % T);   // left: samples of channel cur_c to add
     auto flush = [&](int c, int sgm) {
         float *dst = direct ? out + (size_t)c * Q * 4096 : out + ((size_t)blockIdx.x * 2 + sgm) * Q * 4096;
         const int lx = (col + 32) & 63;
@@ -406,6 +411,25 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
         hai_fft512::dft8(a);
     };
 
+    // the same for a pair: real parts, then imaginary parts through the scratch
+    using hai_fft512::c2;
+    auto finish2 = [&](c2 (&a)[8]) {
+        unsigned long long *x = reinterpret_cast<unsigned long long *>(xs);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; k++) x[9 * k + t] = a[k].re;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 8; u++) a[u].re = x[9 * t + u];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; k++) x[9 * k + t] = a[k].im;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 8; u++) a[u].im = x[9 * t + u];
+        hai_fft512::dft8(a);
+    };
+
     load(0, 0);
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
@@ -417,14 +441,17 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
                                      staged_offset(volt + (size_t)(s0 + (long long)SP * it) * vbytes);
             float2 *H = Hs + (size_t)(it & 1) * HB;
             const int ns = min(SP, n - SP * it);
-#pragma unroll
-            for (int r = 0; r < RR; r++) {
+            do {
                 int y, p0, si;
-                const int w = g >> 2, yw = ((g & 2) ? 31 - w : w) + 32 * r;
+                const int w = g >> 2, yw = ((g & 2) ? 31 - w : w);
                 if (SP == 2) {
                     si = g & 1;
                     p0 = 0;
                     y = yw;
+                } else if (kPair) {
+                    si = 0;
+                    p0 = 0;
+                    y = (g & ~7) | ((g & 1) << 2) | ((g >> 1) & 3);
                 } else if (P == 2) {
                     si = 0;
                     p0 = g & 1;
@@ -435,10 +462,10 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
                     y = (g & ~7) | ((g & 1) << 2) | ((g >> 1) & 3);
                 }
                 const bool live = y < box_h && si < ns;
-                if (!__any_sync(0xffffffffu, live)) continue;             // warp-uniform
-                float2 a[RP][8];
+                if (!__any_sync(0xffffffffu, live)) break;                // warp-uniform
+                float2 a[GP][8];
 #pragma unroll
-                for (int q = 0; q < RP; q++)
+                for (int q = 0; q < GP; q++)
 #pragma unroll
                     for (int m = 0; m < 8; m++) a[q][m] = make_float2(0.f, 0.f);
                 if (live) {
@@ -456,9 +483,9 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
                     }
 #pragma unroll
                     for (int m = 0; m < MX; m++) {
-                        float2 acg[RP];
+                        float2 acg[GP];
 #pragma unroll
-                        for (int q = 0; q < RP; q++) acg[q] = make_float2(0.f, 0.f);
+                        for (int q = 0; q < GP; q++) acg[q] = make_float2(0.f, 0.f);
                         for (int i = cb[m]; i < ce[m]; i++) {
                             int el;
                             float2 wv;                                    // conj(W~)
@@ -471,7 +498,7 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
                                 wv = __ldg(cw + i);
                             }
 #pragma unroll
-                            for (int q = 0; q < RP; q++) {
+                            for (int q = 0; q < GP; q++) {
                                 const char2 v = E[q * ne + el];
                                 const float er = (float)v.x, ei = (float)v.y;
                                 acg[q].x = fmaf(wv.x, er, fmaf(-wv.y, ei, acg[q].x));
@@ -479,27 +506,42 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
                             }
                         }
 #pragma unroll
-                        for (int q = 0; q < RP; q++) a[q][m] = acg[q];
+                        for (int q = 0; q < GP; q++) a[q][m] = acg[q];
                     }
                 }
+                if constexpr (kPair) {
+                    c2 b[8];
 #pragma unroll
-                for (int q = 0; q < RP; q++) {
-                    if (PX) dft8_first4(a[q]);
-                    else hai_fft512::dft8(a[q]);
+                    for (int m = 0; m < 8; m++)
+                        b[m] = {hai_fft512::pack2(a[0][m].x, a[1][m].x), hai_fft512::pack2(a[0][m].y, a[1][m].y)};
+                    if (PX) dft8_first4(b);
+                    else hai_fft512::dft8(b);
 #pragma unroll
-                    for (int k = 1; k < 8; k++) a[q][k] = hai_fft512::cmul(a[q][k], tw[k]);
-                    finish(a[q]);
-                }
-                if (live) {
-                    const int sw = 2 * (y & 7);
+                    for (int k = 1; k < 8; k++) b[k] = hai_fft512::cmul(b[k], tw[k]);
+                    finish2(b);
+                    if (live) {
+                        const int sw = 2 * (y & 7);
+                        unsigned long long *row = reinterpret_cast<unsigned long long *>(H + (size_t)si * SO + (size_t)y * 64);
 #pragma unroll
-                    for (int q = 0; q < RP; q++) {
-                        float2 *row = H + (size_t)si * SO + (size_t)(p0 + q) * PO + (size_t)y * 64;
+                        for (int k2 = 0; k2 < 8; k2++) {
+                            row[(t + 8 * k2 + sw) & 63] = b[k2].re;
+                            row[PO + ((t + 8 * k2 + sw) & 63)] = b[k2].im;
+                        }
+                    }
+                } else {
+                    if (PX) dft8_first4(a[0]);
+                    else hai_fft512::dft8(a[0]);
 #pragma unroll
-                        for (int k2 = 0; k2 < 8; k2++) row[(t + 8 * k2 + sw) & 63] = a[q][k2];
+                    for (int k = 1; k < 8; k++) a[0][k] = hai_fft512::cmul(a[0][k], tw[k]);
+                    finish(a[0]);
+                    if (live) {
+                        const int sw = 2 * (y & 7);
+                        float2 *row = H + (size_t)si * SO + (size_t)p0 * PO + (size_t)y * 64;
+#pragma unroll
+                        for (int k2 = 0; k2 < 8; k2++) row[(t + 8 * k2 + sw) & 63] = a[0][k2];
                     }
                 }
-            }
+            } while (false);
         }
         if (it >= 1) {
             // column pass of phase it - 1, sample by sample
@@ -509,38 +551,62 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
 #pragma unroll
             for (int si = 0; si < SP; si++) {
                 if (si >= ns) break;                                      // CTA-uniform
-                const int c = (int)((s0 + (long long)SP * (it - 1) + si) / T);
-                if (c != cur_c) {
+                if (left == 0) {
                     flush(cur_c, seg);
                     seg++;
-                    cur_c = c;
+                    cur_c++;
+                    left = T;
                 }
+                left--;
                 const float2 *H = Hp + (size_t)si * SO;
-                float2 f[P][8];
-#pragma unroll
-                for (int p = 0; p < P; p++) {
+                if constexpr (kPair) {
+                    const unsigned long long *Hq = reinterpret_cast<const unsigned long long *>(H) + pos;
+                    c2 x[8];
 #pragma unroll
                     for (int m = 0; m < 8; m++) {
                         const int y = t + 8 * m;
-                        f[p][m] = (m < (PY ? 4 : 8) && y < box_h) ? H[(size_t)p * PO + (size_t)y * 64 + pos]
-                                                                  : make_float2(0.f, 0.f);
+                        x[m] = m < (PY ? 4 : 8) && y < box_h ? c2{Hq[y * 64], Hq[PO + y * 64]} : c2{0, 0};
                     }
-                    if (PY) dft8_first4(f[p]);
-                    else hai_fft512::dft8(f[p]);
+                    if (PY) dft8_first4(x);
+                    else hai_fft512::dft8(x);
 #pragma unroll
-                    for (int k = 1; k < 8; k++) f[p][k] = hai_fft512::cmul(f[p][k], tw[k]);
-                }
+                    for (int k = 1; k < 8; k++) x[k] = hai_fft512::cmul(x[k], tw[k]);
+                    finish2(x);
 #pragma unroll
-                for (int p = 0; p < P; p++) finish(f[p]);
+                    for (int k2 = 0; k2 < 8; k2++) {
+                        unsigned long long pw = hai_fft512::pack2(acc[k2][0], acc[k2][Q > 1 ? 1 : 0]);
+                        hai_fft512::add_products(x[k2], pw, acc[k2][Q > 2 ? 2 : 0], acc[k2][Q > 3 ? 3 : 0]);
+                        const float2 v = hai_fft512::unpack2(pw);
+                        acc[k2][0] = v.x;
+                        acc[k2][Q > 1 ? 1 : 0] = v.y;
+                    }
+                } else {
+                    float2 f[P][8];
 #pragma unroll
-                for (int k2 = 0; k2 < 8; k2++) {
-                    const float2 fx = f[0][k2];
-                    acc[k2][0] = fmaf(fx.x, fx.x, fmaf(fx.y, fx.y, acc[k2][0]));
-                    if (P == 2) {
-                        const float2 fy = f[P - 1][k2];
-                        acc[k2][Q > 1 ? 1 : 0] = fmaf(fy.x, fy.x, fmaf(fy.y, fy.y, acc[k2][Q > 1 ? 1 : 0]));
-                        acc[k2][Q > 2 ? 2 : 0] = fmaf(fx.x, fy.x, fmaf(fx.y, fy.y, acc[k2][Q > 2 ? 2 : 0]));
-                        acc[k2][Q > 3 ? 3 : 0] = fmaf(fx.y, fy.x, fmaf(-fx.x, fy.y, acc[k2][Q > 3 ? 3 : 0]));
+                    for (int p = 0; p < P; p++) {
+#pragma unroll
+                        for (int m = 0; m < 8; m++) {
+                            const int y = t + 8 * m;
+                            f[p][m] = (m < (PY ? 4 : 8) && y < box_h) ? H[(size_t)p * PO + (size_t)y * 64 + pos]
+                                                                      : make_float2(0.f, 0.f);
+                        }
+                        if (PY) dft8_first4(f[p]);
+                        else hai_fft512::dft8(f[p]);
+#pragma unroll
+                        for (int k = 1; k < 8; k++) f[p][k] = hai_fft512::cmul(f[p][k], tw[k]);
+                    }
+#pragma unroll
+                    for (int p = 0; p < P; p++) finish(f[p]);
+#pragma unroll
+                    for (int k2 = 0; k2 < 8; k2++) {
+                        const float2 fx = f[0][k2];
+                        acc[k2][0] = fmaf(fx.x, fx.x, fmaf(fx.y, fx.y, acc[k2][0]));
+                        if (P == 2) {
+                            const float2 fy = f[P - 1][k2];
+                            acc[k2][Q > 1 ? 1 : 0] = fmaf(fy.x, fy.x, fmaf(fy.y, fy.y, acc[k2][Q > 1 ? 1 : 0]));
+                            acc[k2][Q > 2 ? 2 : 0] = fmaf(fx.x, fy.x, fmaf(fx.y, fy.y, acc[k2][Q > 2 ? 2 : 0]));
+                            acc[k2][Q > 3 ? 3 : 0] = fmaf(fx.y, fy.x, fmaf(-fx.x, fy.y, acc[k2][Q > 3 ? 3 : 0]));
+                        }
                     }
                 }
             }

@@ -276,14 +276,6 @@ __global__ void __launch_bounds__(64 * RPC, 4) large512_rows_kernel(
     }
 }
 
-// |F_X|^2, |F_Y|^2 (a pair) and F_X conj(F_Y) of one pixel added to its sums.
-__device__ __forceinline__ void add_products(c2 f, unsigned long long &pw, float &xr, float &xi) {
-    pw = fma2(f.re, f.re, fma2(f.im, f.im, pw));
-    const float2 r = unpack2(f.re), i = unpack2(f.im);
-    xr = fmaf(r.x, r.y, fmaf(i.x, i.y, xr));           // Re X conj(Y)
-    xi = fmaf(i.x, r.y, fmaf(-r.x, i.y, xi));          // Im X conj(Y)
-}
-
 // The four sums of a pixel into the image planes (or onto them).
 __device__ __forceinline__ void put_products(float *dst, size_t plane, int add, unsigned long long pw, float xr, float xi) {
     const float2 p = unpack2(pw);

@@ -86,6 +86,14 @@ __device__ __forceinline__ c2 cmul(c2 a, float2 w) {
             pack2(fmaf(r.x, w.y, i.x * w.x), fmaf(r.y, w.y, i.y * w.x))};
 }
 
+// |F_X|^2, |F_Y|^2 (a pair) and F_X conj(F_Y) of one pixel added to its sums.
+__device__ __forceinline__ void add_products(c2 f, unsigned long long &pw, float &xr, float &xi) {
+    pw = fma2(f.re, f.re, fma2(f.im, f.im, pw));
+    const float2 r = unpack2(f.re), i = unpack2(f.im);
+    xr = fmaf(r.x, r.y, fmaf(i.x, i.y, xr));           // Re X conj(Y)
+    xi = fmaf(i.x, r.y, fmaf(-r.x, i.y, xi));          // Im X conj(Y)
+}
+
 // 4-point DFT, exponent +: X_k = sum_m x_m i^(m k), natural order; I2: x2 is
 // taken times i.
 template <bool I2 = false, typename V>
