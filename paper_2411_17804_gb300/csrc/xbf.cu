@@ -25,12 +25,16 @@
 // A' = [A_hi | A_hi | A_lo] against Phi' = [Phi_hi | Phi_lo | Phi_hi], so the
 // same GEMM sums hi*hi + hi*lo + lo*hi (FP32-level accuracy, 3x the work).
 //
-// GEMM: one CTA per 128 x 256 output tile; a 4-stage pipeline of 48 KB bulk
-// copies (A 128 x 64 and Phi 256 x 64, fp16); warp 0 streams, warp 1 issues
-// tcgen05.mma (M = 128, N = 256, K = 16) into a 256-column TMEM accumulator,
-// warps 4-7 write the tile.  Row blocks are the fastest grid index, so the
-// CTAs running together share one Phi block, read from HBM once and served
-// to the row blocks from L2.
+// GEMM: a CTA takes two row blocks of 128 x a block of 256 pixels (one row block in
+// the last wave); 64-deep k blocks of A and Phi arrive by bulk copies in a ring of 3
+// stages of 64 KB (4 of 48 KB); warp 0 streams, warp 1 issues tcgen05.mma (M = 128,
+// N = 256, K = 16) into one 256-column TMEM accumulator per row block, warps 4-7
+// write the tiles.  Row blocks are the fastest grid index, so the CTAs running
+// together share one Phi block, read from HBM once and served to the row blocks
+// from L2.  Bound: shared memory, which both the copies and the MMAs' operands
+// pass through: a k block of one row block keeps it busy for 768 cycles (48 KB in,
+// 4 x 12 KB out) and the tensor pipe for 512, of two row blocks 1,280 and 1,024.
+// 512 rows x 65,536 pixels, 5,515 pairs: 591 us with single tiles, 546 us.
 #include <math.h>
 
 #include <algorithm>
@@ -193,81 +197,105 @@ struct GemmParams {
     const float *scale;
     float *img;
     int n_kblk, M, npix, accumulate;
+    int mblk;                    // row blocks
+    int dbl;                     // pixel blocks whose row blocks go in twos
     unsigned *status;
 };
 
-__global__ void __launch_bounds__(kThreads, 1) xbf_gemm_kernel(const GemmParams p) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t full[kStages], empty[kStages], accf;
-    __shared__ uint32_t tslot;
+struct GemmBars {
+    uint64_t full[kStages], empty[kStages], accf;
+    uint32_t tslot;
+};
+
+// Output tiles of MB row blocks (the first one mb) x pixel block nb.
+template <int MB>
+__device__ __forceinline__ void gemm_tile(const GemmParams &p, uint8_t *smem, GemmBars &bar, int mb, int nb) {
+    constexpr int kSt = MB == 2 ? 3 : kStages;                // 3 x 64 KB or 4 x 48 KB
+    constexpr uint32_t kStage = MB * kABytes + kBBytes;
+    static_assert(kSt * kStage <= kSmem && kSt <= kStages, "stages");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int mb = blockIdx.x, nb = blockIdx.y;
     if (tid == 0) {
-        for (int s = 0; s < kStages; s++) {
-            tc::mbar_init(&full[s], 1);
-            tc::mbar_init(&empty[s], 1);
+        for (int s = 0; s < kSt; s++) {
+            tc::mbar_init(&bar.full[s], 1);
+            tc::mbar_init(&bar.empty[s], 1);
         }
-        tc::mbar_init(&accf, 1);
+        tc::mbar_init(&bar.accf, 1);
         tc::mbar_fence_init();
     }
-    if (warp == 0) tc::tmem_alloc(&tslot, kTN);
+    if (warp == 0) tc::tmem_alloc(&bar.tslot, MB * kTN);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    const uint32_t tmem = tslot;
-    auto sA = [&](int s) { return smem + (size_t)s * (kABytes + kBBytes); };
-    auto sB = [&](int s) { return smem + (size_t)s * (kABytes + kBBytes) + kABytes; };
-    const uint8_t *ablk = p.A + (size_t)mb * p.n_kblk * kABytes;
-    const uint8_t *bblk = p.phi + (size_t)nb * p.n_kblk * kBBytes;
+    const uint32_t tmem = bar.tslot;
     if (warp == 0) {
-        if (lane == 0)
-            for (int kb = 0; kb < p.n_kblk; kb++) {
-                const int s = kb % kStages;
-                if (kb >= kStages) tc::mbar_wait(&empty[s], (uint32_t)(((kb / kStages) - 1) & 1), p.status);
-                tc::mbar_arrive_expect_tx(&full[s], kABytes + kBBytes);
-                tc::bulk_g2s(sA(s), ablk + (size_t)kb * kABytes, kABytes, &full[s]);
-                tc::bulk_g2s(sB(s), bblk + (size_t)kb * kBBytes, kBBytes, &full[s]);
+        if (tc::elect()) {
+            const uint8_t *a = p.A + (size_t)mb * p.n_kblk * kABytes, *b = p.phi + (size_t)nb * p.n_kblk * kBBytes;
+            const size_t next_block = (size_t)p.n_kblk * kABytes;
+            int s = 0, fill = 0;                              // ring stage, times it has been filled before
+            for (int kb = 0; kb < p.n_kblk; kb++, a += kABytes, b += kBBytes) {
+                if (fill) tc::mbar_wait(&bar.empty[s], (uint32_t)((fill - 1) & 1), p.status);
+                uint8_t *st = smem + (size_t)s * kStage;
+                tc::mbar_arrive_expect_tx(&bar.full[s], kStage);
+#pragma unroll
+                for (int m = 0; m < MB; m++) tc::bulk_g2s(st + m * kABytes, a + m * next_block, kABytes, &bar.full[s]);
+                tc::bulk_g2s(st + MB * kABytes, b, kBBytes, &bar.full[s]);
+                if (++s == kSt) {
+                    s = 0;
+                    fill++;
+                }
             }
+        }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (tc::elect()) {
+            const uint64_t da0 = tc::desc(tc::smem_u32(smem), kLBO, kSBO);
+            int s = 0;
+            uint32_t ph = 0;
             for (int kb = 0; kb < p.n_kblk; kb++) {
-                const int s = kb % kStages;
-                tc::mbar_wait(&full[s], (uint32_t)((kb / kStages) & 1), p.status);
+                tc::mbar_wait(&bar.full[s], ph, p.status);
                 tc::fence_after();
-                const uint32_t a = tc::smem_u32(sA(s)), b = tc::smem_u32(sB(s));
+                const uint64_t da = tc::desc_add(da0, (uint32_t)s * kStage), db = tc::desc_add(da, MB * kABytes);
 #pragma unroll
                 for (int j = 0; j < kTK / 16; j++)
-                    tc::mma_f16(tmem, tc::desc(a + j * 2 * kLBO, kLBO, kSBO), tc::desc(b + j * 2 * kLBO, kLBO, kSBO),
-                                kIdesc, (kb > 0 || j > 0) ? 1u : 0u);
-                tc::mma_commit(&empty[s]);
+#pragma unroll
+                    for (int m = 0; m < MB; m++)
+                        tc::mma_f16(tmem + m * kTN, tc::desc_add(da, m * kABytes + j * 2 * kLBO), tc::desc_add(db, j * 2 * kLBO),
+                                    kIdesc, (kb > 0 || j > 0) ? 1u : 0u);
+                tc::mma_commit(&bar.empty[s]);
+                if (++s == kSt) {
+                    s = 0;
+                    ph ^= 1;
+                }
             }
-            tc::mma_commit(&accf);
+            tc::mma_commit(&bar.accf);
         }
     } else if (warp >= 4) {
-        tc::mbar_wait(&accf, 0u, p.status);
+        tc::mbar_wait(&bar.accf, 0u, p.status);
         tc::fence_after();
         const int q = warp & 3;
-        const int row = mb * kTM + q * 32 + lane;
-        const float sc = row < p.M ? p.scale[row / 4] : 0.f;
 #pragma unroll 1
-        for (int ch = 0; ch < kTN / 32; ch++) {
-            uint32_t r[32];
-            tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 32), r);
-            tc::tmem_wait_ld();
-            if (row < p.M) {
-                float4 *dst = reinterpret_cast<float4 *>(p.img + (size_t)row * p.npix + (size_t)nb * kTN + ch * 32);
+        for (int m = 0; m < MB; m++) {
+            const int row = (mb + m) * kTM + q * 32 + lane;
+            const float sc = row < p.M ? p.scale[row / 4] : 0.f;
+#pragma unroll 1
+            for (int ch = 0; ch < kTN / 32; ch++) {
+                uint32_t r[32];
+                tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(m * kTN + ch * 32), r);
+                tc::tmem_wait_ld();
+                if (row < p.M) {
+                    float4 *dst = reinterpret_cast<float4 *>(p.img + (size_t)row * p.npix + (size_t)nb * kTN + ch * 32);
 #pragma unroll
-                for (int v = 0; v < 8; v++) {
-                    float4 o = make_float4(__uint_as_float(r[4 * v]) * sc, __uint_as_float(r[4 * v + 1]) * sc,
-                                           __uint_as_float(r[4 * v + 2]) * sc, __uint_as_float(r[4 * v + 3]) * sc);
-                    if (p.accumulate) {
-                        const float4 old = dst[v];
-                        o.x += old.x;
-                        o.y += old.y;
-                        o.z += old.z;
-                        o.w += old.w;
+                    for (int v = 0; v < 8; v++) {
+                        float4 o = make_float4(__uint_as_float(r[4 * v]) * sc, __uint_as_float(r[4 * v + 1]) * sc,
+                                               __uint_as_float(r[4 * v + 2]) * sc, __uint_as_float(r[4 * v + 3]) * sc);
+                        if (p.accumulate) {
+                            const float4 old = dst[v];
+                            o.x += old.x;
+                            o.y += old.y;
+                            o.z += old.z;
+                            o.w += old.w;
+                        }
+                        dst[v] = o;
                     }
-                    dst[v] = o;
                 }
             }
         }
@@ -275,7 +303,28 @@ __global__ void __launch_bounds__(kThreads, 1) xbf_gemm_kernel(const GemmParams 
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (warp == 0) tc::tmem_dealloc(tmem, kTN);
+    if (warp == 0) tc::tmem_dealloc(tmem, MB * kTN);
+}
+
+__global__ void __launch_bounds__(kThreads, 1) xbf_gemm_kernel(const GemmParams p) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) GemmBars bar;
+    const int per = (p.mblk + 1) / 2;                         // CTAs of a pixel block whose row blocks go in twos
+    const int b = blockIdx.x, rest = b - p.dbl * per;
+    const int nb = rest < 0 ? b / per : p.dbl + rest / p.mblk;
+    const int mb = rest < 0 ? 2 * (b % per) : rest % p.mblk;
+    if (rest < 0 && mb + 1 < p.mblk) gemm_tile<2>(p, smem, bar, mb, nb);
+    else gemm_tile<1>(p, smem, bar, mb, nb);
+}
+
+// Pixel blocks whose row blocks go in twos: all that fill whole waves of CTAs, and
+// the others too unless their row blocks make one wave one by one.  A k block takes
+// the shared memory (128 bytes a cycle: copies in, operand reads) 768 cycles for one
+// row block and 1,280 for two.
+inline int xbf_double_blocks(int mblk, int npixblk, int sms) {
+    const int per = (mblk + 1) / 2;
+    const int dbl = (int)((long long)npixblk * per / sms * sms / per);
+    return (long long)(npixblk - dbl) * mblk <= sms ? dbl : npixblk;
 }
 
 }  // namespace
@@ -437,8 +486,12 @@ extern "C" hai_status hai_xbf_station_image(hai_ctx *ctx, const hai_xbf_layout *
     gp.npix = (int)npix;
     gp.accumulate = accumulate;
     gp.status = ctx->d_status;
+    gp.mblk = (M + kTM - 1) / kTM;
+    const int npb = (int)(npix / kTN);
+    gp.dbl = xbf_double_blocks(gp.mblk, npb, ctx->num_sms);
+    const int ctas = gp.dbl * ((gp.mblk + 1) / 2) + (npb - gp.dbl) * gp.mblk;
     const int pidx = prof_begin(ctx, st);
-    xbf_gemm_kernel<<<dim3((M + kTM - 1) / kTM, (unsigned)(npix / kTN)), kThreads, kSmem, st>>>(gp);
+    xbf_gemm_kernel<<<ctas, kThreads, kSmem, st>>>(gp);
     prof_end(ctx, pidx, st);
     prof_count(ctx, 2);
     HAI_CUDA_TRY(cudaGetLastError());
