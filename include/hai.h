@@ -432,7 +432,7 @@ hai_status hai_xfft_image(hai_ctx *ctx, const hai_layout *layout, const int32_t 
  *   grid  device float complex [C][P][P][N][N][2], 8-byte aligned; lag d at
  *         cell (dx mod N, dy mod N) of the row-major plane (zero lag at
  *         (0, 0)); overwritten.  YX is conj(XY) mirrored.
- * N a power of two in [16, 512] (else HAI_ERR_UNSUPPORTED).  FP32 radix-2
+ * N a power of two in [16, 512] (else HAI_ERR_UNSUPPORTED).  FP32
  * transforms; no scratch memory. */
 hai_status hai_fft_correlate(hai_ctx *ctx, const float *img, int C, int N, int P, float *grid, void *stream);
 
@@ -487,8 +487,8 @@ typedef struct hai_vis_layout hai_vis_layout;
  * steering phasors exp(+2 pi i s_k.(r_m - r_n) / lambda), computed in FP64 on
  * the GPU and stored in FP32.  Pairs whose footprint, or its mirror's, leaves
  * [-N/2, N/2 - 1]^2 are dropped (hai_vis_layout_offgrid counts them).
- * HAI_ERR_UNSUPPORTED if the uv window of the kept pairs does not fit in
- * shared memory or n_pol != 2. */
+ * HAI_ERR_UNSUPPORTED if n_pol != 2 or the station pairs' footprints exceed
+ * 2^28. */
 hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_desc *desc, hai_vis_layout **out);
 void hai_vis_layout_destroy(hai_vis_layout *layout);
 /* Station pairs (unordered, autos never) dropped off the grid, per image. */
@@ -502,7 +502,8 @@ hai_status hai_vis_layout_offgrid(const hai_vis_layout *layout, long long *n_off
  *        autos must have real XX and YY and YX = conj(XY): the XX and YY
  *        images are real and are computed together as one complex FFT.
  *   img  device float [K][C][4][N][N]: XX, YY, Re XY, Im XY (overwritten; the
- *        planes also serve as the gridding scratch)
+ *        grids are built in the planes: no scratch).  Every cell sums its pairs
+ *        in a fixed order, so results are deterministic.
  * Phase centre at pixel (N/2, N/2); pixel l looks along s_k + (l - N/2) *
  * lambda / (N cell). */
 hai_status hai_xfft_station_image(hai_ctx *ctx, const hai_vis_layout *layout, const int32_t *vis, int C, float *img,
