@@ -18,7 +18,8 @@
 //           A1[field][k block] = 128 rows y x 64 (x, re/im);
 //   stage1: H[y][l_x] = sum_x G[y][x] W'[x][l_x]: persistent CTAs over
 //           contiguous ranges of (l_x block, field) tiles, the l_x block's DFT
-//           operand resident in shared memory, A1 streamed by bulk copies,
+//           operand resident in shared memory (W1 is halved for boxes of more than
+//           128 columns, so that theirs fits), A1 streamed by bulk copies,
 //           tcgen05.mma M = 128 (y), N = 2 W1 (re, im of W1 l_x), accumulator
 //           double-buffered in TMEM; the epilogue stores H (16-bit),
 //           transposed, into the stage-2 operand:
@@ -37,7 +38,8 @@
 //   fixup:  adds the slots of every split item to the image in CTA order
 //           (deterministic: the same order on every run).
 // W1 = W2 = 128 (MMA N = 256) for plain operands, 64 (N = 128) for split ones
-// (the hi and lo DFT operands then fit shared memory together).
+// (the hi and lo DFT operands then fit shared memory together); W1 = 64 and 32
+// for wide boxes.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -56,7 +58,7 @@ constexpr uint32_t kMKs = 2048;          // MN-major (128 rows): K-group stride
 constexpr uint32_t kMMN = 128;           // MN-major: MN-group stride
 constexpr uint32_t kTile16 = 16384;      // 128 rows x 64 K x 2 bytes
 constexpr int kKb2 = 4;                  // k blocks of stage 2 (box rows padded to 128: 2 x 128 / 64)
-constexpr int kMaxKb1 = 4;               // k blocks of stage 1 (box <= 128 columns)
+constexpr int kMaxKb1 = 4;               // k blocks of stage 1 for boxes of <= 128 columns; up to 8 for wide ones
 
 struct BigGeo {
     int N, P, bx, by;            // grid, pols, box (cells)
@@ -383,6 +385,9 @@ __global__ void __launch_bounds__(kGridThreads) big_grid_dense_kernel(
 }
 
 // ------------------------------------------------------------------ stage 1
+// l_x values per tile: wide boxes (more k blocks than kMaxKb1) take half as many.
+__host__ __device__ constexpr int s1_width(bool split, bool wide) { return (split ? 64 : 128) / (wide ? 2 : 1); }
+
 struct S1Params {
     const uint8_t *a1, *a1lo;    // A1 (hi, lo)
     const uint8_t *b1, *b1lo;    // DFT operand (hi, lo): [l_x block][k block] tiles
@@ -395,18 +400,24 @@ struct S1Params {
 
 constexpr int kS1Threads = 640;             // warp 0 loads, warp 1 MMA, warps 4-19 epilogue
 
-template <bool BF, bool SP>
+// WIDE: boxes of 129 to 256 columns (5 to 8 k blocks), tiles of half as many l_x:
+// the resident operand takes at most the shared memory of the other form's.
+template <bool BF, bool SP, bool WIDE>
 __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p) {
     using V = Var<SP>;
+    constexpr int kW = s1_width(SP, WIDE), kNM = 2 * kW;             // l_x per tile, MMA N
+    constexpr uint32_t kBTile = (uint32_t)kNM * 128u;                 // one k block of an operand part
+    constexpr uint32_t kBPart = (WIDE ? 2 : 1) * kMaxKb1 * kBTile;    // the most an operand part takes
+    static_assert(kBPart == kMaxKb1 * V::BTile && kNM <= V::NM, "shared memory, TMEM");
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[V::S1Stages], empty[V::S1Stages], dfull[2], dempty[2], bfull;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const BigGeo g = p.g;
-    constexpr uint32_t kIdesc = tc::idesc_f16_as(BF, 128, V::NM, 0, 0);
-    const uint32_t bpart = (uint32_t)g.kb1 * V::BTile;                 // one DFT operand part of a block
-    uint8_t *sB = smem;                                                 // [part][kb1][BTile]
-    uint8_t *sA0 = smem + (size_t)kMaxKb1 * V::BTile * V::Parts;       // ring [stage][part][16 KB]
+    constexpr uint32_t kIdesc = tc::idesc_f16_as(BF, 128, kNM, 0, 0);
+    const uint32_t bpart = (uint32_t)g.kb1 * kBTile;                   // one DFT operand part of a block
+    uint8_t *sB = smem;                                                 // [part][kb1][kBTile]
+    uint8_t *sA0 = smem + (size_t)kBPart * V::Parts;                    // ring [stage][part][16 KB]
     if (tid == 0) {
         for (int s = 0; s < V::S1Stages; s++) {
             tc::mbar_init(&full[s], 1);
@@ -424,7 +435,6 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = tslot;
-    const int lbs = g.N / V::W;
     const long long nf = p.nfield;
     // contiguous tile range of this CTA; tiles are (l_x block, field), field fastest
     const long long r0 = p.ntiles * blockIdx.x / gridDim.x, r1 = p.ntiles * (blockIdx.x + 1) / gridDim.x;
@@ -443,7 +453,7 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
                     tc::mbar_arrive_expect_tx(&bfull, bpart * V::Parts);
                     for (int part = 0; part < V::Parts; part++) {
                         const uint8_t *src = (part ? p.b1lo : p.b1) + (size_t)lb * bpart;
-                        tc::bulk_g2s(sB + (size_t)part * kMaxKb1 * V::BTile, src, bpart, &bfull);
+                        tc::bulk_g2s(sB + (size_t)part * kBPart, src, bpart, &bfull);
                     }
                     cur_lb = lb;
                 }
@@ -479,13 +489,13 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
                 const int b = (int)(gt & 1);
                 if (gt >= 2) tc::mbar_wait(&dempty[b], (uint32_t)(((gt >> 1) - 1) & 1), p.status);
                 tc::fence_after();
-                const uint32_t d = tmem + (uint32_t)b * V::NM;
+                const uint32_t d = tmem + (uint32_t)b * kNM;
                 for (int kb = 0; kb < g.kb1; kb++, gs++) {
                     const int s = (int)(gs % V::S1Stages);
                     // bulk-copied stage: no tcgen05 fence needed (see stage 2)
                     tc::mbar_wait(&full[s], (uint32_t)((gs / V::S1Stages) & 1), p.status);
                     const uint32_t a = tc::smem_u32(sA0 + (size_t)s * V::AStage);
-                    const uint32_t bq = tc::smem_u32(sB + (size_t)kb * V::BTile);
+                    const uint32_t bq = tc::smem_u32(sB + (size_t)kb * kBTile);
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
                         const uint32_t acc0 = (kb > 0 || j > 0) ? 1u : 0u;
@@ -494,7 +504,7 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
                         tc::mma_f16(d, da, db, kIdesc, acc0);
                         if constexpr (SP) {
                             const uint64_t dal = tc::desc(a + kTile16 + j * 2 * kKBytes, kKBytes, kKMN);
-                            const uint64_t dbl = tc::desc(bq + kMaxKb1 * V::BTile + j * 2 * kKBytes, kKBytes, kKMN);
+                            const uint64_t dbl = tc::desc(bq + kBPart + j * 2 * kKBytes, kKBytes, kKMN);
                             tc::mma_f16(d, da, dbl, kIdesc, 1u);
                             tc::mma_f16(d, dal, db, kIdesc, 1u);
                         }
@@ -510,7 +520,7 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
         // re/im
         const int q = warp & 3, y = q * 32 + lane, h = (warp - 4) >> 2;
         const int kb2 = (2 * y) / 64, kk = (2 * y) % 64;   // K of the real part; imag at kk + 1
-        constexpr int kChunks = V::W / 64;                   // 16 l_x per chunk, per quarter
+        constexpr int kChunks = kW / 16, kEach = (kChunks + 3) / 4;   // 16 l_x per chunk; per quarter
         long long gt = 0;
         for (long long tile = r0; tile < r1; tile++, gt++) {
             const int b = (int)(gt & 1);
@@ -524,13 +534,13 @@ __global__ void __launch_bounds__(kS1Threads, 1) big_s1_kernel(const S1Params p)
             __syncwarp();
             tc::fence_after();
 #pragma unroll 1
-            for (int ch = kChunks * h; ch < kChunks * h + kChunks; ch++) {
+            for (int ch = kEach * h; ch < min(kChunks, kEach * (h + 1)); ch++) {
                 uint32_t rr[16], ri[16];
-                const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * V::NM + (uint32_t)(16 * ch);
+                const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * kNM + (uint32_t)(16 * ch);
                 tc::tmem_ld16(t0, rr);
-                tc::tmem_ld16(t0 + V::W, ri);
+                tc::tmem_ld16(t0 + kW, ri);
                 tc::tmem_wait_ld();
-                const int lx = lb * V::W + 16 * ch;             // first l_x of the chunk
+                const int lx = lb * kW + 16 * ch;             // first l_x of the chunk
                 const int lxb = lx / 64, lx64 = lx % 64;
                 const size_t toff = (((size_t)ct * g.lb2 + lxb) * kKb2 + kb2) * kTile16;
                 // rows (l_x, pol): m = (l_x >> 4) 32 + pol 16 + (l_x & 15)
@@ -931,7 +941,9 @@ hai_status launch_variant(const hai_layout *L, const int8_t *volt, int C, int T,
         return hai_fail(HAI_ERR_UNSUPPORTED, "epic tensor cores (large grid): shared memory");
     HAI_CUDA_TRY(hai_allow_dyn_smem(big_grid_smem_kernel<BF, SP>, ctx->smem_optin));
     HAI_CUDA_TRY(hai_allow_dyn_smem(big_grid_dense_kernel<BF, SP>, ctx->smem_optin));
-    HAI_CUDA_TRY(hai_allow_dyn_smem(big_s1_kernel<BF, SP>, ctx->smem_optin));
+    const bool wide = g.kb1 > kMaxKb1;
+    const auto stage1 = wide ? big_s1_kernel<BF, SP, true> : big_s1_kernel<BF, SP, false>;
+    HAI_CUDA_TRY(hai_allow_dyn_smem(stage1, ctx->smem_optin));
     HAI_CUDA_TRY(hai_allow_dyn_smem(big_s2_kernel<BF, SP>, ctx->smem_optin));
     // the scratch holds big_batch (channel, sample) pairs of plain operands,
     // half as many split ones: channels in chunks of at most that many, and
@@ -981,9 +993,9 @@ hai_status launch_variant(const hai_layout *L, const int8_t *volt, int C, int T,
         p1.a2lo = a2lo;
         p1.g = g;
         p1.nfield = nfield;
-        p1.ntiles = nfield * (g.N / V::W);
+        p1.ntiles = nfield * (g.N / s1_width(SP, wide));
         p1.status = ctx->d_status;
-        big_s1_kernel<BF, SP><<<(unsigned)std::min<long long>(p1.ntiles, G1), kS1Threads, V::S1Smem, st>>>(p1);
+        stage1<<<(unsigned)std::min<long long>(p1.ntiles, G1), kS1Threads, V::S1Smem, st>>>(p1);
         S2Params p2;
         p2.a2 = a2;
         p2.a2lo = a2lo;
@@ -1054,12 +1066,12 @@ hai_status epic_big_prepare(hai_layout *L) {
     size_t op_bytes = 0;
     for (int vi = 0; vi < 4; vi++) {
         const bool bf = vi & 1, sp = vi >= 2;
-        const int w = sp ? 64 : 128;
+        const int w1 = s1_width(sp, g.kb1 > kMaxKb1), w2 = sp ? 64 : 128;
         for (int stage = 0; stage < 2; stage++)
             for (int part = 0; part < 2; part++) {
                 ops.emplace_back();
                 if ((part && !sp) || (split_only && !sp)) continue;
-                dft_operand(g.N, stage == 0 ? g.kb1 * 32 : 128, w, bf, part, ops.back());
+                dft_operand(g.N, stage == 0 ? g.kb1 * 32 : 128, stage == 0 ? w1 : w2, bf, part, ops.back());
                 op_bytes += (ops.back().size() * 2 + 1023) & ~(size_t)1023;
             }
     }
