@@ -22,14 +22,15 @@
 // grid.  The two complex grids are built in the caller's image planes
 // [XX, YY, Re XY, Im XY] (as split re / im planes), which the FFT then
 // transforms in place: no scratch memory.  Gridding runs over tiles of the uv
-// grid with a thread per cell, the pairs binned to tiles on the host, and
-// writes its cells with the (-1)^(u+v) checkerboard that puts the phase
+// grid with threads per cell, the pairs binned to tiles on the host and listed
+// per cell on the GPU when the layout is made, and writes its cells with the (-1)^(u+v) checkerboard that puts the phase
 // centre at pixel (N/2, N/2).  The FFTs hold their lines in registers
 // (fft_line.cuh).
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "fft_line.cuh"
@@ -37,13 +38,13 @@
 
 namespace {
 
-// Tiles of the periodic uv grid (x = u mod N, y = v mod N), 16 x 16 cells with a
-// thread per cell.  The unit of gridding work is a tile and its mirror: tile t
-// along an axis holds the lower corners 16 t .. 16 t + 15, whose mirrors' lower
-// corners fall in tile -t - 1, so that a pair's visibilities are read once for
-// both of its footprints.
+// Tiles of the periodic uv grid (x = u mod N, y = v mod N), 16 x 16 cells.  The
+// unit of gridding work is a tile and its mirror: tile t along an axis holds the
+// lower corners 16 t .. 16 t + 15, whose mirrors' lower corners fall in tile
+// -t - 1, so that a pair's visibilities are read once for both of its footprints.
 constexpr int kTile = 16, kTcells = kTile * kTile;
-constexpr int kGridThreads = 2 * kTcells;         // the tile's cells, then the mirror tile's
+constexpr int kUcells = 2 * kTcells;              // cells of a unit: the tile's, then the mirror tile's
+constexpr int kGridThreads = kUcells;
 constexpr int kGridWarps = kGridThreads / 32;
 constexpr int kImgs = 4;                          // images (beam, channel) a CTA grids together
 constexpr int kFoot = 512;                        // pairs staged at a time
@@ -52,8 +53,9 @@ constexpr int kFootRow = kFoot + 4;               // float4 per staged row: dire
 // One chunk of a unit's pairs and, per warp, its gather entries: slot k of lane
 // l at entry base[w] + 32 k + l (zero weights pad the shorter lists).
 struct TileChunk {
-    int32_t foot, nfoot;
-    int32_t base[kGridWarps + 1];
+    long long foot;
+    int32_t nfoot, unit;
+    long long base[kGridWarps + 1];
 };
 struct TileEnt {
     float w;             // bilinear weight
@@ -63,6 +65,17 @@ struct TileEnt {
 struct TileUnit {
     int32_t tile, mirror, chunk;
 };
+// A pair in a unit's list: lower corners of its footprint and of its mirror's
+// (periodic grid), and the fractions; mfu < 0: no mirror (an auto).
+struct FootRec {
+    uint8_t x, y, mx, my;
+    float fu, fv, mfu, mfv;
+};
+static_assert(sizeof(FootRec) == 20, "copied by words");
+
+__host__ __device__ __forceinline__ float bilinear(int dx, int dy, float fu, float fv) {
+    return (dx ? fu : 1.f - fu) * (dy ? fv : 1.f - fv);
+}
 
 __device__ __forceinline__ void pair_of(long long bl, int &m, int &n) {
     int a = (int)((sqrt(8.0 * (double)bl + 1.0) - 1.0) * 0.5);
@@ -93,6 +106,123 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// ---- The gather lists, made once per layout (a CTA per chunk, a thread per cell
+// or list).  Each thread compares its cell with every pair of the chunk, so the
+// lists are in pair order whatever the threads' timing.  By the host, in passes
+// over the pairs, they took 9 ms for 256 stations and 562 ms for 2,048; here, with
+// the binning, 1 and 43 ms.
+__device__ __forceinline__ FootRec foot_rec(long long pair, const double *__restrict__ pos, double cell, int N) {
+    int m, n;
+    pair_of(pair, m, n);
+    // the host's operations (nothing to contract): the same corners
+    const double du = (pos[2 * m] - pos[2 * n]) / cell, dv = (pos[2 * m + 1] - pos[2 * n + 1]) / cell;
+    const double a = floor(du), b = floor(dv), ma = floor(-du), mb = floor(-dv);
+    FootRec r;
+    r.x = (uint8_t)((int)a & (N - 1));
+    r.y = (uint8_t)((int)b & (N - 1));
+    r.mx = (uint8_t)((int)ma & (N - 1));
+    r.my = (uint8_t)((int)mb & (N - 1));
+    r.fu = (float)(du - a);
+    r.fv = (float)(dv - b);
+    r.mfu = m == n ? -1.f : (float)(-du - ma);
+    r.mfv = (float)(-dv - mb);
+    return r;
+}
+__global__ void foot_rec_kernel(const uint32_t *__restrict__ foot, long long nfoot, const double *__restrict__ pos, double cell,
+                                int N, FootRec *__restrict__ recs) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nfoot) recs[i] = foot_rec(foot[i], pos, cell, N);
+}
+
+__device__ __forceinline__ bool unit_cell(const TileUnit &u, int cell, int N, int &X, int &Y) {
+    const int t = cell < kTcells ? u.tile : u.mirror, c = cell % kTcells;
+    X = t % (N / kTile) * kTile + c % kTile;
+    Y = t / (N / kTile) * kTile + c / kTile;
+    return t >= 0;
+}
+
+// f(weight, slot) for the entries of cell (X, Y) from the n staged pairs
+template <typename F>
+__device__ __forceinline__ void each_entry(const FootRec *rec, int n, int N, int X, int Y, F &&f) {
+    for (int i = 0; i < n; i++) {
+        const FootRec r = rec[i];
+        const int dx = (X - r.x) & (N - 1), dy = (Y - r.y) & (N - 1);
+        if (dx < 2 && dy < 2) {
+            const float w = bilinear(dx, dy, r.fu, r.fv);
+            if (w != 0.f) f(w, i);
+        }
+        const int mx = (X - r.mx) & (N - 1), my = (Y - r.my) & (N - 1);
+        if (mx < 2 && my < 2 && r.mfu >= 0.f) {
+            const float w = bilinear(mx, my, r.mfu, r.mfv);
+            if (w != 0.f) f(w, i + kFootRow);
+        }
+    }
+}
+
+__device__ __forceinline__ int stage_recs(const TileChunk &ch, const FootRec *recs, FootRec *rec) {
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(recs + ch.foot);
+    uint32_t *dst = reinterpret_cast<uint32_t *>(rec);
+    for (int i = threadIdx.x; i < ch.nfoot * (int)(sizeof(FootRec) / 4); i += blockDim.x) dst[i] = src[i];
+    __syncthreads();
+    return ch.nfoot;
+}
+
+// entries of every cell of a unit: total[unit][kUcells]
+__global__ void __launch_bounds__(kUcells) tile_total_kernel(const TileChunk *__restrict__ chunks,
+                                                            const TileUnit *__restrict__ unit,
+                                                            const FootRec *__restrict__ recs, int N, int *__restrict__ total) {
+    __shared__ FootRec rec[kFoot];
+    const TileChunk &ch = chunks[blockIdx.x];
+    const int nf = stage_recs(ch, recs, rec), cell = threadIdx.x;
+    int X, Y, n = 0;
+    if (!unit_cell(unit[ch.unit], cell, N, X, Y)) return;
+    each_entry(rec, nf, N, X, Y, [&](float, int) { n++; });
+    if (n) atomicAdd(&total[(size_t)ch.unit * kUcells + cell], n);
+}
+
+// Threads of a unit's cells, longest lists first (so that a warp's lanes end
+// together): lists[unit][thread] = cell (or kUcells: none), cells[unit][cell] =
+// its thread.
+__global__ void __launch_bounds__(kUcells) tile_assign_kernel(const int *__restrict__ total, uint32_t *__restrict__ lists,
+                                                             uint32_t *__restrict__ cells) {
+    __shared__ int load[kUcells];
+    const size_t o = (size_t)blockIdx.x * kUcells;
+    const int cell = threadIdx.x, mine = total[o + cell];
+    load[cell] = mine;
+    __syncthreads();
+    int first = 0;
+    for (int c = 0; c < kUcells; c++) first += load[c] > mine || (load[c] == mine && c < cell);
+    lists[o + first] = cell;
+    cells[o + cell] = first;
+}
+
+// FILL false: the longest list of every warp, slots[chunk][warp]; true: the
+// entries at the chunk's bases, padded to that length.
+template <bool FILL>
+__global__ void __launch_bounds__(kGridThreads) tile_lists_kernel(const TileChunk *__restrict__ chunks,
+                                                                 const TileUnit *__restrict__ unit,
+                                                                 const FootRec *__restrict__ recs, int N,
+                                                                 const uint32_t *__restrict__ lists,
+                                                                 int *__restrict__ slots, TileEnt *__restrict__ ent) {
+    __shared__ FootRec rec[kFoot];
+    const TileChunk &ch = chunks[blockIdx.x];
+    const int nf = stage_recs(ch, recs, rec), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    TileEnt *dst = FILL ? ent + ch.base[warp] + lane : nullptr;
+    int X, Y, n = 0;
+    if (unit_cell(unit[ch.unit], lists[(size_t)ch.unit * kGridThreads + threadIdx.x], N, X, Y))
+        each_entry(rec, nf, N, X, Y, [&](float w, int slot) {
+            if (FILL) dst[32ll * n] = TileEnt{w, slot};
+            n++;
+        });
+    if (FILL) {
+        const int most = (int)((ch.base[warp + 1] - ch.base[warp]) / 32);
+        for (; n < most; n++) dst[32ll * n] = TileEnt{0.f, 0};
+    } else {
+        n = __reduce_max_sync(0xffffffffu, n);
+        if (lane == 0) slots[(size_t)blockIdx.x * kGridWarps + warp] = n;
+    }
+}
+
 // G_XX + i G_YY into planes 0 / 1 and G_XY into planes 2 / 3 of kImgs images per
 // CTA, one tile of the grid and its mirror, with the checkerboard.  The unit's
 // pairs are phased once into shared memory, a chunk at a time, as the value of
@@ -116,7 +246,7 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
 template <bool VEC>
 __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
     const int32_t *__restrict__ vis, const uint32_t *__restrict__ foot, const TileEnt *__restrict__ ent,
-    const TileChunk *__restrict__ chunks, const TileUnit *__restrict__ unit, const uint8_t *__restrict__ cell_of,
+    const TileChunk *__restrict__ chunks, const TileUnit *__restrict__ unit, const uint32_t *__restrict__ cell_tab,
     int nunit, const float2 *__restrict__ phasor, int C, int images, long long nbl, int N, float *__restrict__ img) {
     extern __shared__ __align__(16) float4 stage[];     // [kImgs][2][kFootRow]; at the end [kImgs][4][512] floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -130,7 +260,8 @@ __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
     const int q0 = unit[o].chunk, q1 = unit[o + 1].chunk;
     for (int q = q0; q < q1; q++) {
         const TileChunk *ch = chunks + q;
-        const int f0 = ch->foot, nf = ch->nfoot;
+        const long long f0 = ch->foot;
+        const int nf = ch->nfoot;
         if (q > q0) __syncthreads();                    // the last chunk's gather is done
         // whole warps stay in the loop for the exchange
         for (int fw = (tid >> 1) & ~15; fw < nf; fw += kGridThreads / 2) {
@@ -162,10 +293,10 @@ __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
             }
         }
         __syncthreads();
-        const int e1 = ch->base[warp + 1];
+        const TileEnt *e1 = ent + ch->base[warp + 1];
 #pragma unroll 2
-        for (int e = ch->base[warp] + lane; e < e1; e += 32) {
-            const float2 x = __ldg(reinterpret_cast<const float2 *>(ent) + e);
+        for (const TileEnt *e = ent + ch->base[warp] + lane; e < e1; e += 32) {
+            const float2 x = __ldg(reinterpret_cast<const float2 *>(e));
             const int slot = __float_as_int(x.y);
 #pragma unroll
             for (int i = 0; i < kImgs; i++) {
@@ -177,32 +308,32 @@ __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
             }
         }
     }
-    // the cells back in row order, then out
-    const int side = tid / kTcells, tc = tid % kTcells;
+    // the sums back in row order of the cells, then out
     float *cells = reinterpret_cast<float *>(stage);
     if (q1 > q0) {
         __syncthreads();
-        const int cell = cell_of[(size_t)o * kGridThreads + tid];
-        const float sgn = ((cell ^ (cell / kTile)) & 1) ? -1.f : 1.f;     // tiles start on even cells
 #pragma unroll
         for (int i = 0; i < kImgs; i++) {
-            float *d = cells + (size_t)i * 4 * kGridThreads + side * kTcells + cell;
-            d[0] = sgn * acc[i].x;
-            d[kGridThreads] = sgn * acc[i].y;
-            d[2 * kGridThreads] = sgn * acc[i].z;
-            d[3 * kGridThreads] = sgn * acc[i].w;
+            float *d = cells + (size_t)i * 4 * kGridThreads + tid;
+            d[0] = acc[i].x;
+            d[kGridThreads] = acc[i].y;
+            d[2 * kGridThreads] = acc[i].z;
+            d[3 * kGridThreads] = acc[i].w;
         }
         __syncthreads();
     }
-    const int t = side ? unit[o].mirror : unit[o].tile;
+    const int t = tid < kTcells ? unit[o].tile : unit[o].mirror, tc = tid % kTcells;
     if (t < 0) return;
+    const int list = q1 > q0 ? (int)cell_tab[(size_t)o * kUcells + tid] : 0;
+    const float sgn = ((tc ^ (tc / kTile)) & 1) ? -1.f : 1.f;             // tiles start on even cells
     const int x = t % (N / kTile) * kTile + tc % kTile, y = t / (N / kTile) * kTile + tc / kTile;
 #pragma unroll
     for (int i = 0; i < kImgs; i++) {
         if (i0 + i >= images) break;
 #pragma unroll
         for (int p = 0; p < 4; p++)
-            img[(((size_t)(i0 + i) * 4 + p) * N + y) * N + x] = q1 > q0 ? cells[(i * 4 + p) * kGridThreads + tid] : 0.f;
+            img[(((size_t)(i0 + i) * 4 + p) * N + y) * N + x] =
+                q1 > q0 ? sgn * cells[(i * 4 + p) * kGridThreads + list] : 0.f;
     }
 }
 
@@ -364,7 +495,7 @@ struct hai_vis_layout {
     TileEnt *d_ent = nullptr;                // gather entries
     TileChunk *d_chunk = nullptr;
     TileUnit *d_unit = nullptr;              // units by pair count [nunit + 1]
-    uint8_t *d_cell = nullptr;               // [nunit][512] cell of each thread
+    uint32_t *d_cell = nullptr;              // [nunit][kUcells] thread of each cell
     int32_t *d_rows = nullptr;               // the written rows
     uint8_t *d_live = nullptr;               // [N] whether a row is written
     float2 *d_phasor = nullptr;
@@ -403,149 +534,82 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     // is recorded once in every unit (tile and mirror tile) that its footprint or
     // its mirror's touches (counted, then placed)
     const int nt = N / kTile;
-    auto mirror_of = [&](int t) { return (nt - 1 - t / nt) * nt + nt - 1 - t % nt; };
-    auto unit_of = [&](int t) { return std::min(t, mirror_of(t)); };
-    struct Hit {
-        int tile, mirrored, cx, cy;            // lower corner in the tile, -1 .. 15
-        float fu, fv;
+    std::vector<int32_t> unit_of((size_t)nt * nt), mirror_of((size_t)nt * nt);
+    for (int t = 0; t < nt * nt; t++) {
+        mirror_of[t] = (nt - 1 - t / nt) * nt + nt - 1 - t % nt;
+        unit_of[t] = std::min(t, mirror_of[t]);
+    }
+    struct Kept {
+        uint32_t pair;
+        uint8_t c[4];                          // lower corners: footprint x, y, its mirror's
     };
-    // the tiles that the two footprints of a pair touch
-    auto hits_of = [&](double du, double dv, bool autos, Hit (&h)[8]) {
-        int n = 0;
-        for (int m = 0; m < (autos ? 1 : 2); m++) {
-            const double u = m ? -du : du, v = m ? -dv : dv, fu = floor(u), fv = floor(v);
-            const int x = (((int)fu % N) + N) % N, y = (((int)fv % N) + N) % N;
-            const int x1 = (x + 1) % N, y1 = (y + 1) % N;
-            // with one tile a side the wrapped column is in the same tile: its own hit
+    // f(unit) once for every unit that the two footprints touch (an auto's mirror
+    // lies on the auto)
+    auto each_unit = [&](const Kept &r, auto &&f) {
+        int seen[8], n = 0;
+        for (int k = 0; k < 4; k += 2) {
+            const int x = r.c[k], y = r.c[k + 1];
             const int nx = x % kTile == kTile - 1 ? 2 : 1, ny = y % kTile == kTile - 1 ? 2 : 1;
             for (int j = 0; j < ny; j++)
-                for (int i = 0; i < nx; i++)
-                    h[n++] = Hit{((j ? y1 : y) / kTile) * nt + (i ? x1 : x) / kTile, m, i ? -1 : x % kTile,
-                                 j ? -1 : y % kTile, (float)(u - fu), (float)(v - fv)};
+                for (int i = 0; i < nx; i++) {
+                    const int u = unit_of[((y + j) & (N - 1)) / kTile * nt + ((x + i) & (N - 1)) / kTile];
+                    bool known = false;
+                    for (int q = 0; q < n; q++) known |= seen[q] == u;
+                    if (known) continue;
+                    seen[n++] = u;
+                    f(u);
+                }
         }
-        return n;
     };
-    long long dropped = 0;
-    auto each_pair = [&](auto &&f) {           // f(pair, hits, n) of the kept pairs
-        dropped = 0;
+    std::vector<Kept> kept;
+    std::vector<int32_t> rows;
+    std::vector<uint8_t> live(N, 0);
+    std::vector<uint32_t> foot;
+    std::vector<TileUnit> units;
+    std::vector<TileChunk> chunks;
+    try {
+        kept.reserve((size_t)nbl);
+        std::vector<long long> count((size_t)nt * nt, 0), fill((size_t)nt * nt, 0);
         long long bl = 0;
-        Hit h[8];
         for (int m = 0; m < S; m++)
             for (int n = 0; n <= m; n++, bl++) {
                 const double du = (d->pos_m[2 * m] - d->pos_m[2 * n]) / d->cell_m;
                 const double dv = (d->pos_m[2 * m + 1] - d->pos_m[2 * n + 1]) / d->cell_m;
-                if (!station_pair_kept(N, du, dv)) {
-                    dropped++;
-                    continue;
-                }
-                f((uint32_t)bl, h, hits_of(du, dv, m == n, h));    // an auto pair has no mirror
+                if (!station_pair_kept(N, du, dv)) continue;
+                auto corner = [&](double u) { return (uint8_t)((int)floor(u) & (N - 1)); };
+                const Kept r = {(uint32_t)bl, {corner(du), corner(dv), corner(-du), corner(-dv)}};
+                kept.push_back(r);
+                each_unit(r, [&](int u) { count[u]++; });
             }
-    };
-    auto each_unit = [&](const Hit *h, int n, auto &&f) {          // f(unit) once for every unit hit
-        for (int i = 0; i < n; i++) {
-            bool seen = false;
-            for (int j = 0; j < i; j++) seen |= unit_of(h[j].tile) == unit_of(h[i].tile);
-            if (!seen) f(unit_of(h[i].tile));
-        }
-    };
-    std::vector<int32_t> count((size_t)nt * nt, 0);
-    each_pair([&](uint32_t, const Hit *h, int n) { each_unit(h, n, [&](int u) { count[u]++; }); });
-    // written rows: those of a tile row (or its mirror's) with a pair in it
-    std::vector<uint8_t> live(N, 0);
-    std::vector<int32_t> rows, tiles;
-    for (int t = 0; t < nt * nt; t++)
-        if (count[t])
-            for (int r : {t / nt, nt - 1 - t / nt}) std::fill(live.begin() + r * kTile, live.begin() + (r + 1) * kTile, 1);
-    for (int y = 0; y < N; y++)
-        if (live[y]) rows.push_back(y);
-    for (int t = 0; t < nt * nt; t++)
-        if (unit_of(t) == t && live[t / nt * kTile]) tiles.push_back(t);
-    std::stable_sort(tiles.begin(), tiles.end(), [&](int x, int y) { return count[x] > count[y]; });
-    std::vector<long long> fill(count.size(), 0);
-    long long nfoot = 0;
-    for (int t : tiles) {
-        fill[t] = nfoot;
-        nfoot += count[t];
-    }
-    if (nfoot > 0x0fffffffll) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: too many station pairs");
-    std::vector<uint32_t> foot(std::max<long long>(1, nfoot));
-    struct Where {
-        int m, n;
-    };
-    std::vector<Where> who(foot.size());
-    {
-        long long bl = 0;
-        std::vector<Where> of((size_t)nbl);
-        for (int m = 0; m < S; m++)
-            for (int n = 0; n <= m; n++) of[bl++] = Where{m, n};
-        each_pair([&](uint32_t pair, const Hit *h, int n) {
-            each_unit(h, n, [&](int u) {
-                who[fill[u]] = of[pair];
-                foot[fill[u]++] = pair;
-            });
-        });
-    }
-    std::vector<TileEnt> ent;
-    std::vector<TileChunk> chunks;
-    std::vector<TileUnit> units;
-    std::vector<uint8_t> cell_of(tiles.size() * kGridThreads);
-    long long f0 = 0;
-    for (size_t o = 0; o < tiles.size(); o++) {
-        const long long f1 = f0 + count[tiles[o]];
-        const int ta = tiles[o], tb = mirror_of(ta) == ta ? -1 : mirror_of(ta);
-        units.push_back(TileUnit{ta, tb, (int32_t)chunks.size()});
-        // f(cell of the unit, weight, mirrored) of the non-zero cells of pair k in the unit
-        auto each_cell = [&](long long k, auto &&f) {
-            Hit h[8];
-            const int m = who[k].m, n = who[k].n;
-            const double du = (d->pos_m[2 * m] - d->pos_m[2 * n]) / d->cell_m;
-            const double dv = (d->pos_m[2 * m + 1] - d->pos_m[2 * n + 1]) / d->cell_m;
-            const int nh = hits_of(du, dv, m == n, h);
-            for (int i = 0; i < nh; i++) {
-                const Hit &r = h[i];
-                if (r.tile != ta && r.tile != tb) continue;
-                for (int t = 0; t < 4; t++) {
-                    const int x = r.cx + (t & 1), y = r.cy + (t >> 1);
-                    const float w = ((t & 1) ? r.fu : 1.f - r.fu) * ((t >> 1) ? r.fv : 1.f - r.fv);
-                    if (x >= 0 && x < kTile && y >= 0 && y < kTile && w != 0.f)
-                        f((r.tile == ta ? 0 : kTcells) + y * kTile + x, w, r.mirrored);
-                }
+        // written rows: those of a tile row (or its mirror's) with a pair in it
+        std::vector<int32_t> tiles;
+        for (int t = 0; t < nt * nt; t++)
+            if (count[t])
+                for (int r : {t / nt, nt - 1 - t / nt}) std::fill(live.begin() + r * kTile, live.begin() + (r + 1) * kTile, 1);
+        for (int y = 0; y < N; y++)
+            if (live[y]) rows.push_back(y);
+        for (int t = 0; t < nt * nt; t++)
+            if (unit_of[t] == t && live[t / nt * kTile]) tiles.push_back(t);
+        std::stable_sort(tiles.begin(), tiles.end(), [&](int x, int y) { return count[x] > count[y]; });
+        long long nfoot = 0;
+        for (int t : tiles) {
+            fill[t] = nfoot;
+            units.push_back(TileUnit{t, mirror_of[t] == t ? -1 : mirror_of[t], (int32_t)chunks.size()});
+            for (long long q = 0; q < count[t]; q += kFoot) {
+                TileChunk ch = {};
+                ch.foot = nfoot + q;
+                ch.nfoot = (int32_t)std::min<long long>(kFoot, count[t] - q);
+                ch.unit = (int32_t)units.size() - 1;
+                chunks.push_back(ch);
             }
-        };
-        int total[kGridThreads] = {}, order[kGridThreads], thread_of[kGridThreads];
-        for (long long k = f0; k < f1; k++) each_cell(k, [&](int c, float, int) { total[c]++; });
-        for (int side = 0; side < 2; side++) {
-            int *o0 = order + side * kTcells;
-            for (int c = 0; c < kTcells; c++) o0[c] = side * kTcells + c;
-            std::stable_sort(o0, o0 + kTcells, [&](int x, int y) { return total[x] > total[y]; });
+            nfoot += count[t];
         }
-        for (int i = 0; i < kGridThreads; i++) {
-            thread_of[order[i]] = i;
-            cell_of[o * kGridThreads + i] = (uint8_t)(order[i] % kTcells);
-        }
-        for (long long q = f0; q < f1; q += kFoot) {
-            TileChunk ch;
-            ch.foot = (int32_t)q;
-            ch.nfoot = (int32_t)std::min<long long>(kFoot, f1 - q);
-            int n[kGridThreads] = {};
-            for (int f = 0; f < ch.nfoot; f++) each_cell(q + f, [&](int c, float, int) { n[thread_of[c]]++; });
-            for (int w = 0; w < kGridWarps; w++) {
-                ch.base[w] = (int32_t)ent.size();
-                ent.resize(ent.size() + 32 * (size_t)*std::max_element(n + 32 * w, n + 32 * w + 32), TileEnt{0.f, 0});
-            }
-            ch.base[kGridWarps] = (int32_t)ent.size();
-            std::fill(n, n + kGridThreads, 0);
-            for (int f = 0; f < ch.nfoot; f++)
-                each_cell(q + f, [&](int c, float w, int mirrored) {
-                    const int i = thread_of[c];
-                    ent[ch.base[i / 32] + 32 * n[i]++ + i % 32] = TileEnt{w, mirrored * kFootRow + f};
-                });
-            chunks.push_back(ch);
-            if (ent.size() > 0x7fffffffull) return hai_fail(HAI_ERR_UNSUPPORTED, "hai_vis_layout_create: too many station pairs");
-        }
-        f0 = f1;
+        units.push_back(TileUnit{-1, -1, (int32_t)chunks.size()});
+        foot.resize((size_t)nfoot);
+        for (const Kept &r : kept) each_unit(r, [&](int u) { foot[fill[u]++] = r.pair; });
+    } catch (const std::bad_alloc &) {
+        return hai_fail(HAI_ERR_NO_MEMORY, "hai_vis_layout_create: host memory for the station pairs");
     }
-    units.push_back(TileUnit{-1, -1, (int32_t)chunks.size()});
     hai_vis_layout *L = new hai_vis_layout();
     L->ctx = ctx;
     L->S = S;
@@ -553,28 +617,60 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     L->P = d->n_pol;
     L->K = K;
     L->nbl = nbl;
-    L->n_offgrid = dropped;
-    L->nunit = (int)tiles.size();
+    L->n_offgrid = nbl - (long long)kept.size();
+    L->nunit = (int)units.size() - 1;
     L->nrow = (int)rows.size();
     double *d_pos = nullptr, *d_dir = nullptr;
     std::vector<double> dirs(2 * (size_t)K, 0.0);
     if (d->dir) std::copy(d->dir, d->dir + 2 * (size_t)K, dirs.begin());
     cudaError_t e = cudaSetDevice(ctx->device);
+    auto room = [&](auto *&dst, size_t n) {
+        if (e == cudaSuccess) e = cudaMalloc(&dst, sizeof(*dst) * n);
+    };
     auto put = [&](auto *&dst, const auto &src) {
-        if (e == cudaSuccess) e = cudaMalloc(&dst, sizeof(src[0]) * src.size());
+        room(dst, src.size());
         if (e == cudaSuccess) e = cudaMemcpy(dst, src.data(), sizeof(src[0]) * src.size(), cudaMemcpyHostToDevice);
     };
     put(L->d_foot, foot);
-    put(L->d_ent, ent);
     put(L->d_chunk, chunks);
     put(L->d_unit, units);
-    put(L->d_cell, cell_of);
     put(L->d_rows, rows);
     put(L->d_live, live);
-    if (e == cudaSuccess) e = cudaMalloc(&L->d_phasor, sizeof(float2) * (size_t)K * nbl);
-    if (e == cudaSuccess) e = cudaMalloc(&d_pos, sizeof(double) * 2 * S);
-    if (e == cudaSuccess) e = cudaMalloc(&d_dir, sizeof(double) * 2 * K);
+    room(d_pos, 2 * (size_t)S);
     if (e == cudaSuccess) e = cudaMemcpy(d_pos, d->pos_m, sizeof(double) * 2 * S, cudaMemcpyHostToDevice);
+    // the gather lists: sizes, then entries
+    const unsigned nchunk = (unsigned)chunks.size();
+    const size_t ncell = (size_t)L->nunit * kUcells, nslot = (size_t)nchunk * kGridWarps;
+    std::vector<int> slots(nslot);
+    uint32_t *d_tmp = nullptr;                 // entries per cell, cells by list, slots, records
+    room(d_tmp, 2 * ncell + nslot + foot.size() * (sizeof(FootRec) / 4));
+    room(L->d_cell, ncell);
+    if (e == cudaSuccess && nchunk) {
+        int *total = reinterpret_cast<int *>(d_tmp), *d_slots = reinterpret_cast<int *>(d_tmp + 2 * ncell);
+        uint32_t *list = d_tmp + ncell;
+        FootRec *rec = reinterpret_cast<FootRec *>(d_slots + nslot);
+        e = cudaMemset(total, 0, sizeof(int) * ncell);
+        foot_rec_kernel<<<(unsigned)((foot.size() + 255) / 256), 256>>>(L->d_foot, (long long)foot.size(), d_pos, d->cell_m, N, rec);
+        tile_total_kernel<<<nchunk, kUcells>>>(L->d_chunk, L->d_unit, rec, N, total);
+        tile_assign_kernel<<<(unsigned)L->nunit, kUcells>>>(total, list, L->d_cell);
+        tile_lists_kernel<false><<<nchunk, kGridThreads>>>(L->d_chunk, L->d_unit, rec, N, list, d_slots, nullptr);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpy(slots.data(), d_slots, sizeof(int) * nslot, cudaMemcpyDeviceToHost);
+        long long nent = 0;
+        for (unsigned q = 0; q < nchunk; q++)
+            for (int w = 0; w <= kGridWarps; w++) {
+                chunks[q].base[w] = nent;
+                if (w < kGridWarps) nent += 32ll * slots[(size_t)q * kGridWarps + w];
+            }
+        room(L->d_ent, (size_t)nent);
+        if (e == cudaSuccess) e = cudaMemcpy(L->d_chunk, chunks.data(), sizeof(TileChunk) * nchunk, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) {
+            tile_lists_kernel<true><<<nchunk, kGridThreads>>>(L->d_chunk, L->d_unit, rec, N, list, d_slots, L->d_ent);
+            e = cudaGetLastError();
+        }
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&L->d_phasor, sizeof(float2) * (size_t)K * nbl);
+    if (e == cudaSuccess) e = cudaMalloc(&d_dir, sizeof(double) * 2 * K);
     if (e == cudaSuccess) e = cudaMemcpy(d_dir, dirs.data(), sizeof(double) * 2 * K, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         const long long n = (long long)K * nbl;
@@ -582,6 +678,7 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    cudaFree(d_tmp);
     cudaFree(d_pos);
     cudaFree(d_dir);
     if (e != cudaSuccess) {
