@@ -23,9 +23,9 @@
 // [XX, YY, Re XY, Im XY] (as split re / im planes), which the FFT then
 // transforms in place: no scratch memory.  Gridding runs over tiles of the uv
 // grid with threads per cell, the pairs binned to tiles on the host and listed
-// per cell on the GPU when the layout is made, and writes its cells with the (-1)^(u+v) checkerboard that puts the phase
-// centre at pixel (N/2, N/2).  The FFTs hold their lines in registers
-// (fft_line.cuh).
+// per cell on the GPU when the layout is made, and writes its cells with the
+// (-1)^(u+v) checkerboard that puts the phase centre at pixel (N/2, N/2).  The
+// FFTs hold their lines in registers (fft_line.cuh).
 #include <math.h>
 #include <string.h>
 
@@ -46,7 +46,8 @@ constexpr int kTile = 16, kTcells = kTile * kTile;
 constexpr int kUcells = 2 * kTcells;              // cells of a unit: the tile's, then the mirror tile's
 constexpr int kGridThreads = kUcells;
 constexpr int kGridWarps = kGridThreads / 32;
-constexpr int kImgs = 4;                          // images (beam, channel) a CTA grids together
+constexpr int kImgs = 4;                          // images (beam, channel) a CTA grids together, at most
+constexpr int kCellLists = 64;                    // lists of one cell, at most
 constexpr int kFoot = 512;                        // pairs staged at a time
 constexpr int kFootRow = kFoot + 4;               // float4 per staged row: direct and mirrored values 4 banks apart
 
@@ -180,20 +181,48 @@ __global__ void __launch_bounds__(kUcells) tile_total_kernel(const TileChunk *__
     if (n) atomicAdd(&total[(size_t)ch.unit * kUcells + cell], n);
 }
 
-// Threads of a unit's cells, longest lists first (so that a warp's lanes end
-// together): lists[unit][thread] = cell (or kUcells: none), cells[unit][cell] =
-// its thread.
+// Lists of a unit's cells, a thread each: a cell without entries has none, one
+// with more entries than `load` has several, dealt in turn, for the smallest load
+// (of 8 or more) with which the unit's lists are at most its 512 threads.  Longest lists first,
+// so that a warp's lanes end together.  lists[unit][thread] = cell | part << 9 |
+// parts << 16 (0: none), cells[unit][cell] = first thread | parts << 16.
+//
+// A short array puts every pair on a few cells: with one thread a cell, 256
+// stations within 57 m (49 cells of 19 m, 128 images) took 4,370 us and 512 within
+// 270 m (32 images) 1,820, where shared-memory atomics had taken 1,118 and 915;
+// now 275 and 760 (whole calls).
 __global__ void __launch_bounds__(kUcells) tile_assign_kernel(const int *__restrict__ total, uint32_t *__restrict__ lists,
                                                              uint32_t *__restrict__ cells) {
-    __shared__ int load[kUcells];
+    __shared__ int2 cell_load[kUcells];                // entries per list, lists
+    __shared__ int need[32], most;                     // lists needed in each try; the largest cell
     const size_t o = (size_t)blockIdx.x * kUcells;
     const int cell = threadIdx.x, mine = total[o + cell];
-    load[cell] = mine;
+    if (cell < 32) need[cell] = 0;
+    if (cell == 0) most = 0;
+    lists[o + cell] = 0;
+    __syncthreads();
+    atomicMax(&most, mine);
+    __syncthreads();
+    auto lists_at = [&](int load) { return mine ? min((mine - 1) / load + 1, kCellLists) : 0; };
+    int hi = max(1, most), lo = min(8, hi);            // at hi a cell has one list
+    for (int k = 0; lo < hi; k++) {                    // the same in every thread; at most 31 halvings
+        const int mid = lo + (hi - lo) / 2;
+        const int n = __reduce_add_sync(0xffffffffu, lists_at(mid));
+        if ((cell & 31) == 0) atomicAdd(&need[k], n);
+        __syncthreads();
+        if (need[k] <= kUcells) hi = mid;
+        else lo = mid + 1;
+    }
+    const int parts = lists_at(hi), each = parts ? (mine - 1) / parts + 1 : 0;
+    cell_load[cell] = make_int2(each, parts);
     __syncthreads();
     int first = 0;
-    for (int c = 0; c < kUcells; c++) first += load[c] > mine || (load[c] == mine && c < cell);
-    lists[o + first] = cell;
-    cells[o + cell] = first;
+    for (int c = 0; c < kUcells; c++) {
+        const int2 x = cell_load[c];
+        if (x.x > each || (x.x == each && c < cell)) first += x.y;
+    }
+    for (int k = 0; k < parts; k++) lists[o + first + k] = cell | k << 9 | parts << 16;
+    cells[o + cell] = first | parts << 16;
 }
 
 // FILL false: the longest list of every warp, slots[chunk][warp]; true: the
@@ -208,9 +237,13 @@ __global__ void __launch_bounds__(kGridThreads) tile_lists_kernel(const TileChun
     const TileChunk &ch = chunks[blockIdx.x];
     const int nf = stage_recs(ch, recs, rec), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     TileEnt *dst = FILL ? ent + ch.base[warp] + lane : nullptr;
-    int X, Y, n = 0;
-    if (unit_cell(unit[ch.unit], lists[(size_t)ch.unit * kGridThreads + threadIdx.x], N, X, Y))
+    const uint32_t list = lists[(size_t)ch.unit * kGridThreads + threadIdx.x];
+    const int parts = list >> 16;
+    int X, Y, n = 0, turn = (list >> 9) & 127;         // entries of other lists before the next one of this
+    if (parts && unit_cell(unit[ch.unit], list & (kUcells - 1), N, X, Y))
         each_entry(rec, nf, N, X, Y, [&](float w, int slot) {
+            if (turn-- > 0) return;
+            turn = parts - 1;
             if (FILL) dst[32ll * n] = TileEnt{w, slot};
             n++;
         });
@@ -223,16 +256,18 @@ __global__ void __launch_bounds__(kGridThreads) tile_lists_kernel(const TileChun
     }
 }
 
-// G_XX + i G_YY into planes 0 / 1 and G_XY into planes 2 / 3 of kImgs images per
+// G_XX + i G_YY into planes 0 / 1 and G_XY into planes 2 / 3 of IMGS images per
 // CTA, one tile of the grid and its mirror, with the checkerboard.  The unit's
 // pairs are phased once into shared memory, a chunk at a time, as the value of
 // the pair (XX + i YY, XY) and that of its mirror (conj(XX) + i conj(YY),
-// conj(YX)), and every cell (thread) then adds its own list of them: no atomics,
-// and a fixed order, so the images are bit-reproducible.  Two lanes share a
+// conj(YX)), and every thread then adds one list of a cell of them; a cell's lists
+// are added in order at the end.  No atomics, and a fixed order, so the images are
+// bit-reproducible.  Two lanes share a
 // pair's 32-byte sector (XX, XY | YX, YY) and exchange XX for YY; one then holds
 // the pair's value and the other the mirror's.  The lists are the same for every
-// image: entries and phasors are read once per kImgs images; cells are dealt to
-// the lanes by list length, so a warp's lanes end together.  Units are the fast
+// image: entries and phasors are read once per IMGS images; lists are dealt to
+// the lanes by length, so a warp's lanes end together.  With one image a CTA (few
+// CTAs, each a long walk) a chunk's loads are issued before the last one's gather.  Units are the fast
 // grid index, so a group's visibilities (1 MB an image for 256 stations) come
 // from HBM once and from L2 for the neighbouring tiles.  Grid rows whose tiles
 // are all empty are left unwritten: the FFT passes do not read them.
@@ -243,63 +278,95 @@ __global__ void __launch_bounds__(kGridThreads) tile_lists_kernel(const TileChun
 // all planes; a lane per image with the cells in registers 798 us (32 lanes a
 // megabyte apart, 1.4 GB read from HBM); a tile at a time with a lane per
 // footprint's two 16-byte loads 616 us (32 lines a load); this form 511 us.
-template <bool VEC>
+template <bool VEC, int IMGS>
 __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
     const int32_t *__restrict__ vis, const uint32_t *__restrict__ foot, const TileEnt *__restrict__ ent,
     const TileChunk *__restrict__ chunks, const TileUnit *__restrict__ unit, const uint32_t *__restrict__ cell_tab,
     int nunit, const float2 *__restrict__ phasor, int C, int images, long long nbl, int N, float *__restrict__ img) {
-    extern __shared__ __align__(16) float4 stage[];     // [kImgs][2][kFootRow]; at the end [kImgs][4][512] floats
+    extern __shared__ __align__(16) float4 stage[];     // [IMGS][2][kFootRow]; at the end [IMGS][4][512] floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = blockIdx.x / nunit, o = blockIdx.x - grp * nunit;
-    const int i0 = grp * kImgs, i1 = min(i0 + kImgs, images) - 1;
+    const int i0 = grp * IMGS, i1 = min(i0 + IMGS, images) - 1;
     const bool same = i0 / C == i1 / C;                 // one beam: one phasor for all images
-    float4 acc[kImgs];
+    float4 acc[IMGS];
 #pragma unroll
-    for (int i = 0; i < kImgs; i++) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < IMGS; i++) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int half = lane & 1;                          // XX, XY or YX, YY
     const int q0 = unit[o].chunk, q1 = unit[o + 1].chunk;
+    constexpr int kPass = 2 * kFoot / kGridThreads;     // pairs a lane pair stages of a chunk
+    constexpr bool kAhead = IMGS == 1;                  // a chunk's loads issued before the last one's gather
+    struct Pair {
+        int4 x[IMGS];
+        float2 w[IMGS];
+    };
+    auto index = [&](int q, int p) -> size_t {
+        const TileChunk *ch = chunks + q;
+        return __ldg(foot + ch->foot + min(p * (kGridThreads / 2) + (tid >> 1), ch->nfoot - 1));
+    };
+    auto fetch = [&](size_t bl, Pair &r) {
+#pragma unroll
+        for (int i = 0; i < IMGS; i++) {
+            const int im = min(i0 + i, images - 1);
+            const int32_t *v = vis + ((size_t)im * nbl + bl) * 8 + 4 * half;
+            if (VEC) {
+                r.x[i] = __ldg(reinterpret_cast<const int4 *>(v));
+            } else {
+                const int2 a = __ldg(reinterpret_cast<const int2 *>(v)), b = __ldg(reinterpret_cast<const int2 *>(v) + 1);
+                r.x[i] = make_int4(a.x, a.y, b.x, b.y);
+            }
+            r.w[i] = i > 0 && same ? r.w[0] : __ldg(phasor + (size_t)(im / C) * nbl + bl);
+        }
+    };
+    auto put = [&](const Pair &r, int f, int nf) {
+#pragma unroll
+        for (int i = 0; i < IMGS; i++) {
+            const float2 u = cmulf(make_float2((float)r.x[i].x, (float)r.x[i].y), r.w[i]);      // XX or YX
+            const float2 v = cmulf(make_float2((float)r.x[i].z, (float)r.x[i].w), r.w[i]);      // XY or YY
+            const float sx = __shfl_xor_sync(0xffffffffu, half ? v.x : u.x, 1);
+            const float sy = __shfl_xor_sync(0xffffffffu, half ? v.y : u.y, 1);                 // YY or XX
+            if (f < nf)
+                stage[(i * 2 + half) * kFootRow + f] = half ? make_float4(sx + v.y, v.x - sy, u.x, -u.y)
+                                                            : make_float4(u.x - sy, u.y + sx, v.x, v.y);
+        }
+    };
+    Pair ahead[kAhead ? kPass : 1];
+    size_t next[kAhead ? kPass : 1];
+    if constexpr (kAhead)
+        if (q0 < q1)
+#pragma unroll
+            for (int p = 0; p < kPass; p++) {
+                fetch(index(q0, p), ahead[p]);
+                next[p] = index(min(q0 + 1, q1 - 1), p);
+            }
     for (int q = q0; q < q1; q++) {
         const TileChunk *ch = chunks + q;
-        const long long f0 = ch->foot;
         const int nf = ch->nfoot;
         if (q > q0) __syncthreads();                    // the last chunk's gather is done
-        // whole warps stay in the loop for the exchange
-        for (int fw = (tid >> 1) & ~15; fw < nf; fw += kGridThreads / 2) {
-            const int f = fw + (lane >> 1);
-            const size_t bl = __ldg(foot + f0 + min(f, nf - 1));
-            int4 x[kImgs];
-            float2 w[kImgs];
-#pragma unroll
-            for (int i = 0; i < kImgs; i++) {
-                const int im = min(i0 + i, images - 1);
-                const int32_t *v = vis + ((size_t)im * nbl + bl) * 8 + 4 * half;
-                if (VEC) {
-                    x[i] = __ldg(reinterpret_cast<const int4 *>(v));
-                } else {
-                    const int2 a = __ldg(reinterpret_cast<const int2 *>(v)), b = __ldg(reinterpret_cast<const int2 *>(v) + 1);
-                    x[i] = make_int4(a.x, a.y, b.x, b.y);
-                }
-                w[i] = i > 0 && same ? w[0] : __ldg(phasor + (size_t)(im / C) * nbl + bl);
+#pragma unroll (kAhead ? kPass : 1)
+        for (int p = 0; p < kPass; p++) {
+            const int f = p * (kGridThreads / 2) + (tid >> 1);
+            if constexpr (!kAhead) {
+                if (f - (lane >> 1) >= nf) break;       // whole warps, for the exchange
+                fetch(index(q, p), ahead[0]);
             }
-#pragma unroll
-            for (int i = 0; i < kImgs; i++) {
-                const float2 u = cmulf(make_float2((float)x[i].x, (float)x[i].y), w[i]);      // XX or YX
-                const float2 v = cmulf(make_float2((float)x[i].z, (float)x[i].w), w[i]);      // XY or YY
-                const float sx = __shfl_xor_sync(0xffffffffu, half ? v.x : u.x, 1);
-                const float sy = __shfl_xor_sync(0xffffffffu, half ? v.y : u.y, 1);           // YY or XX
-                if (f < nf)
-                    stage[(i * 2 + half) * kFootRow + f] = half ? make_float4(sx + v.y, v.x - sy, u.x, -u.y)
-                                                                : make_float4(u.x - sy, u.y + sx, v.x, v.y);
-            }
+            put(ahead[kAhead ? p : 0], f, nf);
         }
         __syncthreads();
-        const TileEnt *e1 = ent + ch->base[warp + 1];
-#pragma unroll 2
-        for (const TileEnt *e = ent + ch->base[warp] + lane; e < e1; e += 32) {
-            const float2 x = __ldg(reinterpret_cast<const float2 *>(e));
+        if constexpr (kAhead)
+            if (q + 1 < q1)
+#pragma unroll
+                for (int p = 0; p < kPass; p++) {
+                    fetch(next[p], ahead[p]);
+                    next[p] = index(min(q + 2, q1 - 1), p);
+                }
+        const float2 *el = reinterpret_cast<const float2 *>(ent + ch->base[warp]) + lane;
+        const int ne = (int)(ch->base[warp + 1] - ch->base[warp]);
+#pragma unroll (8 / IMGS)
+        for (int e = 0; e < ne; e += 32) {
+            const float2 x = __ldg(el + e);
             const int slot = __float_as_int(x.y);
 #pragma unroll
-            for (int i = 0; i < kImgs; i++) {
+            for (int i = 0; i < IMGS; i++) {
                 const float4 g = stage[i * 2 * kFootRow + slot];
                 acc[i].x = fmaf(x.x, g.x, acc[i].x);
                 acc[i].y = fmaf(x.x, g.y, acc[i].y);
@@ -313,7 +380,7 @@ __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
     if (q1 > q0) {
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < kImgs; i++) {
+        for (int i = 0; i < IMGS; i++) {
             float *d = cells + (size_t)i * 4 * kGridThreads + tid;
             d[0] = acc[i].x;
             d[kGridThreads] = acc[i].y;
@@ -324,16 +391,20 @@ __global__ void __launch_bounds__(kGridThreads, 2) station_grid_kernel(
     }
     const int t = tid < kTcells ? unit[o].tile : unit[o].mirror, tc = tid % kTcells;
     if (t < 0) return;
-    const int list = q1 > q0 ? (int)cell_tab[(size_t)o * kUcells + tid] : 0;
+    const uint32_t list = q1 > q0 ? cell_tab[(size_t)o * kUcells + tid] : 0u;
+    const int l0 = list & 0xffff, l1 = l0 + (int)(list >> 16);
     const float sgn = ((tc ^ (tc / kTile)) & 1) ? -1.f : 1.f;             // tiles start on even cells
     const int x = t % (N / kTile) * kTile + tc % kTile, y = t / (N / kTile) * kTile + tc / kTile;
+    float v[4 * IMGS];
 #pragma unroll
-    for (int i = 0; i < kImgs; i++) {
-        if (i0 + i >= images) break;
+    for (int k = 0; k < 4 * IMGS; k++) v[k] = l1 > l0 ? sgn * cells[k * kGridThreads + l0] : 0.f;
+    for (int l = l0 + 1; l < l1; l++)
 #pragma unroll
-        for (int p = 0; p < 4; p++)
-            img[(((size_t)(i0 + i) * 4 + p) * N + y) * N + x] =
-                q1 > q0 ? sgn * cells[(i * 4 + p) * kGridThreads + list] : 0.f;
+        for (int k = 0; k < 4 * IMGS; k++) v[k] += sgn * cells[k * kGridThreads + l];
+#pragma unroll
+    for (int k = 0; k < 4 * IMGS; k++) {
+        if (i0 + k / 4 >= images) break;
+        img[(((size_t)i0 * 4 + k) * N + y) * N + x] = v[k];
     }
 }
 
@@ -491,11 +562,12 @@ struct hai_vis_layout {
     long long nbl = 0;
     long long n_offgrid = 0;
     int nunit = 0, nrow = 0;                 // tile units in written rows; written rows
+    int nchunk = 0, most_chunks = 0;         // chunks of all units, of the largest
     uint32_t *d_foot = nullptr;              // stored pairs, unit after unit
     TileEnt *d_ent = nullptr;                // gather entries
     TileChunk *d_chunk = nullptr;
     TileUnit *d_unit = nullptr;              // units by pair count [nunit + 1]
-    uint32_t *d_cell = nullptr;              // [nunit][kUcells] thread of each cell
+    uint32_t *d_cell = nullptr;              // [nunit][kUcells] lists of each cell
     int32_t *d_rows = nullptr;               // the written rows
     uint8_t *d_live = nullptr;               // [N] whether a row is written
     float2 *d_phasor = nullptr;
@@ -619,6 +691,8 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     L->nbl = nbl;
     L->n_offgrid = nbl - (long long)kept.size();
     L->nunit = (int)units.size() - 1;
+    L->nchunk = (int)chunks.size();
+    L->most_chunks = L->nunit ? units[1].chunk : 0;      // the units are in order of their pairs
     L->nrow = (int)rows.size();
     double *d_pos = nullptr, *d_dir = nullptr;
     std::vector<double> dirs(2 * (size_t)K, 0.0);
@@ -642,7 +716,7 @@ extern "C" hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_d
     const unsigned nchunk = (unsigned)chunks.size();
     const size_t ncell = (size_t)L->nunit * kUcells, nslot = (size_t)nchunk * kGridWarps;
     std::vector<int> slots(nslot);
-    uint32_t *d_tmp = nullptr;                 // entries per cell, cells by list, slots, records
+    uint32_t *d_tmp = nullptr;                 // entries per cell, lists, slots, records
     room(d_tmp, 2 * ncell + nslot + foot.size() * (sizeof(FootRec) / 4));
     room(L->d_cell, ncell);
     if (e == cudaSuccess && nchunk) {
@@ -712,13 +786,19 @@ extern "C" hai_status hai_xfft_station_image(hai_ctx *ctx, const hai_vis_layout 
     HAI_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
     const int N = L->N, images = L->K * C;
-    const int groups = (images + kImgs - 1) / kImgs;
-    if ((long long)images * 2 > 0x7fffffffll || (long long)L->nunit * groups > 0x7fffffffll)
+    if ((long long)images * 2 > 0x7fffffffll || (long long)L->nunit * ((images + kImgs - 1) / kImgs) > 0x7fffffffll)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_station_image: too many images");
+    // images per CTA: four share a unit's entries and phasors; fewer when the walk
+    // over the largest unit is longer than what the work comes to per resident CTA
+    int imgs = kImgs;
+    while (imgs > 1 && 2ll * ctx->num_sms * L->most_chunks > (long long)L->nchunk * ((images + imgs - 1) / imgs)) imgs /= 2;
+    const bool vec = ((uintptr_t)vis & 15) == 0;
     const int pidx = prof_begin(ctx, st);
-    auto grid = (((uintptr_t)vis & 15) == 0) ? station_grid_kernel<true> : station_grid_kernel<false>;
+    const auto grid = imgs == 4   ? vec ? station_grid_kernel<true, 4> : station_grid_kernel<false, 4>
+                      : imgs == 2 ? vec ? station_grid_kernel<true, 2> : station_grid_kernel<false, 2>
+                                  : vec ? station_grid_kernel<true, 1> : station_grid_kernel<false, 1>;
     HAI_CUDA_TRY(hai_allow_dyn_smem(grid, ctx->smem_optin));
-    grid<<<(unsigned)(L->nunit * groups), kGridThreads, sizeof(float4) * kImgs * 2 * kFootRow, st>>>(
+    grid<<<(unsigned)(L->nunit * ((images + imgs - 1) / imgs)), kGridThreads, sizeof(float4) * imgs * 2 * kFootRow, st>>>(
         vis, L->d_foot, L->d_ent, L->d_chunk, L->d_unit, L->d_cell, L->nunit, L->d_phasor, C, images, L->nbl, N, img);
     prof_end(ctx, pidx, st);
     HAI_CUDA_TRY(cudaGetLastError());

@@ -1,5 +1,6 @@
 """Gather lists of the inter-station XFFT: units of several chunks against the
-FP64 oracle and bit for bit on repeat, and what creating a large layout costs."""
+FP64 oracle and bit for bit on repeat, what creating a large layout costs, and the time of a short
+array."""
 import time
 
 import numpy as np
@@ -68,3 +69,28 @@ def test_creating_a_large_layout_is_quick(hai):
         hai.hai_vis_layout_destroy(lay)
     hai.hai_destroy(ctx)
     assert best < 0.2
+
+
+def test_a_short_array_is_not_slow(hai):
+    """256 stations within 57 m, 128 images: every pair on 49 cells.  0.28 ms;
+    with one thread a cell 4.4 ms (by shared-memory atomics 1.1 ms)."""
+    rng = np.random.default_rng(2)
+    S, C, n = 256, 128, 256
+    pos = rng.uniform(-1.5, 1.5, (S, 2)) * 19.0
+    vis = torch.randint(-1000, 1000, (C, S * (S + 1) // 2, 2, 2, 2), device="cuda", dtype=torch.int32)
+    img = torch.empty((C, 4, n, n), device="cuda")
+    ctx = hai.hai_create(0)
+    lay = hai.hai_vis_layout_create(ctx, pos, 3.0, 19.0, n, None)
+    try:
+        best = float("inf")
+        for _ in range(10):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            hai.hai_xfft_station_image(ctx, lay, vis, C, img)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        assert best < 1.0
+    finally:
+        hai.hai_vis_layout_destroy(lay)
+        hai.hai_destroy(ctx)
