@@ -712,8 +712,8 @@ const void *epic_tc_dft(hai_ctx *ctx, int N, bool bf16) {
 
 void epic_tc_build_gather(int box_w, int box_h, const std::vector<int32_t> &cstart,
                           const std::vector<int32_t> &elem, const std::vector<float2> &w, uint32_t k_stride,
-                          uint32_t mn_stride, int F, std::vector<uint8_t> &out, int &ntile, int &nent, int &cplx,
-                          int n_warps) {
+                          uint32_t mn_stride, int F, size_t room, std::vector<uint8_t> &out, int &ntile, int &nent,
+                          int &cplx, int n_warps) {
     std::vector<int> cells, cnt((size_t)box_w * box_h, 0);
     cplx = 0;
     for (int y = 0; y < box_h; y++)
@@ -759,64 +759,84 @@ void epic_tc_build_gather(int box_w, int box_h, const std::vector<int32_t> &csta
     uint16_t *o_e = reinterpret_cast<uint16_t *>(&out[gl.off_e]);
     for (int t = 0; t <= ntile; t++) o_base[t] = base[t];
     for (int v = 0; v <= kGatherWarps; v++) o_warp[v] = wrange[v];
-    const int phase = 32 / F;                // lanes whose voltages one shared-memory phase reads
+    // Order within the lists: for every slot a lane looks through its next 16 entries,
+    // so that the cost is linear in the entries, and only when the table can be used
+    // (a host core: 256 elements at 64^2 0.10 ms, as the entries come 0.04; 1,024 at
+    // 128^2 0.63, 0.42; through all of a lane's entries 0.26 and 1.2, and 361 ms for
+    // 16,000 elements on one cell, now 1.9).
+    const int most = gl.bytes <= room ? 16 : 1;
+    const int phase = 32 / F;                // 8 or 16 lanes, whose voltages one shared-memory phase reads
+    struct Left {
+        int k, e;                            // entry, its element
+    };
+    std::vector<Left> list;                  // what the phase's lanes still have to place
+    std::vector<int> read(elem.empty() ? 0 : (size_t)*std::max_element(elem.begin(), elem.end()) + 1, 0);
+    int now = 0;                             // slot of a phase: read[e] == now if a lane reads element e in it
     for (int t = 0; t < ntile; t++)
         for (int l0 = 0; l0 < 32; l0 += phase) {
-            std::vector<std::vector<int>> left(phase);       // entries each lane still has to place
+            int head[16], end[16];
+            list.clear();
             for (int i = 0; i < phase; i++) {
                 const int ci = order[t] * 32 + l0 + i;       // cell of this lane of the tile now at position t
                 o_cell[t * 32 + l0 + i] = ci < (int)cells.size() ? a1off(cells[ci]) : 0xffffffffu;
-                if (ci >= (int)cells.size()) continue;
-                for (int k = cstart[cells[ci]]; k < cstart[cells[ci] + 1]; k++)
-                    if (w[k].x != 0.f || w[k].y != 0.f) left[i].push_back(k);
+                head[i] = (int)list.size();
+                if (ci < (int)cells.size())
+                    for (int k = cstart[cells[ci]]; k < cstart[cells[ci] + 1]; k++)
+                        if (w[k].x != 0.f || w[k].y != 0.f) list.push_back({k, elem[k]});
+                end[i] = (int)list.size();
             }
             const int ns = slots[order[t]];
             for (int s = 0; s < ns; s++) {
-                std::vector<std::vector<int>> bank(phase);   // elements already read from each bank group
+                int used[16] = {};                           // elements already read from each bank group
+                now++;
                 int any = 0;
-                std::vector<int> empty;
+                uint32_t empty = 0;
                 for (int i = 0; i < phase; i++) {
+                    Left *const mine = list.data() + head[i];
+                    const int left = end[i] - head[i], look = std::min(left, most);
                     int best = -1, cost = 1 << 30;
-                    for (int j = 0; j < (int)left[i].size(); j++) {
-                        const std::vector<int> &b = bank[elem[left[i][j]] % phase];
-                        const int c = std::find(b.begin(), b.end(), elem[left[i][j]]) != b.end() ? -1 : (int)b.size();
+                    for (int j = 0; j < look && cost >= 0; j++) {
+                        const int e = mine[j].e, c = read[e] == now ? -1 : used[e & (phase - 1)];
                         if (c < cost) {
                             cost = c;
                             best = j;
                         }
                     }
                     // a lane with slots to spare leaves one empty rather than conflict
-                    if (best < 0 || (cost > 0 && (int)left[i].size() < ns - s)) {
-                        empty.push_back(i);
+                    if (best < 0 || (cost > 0 && left < ns - s)) {
+                        empty |= 1u << i;
                         continue;
                     }
-                    const int k = left[i][best], q = base[t] + 32 * s + l0 + i;
-                    if (cost >= 0) bank[elem[k] % phase].push_back(elem[k]);
-                    o_e[q] = (uint16_t)elem[k];
+                    const int k = mine[best].k, e = mine[best].e, q = base[t] + 32 * s + l0 + i;
+                    for (int j = best; j > 0; j--) mine[j] = mine[j - 1];
+                    head[i]++;
+                    used[e & (phase - 1)] += cost >= 0;
+                    read[e] = now;
+                    o_e[q] = (uint16_t)e;
                     if (cplx) {
                         o_w[2 * q] = w[k].x;                 // conj(W~) = a + ib
                         o_w[2 * q + 1] = w[k].y;
                     } else {
                         o_w[q] = w[k].x;
                     }
-                    any = elem[k];
-                    left[i].erase(left[i].begin() + best);
+                    any = e;
                 }
-                for (int i : empty) o_e[base[t] + 32 * s + l0 + i] = (uint16_t)any;   // weight 0
+                for (int i = 0; i < phase; i++)
+                    if (empty >> i & 1) o_e[base[t] + 32 * s + l0 + i] = (uint16_t)any;   // weight 0
             }
         }
 }
 
 void epic_tc_station_table(int grid_n, int box_w, int box_h, const std::vector<int32_t> &cstart,
-                           const std::vector<int32_t> &elem, const std::vector<float2> &w, std::vector<uint8_t> &out,
-                           TcStation &rec, uint32_t &shared_bytes, long long &entries) {
+                           const std::vector<int32_t> &elem, const std::vector<float2> &w, size_t room,
+                           std::vector<uint8_t> &out, TcStation &rec, uint32_t &shared_bytes, long long &entries) {
     if (grid_n == 128) {
-        epic_tc128_build_blob(box_w, box_h, cstart, elem, w, out, shared_bytes, entries);
+        epic_tc128_build_blob(box_w, box_h, cstart, elem, w, room, out, shared_bytes, entries);
         return;
     }
     uint32_t ks, mns;
     epic_tc_a1_strides(grid_n, ks, mns);
-    epic_tc_build_gather(box_w, box_h, cstart, elem, w, ks, mns, 4, out, rec.ntile, rec.nent, rec.cplx);
+    epic_tc_build_gather(box_w, box_h, cstart, elem, w, ks, mns, 4, room, out, rec.ntile, rec.nent, rec.cplx);
     shared_bytes = (uint32_t)out.size();
     entries = rec.nent;
 }

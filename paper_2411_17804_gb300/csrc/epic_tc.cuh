@@ -200,10 +200,12 @@ __device__ __forceinline__ void cell_sum(const uint8_t *tab, const GatherLayout 
 // lands at byte tc::off_kmajor(y, 2 x, k_stride, mn_stride) of the stage-1
 // operand.
 // Entries of zero weight are left out.  F: half2 fields read per element (the
-// phase is 32 / F lanes).  n_warps (<= kGatherWarps) get tiles; the others none.
+// phase is 32 / F lanes).  room: the most bytes a kernel can keep; a larger table
+// is not ordered, as none can read it.  n_warps (<= kGatherWarps) get tiles; the
+// others none.
 void epic_tc_build_gather(int box_w, int box_h, const std::vector<int32_t> &cstart,
                           const std::vector<int32_t> &elem, const std::vector<float2> &w, uint32_t k_stride,
-                          uint32_t mn_stride, int F, std::vector<uint8_t> &out, int &ntile, int &nent, int &cplx,
+                          uint32_t mn_stride, int F, size_t room, std::vector<uint8_t> &out, int &ntile, int &nent, int &cplx,
                           int n_warps = kGatherWarps);
 
 // fp16 W'[j][l] = (-1)^j exp(+2 pi i l j / N) as a real matrix entry: row
@@ -255,12 +257,12 @@ size_t epic_tc128_smem(int ne_max, uint32_t table_max);
 // Gather table (N = 128: blob) of one station: fills the record's table fields;
 // shared_bytes = what the kernel keeps in shared memory.
 void epic_tc_station_table(int grid_n, int box_w, int box_h, const std::vector<int32_t> &cstart,
-                           const std::vector<int32_t> &elem, const std::vector<float2> &w, std::vector<uint8_t> &out,
-                           TcStation &rec, uint32_t &shared_bytes, long long &entries);
+                           const std::vector<int32_t> &elem, const std::vector<float2> &w, size_t room,
+                           std::vector<uint8_t> &out, TcStation &rec, uint32_t &shared_bytes, long long &entries);
 // Per-rank gather blob of one station for the N = 128 kernel;
 // max_rank_bytes = the largest rank table (what a CTA keeps in shared memory).
 void epic_tc128_build_blob(int box_w, int box_h, const std::vector<int32_t> &cstart,
-                           const std::vector<int32_t> &elem, const std::vector<float2> &w,
+                           const std::vector<int32_t> &elem, const std::vector<float2> &w, size_t room,
                            std::vector<uint8_t> &out, uint32_t &max_rank_bytes, long long &max_rank_entries);
 // Clusters of the N = 128 kernel resident at once (0 if it cannot run).
 int epic_tc128_max_groups(hai_ctx *ctx, int ne_max, uint32_t table_max);

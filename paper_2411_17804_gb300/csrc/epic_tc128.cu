@@ -536,7 +536,7 @@ size_t epic_tc128_smem(int ne_max, uint32_t table_max) {
 // dealt to the four ranks (largest entry count first, to the least loaded
 // rank), then one gather table per rank with the cells of its groups.
 void epic_tc128_build_blob(int box_w, int box_h, const std::vector<int32_t> &cstart,
-                           const std::vector<int32_t> &elem, const std::vector<float2> &w,
+                           const std::vector<int32_t> &elem, const std::vector<float2> &w, size_t room,
                            std::vector<uint8_t> &out, uint32_t &max_rank_bytes, long long &max_rank_entries) {
     long long cnt[8] = {0};
     for (int y = 0; y < box_h; y++)
@@ -578,7 +578,7 @@ void epic_tc128_build_blob(int box_w, int box_h, const std::vector<int32_t> &cst
                     }
                 cs[c + 1] = (int32_t)el.size();
             }
-        epic_tc_build_gather(box_w, box_h, cs, el, ww, kKs, kMNs, 2, tabs[r], hd.ntile[r], hd.nent[r], hd.cplx[r],
+        epic_tc_build_gather(box_w, box_h, cs, el, ww, kKs, kMNs, 2, room, tabs[r], hd.ntile[r], hd.nent[r], hd.cplx[r],
                              kGridWarps);
         hd.bytes[r] = (uint32_t)tabs[r].size();
         max_rank_bytes = std::max(max_rank_bytes, hd.bytes[r]);

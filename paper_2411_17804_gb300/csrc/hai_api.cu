@@ -349,7 +349,9 @@ extern "C" hai_status hai_layout_create(hai_ctx *ctx, const hai_layout_desc *d, 
         std::vector<uint8_t> tab;
         TcStation rec = {};
         uint32_t shared_bytes = 0;
-        epic_tc_station_table(n, L->box_w, L->box_h, count, elem, w, tab, rec, shared_bytes, L->tc_entries);
+        const size_t fixed = epic_tc_smem(ctx, n, ne, 0) + kStaticSmem, limit = (size_t)ctx->smem_optin;
+        epic_tc_station_table(n, L->box_w, L->box_h, count, elem, w, fixed < limit ? limit - fixed : 0, tab, rec,
+                              shared_bytes, L->tc_entries);
         L->tc_tables_bytes = shared_bytes;
         L->tc_blob_bytes = tab.size();
         e = dmalloc(&L->d_tc_tables, tab.size());
