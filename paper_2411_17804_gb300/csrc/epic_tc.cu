@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1) epic_tc_kernel(const Params p) {
             auto grid_step = [&](int i) {
                 uint8_t *A = sA1 + (i & 1) * G::kSet * G::kA1Bytes;
                 const int32_t *base = reinterpret_cast<const int32_t *>(sT + gl.off_base);
-                const int32_t *wr = reinterpret_cast<const int32_t *>(sT + gl.off_warp);
+                const uint16_t *wr = reinterpret_cast<const uint16_t *>(sT + gl.off_warp);
                 const int t1 = wr[gw + 1];
                 for (int t = wr[gw]; t < t1; t++) {
                     const uint32_t off = reinterpret_cast<const uint32_t *>(sT + gl.off_cell)[t * 32 + lane];
@@ -754,11 +754,11 @@ void epic_tc_build_gather(int box_w, int box_h, const std::vector<int32_t> &csta
     out.assign(gl.bytes, 0);
     uint32_t *o_cell = reinterpret_cast<uint32_t *>(&out[gl.off_cell]);
     int32_t *o_base = reinterpret_cast<int32_t *>(&out[gl.off_base]);
-    int32_t *o_warp = reinterpret_cast<int32_t *>(&out[gl.off_warp]);
+    uint16_t *o_warp = reinterpret_cast<uint16_t *>(&out[gl.off_warp]);
     float *o_w = reinterpret_cast<float *>(&out[gl.off_w]);
     uint16_t *o_e = reinterpret_cast<uint16_t *>(&out[gl.off_e]);
     for (int t = 0; t <= ntile; t++) o_base[t] = base[t];
-    for (int v = 0; v <= kGatherWarps; v++) o_warp[v] = wrange[v];
+    for (int v = 0; v <= kGatherWarps; v++) o_warp[v] = (uint16_t)wrange[v];
     // Order within the lists: for every slot a lane looks through its next 16 entries,
     // so that the cost is linear in the entries, and only when the table can be used
     // (a host core: 256 elements at 64^2 0.10 ms, as the entries come 0.04; 1,024 at

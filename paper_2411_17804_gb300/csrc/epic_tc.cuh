@@ -119,7 +119,7 @@ __device__ __forceinline__ int tc_count_steps(long long s0, long long s1, int T,
 //                                       stage-1 operand (field 0), or
 //                                       0xffffffff for an unused lane
 //   tile bases     int32 [ntile + 1]    first entry of each tile
-//   warp ranges    int32 [kGatherWarps + 1]  warp w grids tiles [r[w], r[w+1]);
+//   warp ranges    uint16 [kGatherWarps + 1] warp w grids tiles [r[w], r[w+1]);
 //                                       tiles are dealt to the warps by
 //                                       longest-first (slots + 2 per tile)
 //   (pad to 16)
@@ -135,7 +135,7 @@ __host__ __device__ inline GatherLayout gather_layout(int ntile, int nent, int c
     t.off_cell = 0;
     t.off_base = 4u * 32u * ntile;
     t.off_warp = t.off_base + 4u * (ntile + 1);
-    t.off_w = (t.off_warp + 4u * (kGatherWarps + 1) + 15u) & ~15u;
+    t.off_w = (t.off_warp + 2u * (kGatherWarps + 1) + 15u) & ~15u;
     t.off_e = t.off_w + (cplx ? 8u : 4u) * nent;
     t.bytes = (t.off_e + 2u * nent + 15u) & ~15u;
     return t;

@@ -247,7 +247,7 @@ __global__ void __cluster_dims__(kRanks, 1, 1) __launch_bounds__(kThreads, 1) ep
                 uint8_t *A = sA1 + (i & 1) * kA1Bytes;
                 const uint2 *E = sE + (size_t)(i & 1) * ((p.ne_max + 1) & ~1);
                 const int32_t *base = reinterpret_cast<const int32_t *>(sT + gl.off_base);
-                const int32_t *wr = reinterpret_cast<const int32_t *>(sT + gl.off_warp);
+                const uint16_t *wr = reinterpret_cast<const uint16_t *>(sT + gl.off_warp);
                 const int t1 = wr[gw + 1];
                 for (int t = wr[gw]; t < t1; t++) {
                     float2 g[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};       // X, Y
