@@ -39,7 +39,8 @@ constexpr int kThreads = 768;
 constexpr int kProd = 512;             // warps 0-15
 constexpr int kMmaWarp = 16;
 constexpr int kEpi = 128;              // warps 20-23
-constexpr int kProdRegs = 96, kMmaRegs = 32, kEpiRegs = 64;   // 4 x 96 + 32 + 64 = 6 x 80
+constexpr int kLaunchRegs = 80, kProdRegs = 96, kMmaRegs = 32, kEpiRegs = 64;
+static_assert(512 * kProdRegs + 128 * kMmaRegs + 128 * kEpiRegs <= kThreads * kLaunchRegs, "register shares");
 constexpr int kGroup = 128;            // producers of one slot
 constexpr int kItems = 8;              // (row, 16-byte group) items per producer thread and chunk
 constexpr int kItemRows = 16;          // rows between a thread's items
@@ -426,7 +427,8 @@ extern "C" hai_status hai_beamform(hai_ctx *ctx, const int8_t *volt, const int8_
     const size_t smem = kAStages * kABytes + (size_t)P * bbytes;
     if (smem > (size_t)ctx->smem_optin)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_beamform: weights of one station exceed shared memory");
-    HAI_CUDA_TRY(cudaFuncSetAttribute(bf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const hai_status ready = hai_allow_dyn_smem_regs(bf_kernel, ctx->smem_optin, kLaunchRegs);
+    if (ready != HAI_OK) return ready;
     const int pidx = prof_begin(ctx, st);
     bf_kernel<<<grid, kThreads, smem, st>>>(p);
     prof_end(ctx, pidx, st);

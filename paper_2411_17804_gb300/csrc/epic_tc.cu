@@ -525,20 +525,6 @@ size_t smem_bytes(int ne_max, uint32_t table_max) {
     return G::kOffE + 32ull * G::kU * ne_max + (size_t)kStages * vstage + table_max;
 }
 
-// Dynamic shared memory a kernel may use: the device's opt-in limit less the
-// kernel's static shared memory.
-template <typename K>
-hai_status raise_limit(hai_ctx *ctx, K kern) {
-    cudaFuncAttributes a;
-    HAI_CUDA_TRY(cudaFuncGetAttributes(&a, kern));
-    // the warpgroups' register shares have to come out of the launch's
-    if (a.numRegs < kLaunchRegs)
-        return hai_fail(HAI_ERR_UNSUPPORTED, "epic tensor cores: the kernel was built with too few registers");
-    HAI_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      ctx->smem_optin - (int)a.sharedSizeBytes));
-    return HAI_OK;
-}
-
 template <int N, bool SP, bool BF>
 hai_status run_n(hai_ctx *ctx, const TcLaunch &l, cudaStream_t st) {
     using G = Geo<N, SP>;
@@ -553,7 +539,7 @@ hai_status run_n(hai_ctx *ctx, const TcLaunch &l, cudaStream_t st) {
         if (s != HAI_OK) return s;
     }
     if (SP || BF) {
-        const hai_status s = raise_limit(ctx, epic_tc_kernel<N, SP, BF>);
+        const hai_status s = hai_allow_dyn_smem_regs(epic_tc_kernel<N, SP, BF>, ctx->smem_optin, kLaunchRegs);
         if (s != HAI_OK) return s;
     }
     Params p;
@@ -601,8 +587,8 @@ size_t epic_tc_smem(hai_ctx *, int N, int ne_max, uint32_t table_max) {
 }
 
 hai_status epic_tc_set_attr(hai_ctx *ctx, int N) {
-    if (N == 32) return raise_limit(ctx, epic_tc_kernel<32, false, false>);
-    if (N == 64) return raise_limit(ctx, epic_tc_kernel<64, false, false>);
+    if (N == 32) return hai_allow_dyn_smem_regs(epic_tc_kernel<32, false, false>, ctx->smem_optin, kLaunchRegs);
+    if (N == 64) return hai_allow_dyn_smem_regs(epic_tc_kernel<64, false, false>, ctx->smem_optin, kLaunchRegs);
     if (N == 128) return epic_tc128_set_attr(ctx);
     return HAI_OK;
 }

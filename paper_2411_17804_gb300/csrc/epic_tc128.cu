@@ -632,16 +632,8 @@ hai_status epic_tc128_run(hai_ctx *ctx, const TcLaunch &l, cudaStream_t st) {
 }
 
 hai_status epic_tc128_set_attr(hai_ctx *ctx) {
-    // the warpgroups' register shares have to come out of the launch's
-    for (auto kern : {epic_tc128_kernel<false>, epic_tc128_kernel<true>}) {
-        cudaFuncAttributes a;
-        HAI_CUDA_TRY(cudaFuncGetAttributes(&a, kern));
-        if (a.numRegs < kLaunchRegs)
-            return hai_fail(HAI_ERR_UNSUPPORTED, "epic tensor cores: the kernel was built with too few registers");
-    }
-    HAI_CUDA_TRY(hai_allow_dyn_smem(epic_tc128_kernel<false>, ctx->smem_optin));
-    HAI_CUDA_TRY(hai_allow_dyn_smem(epic_tc128_kernel<true>, ctx->smem_optin));
-    return HAI_OK;
+    const hai_status s = hai_allow_dyn_smem_regs(epic_tc128_kernel<false>, ctx->smem_optin, kLaunchRegs);
+    return s != HAI_OK ? s : hai_allow_dyn_smem_regs(epic_tc128_kernel<true>, ctx->smem_optin, kLaunchRegs);
 }
 
 // Clusters of four of this kernel that can be resident at once.

@@ -26,7 +26,7 @@ hai_status hai_cuda_fail(cudaError_t e, const char *what) {
     return HAI_ERR_CUDA;
 }
 
-// HAI_FAULT is a comma-separated list of sites ("alloc", "launch", "timeout")
+// HAI_FAULT is a comma-separated list of sites ("alloc", "launch", "registers", "timeout")
 // at which the host wrapper reports a failure without touching the GPU.
 bool hai_fault_injected(const char *site) {
     const char *env = getenv("HAI_FAULT");

@@ -125,6 +125,20 @@ inline cudaError_t hai_allow_dyn_smem(K kern, int smem_optin) {
         if (_e != cudaSuccess) return hai_cuda_fail(_e, #call);    \
     } while (0)
 
+// The same for a kernel whose warpgroups move registers (setmaxnreg): it must have
+// been built with at least the registers a thread that their shares add up to.  A
+// share beyond the launch's own is waited for without end, and no bounded wait
+// would give up.
+template <typename K>
+inline hai_status hai_allow_dyn_smem_regs(K kern, int smem_optin, int launch_regs) {
+    cudaFuncAttributes a;
+    HAI_CUDA_TRY(cudaFuncGetAttributes(&a, kern));
+    if (a.numRegs < launch_regs || hai_fault_injected("registers"))
+        return hai_fail(HAI_ERR_UNSUPPORTED, "a kernel was built with fewer registers than its warpgroups share");
+    HAI_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - (int)a.sharedSizeBytes));
+    return HAI_OK;
+}
+
 // ---------------------------------------------------------------- EPIC split
 // The (channel, sample) space is cut into n_cta contiguous ranges of the
 // flattened index c * T + t; each CTA sums its range per channel segment into
