@@ -1074,6 +1074,10 @@ hai_status launch_n(const hai_layout *L, const int8_t *volt, int C, int T, float
     float *dst = sp.direct ? img : L->d_partials;
     bool launched = false;
     const int pidx = prof_begin(L->ctx, st);
+    auto refuse = [&](hai_status s) {
+        prof_cancel(L->ctx, pidx);
+        return s;
+    };
     hai_status s = HAI_OK;
     if constexpr (N == 64)
         s = launch64<P>(volt, C, T, L->n_elem, sp, L->box_w, L->box_h, L->d_cell_start, L->d_entry_elem,
@@ -1081,12 +1085,12 @@ hai_status launch_n(const hai_layout *L, const int8_t *volt, int C, int T, float
     else
         s = launch_small<N, P>(volt, C, T, L->n_elem, sp, L->box_w, L->box_h, L->d_cell_start, L->d_entry_elem,
                                L->d_entry_w, L->nnz, dst, accumulate, optin, st, &launched);
-    if (s != HAI_OK) return s;
+    if (s != HAI_OK) return refuse(s);
     if (!launched) {
         const size_t smem = sizeof(float2) * EpicSmem<N, P>::kBuf +
                             ((size_t)kSamples * P * L->n_elem * 2 + 15) / 16 * 16;
         if (smem > (size_t)optin)
-            return hai_fail(HAI_ERR_UNSUPPORTED, "epic fp32: shared memory need exceeds the device limit");
+            return refuse(hai_fail(HAI_ERR_UNSUPPORTED, "epic fp32: shared memory need exceeds the device limit"));
         auto kern = epic_fp32_kernel<N, P>;
         HAI_CUDA_TRY(hai_allow_dyn_smem(kern, optin));
         kern<<<sp.n_cta, kThreads, smem, st>>>(volt, C, T, L->n_elem, sp.len, L->box_w, L->box_h,

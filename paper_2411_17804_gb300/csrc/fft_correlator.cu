@@ -284,9 +284,9 @@ extern "C" hai_status hai_fft_correlate(hai_ctx *ctx, const float *img, int C, i
         const size_t smem512 = sizeof(float2) * (hai_fft512::kTwFloat2 + 8 * (size_t)hai_fft512::kFftBuf);
         HAI_CUDA_TRY(hai_allow_dyn_smem(fc512_rows_kernel, ctx->smem_optin));
         HAI_CUDA_TRY(hai_allow_dyn_smem(fc512_cols_kernel, ctx->smem_optin));
-        const int pidx = prof_begin(ctx, st);
         if ((long long)C * fc512_items(P, true) > 0x7fffffffll)
             return hai_fail(HAI_ERR_UNSUPPORTED, "hai_fft_correlate: too many channels");
+        const int pidx = prof_begin(ctx, st);
         const int resident = 3 * ctx->num_sms;
         fc512_rows_kernel<<<std::min(resident, C * fc512_items(P, false)), 512, smem512, st>>>(img, P, C, out);
         fc512_cols_kernel<<<std::min(resident, C * fc512_items(P, true)), 512, smem512, st>>>(P, C, out);

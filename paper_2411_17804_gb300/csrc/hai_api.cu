@@ -153,6 +153,10 @@ void prof_end(hai_ctx *ctx, int idx, cudaStream_t st) {
     if (idx >= 0) cudaEventRecord(ctx->prof_ev[2 * idx + 1], st);
 }
 
+void prof_cancel(hai_ctx *ctx, int idx) {
+    if (idx >= 0) ctx->prof_used = (size_t)idx;
+}
+
 extern "C" hai_status hai_profile_read(hai_ctx *ctx, double *ms, long long *n_dom, long long *n_all) {
     if (!ctx || !ms || !n_dom || !n_all) return hai_fail(HAI_ERR_INVALID_ARG, "hai_profile_read: NULL argument");
     HAI_CUDA_TRY(cudaSetDevice(ctx->device));

@@ -41,9 +41,11 @@ struct hai_ctx {
 constexpr size_t kCorrWorkspaceBytes = (size_t)512 << 20;
 hai_status hai_workspace(hai_ctx *ctx);
 
-// Profiling helpers: prof_begin returns the pair index or -1.
+// Profiling helpers: prof_begin returns the pair index or -1; prof_cancel gives
+// the latest pair back when nothing was launched after all.
 int prof_begin(hai_ctx *ctx, cudaStream_t st);
 void prof_end(hai_ctx *ctx, int idx, cudaStream_t st);
+void prof_cancel(hai_ctx *ctx, int idx);
 inline void prof_count(hai_ctx *ctx, int n) { if (ctx->prof_on) ctx->prof_launches += n; }
 
 // Gather table of the gridding step: for every cell of the kernel's bounding
