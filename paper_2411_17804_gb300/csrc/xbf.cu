@@ -320,9 +320,15 @@ __global__ void __launch_bounds__(kThreads, 1) xbf_gemm_kernel(const GemmParams 
 // Pixel blocks whose row blocks go in twos: all that fill whole waves of CTAs, and
 // the others too unless their row blocks make one wave one by one.  A k block takes
 // the shared memory (128 bytes a cycle: copies in, operand reads) 768 cycles for one
-// row block and 1,280 for two.
-inline int xbf_double_blocks(int mblk, int npixblk, int sms) {
+// row block and 1,280 for two.  With an odd number the one left over runs ahead of
+// its pixel block's twos, by two fifths of the Phi block at their end; once that, over
+// the pixel blocks in flight, is more than L2 holds, Phi comes from HBM twice and all
+// go one by one (384 rows: 4,528 pairs 416 us one by one, 403 in twos; 6,109 pairs
+// 536 and 545; 12,572 pairs 1,053 and 1,067; 1,408 rows are faster in twos to the end).
+inline int xbf_double_blocks(int mblk, int npixblk, int n_kblk, int sms) {
+    constexpr double kL2 = 1.25 * 129e6;
     const int per = (mblk + 1) / 2;
+    if (mblk % 2 && 0.4 * n_kblk * kBBytes * std::min(npixblk, sms / per) > kL2) return 0;
     const int dbl = (int)((long long)npixblk * per / sms * sms / per);
     return (long long)(npixblk - dbl) * mblk <= sms ? dbl : npixblk;
 }
@@ -488,7 +494,7 @@ extern "C" hai_status hai_xbf_station_image(hai_ctx *ctx, const hai_xbf_layout *
     gp.status = ctx->d_status;
     gp.mblk = (M + kTM - 1) / kTM;
     const int npb = (int)(npix / kTN);
-    gp.dbl = xbf_double_blocks(gp.mblk, npb, ctx->num_sms);
+    gp.dbl = xbf_double_blocks(gp.mblk, npb, gp.n_kblk, ctx->num_sms);
     const int ctas = gp.dbl * ((gp.mblk + 1) / 2) + (npb - gp.dbl) * gp.mblk;
     const int pidx = prof_begin(ctx, st);
     xbf_gemm_kernel<<<ctas, kThreads, kSmem, st>>>(gp);
