@@ -106,7 +106,9 @@ __global__ void __launch_bounds__(256) corr_pack_kernel(const int8_t *__restrict
     const int a0 = jg * ge;
     const int8_t *vc = volt + (size_t)(c0 + cb) * g.T * g.P * g.ne * 2;
     const int tb = (kb0 + kb) * kKbT;
-    // load: rows (t, pol) of ge elements; 16-byte vectors where the rows allow
+    const int nj = min(kPackJ, g.nimg - jg * kPackJ);
+    // load: rows (t, pol) of the images' elements; 16-byte vectors where the rows
+    // allow
     if (vec16 && a0 + ge <= g.ne) {
         const int nv = ge / 8;                   // 8 elements per 16 bytes
         for (int i = threadIdx.x; i < kKbT * g.P * nv; i += blockDim.x) {
@@ -117,16 +119,16 @@ __global__ void __launch_bounds__(256) corr_pack_kernel(const int8_t *__restrict
             *reinterpret_cast<uint4 *>(&tile[t][pol * ge + 8 * v]) = x;
         }
     } else {
-        for (int i = threadIdx.x; i < kKbT * g.P * ge; i += blockDim.x) {
-            const int e = i % ge, tp = i / ge, t = tp / g.P, pol = tp % g.P;
-            char2 x = make_char2(0, 0);
-            if (tb + t < g.T && a0 + e < g.ne)
-                x = reinterpret_cast<const char2 *>(vc)[((size_t)(tb + t) * g.P + pol) * g.ne + a0 + e];
-            tile[t][pol * ge + e] = x;
+        // a warp per row: the images' elements only (a station of 8 fills a 64th of a group)
+        const int gu = nj * g.E, lane = threadIdx.x & 31;
+        for (int tp = threadIdx.x >> 5; tp < kKbT * g.P; tp += 8) {
+            const int t = tp / g.P, pol = tp % g.P, left = tb + t < g.T ? g.ne - a0 : 0;
+            const char2 *src = reinterpret_cast<const char2 *>(vc) + ((size_t)(tb + t) * g.P + pol) * g.ne + a0;
+#pragma unroll 4
+            for (int e = lane; e < gu; e += 32) tile[t][pol * ge + e] = e < left ? src[e] : make_char2(0, 0);
         }
     }
     __syncthreads();
-    const int nj = min(kPackJ, g.nimg - jg * kPackJ);
     const int le = g.P == 2 ? 5 : 6;             // log2 of the elements per column block
     const __half2 bias = __floats2half2_rn(1152.f, 1152.f);
     for (int i = threadIdx.x; i < nj * 512; i += blockDim.x) {
