@@ -72,23 +72,12 @@ __device__ __forceinline__ int4 load16(const int8_t *p) {
 }
 __device__ __forceinline__ void bar_prod() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
-// 16 int8 -> 16 fp16 (two 8-value K groups), exact: bits 0x6400 + (x ^ 0x80) minus 1152
+// 16 int8 -> 16 fp16 (two 8-value K groups), exact
 __device__ __forceinline__ void widen16(const int4 raw, uint4 &lo, uint4 &hi) {
-    const uint32_t w[4] = {(uint32_t)raw.x ^ 0x80808080u, (uint32_t)raw.y ^ 0x80808080u,
-                           (uint32_t)raw.z ^ 0x80808080u, (uint32_t)raw.w ^ 0x80808080u};
-    const __half2 bias = __floats2half2_rn(1152.f, 1152.f);
-    uint32_t o[8];
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const uint32_t p0 = __byte_perm(w[k], 0x64646464u, 0x4140);   // bytes 0, 1
-        const uint32_t p1 = __byte_perm(w[k], 0x64646464u, 0x4342);   // bytes 2, 3
-        __half2 h0 = __hsub2(*reinterpret_cast<const __half2 *>(&p0), bias);
-        __half2 h1 = __hsub2(*reinterpret_cast<const __half2 *>(&p1), bias);
-        o[2 * k] = *reinterpret_cast<uint32_t *>(&h0);
-        o[2 * k + 1] = *reinterpret_cast<uint32_t *>(&h1);
-    }
-    lo = make_uint4(o[0], o[1], o[2], o[3]);
-    hi = make_uint4(o[4], o[5], o[6], o[7]);
+    tc::widen4(raw.x, lo.x, lo.y);
+    tc::widen4(raw.y, lo.z, lo.w);
+    tc::widen4(raw.z, hi.x, hi.y);
+    tc::widen4(raw.w, hi.z, hi.w);
 }
 
 __device__ __forceinline__ int requant(int x, int shift, int &sat) {

@@ -542,8 +542,11 @@ hai_status epic_large_prepare(hai_layout *L) {
     e = cudaStreamCreateWithFlags(&L->large_stream, cudaStreamNonBlocking);
     for (int i = 0; i < 5 && e == cudaSuccess; i++) e = cudaEventCreateWithFlags(&L->large_ev[i], cudaEventDisableTiming);
     if (e != cudaSuccess) return hai_cuda_fail(e, "epic fp32 (large grid): stream");
-    // per-cell table of the box when no cell holds more than one gather entry
-    // (the row pass then reads element and weight in one 16-byte load)
+    // per-cell table of the box when no cell holds more than one gather entry: the
+    // row pass of boxes of at most 128 columns then keeps element and weight of its
+    // cells in registers (wider ones walk the lists: 256 x 64 cells, 2 channels x
+    // 100 samples, 240 us; 263 with a table and a block per 8 rows)
+    if (L->n_pol != 2 || L->box_w > 128) return HAI_OK;
     const int ncell = L->box_w * L->box_h;
     std::vector<int32_t> cstart(ncell + 1);
     e = cudaMemcpy(cstart.data(), L->d_cell_start, sizeof(int32_t) * (ncell + 1), cudaMemcpyDeviceToHost);
@@ -619,7 +622,7 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
         const size_t cs_smem = sizeof(float2) * (kTwFloat2 + 2 * kCols512 * (size_t)kFftBuf);
         const size_t cq_smem = sizeof(float2) * (kTwq + 2 * (kPfq * (size_t)kStageQ + kColsQ * (size_t)kXq));
         const int4 *cell_tab = static_cast<const int4 *>(L->d_large_cell);
-        const auto rows = cell_tab && L->box_w <= 128 ? large512_rows_kernel<kRpc, true> : large512_rows_kernel<kRpc, false>;
+        const auto rows = cell_tab ? large512_rows_kernel<kRpc, true> : large512_rows_kernel<kRpc, false>;
         const int row_groups = (L->box_h + kRpc - 1) / kRpc, row_ctas = std::max(1, 4 * L->ctx->num_sms / row_groups);
         HAI_CUDA_TRY(hai_allow_dyn_smem(rows, L->ctx->smem_optin));
         HAI_CUDA_TRY(hai_allow_dyn_smem(large512_cols_kernel, L->ctx->smem_optin));

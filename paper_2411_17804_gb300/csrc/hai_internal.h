@@ -75,7 +75,7 @@ struct hai_layout {
     // FP32 path of large grids (N >= 128): L2-resident row-transform scratch
     void *d_large_scratch = nullptr;
     size_t large_scratch_bytes = 0;
-    void *d_large_cell = nullptr;       // N = 512, at most one entry per cell: int4 {element, conj(W~)} per box cell
+    void *d_large_cell = nullptr;       // N = 512, P = 2, box of <= 128 columns, at most one entry per cell: int4 {element, conj(W~)} per box cell
     cudaStream_t large_stream = nullptr;   // N = 512: the row pass's stream
     cudaEvent_t large_ev[5] = {};          // rows done (2), columns done (2), fork / join
     void *d_tc_station = nullptr;
