@@ -416,8 +416,11 @@ extern "C" hai_status hai_beamform(hai_ctx *ctx, const int8_t *volt, const int8_
     const size_t smem = kAStages * kABytes + (size_t)P * bbytes;
     if (smem > (size_t)ctx->smem_optin)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_beamform: weights of one station exceed shared memory");
-    const hai_status ready = hai_allow_dyn_smem_regs(bf_kernel, ctx->smem_optin, kLaunchRegs);
-    if (ready != HAI_OK) return ready;
+    if (!ctx->bf_ready || hai_fault_injected("registers")) {      // once: both are the build's and the device's
+        const hai_status ready = hai_allow_dyn_smem_regs(bf_kernel, ctx->smem_optin, kLaunchRegs);
+        if (ready != HAI_OK) return ready;
+        ctx->bf_ready = true;
+    }
     const int pidx = prof_begin(ctx, st);
     bf_kernel<<<grid, kThreads, smem, st>>>(p);
     prof_end(ctx, pidx, st);

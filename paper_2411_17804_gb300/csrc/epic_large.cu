@@ -625,8 +625,8 @@ hai_status epic_large_launch(const hai_layout *L, const int8_t *volt, int C, int
         const auto rows = cell_tab ? large512_rows_kernel<kRpc, true> : large512_rows_kernel<kRpc, false>;
         const int row_groups = (L->box_h + kRpc - 1) / kRpc, row_ctas = std::max(1, 4 * L->ctx->num_sms / row_groups);
         HAI_CUDA_TRY(hai_allow_dyn_smem(rows, L->ctx->smem_optin));
-        HAI_CUDA_TRY(hai_allow_dyn_smem(large512_cols_kernel, L->ctx->smem_optin));
-        HAI_CUDA_TRY(hai_allow_dyn_smem(large512q_cols_kernel, L->ctx->smem_optin));
+        HAI_CUDA_TRY(L->box_h <= 128 ? hai_allow_dyn_smem(large512q_cols_kernel, L->ctx->smem_optin)
+                                     : hai_allow_dyn_smem(large512_cols_kernel, L->ctx->smem_optin));
         cudaStream_t rst = L->large_stream;
         cudaEvent_t const *ev = L->large_ev;            // 0, 1: rows done (scratch 0, 1); 2, 3: columns done; 4: fork / join
         HAI_CUDA_TRY(cudaEventRecord(ev[4], st));

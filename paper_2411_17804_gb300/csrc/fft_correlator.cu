@@ -275,10 +275,6 @@ extern "C" hai_status hai_fft_correlate(hai_ctx *ctx, const float *img, int C, i
     if (hai_fault_injected("launch")) return hai_fail(HAI_ERR_CUDA, "hai_fft_correlate: injected launch failure");
     HAI_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
-    const int np = (P == 2) ? 3 : 1;
-    const size_t smem = sizeof(float2) * ((size_t)N / 2 + (size_t)kCols * (N + 1));   // both passes
-    HAI_CUDA_TRY(hai_allow_dyn_smem(fc_rows_kernel, ctx->smem_optin));
-    HAI_CUDA_TRY(hai_allow_dyn_smem(fc_cols_kernel, ctx->smem_optin));
     float2 *out = reinterpret_cast<float2 *>(grid);
     if (N == 512) {
         const size_t smem512 = sizeof(float2) * (hai_fft512::kTwFloat2 + 8 * (size_t)hai_fft512::kFftBuf);
@@ -295,6 +291,10 @@ extern "C" hai_status hai_fft_correlate(hai_ctx *ctx, const float *img, int C, i
         HAI_CUDA_TRY(cudaGetLastError());
         return HAI_OK;
     }
+    const int np = (P == 2) ? 3 : 1;
+    const size_t smem = sizeof(float2) * ((size_t)N / 2 + (size_t)kCols * (N + 1));   // both passes
+    HAI_CUDA_TRY(hai_allow_dyn_smem(fc_rows_kernel, ctx->smem_optin));
+    HAI_CUDA_TRY(hai_allow_dyn_smem(fc_cols_kernel, ctx->smem_optin));
     const int pidx = prof_begin(ctx, st);
     fc_rows_kernel<<<dim3(C * np, (N + kThreads / 32 - 1) / (kThreads / 32)), kThreads, smem, st>>>(img, N, log2n,
                                                                                                      P, out);

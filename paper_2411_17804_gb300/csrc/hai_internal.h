@@ -5,6 +5,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -34,6 +35,7 @@ struct hai_ctx {
     void *d_stage = nullptr;
     size_t stage_bytes = 0;
     size_t dev_bytes = 0;               // other device memory the context holds (status, DFT operands)
+    std::atomic<bool> bf_ready{false};  // the beamformer's registers checked, its shared-memory limit raised
 };
 
 // Operand workspace of the correlator and the XFFT (allocated on first use by
