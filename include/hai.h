@@ -411,7 +411,8 @@ hai_status hai_correlate(hai_ctx *ctx, const int8_t *volt, int C, int T, int N, 
  * deterministic.  The first call for a layout builds (synchronously, on the
  * host and the device) the table of K_ab contributions by patches of the grid
  * (layout-only data, freed with the layout; HAI_ERR_UNSUPPORTED beyond 2e8
- * entries, i.e. N_e(N_e+1)(2K-1)^2 > 2e8); the channels are staged through
+ * entries, i.e. N_e(N_e+1)(2K-1)^2 > 2e8, or if one channel's visibilities and
+ * grids as floats exceed 512 MB); the partial sums of the channels go through
  * the context's operand workspace, so calls on one context must not run
  * concurrently on different streams.  N = 16, 32 or 64. */
 hai_status hai_xfft_image(hai_ctx *ctx, const hai_layout *layout, const int32_t *vis, int C,
@@ -482,13 +483,12 @@ typedef struct {
 } hai_vis_layout_desc;
 typedef struct hai_vis_layout hai_vis_layout;
 
-/* Build the gridding records (FP64 on the host: the 2x2 bilinear footprint of
+/* Build the gridding lists (FP64: the 2x2 bilinear footprint of
  * every station pair at uv = (r_m - r_n) / cell and of its mirror) and the
  * steering phasors exp(+2 pi i s_k.(r_m - r_n) / lambda), computed in FP64 on
  * the GPU and stored in FP32.  Pairs whose footprint, or its mirror's, leaves
  * [-N/2, N/2 - 1]^2 are dropped (hai_vis_layout_offgrid counts them).
- * HAI_ERR_UNSUPPORTED if n_pol != 2 or the station pairs' footprints exceed
- * 2^28. */
+ * HAI_ERR_UNSUPPORTED if n_pol != 2. */
 hai_status hai_vis_layout_create(hai_ctx *ctx, const hai_vis_layout_desc *desc, hai_vis_layout **out);
 void hai_vis_layout_destroy(hai_vis_layout *layout);
 /* Station pairs (unordered, autos never) dropped off the grid, per image. */

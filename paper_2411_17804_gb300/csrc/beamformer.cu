@@ -7,9 +7,9 @@
 //   D_p[t][n] = sum_kappa A_p[t][kappa] B_p[n][kappa],  kappa = (element, re/im)
 // with A_p the voltages (int8 widened to fp16, exact) and B_p the weights:
 // row n = 2k holds (w_r, w_i) per element (real part of conj(w) E), row 2k+1
-// holds (-w_i, w_r) (imaginary part).  Products are below 2^14 and an output
-// sums 2 N_e of them, so for N_e <= 512 every FP32 partial sum is an integer
-// below 2^24: exact.
+// holds (-w_i, w_r) (imaginary part).  Products are at most 2^14 in magnitude and
+// an output sums 2 N_e of them, so for N_e <= 512 every FP32 partial sum is an
+// integer of at most 2^24: exact.
 //
 // CTA = 24 warps, persistent over a contiguous range of (s, c, tile) units:
 //   warps 0-15 producers, in four groups of 4 warps: group g fills slot g of the
@@ -29,7 +29,9 @@
 // two block barriers a chunk; 739 us with 16 warps loading into registers for every
 // slot in turn; 760 us in groups, all with a warp on half lines of 8 rows; 521 us
 // with a warp on whole 128-byte lines of 4 rows.  Neighbouring units dealt to the
-// CTAs side by side instead of in ranges change stations more often: 546 us.
+// CTAs side by side instead of in ranges change stations more often: 546 us.  The
+// launch's 80 registers a thread hold for the whole kernel, so the producers (two
+// buffers of 32, the walkers) spill 112 bytes.
 #include "hai_internal.h"
 #include "tc.cuh"
 

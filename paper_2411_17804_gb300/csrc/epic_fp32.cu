@@ -2,11 +2,12 @@
 // the squaring and temporal sum of Eq. intra-station squaring), for grids of
 // N = 16, 32, 64 (larger grids: epic_large.cu).
 //
-// In both kernels here one CTA sums a contiguous range of the flattened
-// (channel, sample) index.  At N = 64 the 64-point lines are held in
-// registers by groups of 8 lanes (epic64_kernel, described below); for
-// N = 16 and 32, and as the fallback when that kernel's shared memory does not
-// fit, epic_fp32_kernel does, per group of kSamples samples:
+// In every kernel here one CTA sums a contiguous range of the flattened
+// (channel, sample) index.  The lines are held in registers, at N = 64 by groups
+// of 8 lanes (epic64_kernel) and at N = 16 and 32 by groups of 4
+// (epic_small_kernel), both described below.  Where even their forms with the
+// gather table in global memory do not fit shared memory, epic_fp32_kernel does,
+// per group of kSamples samples:
 //   1. stages the int8 voltages of the group in shared memory;
 //   2. row pass: one thread per (sample, pol, box row) gathers the gridded
 //      row sum_a conj(W~) E_a from the layout's gather table and transforms
@@ -632,7 +633,7 @@ epic64_kernel(const int8_t *__restrict__ volt, int C, int T, int ne, long long l
 //
 // These grids are latency-bound: one CTA per SM has a few samples of a short
 // cadence, so the time is the chain gather -> row -> column of a phase times
-// the number of phases.  The kernel before this one (below; one thread per
+// the number of phases.  The kernel before this one (above; one thread per
 // whole row and column, two samples per phase) left all but 32 threads idle in
 // its passes and re-walked 32 cells serially per thread.  One 64-element
 // station, one pol, 1024 samples at N = 32: 100.3 -> 18.0 us a call, with the

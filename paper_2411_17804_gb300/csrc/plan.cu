@@ -58,7 +58,8 @@ struct PlanClass {
 // N = 128 cluster.  On 96 uneven stations (32 channels, 64 samples) shares
 // from 350 + 0.5, 700 + 0.75 and 1,100 + 1.0 an entry, the last without the
 // other three SMs, kept the N = 128 class running alone for a third of a replay:
-// 5,504 us, with these 3,322 us (the three classes end within 12% of each other).
+// 5,504 us, with these 3,270 us in a process of its own (the three classes end
+// within 12% of each other) and 3,950 us in one that had run other work first.
 double model_fixed(int N) { return N == 32 ? 910.0 : N == 64 ? 1380.0 : 8500.0; }
 double model_entry(int N) { return N == 32 ? 0.05 : N == 64 ? 0.21 : 2.0; }
 

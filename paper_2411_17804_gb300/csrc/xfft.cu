@@ -421,7 +421,8 @@ extern "C" hai_status hai_xfft_image(hai_ctx *ctx, const hai_layout *L, const in
     // channels per batch: partial sums in the context's workspace
     const size_t per_chan = sizeof(float2) * (size_t)P * P * L->xfft_nchunk * kPcells;
     const int cmax = (int)std::min<size_t>({(size_t)C, ctx->corr_ws_bytes / per_chan, (size_t)32768});
-    // one channel's visibilities and grids as floats keep to the workspace's size too
+    // the interface's limit: one channel's visibilities and grids as floats would fit
+    // the workspace (the partial sums take less)
     if (cmax < 1 || sizeof(float2) * ((size_t)nbl * P * P + (size_t)(P == 2 ? 3 : 1) * N * N) > ctx->corr_ws_bytes)
         return hai_fail(HAI_ERR_UNSUPPORTED, "hai_xfft_image: one channel exceeds the workspace");
     float2 *part = static_cast<float2 *>(ctx->d_corr_ws);
